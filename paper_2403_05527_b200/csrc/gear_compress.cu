@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(128) quant_fast_kernel(CompressArgs p) {
   const SegDesc& sd = p.seg;
   const int bhl = blockIdx.y, blk = blockIdx.x, tid = threadIdx.x;
   if (tid == 0) { dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u; }
+  __syncthreads();
   const __half* X = (side == 0 ? p.K : p.V) + ((size_t)bhl * sd.n_c + (size_t)blk * L) * kHeadDim;
   float* R = p.R ? p.R + (((size_t)bhl * 2 + side) * sd.n_c + (size_t)blk * L) * kHeadDim : nullptr;
   unsigned char* rec = p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride + sd.bfac_bytes +

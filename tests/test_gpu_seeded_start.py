@@ -231,3 +231,39 @@ def test_same_inputs_give_the_same_bits_from_run_to_run():
         assert np.array_equal(runs[0][0][rep].view(np.uint32), runs[1][0][rep].view(np.uint32)), "runs differ"
     for key, arr in runs[0][1].items():
         assert np.array_equal(arr.view(np.uint8), runs[1][1][key].view(np.uint8)), key
+
+
+def test_equal_inputs_give_equal_arenas():
+    """Every byte of the compressed caches, the block headers among them (largest outlier delta and scale of a block,
+    maxima over a CTA's warps in shared memory, which gear_export does not show), is the same from run to run."""
+    import torch
+    from paper_2403_05527_b200 import binding as G, synth
+
+    dev = torch.device("cuda:0")
+    w = synth.WORKLOADS[2]
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(5)
+    k, v = (torch.randn((w.batch, w.n_kv_heads, w.n, 128), generator=gen, device=dev).half() for _ in range(2))
+    held = {}
+
+    def alloc(nbytes, _ctx):
+        t = torch.zeros(max(int(nbytes), 1), dtype=torch.uint8, device=dev)
+        held[t.data_ptr()] = t
+        return t.data_ptr()
+
+    def free(ptr, _ctx):
+        del held[ptr]
+
+    a_cb, f_cb = G.ALLOC_FN(alloc), G.FREE_FN(free)
+    cfg = G.make_config(w.batch, w.n_q_heads, w.n_kv_heads, w.bits, w.group, w.s_pct, w.buffer_cap, 0, w.n + 64)
+    arenas = []
+    G.gear_set_allocator(a_cb, f_cb)
+    try:
+        for _ in range(4):
+            cache = G.gear_compress(None, cfg, k, v, w.n, 0)
+            torch.cuda.synchronize()
+            arenas.append(max(held.values(), key=lambda t: t.numel()).clone())
+            G.gear_free(cache)
+    finally:
+        G.gear_set_allocator(None, None)
+    assert all(torch.equal(a, arenas[0]) for a in arenas)
