@@ -107,23 +107,39 @@ def strerror(status: int) -> str:
 
 
 def _ptr(t):
-    """Device / host address of a torch tensor or numpy array (None -> NULL)."""
+    """Device / host address of a torch tensor or numpy array (None -> NULL), as the plain integer that ctypes takes for
+    a pointer argument (wrapping it in a c_void_p first costs as much again as reading the address)."""
     if t is None:
         return None
     if hasattr(t, "data_ptr"):
         if not t.is_contiguous():
             raise ValueError("tensor must be contiguous")
-        return C.c_void_p(t.data_ptr())
+        return t.data_ptr()
     if not t.flags["C_CONTIGUOUS"]:
         raise ValueError("array must be contiguous")
-    return C.c_void_p(t.ctypes.data)
+    return t.ctypes.data
+
+
+def _torch_stream():
+    """Handle of torch's current stream on the current device: 0.2 us through the raw accessor, 3.5 us through the
+    torch.cuda.Stream object, which is a third of a small call's host time.  The object is the way in until CUDA is
+    initialised and where the accessor does not exist."""
+    global _raw_stream
+    import torch
+    if _raw_stream is None:
+        handle = torch.cuda.current_stream().cuda_stream
+        accessor, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if accessor is None or device is None:
+            return handle
+        _raw_stream = lambda: accessor(device())  # noqa: E731
+    return _raw_stream()
+
+
+_raw_stream = None
 
 
 def _stream(stream):
-    if stream is None:
-        import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
-    return C.c_void_p(int(stream))
+    return _torch_stream() if stream is None else int(stream)
 
 
 def make_config(batch, n_q_heads, n_kv_heads, bits, group, outlier_pct, buffer_cap, rank_flush, max_tokens,

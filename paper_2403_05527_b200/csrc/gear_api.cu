@@ -124,7 +124,7 @@ struct gear_cache {
   long long n_compressed;
   int n_blocks_c;
   // cached launch plan of the decode kernel (depends on the segments' shapes)
-  int plan_key, plan_occ;
+  long long plan_key; int plan_occ;
   DecodeArgs plan;
   int test_dead_wait;            // gear_test_dead_wait: the next decode calls wait on a barrier nothing completes
   int max_queries, units_alloc;  // query rows per head the scratch was sized for; units of that size
@@ -442,7 +442,6 @@ extern "C" gear_status gear_append_buffer(gear_cache* c, const void* k_new, cons
     return GEAR_ERR_CUDA;
   }
   c->buf_len += 1;
-  c->plan_key = -1;
   c->write_stream = st; c->write_call = next_call_number(st); c->written = true;
   if (c->buf_len < n_b) return GEAR_OK;
   gear_status s = compress_segment(c, c->buf_k, c->buf_v, n_b, c->cfg.rank_flush, B0_flush, true, st);
@@ -452,8 +451,6 @@ extern "C" gear_status gear_append_buffer(gear_cache* c, const void* k_new, cons
 }
 
 static gear_status plan_decode(gear_cache* c, int Gq) {
-  const int key = (int)c->segs.size() * 4096 + Gq;
-  if (c->plan_key == key) return GEAR_OK;
   // One-head passes: with four warps per scheduler the warps of a scheduler slow one another down by more than
   // the fourth warp adds (measured: 3 warps finish 0.85 blocks per microsecond and scheduler, 4 warps 0.79), so
   // long streams run with twelve resident warps.  Short streams (few blocks per warp) keep sixteen: there the
@@ -463,6 +460,10 @@ static gear_status plan_decode(gear_cache* c, int Gq) {
     const long long blocks = (long long)c->cc.BH * (c->n_blocks_c + (c->buf_len + 15) / 16);
     if (blocks >= 24LL * 16 * c->sm_count) warps_cap = 12;
   }
+  // everything else the plan depends on is fixed by the segments: a push that does not flush keeps it (asking the driver
+  // for the occupancy again costs a microsecond and a half per decoding step)
+  const long long key = ((long long)c->segs.size() * 4096 + Gq) * 2 + (warps_cap ? 1 : 0);
+  if (c->plan_key == key) return GEAR_OK;
   int max_k = 0, max_v = 0, max_bfac = 0, max_T = 16;
   for (const SegDesc& s : c->segs) {
     if (s.off_vpart > max_k) max_k = s.off_vpart;
@@ -470,7 +471,7 @@ static gear_status plan_decode(gear_cache* c, int Gq) {
     if (s.bfac_bytes > max_bfac) max_bfac = s.bfac_bytes;
     if ((s.T + 31) / 32 * 32 > max_T) max_T = (s.T + 31) / 32 * 32;
   }
-  if (!decode_plan(c->cc.bits, Gq, c->cc.ngv, max_k, max_v, max_bfac, max_T, 227 * 1024, warps_cap, &c->plan))
+  if (!decode_plan(c->cc.bits, Gq, c->cc.ngv, max_k, max_v, max_bfac, max_T, kDecodeSmemBudget, warps_cap, &c->plan))
     return GEAR_ERR_SHAPE;
   const int occ = decode_occupancy(c->cc.bits, Gq, c->cc.ngv, c->plan.wide, (size_t)c->plan.ws.total);
   if (occ < 1) return GEAR_ERR_CUDA;

@@ -1469,8 +1469,6 @@ cudaError_t launch_decode(const DecodeArgs& a, int grid, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   const size_t smem = (size_t)a.ws.total;
   const bool ok = with_decode_kernel(a.cc.bits, a.group_heads, a.cc.ngv, a.wide, [&](auto kern) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return;
     // Programmatic dependent launch: the CTAs of this launch may become resident while the kernel before it on the
     // stream drains (the kernel below announces that at once, and waits for its predecessor before its first read of
     // global memory), so that back-to-back decode calls do not pay the launch ramp one after the other.
@@ -1492,7 +1490,9 @@ int decode_occupancy(int bits, int heads, int ngv, int wide, size_t smem) {
   int occ = 0;
   cudaError_t e = cudaErrorInvalidValue;
   with_decode_kernel(bits, heads, ngv, wide, [&](auto kern) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // every launch is planned first, through here: the kernel may then ask for any amount (the plans of different caches
+    // differ), and the launches themselves need no attribute call
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecodeSmemBudget);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32, smem);
   });
   if (e != cudaSuccess) { cudaGetLastError(); return 0; }

@@ -131,6 +131,7 @@ int static_shape_id(const SegDesc& s, const CacheConst& c);
 // query heads one pass of the kernel takes for G query heads per kv head, and the number of passes
 inline int decode_heads_per_pass(int G) { return G == 1 ? 1 : 4; }
 inline int decode_passes(int G) { return (G + decode_heads_per_pass(G) - 1) / decode_heads_per_pass(G); }
+constexpr int kDecodeSmemBudget = 227 * 1024;    // shared memory of an SM that a launch may spread over its warps
 constexpr int kDecodeSpinLimit = 4000000;
 
 // fp16-cache attention
