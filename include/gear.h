@@ -99,7 +99,8 @@ typedef struct gear_cache gear_cache;   /* opaque */
 gear_status gear_set_allocator(gear_alloc_fn alloc_fn, gear_free_fn free_fn, void* ctx);
 
 /* Create an empty cache (no segment, empty buffer) on the current device.
- * Allocates everything the cache will ever use.  *cache must be NULL. */
+ * Allocates all the device memory the cache will ever use, without waiting for the device; the pinned host memory of the
+ * *_host calls is made by the first of them.  *cache must be NULL. */
 gear_status gear_create(gear_cache** cache, const gear_config* cfg);
 
 /* Algorithm 1, prefill body, applied to a block of n tokens: for X in {K, V}
@@ -153,7 +154,8 @@ void gear_free(gear_cache* cache);
 
 /* gear_compress takes its transient workspace (the residual of the block being compressed, up to 3 GB)
  * from a stream-ordered pool that the library keeps per device, so that repeated calls do not go back
- * to the driver.  This call synchronises the current device and returns that memory to the driver. */
+ * to the driver; the pinned rows of the *_host calls (64 MB at most) are kept the same way when a cache is freed.
+ * This call synchronises the current device and returns both kinds of memory to the driver. */
 gear_status gear_release_workspace(void);
 
 /* ---- host-buffer variants (copies inside the call) ---- */
@@ -167,21 +169,21 @@ gear_status gear_append_buffer_host(gear_cache* cache, const void* k_new_host, c
 /* gear_decode_attn with q and out in HOST memory; waits for the result (out_host is valid on return). */
 gear_status gear_decode_attn_host(gear_cache* cache, const void* q_host, float* out_host,
                                   float softmax_scale, void* stream);
-/* The same without the wait: the copies and the kernel are queued and the call returns.  q_host must stay
- * unchanged, and out_host is not valid, until gear_cache_wait(cache) has returned.  A model step queues all its
- * layers this way and then waits for each cache once.  Errors as gear_decode_attn. */
+/* The same without the wait: the kernels are queued and the call returns.  q_host must stay unchanged, and
+ * out_host is not valid, until gear_cache_wait(cache) has returned.  A model step queues all its layers this way
+ * and then waits for each cache once.  A pinned out_host is written by the attention kernel itself; a pageable one
+ * takes a copy that makes the call wait.  Errors as gear_decode_attn. */
 gear_status gear_decode_attn_host_async(gear_cache* cache, const void* q_host, float* out_host,
                                         float softmax_scale, void* stream);
 /* One decoding step of one layer through HOST buffers, queued like gear_decode_attn_host_async: the new key / value
- * rows and the query go up in one copy (through pinned memory of the library: k_new_host, v_new_host and q_host may
+ * rows and the query go up together (through pinned memory of the library: k_new_host, v_new_host and q_host may
  * be reused on return), the rows are pushed (gear_append_buffer with library-drawn start vectors if the push
  * flushes), the query attends to the cache including the new token, and the result comes down into out_host, valid
  * after gear_cache_wait(cache).  Returns GEAR_OK, GEAR_FLUSHED or an error of the two calls it combines. */
 gear_status gear_step_host(gear_cache* cache, const void* k_new_host, const void* v_new_host, const void* q_host,
                            float* out_host, float softmax_scale, void* stream);
-/* Blocks the calling host thread until the host-buffer calls queued on `cache` so far have finished: their copies
- * run on a stream of the cache's own (ordered against the caller's stream by events, so that one cache's copies run
- * beside another cache's kernels), which this call waits for.  GEAR_ERR_CUDA if that stream reports an error. */
+/* Blocks the calling host thread until the host-buffer calls queued on `cache` so far have finished.  GEAR_ERR_CUDA
+ * if the stream they ran on reports an error. */
 gear_status gear_cache_wait(gear_cache* cache);
 
 /* ---- FP16-cache reference point for the same decode step (Eq. 1 on uncompressed K, V) ---- */

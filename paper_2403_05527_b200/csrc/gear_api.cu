@@ -53,9 +53,76 @@ static cudaMemPool_t workspace_pool(int dev) {
   return g_pool[dev];
 }
 
+// Pinned rows of the host-buffer calls (a ring of kHostSlots slots with an event each).  Pinning costs up to a
+// millisecond and waits for the device, so the blocks of freed caches are kept for the next ones: at most kHostPoolBlocks
+// blocks and kHostPoolBytes in the process, given back by gear_release_workspace.
+constexpr int kHostSlots = 4;
+constexpr int kHostPoolBlocks = 64;
+constexpr size_t kHostPoolBytes = (size_t)64 << 20;
+struct HostBlock {
+  unsigned char* mem; size_t bytes; int device;
+  cudaEvent_t ev[kHostSlots];
+};
+static std::mutex g_host_mutex;
+static std::vector<HostBlock> g_host_pool;
+static size_t g_host_pool_bytes = 0;
+
+static void host_block_destroy(HostBlock& b) {
+  if (b.mem) cudaFreeHost(b.mem);
+  for (cudaEvent_t& e : b.ev)
+    if (e) cudaEventDestroy(e);
+  b.mem = nullptr;
+}
+static bool host_block_get(size_t need, int device, HostBlock* out) {
+  {
+    std::lock_guard<std::mutex> lock(g_host_mutex);
+    for (size_t i = 0; i < g_host_pool.size(); ++i) {
+      const HostBlock b = g_host_pool[i];
+      if (b.device != device || b.bytes < need || b.bytes > 4 * need + 65536) continue;
+      g_host_pool[i] = g_host_pool.back();
+      g_host_pool.pop_back();
+      g_host_pool_bytes -= b.bytes;
+      *out = b;
+      return true;
+    }
+  }
+  HostBlock b;
+  memset(&b, 0, sizeof(b));
+  b.device = device;
+  b.bytes = (need + 65535) / 65536 * 65536;
+  bool ok = cudaHostAlloc((void**)&b.mem, b.bytes, cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess;
+  for (cudaEvent_t& e : b.ev) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) { cudaGetLastError(); host_block_destroy(b); return false; }
+  *out = b;
+  return true;
+}
+static void host_block_put(HostBlock& b) {      // nothing on the device uses it any more
+  if (!b.mem) return;
+  {
+    std::lock_guard<std::mutex> lock(g_host_mutex);
+    if ((int)g_host_pool.size() < kHostPoolBlocks && g_host_pool_bytes + b.bytes <= kHostPoolBytes) {
+      g_host_pool.push_back(b);
+      g_host_pool_bytes += b.bytes;
+      b.mem = nullptr;
+      return;
+    }
+  }
+  host_block_destroy(b);
+}
+
 extern "C" gear_status gear_release_workspace(void) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
+  {
+    std::lock_guard<std::mutex> lock(g_host_mutex);
+    for (size_t i = 0; i < g_host_pool.size();) {
+      if (g_host_pool[i].device != dev) { ++i; continue; }
+      g_host_pool_bytes -= g_host_pool[i].bytes;
+      host_block_destroy(g_host_pool[i]);
+      g_host_pool[i] = g_host_pool.back();
+      g_host_pool.pop_back();
+    }
+  }
   std::lock_guard<std::mutex> lock(g_pool_mutex);
   if (dev >= 0 && dev < 64 && g_pool_ready[dev] && cudaMemPoolTrimTo(g_pool[dev], 0) != cudaSuccess) {
     cudaGetLastError();
@@ -107,16 +174,13 @@ struct gear_cache {
   void* buf_k; void* buf_v;                              // [BH][n_b][128] fp16
   unsigned char* flush_ws; size_t flush_ws_bytes;
   float* partial; size_t partial_bytes; int max_parts;
-  int* tickets; int* status;
-  void* stage_k; void* stage_v; void* stage_q; float* stage_out; float* stage_b0;   // for the *_host calls
-  // gear_append_buffer_host: pinned copies of the caller's rows, so that the call neither waits for the device nor
-  // holds on to the caller's memory.  A slot is reused once the copy that read it has finished (its event).
-  static constexpr int kHostSlots = 4;
-  unsigned char* host_ring[kHostSlots]; cudaEvent_t host_ev[kHostSlots]; bool host_used[kHostSlots]; int host_next;
-  // The host-buffer entry points copy on a stream of the cache's own, tied to the caller's stream by events, so that
-  // the copies of one cache run beside the kernels of another that shares the caller's stream.
-  cudaStream_t copy_st;
-  cudaEvent_t ev_rows_up, ev_rows_used, ev_q_up, ev_attn_done, ev_out_down;
+  int* tickets; int* status;                             // one block; zeroed on the caller's stream by the first call (scratch_clean)
+  bool scratch_clean;
+  void* stage_q; float* stage_out; float* stage_b0;      // for the *_host calls: query; result for pageable destinations; B0
+  // The *_host calls copy the caller's rows and query into a slot of a pinned ring, from which the push kernel reads them
+  // itself: no copy engine and no second stream, hence no event waits between the kernels of a step.  A slot is filled
+  // again once the call that used it four calls ago has finished (its event).
+  HostBlock host; bool host_used[kHostSlots]; int host_next, host_last;   // host_last: slot of the latest call, -1 = none
   // host state
   std::vector<SegDesc> segs;
   std::vector<long long> dbgA_off, dbgB_off;             // float offsets into dbg (or -1)
@@ -188,20 +252,50 @@ static SegDesc shape_segment(const gear_cache* c, int n_c, int rank) {
 
 extern "C" void gear_free(gear_cache* c) {
   if (!c) return;
-  if (c->copy_st) cudaStreamSynchronize(c->copy_st);      // copies queued by the host-buffer calls still use the staging rows
+  // kernels queued by the host-buffer calls still read the ring and write the caller's memory
+  if (c->host_last >= 0) cudaEventSynchronize(c->host.ev[c->host_last]);
   const DeviceAllocator& m = c->mem;
-  m.put(c->arena); m.put(c->dbg); m.put(c->table_dev); m.put(c->blk2seg); m.put(c->buf_k); m.put(c->buf_v);
-  m.put(c->flush_ws); m.put(c->partial); m.put(c->tickets); m.put(c->status);
-  m.put(c->stage_k); m.put(c->stage_out); m.put(c->stage_b0);
-  for (int i = 0; i < gear_cache::kHostSlots; ++i) {
-    if (c->host_ring[i]) cudaFreeHost(c->host_ring[i]);
-    if (c->host_ev[i]) cudaEventDestroy(c->host_ev[i]);
-  }
-  cudaEvent_t* evs[5] = {&c->ev_rows_up, &c->ev_rows_used, &c->ev_q_up, &c->ev_attn_done, &c->ev_out_down};
-  for (cudaEvent_t* e : evs)
-    if (*e) cudaEventDestroy(*e);
-  if (c->copy_st) cudaStreamDestroy(c->copy_st);
+  m.put(c->arena); m.put(c->dbg); m.put(c->table_dev); m.put(c->buf_k);
+  m.put(c->flush_ws); m.put(c->partial); m.put(c->tickets);
+  m.put(c->stage_q); m.put(c->stage_b0);
+  host_block_put(c->host);
   delete c;
+}
+
+// Next slot of the pinned ring: key rows, value rows, query.  The ring is made by the first host-buffer call: a cache that
+// lives on device buffers alone does not pay for it.
+static size_t host_row_bytes(const gear_cache* c) { return (size_t)c->cc.BH * kHeadDim * 2; }
+static size_t host_query_bytes(const gear_cache* c) { return (size_t)c->cfg.batch * c->cfg.n_q_heads * kHeadDim * 2; }
+static gear_status host_slot(gear_cache* c, unsigned char** mem, int* slot) {
+  const size_t bytes = 2 * host_row_bytes(c) + host_query_bytes(c);       // a multiple of 256
+  if (!c->host.mem && !host_block_get(bytes * kHostSlots, c->device, &c->host)) return GEAR_ERR_ALLOC;
+  const int i = c->host_next;
+  if (c->host_used[i] && cudaEventSynchronize(c->host.ev[i]) != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
+  c->host_used[i] = false;
+  c->host_next = (i + 1) % kHostSlots;
+  *mem = c->host.mem + (size_t)i * bytes;
+  *slot = i;
+  return GEAR_OK;
+}
+static bool host_slot_done(gear_cache* c, int slot, cudaStream_t st) {    // everything that uses the slot has been queued
+  if (cudaEventRecord(c->host.ev[slot], st) != cudaSuccess) { cudaGetLastError(); return false; }
+  c->host_used[slot] = true;
+  c->host_last = slot;
+  return true;
+}
+// A call that fails between taking a slot and queueing its event may have queued a reader of it.
+static gear_status host_slot_failed(gear_cache* c, int slot, cudaStream_t st, gear_status s) {
+  host_slot_done(c, slot, st);
+  return s;
+}
+
+// The merge counters and the status word start at zero on the stream of the first call that writes the cache, so that
+// creating one neither waits for the device nor orders itself against other streams.
+static bool scratch_zeroed(gear_cache* c, cudaStream_t st) {
+  if (c->scratch_clean) return true;
+  if (cudaMemsetAsync(c->tickets, 0, ((size_t)c->units_alloc + 1) * 4, st) != cudaSuccess) { cudaGetLastError(); return false; }
+  c->scratch_clean = true;
+  return true;
 }
 
 #define GEAR_TRY_ALLOC(ptr, bytes)                                                   \
@@ -228,11 +322,11 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
   c->write_stream = nullptr; c->write_call = 0; c->written = false;
   c->arena = nullptr; c->dbg = nullptr; c->table_dev = nullptr; c->blk2seg = nullptr; c->buf_k = c->buf_v = nullptr; c->flush_ws = nullptr;
   c->partial = nullptr; c->tickets = nullptr; c->status = nullptr;
-  c->stage_k = c->stage_v = c->stage_q = nullptr; c->stage_out = nullptr; c->stage_b0 = nullptr;
-  for (int i = 0; i < gear_cache::kHostSlots; ++i) { c->host_ring[i] = nullptr; c->host_ev[i] = nullptr; c->host_used[i] = false; }
-  c->host_next = 0;
-  c->copy_st = nullptr;
-  c->ev_rows_up = c->ev_rows_used = c->ev_q_up = c->ev_attn_done = c->ev_out_down = nullptr;
+  c->scratch_clean = false;
+  c->stage_q = nullptr; c->stage_out = nullptr; c->stage_b0 = nullptr;
+  memset(&c->host, 0, sizeof(c->host));
+  for (bool& u : c->host_used) u = false;
+  c->host_next = 0; c->host_last = -1;
   c->cc.bits = cfg->bits;
   c->cc.g_v = cfg->group == GEAR_GROUP_PER_VECTOR || cfg->group > kHeadDim ? kHeadDim : cfg->group;
   c->cc.ngv = kHeadDim / c->cc.g_v;
@@ -265,11 +359,11 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
   c->arena_used = 0;
   GEAR_TRY_ALLOC(c->arena, c->arena_bytes);
   c->table_cap = (int)(cfg->max_tokens / 16 + 8);
-  GEAR_TRY_ALLOC(c->table_dev, sizeof(SegDesc) * (size_t)c->table_cap);
-  c->blk_cap = (int)(cfg->max_tokens / 16 + 8);
-  GEAR_TRY_ALLOC(c->blk2seg, sizeof(int) * (size_t)c->blk_cap);
-  GEAR_TRY_ALLOC(c->buf_k, BH * n_b * kHeadDim * 2);
-  GEAR_TRY_ALLOC(c->buf_v, BH * n_b * kHeadDim * 2);
+  c->blk_cap = c->table_cap;
+  GEAR_TRY_ALLOC(c->table_dev, (sizeof(SegDesc) + sizeof(int)) * (size_t)c->table_cap);
+  c->blk2seg = reinterpret_cast<int*>(c->table_dev + c->table_cap);
+  GEAR_TRY_ALLOC(c->buf_k, 2 * BH * n_b * kHeadDim * 2);
+  c->buf_v = reinterpret_cast<__half*>(c->buf_k) + BH * n_b * kHeadDim;
   c->flush_ws_bytes = compress_workspace_bytes((int)BH, n_b, cfg->rank_flush);
   GEAR_TRY_ALLOC(c->flush_ws, c->flush_ws_bytes);
   if (cfg->flags & GEAR_FLAG_KEEP_FP32_FACTORS) {
@@ -289,37 +383,12 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
   c->max_parts = (int)(nw_max / units + 3);
   c->partial_bytes = units * c->max_parts * (size_t)hp * kPartRow * 4;
   GEAR_TRY_ALLOC(c->partial, c->partial_bytes);
-  GEAR_TRY_ALLOC(c->tickets, units * 4);
-  GEAR_TRY_ALLOC(c->status, 4);
-  cudaMemset(c->tickets, 0, units * 4);
-  cudaMemset(c->status, 0, 4);
-  const size_t tok_bytes = BH * kHeadDim * 2;
-  // key row, value row, query: one copy can bring all three (gear_step_host)
-  const size_t q_bytes = (size_t)cfg->batch * cfg->n_q_heads * kHeadDim * 2;
-  GEAR_TRY_ALLOC(c->stage_k, 2 * tok_bytes + q_bytes);
-  c->stage_v = reinterpret_cast<unsigned char*>(c->stage_k) + tok_bytes;
-  c->stage_q = reinterpret_cast<unsigned char*>(c->stage_k) + 2 * tok_bytes;
-  for (int i = 0; i < gear_cache::kHostSlots; ++i) {
-    if (cudaHostAlloc((void**)&c->host_ring[i], 2 * tok_bytes + q_bytes, cudaHostAllocDefault) != cudaSuccess ||
-        cudaEventCreateWithFlags(&c->host_ev[i], cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
-      gear_free(c);
-      return GEAR_ERR_ALLOC;
-    }
-  }
-  {
-    cudaEvent_t* evs[5] = {&c->ev_rows_up, &c->ev_rows_used, &c->ev_q_up, &c->ev_attn_done, &c->ev_out_down};
-    bool ok = cudaStreamCreateWithFlags(&c->copy_st, cudaStreamNonBlocking) == cudaSuccess;
-    for (cudaEvent_t* e : evs) ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
-    if (!ok) {
-      cudaGetLastError();
-      gear_free(c);
-      return GEAR_ERR_ALLOC;
-    }
-  }
-  GEAR_TRY_ALLOC(c->stage_out, (size_t)cfg->batch * cfg->n_q_heads * kHeadDim * 4);
+  GEAR_TRY_ALLOC(c->tickets, (units + 1) * 4);
+  c->status = c->tickets + units;
+  const size_t q_bytes = host_query_bytes(c);
+  GEAR_TRY_ALLOC(c->stage_q, 3 * q_bytes);                                // the query (fp16), then a result (fp32)
+  c->stage_out = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(c->stage_q) + q_bytes);
   GEAR_TRY_ALLOC(c->stage_b0, BH * 2 * kHeadDim * (size_t)(cfg->rank_flush > 0 ? cfg->rank_flush : 1) * 4);
-  if (cudaDeviceSynchronize() != cudaSuccess) { gear_free(c); return GEAR_ERR_CUDA; }
   *out = c;
   return GEAR_OK;
 }
@@ -361,6 +430,7 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
   job.seed = c->cfg.seed; job.segment_index = (int)c->segs.size(); job.iters = c->cfg.power_iters;
 
   cudaError_t e = cudaSuccess;
+  if (!scratch_zeroed(c, st)) return GEAR_ERR_CUDA;
   if (sd.T % 16) {     // the last slab of every block is partly empty: its codes, factor rows and scales read as zero
     if (cudaMemsetAsync(c->arena + sd.seg_base, 0, need, st) != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
     if (!compress_tile_fits(sd.T, sd.n_c, sd.rank)) return GEAR_ERR_SHAPE;
@@ -428,16 +498,19 @@ extern "C" gear_status gear_compress(gear_cache** cache, const gear_config* cfg,
   return st;
 }
 
-extern "C" gear_status gear_append_buffer(gear_cache* c, const void* k_new, const void* v_new, const float* B0_flush,
-                                          void* stream) {
-  if (!c || !k_new || !v_new) return GEAR_ERR_ARG;
-  if (((uintptr_t)k_new | (uintptr_t)v_new) & 15) return GEAR_ERR_ALIGN;
-  cudaStream_t st = (cudaStream_t)stream;
+// Push one token's rows (and bring a query along, q_src != nullptr); compresses the buffer when the push fills it.
+static gear_status push_rows(gear_cache* c, const void* k_new, const void* v_new, const void* q_src, bool host_src,
+                             const float* B0_flush, cudaStream_t st) {
   const int n_b = c->cfg.buffer_cap;
   if (c->buf_len + 1 == n_b) {     // this push will flush: make sure the segment fits before touching anything
     if (c->n_compressed + n_b > c->cfg.max_tokens || (int)c->segs.size() >= c->table_cap) return GEAR_ERR_CAPACITY;
   }
-  if (launch_append(c->buf_k, c->buf_v, k_new, v_new, c->cc.BH, n_b, c->buf_len, st) != cudaSuccess) {
+  if (!scratch_zeroed(c, st)) return GEAR_ERR_CUDA;
+  PushArgs a;
+  a.buf_k = (__half*)c->buf_k; a.buf_v = (__half*)c->buf_v; a.k_new = (const __half*)k_new; a.v_new = (const __half*)v_new;
+  a.q_src = (const __half*)q_src; a.q_dst = (__half*)c->stage_q; a.q_pieces = q_src ? (int)(host_query_bytes(c) / 16) : 0;
+  a.BH = c->cc.BH; a.n_b = n_b; a.slot = c->buf_len; a.host_src = host_src ? 1 : 0;
+  if (launch_push(a, st) != cudaSuccess) {
     cudaGetLastError();
     return GEAR_ERR_CUDA;
   }
@@ -448,6 +521,13 @@ extern "C" gear_status gear_append_buffer(gear_cache* c, const void* k_new, cons
   if (s != GEAR_OK) { c->buf_len -= 1; return s; }
   c->buf_len = 0;
   return GEAR_FLUSHED;
+}
+
+extern "C" gear_status gear_append_buffer(gear_cache* c, const void* k_new, const void* v_new, const float* B0_flush,
+                                          void* stream) {
+  if (!c || !k_new || !v_new) return GEAR_ERR_ARG;
+  if (((uintptr_t)k_new | (uintptr_t)v_new) & 15) return GEAR_ERR_ALIGN;
+  return push_rows(c, k_new, v_new, nullptr, false, B0_flush, (cudaStream_t)stream);
 }
 
 static gear_status plan_decode(gear_cache* c, int Gq) {
@@ -565,24 +645,13 @@ extern "C" gear_status gear_append_buffer_host(gear_cache* c, const void* k_host
                                                const float* B0_host, void* stream) {
   if (!c || !k_host || !v_host) return GEAR_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  const size_t tok_bytes = (size_t)c->cc.BH * kHeadDim * 2;
-  // the rows go through a pinned slot of the library's own, so the caller's memory is free again on return and
-  // nothing waits for the device (a slot is waited for only if its copy of four calls ago is still running)
-  const int slot = c->host_next;
-  c->host_next = (slot + 1) % gear_cache::kHostSlots;
-  if (c->host_used[slot] && cudaEventSynchronize(c->host_ev[slot]) != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
-  memcpy(c->host_ring[slot], k_host, tok_bytes);
-  memcpy(c->host_ring[slot] + tok_bytes, v_host, tok_bytes);
-  // copy stream: after the previous push has read the staging rows; caller's stream: after the copy
-  if (cudaStreamWaitEvent(c->copy_st, c->ev_rows_used, 0) != cudaSuccess ||
-      cudaMemcpyAsync(c->stage_k, c->host_ring[slot], 2 * tok_bytes, cudaMemcpyHostToDevice, c->copy_st) != cudaSuccess ||
-      cudaEventRecord(c->host_ev[slot], c->copy_st) != cudaSuccess ||
-      cudaEventRecord(c->ev_rows_up, c->copy_st) != cudaSuccess ||
-      cudaStreamWaitEvent(st, c->ev_rows_up, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return GEAR_ERR_CUDA;
-  }
-  c->host_used[slot] = true;
+  const size_t rows = host_row_bytes(c);
+  unsigned char* mem = nullptr;
+  int slot = 0;
+  gear_status s = host_slot(c, &mem, &slot);
+  if (s != GEAR_OK) return s;
+  memcpy(mem, k_host, rows);
+  memcpy(mem + rows, v_host, rows);
   const float* b0 = nullptr;
   const bool with_b0 = B0_host && c->cfg.rank_flush > 0 && c->buf_len + 1 == c->cfg.buffer_cap;
   if (with_b0) {
@@ -593,40 +662,49 @@ extern "C" gear_status gear_append_buffer_host(gear_cache* c, const void* k_host
     }
     b0 = c->stage_b0;
   }
-  gear_status s = gear_append_buffer(c, c->stage_k, c->stage_v, b0, stream);
-  if (s < 0) return s;
-  if (cudaEventRecord(c->ev_rows_used, st) != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
+  s = push_rows(c, mem, mem + rows, nullptr, true, b0, st);
+  if (s < 0) return host_slot_failed(c, slot, st, s);
+  if (!host_slot_done(c, slot, st)) return GEAR_ERR_CUDA;
   // the start vectors are read straight from the caller's memory: only then wait for the copy
   if (with_b0 && cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
   return s;
 }
 
-static gear_status decode_host(gear_cache* c, const void* q_host, float* out_host, float softmax_scale, void* stream,
-                               bool wait) {
-  if (!c || !q_host || !out_host) return GEAR_ERR_ARG;
-  cudaStream_t st = (cudaStream_t)stream;
-  const size_t nq = (size_t)c->cfg.batch * c->cfg.n_q_heads * kHeadDim;
-  // query up on the copy stream once the previous call's kernel has read the staging query; the kernel after that
-  // copy and after the previous call's result has left the staging output
-  if (cudaStreamWaitEvent(c->copy_st, c->ev_attn_done, 0) != cudaSuccess ||
-      cudaMemcpyAsync(c->stage_q, q_host, nq * 2, cudaMemcpyHostToDevice, c->copy_st) != cudaSuccess ||
-      cudaEventRecord(c->ev_q_up, c->copy_st) != cudaSuccess ||
-      cudaStreamWaitEvent(st, c->ev_q_up, 0) != cudaSuccess ||
-      cudaStreamWaitEvent(st, c->ev_out_down, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return GEAR_ERR_CUDA;
-  }
-  gear_status s = gear_decode_attn(c, c->stage_q, c->stage_out, softmax_scale, stream);
-  if (s != GEAR_OK) return s;
-  if (cudaEventRecord(c->ev_attn_done, st) != cudaSuccess ||
-      cudaStreamWaitEvent(c->copy_st, c->ev_attn_done, 0) != cudaSuccess ||
-      cudaMemcpyAsync(out_host, c->stage_out, nq * 4, cudaMemcpyDeviceToHost, c->copy_st) != cudaSuccess ||
-      cudaEventRecord(c->ev_out_down, c->copy_st) != cudaSuccess ||
-      (wait && cudaStreamSynchronize(c->copy_st) != cudaSuccess)) {
+// Attention for the query in stage_q into host memory.  A pinned destination is written by the kernel itself (posted
+// writes across the bus); any other goes through the device copy of the result.
+static gear_status decode_to_host(gear_cache* c, float* out_host, float softmax_scale, cudaStream_t st) {
+  cudaPointerAttributes at;
+  float* direct = nullptr;
+  if (cudaPointerGetAttributes(&at, out_host) != cudaSuccess) cudaGetLastError();
+  else if (at.type == cudaMemoryTypeHost && at.devicePointer && ((uintptr_t)at.devicePointer & 15) == 0)
+    direct = reinterpret_cast<float*>(at.devicePointer);
+  gear_status s = gear_decode_attn(c, c->stage_q, direct ? direct : c->stage_out, softmax_scale, st);
+  if (s != GEAR_OK || direct) return s;
+  if (cudaMemcpyAsync(out_host, c->stage_out, 2 * host_query_bytes(c), cudaMemcpyDeviceToHost, st) != cudaSuccess) {
     cudaGetLastError();
     return GEAR_ERR_CUDA;
   }
   return GEAR_OK;
+}
+
+static gear_status decode_host(gear_cache* c, const void* q_host, float* out_host, float softmax_scale, void* stream,
+                               bool wait) {
+  if (!c || !q_host || !out_host) return GEAR_ERR_ARG;
+  if (c->n_compressed == 0 && c->buf_len == 0) return GEAR_ERR_STATE;
+  cudaStream_t st = (cudaStream_t)stream;
+  unsigned char* mem = nullptr;
+  int slot = 0;
+  gear_status s = host_slot(c, &mem, &slot);
+  if (s != GEAR_OK) return s;
+  memcpy(mem, q_host, host_query_bytes(c));
+  PushArgs a;
+  memset(&a, 0, sizeof(a));
+  a.q_src = (const __half*)mem; a.q_dst = (__half*)c->stage_q; a.q_pieces = (int)(host_query_bytes(c) / 16); a.host_src = 1;
+  if (launch_push(a, st) != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
+  s = decode_to_host(c, out_host, softmax_scale, st);
+  if (s != GEAR_OK) return host_slot_failed(c, slot, st, s);
+  if (!host_slot_done(c, slot, st)) return GEAR_ERR_CUDA;
+  return wait ? gear_cache_wait(c) : GEAR_OK;
 }
 
 extern "C" gear_status gear_decode_attn_host(gear_cache* c, const void* q_host, float* out_host, float softmax_scale,
@@ -639,50 +717,30 @@ extern "C" gear_status gear_decode_attn_host_async(gear_cache* c, const void* q_
   return decode_host(c, q_host, out_host, softmax_scale, stream, false);
 }
 
-// One token of one layer through host buffers: push the rows, attend, all queued.  One copy up (rows and query
-// through one pinned slot), one copy down.
+// One token of one layer through host buffers: push the rows, attend, all queued; two kernels.
 extern "C" gear_status gear_step_host(gear_cache* c, const void* k_host, const void* v_host, const void* q_host,
                                       float* out_host, float softmax_scale, void* stream) {
   if (!c || !k_host || !v_host || !q_host || !out_host) return GEAR_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  const size_t tok_bytes = (size_t)c->cc.BH * kHeadDim * 2;
-  const size_t nq = (size_t)c->cfg.batch * c->cfg.n_q_heads * kHeadDim;
-  const int slot = c->host_next;
-  c->host_next = (slot + 1) % gear_cache::kHostSlots;
-  if (c->host_used[slot] && cudaEventSynchronize(c->host_ev[slot]) != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
-  memcpy(c->host_ring[slot], k_host, tok_bytes);
-  memcpy(c->host_ring[slot] + tok_bytes, v_host, tok_bytes);
-  memcpy(c->host_ring[slot] + 2 * tok_bytes, q_host, nq * 2);
-  // copy stream: after the previous push and the previous kernel have read the staging area; caller's stream: after the
-  // copy, and after the previous result has left the staging output
-  if (cudaStreamWaitEvent(c->copy_st, c->ev_rows_used, 0) != cudaSuccess ||
-      cudaStreamWaitEvent(c->copy_st, c->ev_attn_done, 0) != cudaSuccess ||
-      cudaMemcpyAsync(c->stage_k, c->host_ring[slot], 2 * tok_bytes + nq * 2, cudaMemcpyHostToDevice, c->copy_st) != cudaSuccess ||
-      cudaEventRecord(c->host_ev[slot], c->copy_st) != cudaSuccess ||
-      cudaStreamWaitEvent(st, c->host_ev[slot], 0) != cudaSuccess ||
-      cudaStreamWaitEvent(st, c->ev_out_down, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return GEAR_ERR_CUDA;
-  }
-  c->host_used[slot] = true;
-  gear_status pushed = gear_append_buffer(c, c->stage_k, c->stage_v, nullptr, stream);
-  if (pushed < 0) return pushed;
-  gear_status s = gear_decode_attn(c, c->stage_q, c->stage_out, softmax_scale, stream);
+  const size_t rows = host_row_bytes(c);
+  unsigned char* mem = nullptr;
+  int slot = 0;
+  gear_status s = host_slot(c, &mem, &slot);
   if (s != GEAR_OK) return s;
-  if (cudaEventRecord(c->ev_attn_done, st) != cudaSuccess ||
-      cudaEventRecord(c->ev_rows_used, st) != cudaSuccess ||
-      cudaStreamWaitEvent(c->copy_st, c->ev_attn_done, 0) != cudaSuccess ||
-      cudaMemcpyAsync(out_host, c->stage_out, nq * 4, cudaMemcpyDeviceToHost, c->copy_st) != cudaSuccess ||
-      cudaEventRecord(c->ev_out_down, c->copy_st) != cudaSuccess) {
-    cudaGetLastError();
-    return GEAR_ERR_CUDA;
-  }
+  memcpy(mem, k_host, rows);
+  memcpy(mem + rows, v_host, rows);
+  memcpy(mem + 2 * rows, q_host, host_query_bytes(c));
+  const gear_status pushed = push_rows(c, mem, mem + rows, mem + 2 * rows, true, nullptr, st);
+  if (pushed < 0) return host_slot_failed(c, slot, st, pushed);
+  s = decode_to_host(c, out_host, softmax_scale, st);
+  if (s != GEAR_OK) return host_slot_failed(c, slot, st, s);
+  if (!host_slot_done(c, slot, st)) return GEAR_ERR_CUDA;
   return pushed;
 }
 
 extern "C" gear_status gear_cache_wait(gear_cache* c) {
   if (!c) return GEAR_ERR_ARG;
-  if (cudaStreamSynchronize(c->copy_st) != cudaSuccess) {
+  if (c->host_last >= 0 && cudaEventSynchronize(c->host.ev[c->host_last]) != cudaSuccess) {
     cudaGetLastError();
     return GEAR_ERR_CUDA;
   }
@@ -827,6 +885,11 @@ extern "C" gear_status gear_cache_bytes(const gear_cache* c, gear_bytes* out) {
 extern "C" gear_status gear_last_device_status(gear_cache* c, int32_t* code) {
   if (!c || !code) return GEAR_ERR_ARG;
   int v = 0;
+  if (!c->scratch_clean) {                                // nothing that could have set the word has run
+    *code = 0;
+    if (cudaDeviceSynchronize() != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
+    return GEAR_OK;
+  }
   if (cudaDeviceSynchronize() != cudaSuccess || cudaMemcpy(&v, c->status, 4, cudaMemcpyDeviceToHost) != cudaSuccess ||
       cudaMemset(c->status, 0, 4) != cudaSuccess) {
     cudaGetLastError();

@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <math.h>
+#include <string.h>
 
 #include "gear_internal.cuh"
 
@@ -1630,14 +1631,33 @@ __global__ void write_desc_kernel(SegDesc* table, int* blk2seg, int index, SegDe
   for (int b = threadIdx.x; b < d.nblk; b += blockDim.x) blk2seg[d.blk_start + b] = index;
 }
 
-__global__ void append_kernel(__half* buf_k, __half* buf_v, const __half* k_new, const __half* v_new,
-                              int BH, int n_b, int slot) {
-  // one 16-byte chunk per thread: BH * 16 chunks per side
+// One decoding step's rows into the streaming buffer (and, for the host-buffer calls, the query into its device copy):
+// one 16-byte piece per thread.  With `host_src` the sources are pinned host memory that the caller filled before the
+// launch: they are read across the bus before the wait for the kernel in front, so that the round trip (2 us) runs
+// while that kernel drains; a device source may be that kernel's output and is read after the wait.  The launch is a
+// programmatic dependent of the kernel before it and keeps the rule of the decode kernel: dependents start only after
+// the own wait.
+__global__ void __launch_bounds__(256) push_kernel(PushArgs p) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= BH * 16 * 2) return;
-  const int side = i / (BH * 16), r = i % (BH * 16), bh = r >> 4, c = r & 15;
-  const uint4 v = reinterpret_cast<const uint4*>(side == 0 ? k_new : v_new)[bh * 16 + c];
-  reinterpret_cast<uint4*>(side == 0 ? buf_k : buf_v)[((size_t)bh * n_b + slot) * 16 + c] = v;
+  const int rows = p.k_new ? p.BH * 16 : 0;                // pieces per side
+  const bool mine = i < 2 * rows + p.q_pieces;
+  const uint4* src = nullptr;
+  uint4* dst = nullptr;
+  if (i < 2 * rows) {
+    const int side = i >= rows, r = side ? i - rows : i, bh = r >> 4, c = r & 15;
+    src = reinterpret_cast<const uint4*>(side == 0 ? p.k_new : p.v_new) + r;
+    dst = reinterpret_cast<uint4*>(side == 0 ? p.buf_k : p.buf_v) + ((size_t)bh * p.n_b + p.slot) * 16 + c;
+  } else if (mine) {
+    src = reinterpret_cast<const uint4*>(p.q_src) + (i - 2 * rows);
+    dst = reinterpret_cast<uint4*>(p.q_dst) + (i - 2 * rows);
+  }
+  uint4 v = make_uint4(0u, 0u, 0u, 0u);
+  if (p.host_src && mine) v = __ldcv(src);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!mine) return;
+  if (!p.host_src) v = *src;
+  *dst = v;
 }
 
 // ---------------------------------------------------------------------------
@@ -1792,13 +1812,18 @@ cudaError_t launch_write_desc(SegDesc* table, int* blk2seg, int index, const Seg
   return cudaGetLastError();
 }
 
-cudaError_t launch_append(void* buf_k, void* buf_v, const void* k_new, const void* v_new, int BH, int n_b, int slot,
-                          cudaStream_t st) {
-  const int n = BH * 16 * 2;
-  append_kernel<<<(n + 255) / 256, 256, 0, st>>>((__half*)buf_k, (__half*)buf_v, (const __half*)k_new,
-                                                 (const __half*)v_new, BH, n_b, slot);
-  count_launches(1);
-  return cudaGetLastError();
+cudaError_t launch_push(const PushArgs& a, cudaStream_t st) {
+  const int n = (a.k_new ? a.BH * 32 : 0) + a.q_pieces;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3((unsigned)((n + 255) / 256)); cfg.blockDim = dim3(256); cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, push_kernel, a);
+  if (e == cudaSuccess) count_launches(1);
+  return e;
 }
 
 }  // namespace gear

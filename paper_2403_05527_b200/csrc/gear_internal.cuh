@@ -75,8 +75,18 @@ bool compress_tile_fits(int T, int n_c, int rank);
 cudaError_t compress_tile(const CompressJob& job, int BH, cudaStream_t st);
 cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned char* ws, cudaStream_t st);
 cudaError_t launch_write_desc(SegDesc* table, int* blk2seg, int index, const SegDesc& d, cudaStream_t st);
-cudaError_t launch_append(void* buf_k, void* buf_v, const void* k_new, const void* v_new, int BH, int n_b, int slot,
-                          cudaStream_t st);
+// Rows of one decoding step into the streaming buffer and / or a query into its device copy
+struct PushArgs {
+  __half* buf_k;        // [BH][n_b][128]
+  __half* buf_v;
+  const __half* k_new;  // [BH][128], or nullptr: no rows
+  const __half* v_new;
+  const __half* q_src;  // q_pieces x 16 bytes
+  __half* q_dst;
+  int BH, n_b, slot, q_pieces;
+  int host_src;         // the sources are pinned host memory, complete before the launch
+};
+cudaError_t launch_push(const PushArgs& a, cudaStream_t st);
 
 // decode attention over the compressed cache
 constexpr int kMaxStages = 4;
