@@ -364,7 +364,8 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
   c->blk2seg = reinterpret_cast<int*>(c->table_dev + c->table_cap);
   GEAR_TRY_ALLOC(c->buf_k, 2 * BH * n_b * kHeadDim * 2);
   c->buf_v = reinterpret_cast<__half*>(c->buf_k) + BH * n_b * kHeadDim;
-  c->flush_ws_bytes = compress_workspace_bytes((int)BH, n_b, cfg->rank_flush);
+  c->flush_ws_bytes = compress_tile_fits(sf.T, n_b, cfg->rank_flush)      // flushed in one launch without a workspace
+                          ? 256 : compress_workspace_bytes((int)BH, n_b, cfg->rank_flush, c->sm_count);
   GEAR_TRY_ALLOC(c->flush_ws, c->flush_ws_bytes);
   if (cfg->flags & GEAR_FLAG_KEEP_FP32_FACTORS) {
     const size_t rm = cfg->rank_max > 0 ? cfg->rank_max : 1;
@@ -428,6 +429,7 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
   job.K = (const __half*)K; job.V = (const __half*)V; job.B0 = B0;
   job.dbgA = dbgA; job.dbgB = dbgB;
   job.seed = c->cfg.seed; job.segment_index = (int)c->segs.size(); job.iters = c->cfg.power_iters;
+  job.sms = c->sm_count; job.status = c->status;
 
   cudaError_t e = cudaSuccess;
   if (!scratch_zeroed(c, st)) return GEAR_ERR_CUDA;
@@ -442,13 +444,12 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
   } else {
     // bounded transient workspace, (batch, head) pairs processed in ranges
     const int csr_k = per_vector ? sd.csr_k : -1;
-    const size_t per_bh = compress_workspace_bytes(1, n, rank, csr_k);
     const size_t budget = (size_t)3 << 30;
-    int chunk = (int)(budget / per_bh);
-    if (chunk < 1) chunk = 1;
-    if (chunk > c->cc.BH) chunk = c->cc.BH;
+    auto bytes_of = [&](int nbh) { return compress_workspace_bytes(nbh, n, rank, c->sm_count, csr_k); };
+    int ranges = 1, chunk = c->cc.BH;
+    while (chunk > 1 && bytes_of(chunk) > budget) chunk = (c->cc.BH + ++ranges - 1) / ranges;      // equal ranges
     unsigned char* ws = nullptr;
-    const size_t ws_bytes = compress_workspace_bytes(chunk, n, rank, csr_k);
+    const size_t ws_bytes = compress_workspace_bytes(chunk, n, rank, c->sm_count, csr_k);
     cudaMemPool_t pool = workspace_pool(c->device);
     if (pool == nullptr || cudaMallocFromPoolAsync((void**)&ws, ws_bytes, pool, st) != cudaSuccess) {
       cudaGetLastError();

@@ -9,6 +9,7 @@
 #include <string.h>
 
 #include "gear_internal.cuh"
+#include "gear_pi.cuh"
 
 namespace gear {
 
@@ -778,17 +779,6 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
   return d;
 }
-// floor(log2 |x|) for a finite x > 0 (0 for x == 0): the power of two that brings x into [1, 2)
-__device__ __forceinline__ int pow2_exponent(float x) { return x > 0.f ? ilogbf(x) : 0; }
-__device__ __forceinline__ float exp2_int(int e) { return scalbnf(1.0f, e); }
-// (x0, x1) -> packed fp16 heads and packed fp16 remainders (x - head, exact in fp32 before its own rounding)
-__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uint32_t& lo) {
-  const __half2 h = __floats2half2_rn(x0, x1);
-  const float2 hf = __half22float2(h);
-  const __half2 l = __floats2half2_rn(x0 - hf.x, x1 - hf.y);
-  hi = *reinterpret_cast<const uint32_t*>(&h);
-  lo = *reinterpret_cast<const uint32_t*>(&l);
-}
 // x -> (head, remainder) packed in one register, head in the low half
 __device__ __forceinline__ void split_pair_hl(float x, uint32_t& hl) {
   const __half h = __float2half_rn(x);
@@ -800,47 +790,9 @@ __device__ __forceinline__ void split_pair_hl(float x, uint32_t& hl) {
 constexpr int kChunkRows = 512;
 constexpr int kPassWarps = 4;
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Counter-based Gaussian for library-drawn start vectors (splitmix64 + Box-Muller).
-__device__ __forceinline__ unsigned long long mix64(unsigned long long z) {
-  z += 0x9E3779B97F4A7C15ull;
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  return z ^ (z >> 31);
-}
-
-__global__ void pi_init_kernel(PiArgs p, const float* B0, int bh0, int BH_total_rank_stride,
-                               unsigned long long seed, int segment) {
-  // one thread per (tile, channel, rho); B0 layout [bh][2][128][rank]
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  const int total = p.ntiles * kHeadDim * kMaxRank;
-  if (idx >= total) return;
-  const int rho = idx % kMaxRank, ch = (idx / kMaxRank) % kHeadDim, tile = idx / (kMaxRank * kHeadDim);
-  float v = 0.f;
-  if (rho < p.rank) {
-    const size_t gtile = (size_t)bh0 * 2 + tile;
-    if (B0 != nullptr) {
-      v = B0[(gtile * kHeadDim + ch) * p.rank + rho];
-    } else {
-      const unsigned long long h = mix64(seed ^ mix64(((unsigned long long)segment << 40) ^ (gtile * 4096ull + ch * 16 + rho)));
-      const float u1 = ((float)(unsigned int)(h >> 40) + 1.0f) * (1.0f / 16777217.0f);
-      const float u2 = (float)(unsigned int)((h >> 8) & 0xFFFFFFu) * (1.0f / 16777216.0f);
-      v = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
-    }
-  }
-  p.Bcur[idx] = v;
-  (void)BH_total_rank_stride;
-}
-
-// One pass over the residual: a = R b for every row, and this chunk's partial of R^T a.
-// mode 0: loops before the last.
-// mode 1: last loop: the rows a are also stored (A0).  Its Gram matrix and the orthonormalising factor W come from
-//         the small kernels below, and since R^T (A0 W) = (R^T A0) W, with W only 16 x 16, R is not read again.
+// The last loop's pass over the residual: the rows a = R b (A0, stored), this chunk's part of R^T a, and of a^T a.  The loops
+// before it run on R^T R alone (gear_gram.cu).  The orthonormalising factor W comes from pi_finish_kernel, and since
+// R^T (A0 W) = (R^T A0) W, with W only 16 x 16, R is not read again.
 //
 // Both products run on the tensor cores (mma.sync.m16n8k16, fp16 operands, fp32 accumulation) with every fp32
 // operand cut into an fp16 head and an fp16 remainder, the four cross products summed in fp32: 22 bits of each
@@ -852,13 +804,13 @@ __global__ void pi_init_kernel(PiArgs p, const float* B0, int bh0, int BH_total_
 // transposed 8 x 8 by movmatrix, are the A fragment of R^T (rows: channels 4j, 4j+1 | 4j+2, 4j+3 of the step).
 // NT = 8-column tiles of n per CTA: one (four rank columns; three CTAs per SM) or two (eight columns, the residual is
 // converted once for both; two CTAs per SM).
-template <int MODE, int NT>
+template <int NT>
 __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kernel(PiArgs p) {
   constexpr int RP = 4 * NT;                       // rank columns per CTA: each gives a (head, remainder) column pair of n
   __shared__ float red[kHeadDim * RP];             // cross-warp sum, accumulated warp by warp
   __shared__ __align__(16) __half bsplit[2 * RP][kHeadDim];   // [2 rho + (0: head, 1: remainder)][channel]
   __shared__ float colmax[kPassWarps][RP];
-  __shared__ float gred[MODE == 1 ? kPassWarps : 1][RP][RP];   // Gram partials of the rows a (last loop, all columns here)
+  __shared__ float gred[kPassWarps][RP][RP];        // Gram partials of the rows a
   // grid (rank column groups, chunks, tiles): the CTAs that read the same chunk of R are neighbours in launch order,
   // so all but the first find it in L2
   const int tile = blockIdx.z, chunk = blockIdx.y;
@@ -908,21 +860,22 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
       const uint2 v = *reinterpret_cast<const uint2*>(&bsplit[8 * nt + gid][16 * c + 4 * t]);
       bf[c][nt][0] = v.x; bf[c][nt][1] = v.y;
     }
-  // |R sr| < 2 and |b 2^-eb| < 2, so |a| < 512 in these units: a 2^-10 stays below one half
-  constexpr float kScaleA = 1.0f / 1024.0f;
-  float inv_a[NT], inv_acc[NT];                    // back to a = R b and to R^T a for column rho = 4 nt + t
+  // The columns of a = R b have a norm of at most one (b carries that scaling), so a 2^14 fits fp16 and entries down to
+  // 2^-18 keep a remainder of full length
+  float inv_a[NT], scale_a[NT];                    // back to a for column rho = 4 nt + t, and to a 2^14
+  const float inv_acc = exp2_int(er - 14);         // back to R^T a
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) {
     int ebt = eb[4 * nt];
 #pragma unroll
     for (int q = 1; q < 4; ++q) ebt = t == q ? eb[4 * nt + q] : ebt;
     inv_a[nt] = exp2_int(er + ebt);
-    inv_acc[nt] = exp2_int(2 * er + ebt + 10);
+    scale_a[nt] = exp2_int(er + ebt + 14);
   }
 
-  // Last loop, and this CTA holds every rank column: the Gram matrix of the rows a (first round of CholeskyQR) is
-  // summed here, so that A0 is not read again for it.  gram[nt][v]: row rho = 4 nt + t of the matrix, column v.
-  const bool with_gram = MODE == 1 && gridDim.x == 1;
+  // Where this CTA holds every rank column, the Gram matrix of the rows a is summed here, so that A0 is not read again for
+  // it.  gram[nt][v]: row rho = 4 nt + t of the matrix, column v.
+  const bool with_gram = gridDim.x == 1;
   float gram[NT][RP];
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt)
@@ -964,7 +917,7 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
     }
     // B fragment of R^T a: k = row, n = (rho, head | remainder): the 8 x 8 tiles [row][2 rho + part], transposed
     uint32_t ab[NT][2];
-    if (MODE == 1 && with_gram) {
+    if (with_gram) {
       float mine[2][NT];                            // a[row gid | gid + 8][rho 4 nt + t]; rows past the chunk are zero
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
@@ -985,13 +938,11 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
       const float a_lo_rows = d[nt][0] + d[nt][1], a_hi_rows = d[nt][2] + d[nt][3];   // a[row gid | gid + 8][rho 4 nt + t], scaled
-      if (MODE == 1) {
-        if (va) A0[(size_t)ra * kMaxRank + 4 * nt + t] = a_lo_rows * inv_a[nt];
-        if (vc) A0[(size_t)rc * kMaxRank + 4 * nt + t] = a_hi_rows * inv_a[nt];
-      }
+      if (va) A0[(size_t)ra * kMaxRank + 4 * nt + t] = a_lo_rows * inv_a[nt];
+      if (vc) A0[(size_t)rc * kMaxRank + 4 * nt + t] = a_hi_rows * inv_a[nt];
       uint32_t m0, m1;
-      split_pair_hl(a_lo_rows * kScaleA, m0);
-      split_pair_hl(a_hi_rows * kScaleA, m1);
+      split_pair_hl(a_lo_rows * scale_a[nt], m0);
+      split_pair_hl(a_hi_rows * scale_a[nt], m1);
       ab[nt][0] = movmatrix_trans(m0);
       ab[nt][1] = movmatrix_trans(m1);
     }
@@ -1009,7 +960,7 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
       }
     }
   }
-  if (MODE == 1 && with_gram) {      // rows of the warp (over gid), then the warps, in a fixed order
+  if (with_gram) {      // rows of the warp (over gid), then the warps, in a fixed order
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -1017,14 +968,14 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
         float g = gram[nt][v];
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-        if (gid == 0) gred[MODE == 1 ? warp : 0][4 * nt + t][v] = g;
+        if (gid == 0) gred[warp][4 * nt + t][v] = g;
       }
     __syncthreads();
     for (int i = threadIdx.x; i < 256; i += blockDim.x) {
       const int u = i / kMaxRank, v = i % kMaxRank;
       float g = 0.f;
       if (u < RP && v < RP)
-        for (int w = 0; w < kPassWarps; ++w) g += gred[MODE == 1 ? w : 0][u][v];
+        for (int w = 0; w < kPassWarps; ++w) g += gred[w][u][v];
       p.Gp[((size_t)tile * p.nchunk + chunk) * 256 + i] = g;
     }
   }
@@ -1036,8 +987,8 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
         const int ch = 16 * c + 4 * (gid >> 1) + (gid & 1);
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
-          red[ch * RP + 4 * nt + t] += (acc[c][nt][0] + acc[c][nt][1]) * inv_acc[nt];
-          red[(ch + 2) * RP + 4 * nt + t] += (acc[c][nt][2] + acc[c][nt][3]) * inv_acc[nt];
+          red[ch * RP + 4 * nt + t] += (acc[c][nt][0] + acc[c][nt][1]) * inv_acc;
+          red[(ch + 2) * RP + 4 * nt + t] += (acc[c][nt][2] + acc[c][nt][3]) * inv_acc;
         }
       }
     }
@@ -1047,7 +998,7 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
     p.Bp[(((size_t)tile * p.nchunk + chunk) * kHeadDim + i / RP) * kMaxRank + rho0 + i % RP] = red[i];
 }
 
-// The stored A = A0 W (W = R1^-1 R2^-1 of the two CholeskyQR rounds): one thread per row.  Keys: a row is r_pad
+// The stored A = A0 W (W = U^-1 of A0's Cholesky factor): one thread per row.  Keys: a row is r_pad
 // consecutive fp16 of its slab; values: the slab is transposed ([r_pad][16 tokens]), so the threads of a slab fill
 // 32 contiguous bytes per rank index.  fp32 copy on request.
 __global__ void __launch_bounds__(256) pi_store_a_kernel(PiArgs p) {
@@ -1094,145 +1045,60 @@ __global__ void __launch_bounds__(256) pi_store_a_kernel(PiArgs p) {
   }
 }
 
-// Sum the chunk partials of R^T a into the factor buffer (fixed order).  With
-// `orth`, orthonormalise its columns (modified Gram-Schmidt, two sweeps per
-// column) -- the QR of B at the top of Algorithm 2's last loop.  With `store`,
-// write the final B as fp16 ([r_pad][128] for keys, [128][r_pad] for values).
-__global__ void __launch_bounds__(kHeadDim) pi_reduce_b_kernel(PiArgs p, int orth, int store, int apply_w) {
-  __shared__ float wsum[4];
-  const int tile = blockIdx.x, j = threadIdx.x, lane = j & 31, warp = j >> 5;
-  float b[kMaxRank];
-#pragma unroll
-  for (int r = 0; r < kMaxRank; ++r) {
+// One CTA per tile: the chunk partials of A0^T A0 and R^T A0 are summed (fixed order), W = U^-1 of the Gram matrix's
+// Cholesky factor orthonormalises A0 (its columns are nearly orthonormal already, see pi_iterate_kernel) and the final
+// factor B = (R^T A0) W is stored as fp16 ([r_pad][128] for keys, [128][r_pad] for values).
+template <int RP>
+__global__ void __launch_bounds__(kHeadDim) pi_finish_kernel(PiArgs p) {
+  __shared__ float Gm[RP][RP + 1], Wm[RP][RP + 1];
+  const int tile = blockIdx.x, j = threadIdx.x, lane = j & 31, warp = j >> 5, r = p.rank;
+  for (int e = j; e < r * r; e += kHeadDim) {
+    const float* src = p.Gp + (size_t)tile * p.nchunk * 256 + (e / r) * kMaxRank + e % r;
     float s = 0.f;
-    if (r < p.rank)
-      for (int c = 0; c < p.nchunk; ++c) s += p.Bp[(((size_t)tile * p.nchunk + c) * kHeadDim + j) * kMaxRank + r];
-    b[r] = s;
+#pragma unroll 4
+    for (int c = 0; c < p.nchunk; ++c) s += src[(size_t)c * 256];
+    Gm[e / r][e % r] = s;
   }
-  if (apply_w) {                 // the sums are R^T A0: the factor of the orthonormalised A = A0 W is (R^T A0) W
-    float bw[kMaxRank];
+  float b[RP];
 #pragma unroll
-    for (int r = 0; r < kMaxRank; ++r) {
+  for (int q = 0; q < RP; ++q) b[q] = 0.f;
+  const float4* bp = reinterpret_cast<const float4*>(p.Bp + ((size_t)tile * p.nchunk * kHeadDim + j) * kMaxRank);
+#pragma unroll 4
+  for (int c = 0; c < p.nchunk; ++c)
+#pragma unroll
+    for (int q = 0; q < RP / 4; ++q) {
+      const float4 v = bp[(size_t)c * (kHeadDim * kMaxRank / 4) + q];
+      b[4 * q] += v.x; b[4 * q + 1] += v.y; b[4 * q + 2] += v.z; b[4 * q + 3] += v.w;
+    }
+  __syncthreads();
+  if (warp == 0) warp_chol_inverse<RP, false>(&Gm[0][0], &Wm[0][0], RP + 1, r, lane);
+  __syncthreads();
+  for (int e = j; e < kMaxRank * kMaxRank; e += kHeadDim) {
+    const int u = e / kMaxRank, v = e % kMaxRank;
+    p.W[(size_t)tile * 256 + e] = u < r && v < r ? Wm[u < RP ? u : 0][v < RP ? v : 0] : 0.f;
+  }
+  const SegDesc& sd = p.seg;
+  const int bhl = tile >> 1, side = tile & 1;
+  __half* bf = reinterpret_cast<__half*>(p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride);
+#pragma unroll
+  for (int c = 0; c < RP; ++c) {
+    if (c < sd.r_pad) {
       float v = 0.f;
 #pragma unroll
-      for (int q = 0; q < kMaxRank; ++q)
-        if (q < p.rank && r < p.rank) v = fmaf(b[q], p.W[(size_t)tile * 256 + q * kMaxRank + r], v);
-      bw[r] = v;
-    }
-#pragma unroll
-    for (int r = 0; r < kMaxRank; ++r) b[r] = bw[r];
-  }
-  auto block_sum = [&](float v) {
-    v = warp_sum(v);
-    __syncthreads();
-    if (lane == 0) wsum[warp] = v;
-    __syncthreads();
-    return (wsum[0] + wsum[1]) + (wsum[2] + wsum[3]);
-  };
-  if (orth) {
-#pragma unroll
-    for (int c = 0; c < kMaxRank; ++c) {
-      if (c < p.rank) {                      // uniform over the block
-#pragma unroll
-        for (int sweep = 0; sweep < 2; ++sweep) {
-#pragma unroll
-          for (int q = 0; q < kMaxRank; ++q) {
-            if (q < c) {
-              const float d = block_sum(b[q] * b[c]);
-              b[c] = fmaf(-d, b[q], b[c]);
-            }
-          }
-        }
-        const float nrm2 = block_sum(b[c] * b[c]);
-        b[c] = nrm2 > 0.f ? b[c] * rsqrtf(nrm2) : 0.f;
-        // one Newton step on the normalisation keeps the column norm at 1 to rounding
-        const float n2 = block_sum(b[c] * b[c]);
-        if (n2 > 0.f) b[c] *= (1.5f - 0.5f * n2);
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < kMaxRank; ++r) p.Bcur[((size_t)tile * kHeadDim + j) * kMaxRank + r] = b[r];
-  if (store) {
-    const SegDesc& sd = p.seg;
-    const int bhl = tile >> 1, side = tile & 1;
-    __half* bf = reinterpret_cast<__half*>(p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride);
-#pragma unroll
-    for (int r = 0; r < kMaxRank; ++r) {
-      if (r < sd.r_pad) {
-        const __half v = __float2half_rn(r < sd.rank ? b[r] : 0.f);
-        if (side == 0) bf[r * kHeadDim + j] = v;
-        else bf[sd.r_pad * kHeadDim + j * sd.r_pad + r] = v;
-        if (p.dbgB != nullptr && r < sd.rank)
-          p.dbgB[(((size_t)(p.bh0 + bhl) * 2 + side) * kHeadDim + j) * sd.rank + r] = b[r];
-      }
+      for (int q = 0; q <= c; ++q) v = q < r && c < r ? fmaf(b[q], Wm[q][c], v) : v;
+      const __half h = __float2half_rn(v);
+      if (side == 0) bf[c * kHeadDim + j] = h;
+      else bf[sd.r_pad * kHeadDim + j * sd.r_pad + c] = h;
+      if (p.dbgB != nullptr && c < r) p.dbgB[(((size_t)(p.bh0 + bhl) * 2 + side) * kHeadDim + j) * r + c] = v;
     }
   }
 }
 
-// Gram matrix of the current A (sum of chunk partials), its Cholesky factor
-// U (G = U^T U) and U^-1.  first = 1: W <- U^-1.  first = 0: W <- W U^-1.
-// A column whose pivot vanishes (rank-deficient residual) is zeroed.
-__global__ void __launch_bounds__(32) pi_chol_kernel(PiArgs p, int first) {
-  __shared__ float G[kMaxRank][kMaxRank + 1], U[kMaxRank][kMaxRank + 1], Ui[kMaxRank][kMaxRank + 1],
-      Wo[kMaxRank][kMaxRank + 1];
-  const int tile = blockIdx.x, lane = threadIdx.x, r = p.rank;
-  for (int i = lane; i < 256; i += 32) {
-    float s = 0.f;
-    for (int c = 0; c < p.nchunk; ++c) s += p.Gp[((size_t)tile * p.nchunk + c) * 256 + i];
-    G[i / kMaxRank][i % kMaxRank] = s;
-    U[i / kMaxRank][i % kMaxRank] = 0.f;
-    Ui[i / kMaxRank][i % kMaxRank] = 0.f;
-    Wo[i / kMaxRank][i % kMaxRank] = first ? 0.f : p.W[(size_t)tile * 256 + i];
-  }
-  __syncwarp();
-  if (lane == 0) {
-    float tr = 0.f;
-    for (int i = 0; i < r; ++i) tr += G[i][i];
-    const float tiny = tr * 1e-12f;
-    for (int j = 0; j < r; ++j) {          // upper-triangular U, row by row
-      float d = G[j][j];
-      for (int k = 0; k < j; ++k) d -= U[k][j] * U[k][j];
-      const bool ok = d > tiny && d > 0.f;
-      const float ujj = ok ? sqrtf(d) : 0.f;
-      U[j][j] = ujj;
-      for (int i = j + 1; i < r; ++i) {
-        float s = G[j][i];
-        for (int k = 0; k < j; ++k) s -= U[k][j] * U[k][i];
-        U[j][i] = ok ? s / ujj : 0.f;
-      }
-    }
-    for (int c = 0; c < r; ++c) {          // U^-1 by back substitution, column by column
-      for (int i = c; i >= 0; --i) {
-        if (U[i][i] == 0.f) { Ui[i][c] = 0.f; continue; }
-        float s = (i == c) ? 1.f : 0.f;
-        for (int k = i + 1; k <= c; ++k) s -= U[i][k] * Ui[k][c];
-        Ui[i][c] = s / U[i][i];
-      }
-      if (U[c][c] == 0.f) for (int i = 0; i <= c; ++i) Ui[i][c] = 0.f;
-    }
-  }
-  __syncwarp();
-  for (int i = lane; i < 256; i += 32) {
-    const int a = i / kMaxRank, b = i % kMaxRank;
-    float v = 0.f;
-    if (a < r && b < r) {
-      if (first) v = Ui[a][b];
-      else for (int k = 0; k < r; ++k) v = fmaf(Wo[a][k], Ui[k][b], v);
-    }
-    p.W[(size_t)tile * 256 + i] = v;
-  }
-}
-
-// Gram partials of A0 W (W = identity in the first round of CholeskyQR): one thread per row.
-__global__ void __launch_bounds__(256) pi_gram2_kernel(PiArgs p, int identity) {
-  __shared__ float Wm[kMaxRank * kMaxRank];
+// Gram partials of A0 for ranks whose columns are spread over two CTAs of the pass: one thread per row.
+__global__ void __launch_bounds__(256) pi_gram2_kernel(PiArgs p) {
   __shared__ float rows[8][32][kMaxRank + 1];
   __shared__ float red[8][256];
   const int tile = blockIdx.y, chunk = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < 256; i += blockDim.x)
-    Wm[i] = identity ? (i / kMaxRank == i % kMaxRank ? 1.f : 0.f) : p.W[(size_t)tile * 256 + i];
-  __syncthreads();
   const int r = p.rank;
   const int row0 = chunk * kChunkRows, row1 = min(p.n_c, row0 + kChunkRows);
   const float* A0 = p.A0 + (size_t)tile * p.n_c * kMaxRank;
@@ -1241,18 +1107,9 @@ __global__ void __launch_bounds__(256) pi_gram2_kernel(PiArgs p, int identity) {
   for (int i = 0; i < 8; ++i) g[i] = 0.f;
   for (int base = row0 + warp * 32; base < row1; base += 8 * 32) {
     const int row = base + lane;
-    float a0[kMaxRank];
 #pragma unroll
-    for (int q = 0; q < kMaxRank; ++q) a0[q] = (row < row1 && q < r) ? A0[(size_t)row * kMaxRank + q] : 0.f;
-#pragma unroll
-    for (int c = 0; c < kMaxRank; ++c) {
-      if (c < r) {                               // uniform over the block: only the rank's columns exist
-        float s = 0.f;
-#pragma unroll
-        for (int q = 0; q < kMaxRank; ++q) s = fmaf(a0[q], Wm[q * kMaxRank + c], s);
-        rows[warp][lane][c] = s;
-      }
-    }
+    for (int q = 0; q < kMaxRank; ++q)
+      if (q < r) rows[warp][lane][q] = row < row1 ? A0[(size_t)row * kMaxRank + q] : 0.f;   // uniform: only the rank's columns exist
     __syncwarp();
     // entry (u, v) of the Gram matrix, u, v < r: pair number i * 32 + lane, so that a small rank takes one round
 #pragma unroll
@@ -1462,11 +1319,7 @@ __global__ void __launch_bounds__(128) compress_tile_kernel(TileArgs p) {
       if (p.B0 != nullptr) {
         v = p.B0[(gtile * kHeadDim + tid) * r + rho];
       } else {
-        const unsigned long long h =
-            mix64(p.seed ^ mix64(((unsigned long long)p.segment_index << 40) ^ (gtile * 4096ull + tid * 16 + rho)));
-        const float u1 = ((float)(unsigned int)(h >> 40) + 1.0f) * (1.0f / 16777217.0f);
-        const float u2 = (float)(unsigned int)((h >> 8) & 0xFFFFFFu) * (1.0f / 16777216.0f);
-        v = sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
+        v = start_value(p.seed, p.segment_index, gtile, tid, rho);
       }
     }
     b[rho] = v;
@@ -1706,21 +1559,21 @@ static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, cudaSt
   return cudaGetLastError();
 }
 
-template <int MODE>
 static void launch_pass(const PiArgs& p, cudaStream_t st) {
   // Four or eight rank columns per CTA; rank 16 is spread over two CTAs that read the same chunk of R one after the
   // other (the second finds it in L2).
-  if (p.rank <= 4) pi_pass_kernel<MODE, 1><<<dim3(1, p.nchunk, p.ntiles), kPassWarps * 32, 0, st>>>(p);
-  else pi_pass_kernel<MODE, 2><<<dim3(p.rank <= 8 ? 1 : 2, p.nchunk, p.ntiles), kPassWarps * 32, 0, st>>>(p);
+  if (p.rank <= 4) pi_pass_kernel<1><<<dim3(1, p.nchunk, p.ntiles), kPassWarps * 32, 0, st>>>(p);
+  else pi_pass_kernel<2><<<dim3(p.rank <= 8 ? 1 : 2, p.nchunk, p.ntiles), kPassWarps * 32, 0, st>>>(p);
 }
 
 // bytes of the power iteration's part of the workspace (a multiple of 256)
-static size_t pi_workspace_bytes(int nbh, int n_c, int rank) {
+static size_t pi_workspace_bytes(int nbh, int n_c, int rank, int sms) {
   if (rank == 0) return 256;
   const size_t ntiles = (size_t)nbh * 2;
   const size_t nchunk = (n_c + kChunkRows - 1) / kChunkRows;
   size_t b = 0;
   b += ntiles * n_c * kHeadDim * 4;               // R
+  b += pi_gram_workspace_bytes((int)ntiles, n_c, sms);   // Gpart
   b += ntiles * kHeadDim * kMaxRank * 4;          // Bcur
   b += ntiles * nchunk * kHeadDim * kMaxRank * 4; // Bp
   b += ntiles * n_c * kMaxRank * 4;               // A0
@@ -1731,8 +1584,8 @@ static size_t pi_workspace_bytes(int nbh, int n_c, int rank) {
 }
 
 // csr_k < 0: a segment with per-block key groups; otherwise one with per-vector keys and csr_k outliers per channel
-size_t compress_workspace_bytes(int nbh, int n_c, int rank, int csr_k) {
-  return pi_workspace_bytes(nbh, n_c, rank) + (csr_k >= 0 ? kcvt_workspace_bytes(nbh, n_c, csr_k) : 0);
+size_t compress_workspace_bytes(int nbh, int n_c, int rank, int sms, int csr_k) {
+  return pi_workspace_bytes(nbh, n_c, rank, sms) + (csr_k >= 0 ? kcvt_workspace_bytes(nbh, n_c, csr_k) : 0);
 }
 
 cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned char* ws, cudaStream_t st) {
@@ -1743,10 +1596,12 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
   PiArgs pa;
   pa.seg = sd; pa.arena = job.arena; pa.bh0 = bh0; pa.ntiles = (int)ntiles; pa.n_c = sd.n_c; pa.rank = sd.rank;
   pa.nchunk = nchunk;
-  pa.R = nullptr; pa.Rmax = nullptr; pa.Bcur = nullptr; pa.Bp = nullptr; pa.A0 = nullptr; pa.Gp = nullptr; pa.W = nullptr;
+  pa.status = job.status;
+  pa.R = nullptr; pa.Rmax = nullptr; pa.Gpart = nullptr; pa.Bcur = nullptr; pa.Bp = nullptr; pa.A0 = nullptr; pa.Gp = nullptr; pa.W = nullptr;
   pa.dbgA = job.dbgA; pa.dbgB = job.dbgB;
   if (sd.rank > 0) {
     pa.R = wsf;       wsf += ntiles * sd.n_c * kHeadDim;
+    pa.Gpart = wsf;   wsf += pi_gram_workspace_bytes((int)ntiles, sd.n_c, job.sms) / 4;
     pa.Bcur = wsf;    wsf += ntiles * kHeadDim * kMaxRank;
     pa.Bp = wsf;      wsf += ntiles * nchunk * kHeadDim * kMaxRank;
     pa.A0 = wsf;      wsf += ntiles * sd.n_c * kMaxRank;
@@ -1770,39 +1625,19 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
   if (per_vector) {
     KcvtArgs ka;
     ka.seg = sd; ka.arena = job.arena; ka.K = ca.K; ka.R = pa.R; ka.Rmax = pa.Rmax; ka.bh0 = bh0;
-    e = launch_kcvt_keys(ka, nbh, job.cc.bits, ws + pi_workspace_bytes(nbh, sd.n_c, sd.rank), st);
+    e = launch_kcvt_keys(ka, nbh, job.cc.bits, ws + pi_workspace_bytes(nbh, sd.n_c, sd.rank, job.sms), st);
     if (e != cudaSuccess) return e;
   }
   if (sd.rank == 0) return cudaSuccess;
-  // init + per early loop (pass, reduce) + last loop (pass, gram, chol, gram, chol, store, reduce)
-  count_launches(1 + 2 * (job.iters - 1) + (sd.rank > 8 ? 7 : 6) + (job.iters == 1 ? 1 : 0));
-
-  const int tot = (int)ntiles * kHeadDim * kMaxRank;
-  const float* b0 = job.B0 ? job.B0 : nullptr;
-  pi_init_kernel<<<(tot + 255) / 256, 256, 0, st>>>(pa, b0, bh0, 0, job.seed, job.segment_index);
-  for (int l = 0; l < job.iters; ++l) {
-    const bool last = l == job.iters - 1;
-    if (!last) {
-      launch_pass<0>(pa, st);                                   // A = R B ; B = R^T A
-      // the loop after this one is the last: its QR of B is folded into the reduction
-      pi_reduce_b_kernel<<<(int)ntiles, kHeadDim, 0, st>>>(pa, (l + 1 == job.iters - 1) ? 1 : 0, 0, 0);
-    } else {
-      if (job.iters == 1) {                                     // single loop: orthonormalise the start itself
-        PiArgs q = pa; q.nchunk = 0;
-        // Bp unused with zero chunks: re-use the reduce kernel on Bcur through a one-chunk view
-        cudaMemcpyAsync(pa.Bp, pa.Bcur, ntiles * kHeadDim * kMaxRank * 4, cudaMemcpyDeviceToDevice, st);
-        q.nchunk = 1;
-        pi_reduce_b_kernel<<<(int)ntiles, kHeadDim, 0, st>>>(q, 1, 0, 0);
-      }
-      launch_pass<1>(pa, st);                                   // A0 = R B, R^T A0; for ranks up to 8 also A0^T A0
-      if (sd.rank > 8) pi_gram2_kernel<<<dim3(nchunk, (int)ntiles), 256, 0, st>>>(pa, 1);
-      pi_chol_kernel<<<(int)ntiles, 32, 0, st>>>(pa, 1);        // A <- Q(A) by CholeskyQR, twice
-      pi_gram2_kernel<<<dim3(nchunk, (int)ntiles), 256, 0, st>>>(pa, 0);
-      pi_chol_kernel<<<(int)ntiles, 32, 0, st>>>(pa, 0);
-      pi_store_a_kernel<<<dim3((sd.n_c + 255) / 256, (int)ntiles), 256, 0, st>>>(pa);   // A = A0 W
-      pi_reduce_b_kernel<<<(int)ntiles, kHeadDim, 0, st>>>(pa, 0, 1, 1);
-    }
-  }
+  e = launch_pi_gram(pa, job.B0, job.seed, job.segment_index, job.iters, job.sms, st);   // the loops, B <- Q(B), its scaling
+  if (e != cudaSuccess) return e;
+  launch_pass(pa, st);                                              // A0 = R B, R^T A0; for ranks up to 8 also A0^T A0
+  if (sd.rank > 8) pi_gram2_kernel<<<dim3(nchunk, (int)ntiles), 256, 0, st>>>(pa);
+  if (sd.rank <= 4) pi_finish_kernel<4><<<(int)ntiles, kHeadDim, 0, st>>>(pa);           // W, B
+  else if (sd.rank <= 8) pi_finish_kernel<8><<<(int)ntiles, kHeadDim, 0, st>>>(pa);
+  else pi_finish_kernel<16><<<(int)ntiles, kHeadDim, 0, st>>>(pa);
+  pi_store_a_kernel<<<dim3((sd.n_c + 255) / 256, (int)ntiles), 256, 0, st>>>(pa);        // A = A0 W
+  count_launches(sd.rank > 8 ? 4 : 3);
   return cudaGetLastError();
 }
 

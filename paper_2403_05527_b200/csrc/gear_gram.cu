@@ -1,0 +1,359 @@
+// Algorithm 2 of a long segment, the loops: every loop of the power iteration multiplies by R^T R, a 128 x 128 matrix
+// whatever the length of the segment.  pi_gram_kernel sums that matrix once per tile on the tensor cores (one pass over
+// the residual instead of one per loop), pi_iterate_kernel runs the loops, the QR of B and the scaling of the last
+// factor on it, on chip.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include "gear_internal.cuh"
+#include "gear_pi.cuh"
+
+namespace gear {
+
+// ------------------------------------------------------------------ tcgen05 / mbarrier helpers
+namespace {
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void bar_init(uint64_t* b) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(b)) : "memory");
+}
+// bounded: false when the phase did not complete within the limit
+__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
+  uint32_t ok = 0;
+#pragma unroll 1
+  for (int i = 0; i < kDecodeSpinLimit && !ok; ++i)
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(smem_addr(b)), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* b) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(b)), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(dst)),
+               "l"(src), "r"(bytes), "r"(smem_addr(b)) : "memory");
+}
+__device__ __forceinline__ void umma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
+               ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void umma_commit(uint64_t* b) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(b)) : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t addr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,"
+      "%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]),
+        "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]),
+        "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(addr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+}  // namespace
+
+// ------------------------------------------------------------------ G = R^T R
+// Work: the 64-row blocks of all tiles, one after the other, cut into equal contiguous ranges, one per CTA (two CTAs per
+// SM); a CTA leaves one partial G per tile it touches.  Partial number = CTA + tile, which is different for all of them.
+constexpr int kGramRows = 64;
+constexpr int kGramStage = kGramRows * kHeadDim * 4;                // fp32 rows as they lie in memory
+constexpr int kGramOperand = kGramRows * kHeadDim * 2;              // fp16 heads or remainders of a block
+constexpr int kGramSmem = 1024 + 2 * kGramOperand + 2 * kGramStage;
+constexpr int kGramMinBlocks = 4;                                   // a partial is 64 KB, a block 32 KB: at least 256 rows per CTA
+
+struct GramSplit { int nb; long long blocks; int ctas; };
+static __host__ __device__ inline GramSplit gram_split(int ntiles, int n_c, int sms) {
+  GramSplit s;
+  s.nb = (n_c + kGramRows - 1) / kGramRows;
+  s.blocks = (long long)ntiles * s.nb;
+  const long long most = (s.blocks + kGramMinBlocks - 1) / kGramMinBlocks;
+  s.ctas = (int)(most < 2LL * sms ? most : 2LL * sms);
+  return s;
+}
+size_t pi_gram_workspace_bytes(int ntiles, int n_c, int sms) {
+  return (size_t)(gram_split(ntiles, n_c, sms).ctas + ntiles) * kHeadDim * kHeadDim * 4;
+}
+
+// Bound: the fp32 residual from HBM, once (32 KB per block; the products of a block take 12 tcgen05.mma of 128 x 128 x 16,
+// a third of the time its bytes take).  Every fp32 entry becomes an fp16 head and an fp16 remainder after exact
+// power-of-two scaling by the tile's largest magnitude; head x head, head x remainder and remainder x head are summed in
+// fp32, so 22 bits of each operand count.  The rows of a block lie in shared memory as they come ([token][channel]), which
+// is the MN-major layout for both operands: G[i][j] = sum over tokens (K) of R[k][i] R[k][j].
+__global__ void __launch_bounds__(256, 2) pi_gram_kernel(PiArgs p, int sms) {
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ uint64_t full[2], mma_done;
+  __shared__ uint32_t tmem_slot;
+  unsigned char* smem = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
+  unsigned char* op_hi = smem;                                      // [2 halves of the channels][8-token groups][8][128 B], 128B swizzle
+  unsigned char* op_lo = smem + kGramOperand;
+  unsigned char* stage = smem + 2 * kGramOperand;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const GramSplit sp = gram_split(p.ntiles, p.n_c, sms);
+  const long long f0 = blockIdx.x * sp.blocks / gridDim.x, f1 = (blockIdx.x + 1LL) * sp.blocks / gridDim.x;
+  if (tid == 0) {
+    bar_init(&full[0]); bar_init(&full[1]); bar_init(&mma_done);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(smem_addr(&tmem_slot)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+
+  auto rows_of = [&](long long f) { return min(kGramRows, p.n_c - (int)(f % sp.nb) * kGramRows); };
+  auto request = [&](long long f) {                                 // thread 0: block f into its stage
+    const int s = (int)(f - f0) & 1;
+    const long long tile = f / sp.nb;
+    const float* src = p.R + ((size_t)tile * p.n_c + (size_t)(f % sp.nb) * kGramRows) * kHeadDim;
+    bulk_load(stage + s * kGramStage, src, (uint32_t)rows_of(f) * kHeadDim * 4, &full[s]);
+  };
+  if (tid == 0) {
+    request(f0);
+    if (f0 + 1 < f1) request(f0 + 1);
+  }
+  // descriptors: 128B swizzle, 64-channel halves 8 KB apart (leading), 8-token groups 1 KB apart (stride)
+  constexpr uint64_t kDesc = ((uint64_t)(kGramOperand / 2 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+  // fp32 accumulator, fp16 operands, both MN-major, N = 128, M = 128
+  constexpr uint32_t kIdesc = (1u << 4) | (1u << 15) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+  const uint64_t d_hi = kDesc | (smem_addr(op_hi) >> 4), d_lo = kDesc | (smem_addr(op_lo) >> 4);
+
+  bool ok = true;
+  uint32_t mma_waits = 0, mma_issued = 0;
+  float sr = 0.f;
+  bool fresh = true;                                                // the accumulator holds nothing of this tile yet
+  long long f = f0;
+  for (; f < f1; ++f) {
+    const int s = (int)(f - f0) & 1, tile = (int)(f / sp.nb), rows = rows_of(f);
+    if (f == f0 || f % sp.nb == 0) sr = exp2_int(-pow2_exponent(__uint_as_float(p.Rmax[tile])));
+    ok = bar_wait(&full[s], (uint32_t)((f - f0) >> 1) & 1u) && ok;
+    while (mma_waits < mma_issued) ok = bar_wait(&mma_done, mma_waits++ & 1u) && ok;   // the operands of the block before are free
+    const float4* src = reinterpret_cast<const float4*>(stage + s * kGramStage);
+#pragma unroll
+    for (int j = 0; j < kGramRows * 32 / 256; ++j) {
+      const int i = tid + 256 * j, row = i >> 5, q = i & 31;        // four channels of a row
+      const float4 v = row < rows ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      uint32_t h0, l0, h1, l1;
+      split_pair(v.x * sr, v.y * sr, h0, l0);
+      split_pair(v.z * sr, v.w * sr, h1, l1);
+      const int at = (q >> 4) * (kGramOperand / 2) + (row >> 3) * 1024 + (row & 7) * 128 + ((((q & 15) >> 1) ^ (row & 7)) << 4) + (q & 1) * 8;
+      *reinterpret_cast<uint2*>(op_hi + at) = make_uint2(h0, h1);
+      *reinterpret_cast<uint2*>(op_lo + at) = make_uint2(l0, l1);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (__syncthreads_or(!ok)) { ok = false; break; }
+    ++mma_issued;
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+      for (int k = 0; k < kGramRows / 16; ++k) {
+        const uint64_t ah = d_hi + k * (2048 >> 4), al = d_lo + k * (2048 >> 4);
+        umma_f16(tmem, ah, ah, kIdesc, (fresh && k == 0) ? 0u : 1u);
+        umma_f16(tmem, ah, al, kIdesc, 1u);
+        umma_f16(tmem, al, ah, kIdesc, 1u);
+      }
+      umma_commit(&mma_done);
+      if (f + 2 < f1) request(f + 2);
+    }
+    fresh = false;
+    if (f + 1 == f1 || (f + 1) % sp.nb == 0) {                      // last block of the tile in this range: leave the partial
+      while (mma_waits < mma_issued) ok = bar_wait(&mma_done, mma_waits++ & 1u) && ok;
+      if (__syncthreads_or(!ok)) { ok = false; ++f; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      // G is symmetric: column c of the accumulator row i goes to row c, so that a warp writes 128 consecutive bytes
+      float* out = p.Gpart + (size_t)(blockIdx.x + tile) * kHeadDim * kHeadDim + (warp & 3) * 32 + lane;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c0 = (warp >> 2) * 64 + h * 32;
+        uint32_t v[32];
+        tmem_ld32(v, tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) out[(size_t)(c0 + c) * kHeadDim] = __uint_as_float(v[c]);
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      fresh = true;
+    }
+  }
+  if (!ok && tid == 0) {                                            // gave up (all threads): report, let the copies in flight land (bounded)
+    atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
+    for (long long g = f; g < f1 && g < f + 2; ++g) bar_wait(&full[(int)(g - f0) & 1], (uint32_t)((g - f0) >> 1) & 1u);
+  }
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem) : "memory");
+}
+
+// ------------------------------------------------------------------ the loops on G
+// One CTA per tile.  Thread (i, half) holds 64 entries of row i of G in registers; B (128 x r) is in shared memory.
+//   B <- G B, iters - 1 times (each time brought back to magnitude one by a power of two, which the QR drops again);
+//   B <- Q(B), classical Gram-Schmidt with each projection taken twice, one warp;
+//   G0 = B^T G B is the Gram matrix of A0 = R B up to rounding: U^-1 of its Cholesky factor, folded into B, makes the
+//   columns of R B nearly orthonormal before they are computed, so one explicit round of CholeskyQR is enough after.
+// Bound: latency of the chain (partials from L2, products, Gram-Schmidt, Cholesky); r^2 and 128 r work per step.
+template <int RP>
+__global__ void __launch_bounds__(256) pi_iterate_kernel(PiArgs p, const float* B0, unsigned long long seed, int segment,
+                                                         int iters, int gram_ctas, int sms) {
+  __shared__ __align__(16) float Bs[kHeadDim][RP];
+  __shared__ __align__(16) float Cs[kHeadDim][RP];
+  __shared__ float Gm[RP][RP + 1], Wm[RP][RP + 1];
+  __shared__ float wmax[4];
+  const int tile = blockIdx.x, tid = threadIdx.x, i = tid & 127, half = tid >> 7, warp = tid >> 5, lane = tid & 31;
+  const int r = p.rank;
+  float g[64];
+  {
+    const GramSplit sp = gram_split(p.ntiles, p.n_c, sms);
+    const long long NW = gram_ctas, b0 = (long long)tile * sp.nb, b1 = b0 + sp.nb;
+    const long long w0 = ((b0 + 1) * NW + sp.blocks - 1) / sp.blocks - 1, w1 = (b1 * NW + sp.blocks - 1) / sp.blocks - 1;
+#pragma unroll
+    for (int k = 0; k < 64; ++k) g[k] = 0.f;
+    for (long long w = w0; w <= w1; ++w) {
+      const float* src = p.Gpart + (size_t)(w + tile) * kHeadDim * kHeadDim + (size_t)(half * 64) * kHeadDim + i;
+#pragma unroll
+      for (int k = 0; k < 64; ++k) g[k] += __ldcg(src + k * kHeadDim);
+    }
+  }
+  if (half == 0) {
+    const size_t gtile = (size_t)p.bh0 * 2 + tile;
+#pragma unroll
+    for (int rho = 0; rho < RP; ++rho)
+      Bs[i][rho] = rho < r ? (B0 ? B0[(gtile * kHeadDim + i) * r + rho] : start_value(seed, segment, gtile, i, rho)) : 0.f;
+  }
+  __syncthreads();
+  float c[RP];
+  auto times_g = [&]() {                          // c = (G B) row i: half 0 holds the sum of both halves
+#pragma unroll
+    for (int rho = 0; rho < RP; ++rho) c[rho] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 64; ++k)
+#pragma unroll
+      for (int q = 0; q < RP / 4; ++q) {
+        const float4 b = *reinterpret_cast<const float4*>(&Bs[half * 64 + k][4 * q]);
+        c[4 * q] = fmaf(g[k], b.x, c[4 * q]);
+        c[4 * q + 1] = fmaf(g[k], b.y, c[4 * q + 1]);
+        c[4 * q + 2] = fmaf(g[k], b.z, c[4 * q + 2]);
+        c[4 * q + 3] = fmaf(g[k], b.w, c[4 * q + 3]);
+      }
+    if (half == 1) {
+#pragma unroll
+      for (int rho = 0; rho < RP; ++rho) Cs[i][rho] = c[rho];
+    }
+    __syncthreads();
+    if (half == 0) {
+#pragma unroll
+      for (int rho = 0; rho < RP; ++rho) c[rho] += Cs[i][rho];
+    }
+  };
+  for (int l = 0; l + 1 < iters; ++l) {
+    times_g();
+    float m = 0.f;
+    if (half == 0) {
+#pragma unroll
+      for (int rho = 0; rho < RP; ++rho) m = fmaxf(m, fabsf(c[rho]));
+      m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+      if (lane == 0) wmax[warp] = m;
+    }
+    __syncthreads();
+    if (half == 0) {
+      const float sc = exp2_int(-pow2_exponent(fmaxf(fmaxf(wmax[0], wmax[1]), fmaxf(wmax[2], wmax[3]))));
+#pragma unroll
+      for (int rho = 0; rho < RP; ++rho) Bs[i][rho] = c[rho] * sc;
+    }
+    __syncthreads();
+  }
+  if (warp == 0) {                                // B <- Q(B)
+    float b[4][RP];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int rho = 0; rho < RP; ++rho) b[j][rho] = Bs[lane + 32 * j][rho];
+#pragma unroll
+    for (int cc = 0; cc < RP; ++cc) {
+      if (cc < r) {
+#pragma unroll
+        for (int sweep = 0; sweep < 2; ++sweep) {
+          float d[RP];
+#pragma unroll
+          for (int q = 0; q < cc; ++q) {
+            d[q] = 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) d[q] = fmaf(b[j][q], b[j][cc], d[q]);
+          }
+#pragma unroll
+          for (int q = 0; q < cc; ++q) d[q] = warp_sum(d[q]);
+#pragma unroll
+          for (int q = 0; q < cc; ++q)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b[j][cc] = fmaf(-d[q], b[j][q], b[j][cc]);
+        }
+        auto norm2 = [&]() {
+          float s = 0.f;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) s = fmaf(b[j][cc], b[j][cc], s);
+          return warp_sum(s);
+        };
+        const float nrm2 = norm2();
+        const float inv = nrm2 > 0.f ? rsqrtf(nrm2) : 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[j][cc] *= inv;
+        const float n2 = norm2();                 // one Newton step keeps the column norm at 1 to rounding
+        const float fix = n2 > 0.f ? 1.5f - 0.5f * n2 : 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) b[j][cc] *= fix;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int rho = 0; rho < RP; ++rho) Bs[lane + 32 * j][rho] = b[j][rho];
+  }
+  __syncthreads();
+  times_g();
+  __syncthreads();
+  if (half == 0) {
+#pragma unroll
+    for (int rho = 0; rho < RP; ++rho) Cs[i][rho] = c[rho];
+  }
+  __syncthreads();
+  for (int e = warp; e < r * r; e += 8) {
+    const int u = e / r, v = e % r;
+    float s = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s = fmaf(Bs[lane + 32 * j][u], Cs[lane + 32 * j][v], s);
+    s = warp_sum(s);
+    if (lane == 0) Gm[u][v] = s;
+  }
+  __syncthreads();
+  if (warp == 0) warp_chol_inverse<RP, true>(&Gm[0][0], &Wm[0][0], RP + 1, r, lane);
+  __syncthreads();
+  if (half == 0) {
+    // G was summed over R 2^-er, so the columns of R (B W) would have norm 2^er
+    const float down = exp2_int(-pow2_exponent(__uint_as_float(p.Rmax[tile])));
+    float* out = p.Bcur + ((size_t)tile * kHeadDim + i) * kMaxRank;
+#pragma unroll
+    for (int rho = 0; rho < kMaxRank; ++rho) {
+      float v = 0.f;
+      if (rho < RP && rho < r) {
+#pragma unroll
+        for (int q = 0; q < RP; ++q)
+          if (q <= rho && q < r) v = fmaf(Bs[i][q], Wm[q][rho < RP ? rho : 0], v);
+      }
+      out[rho] = v * down;
+    }
+  }
+}
+
+cudaError_t launch_pi_gram(const PiArgs& p, const float* B0, unsigned long long seed, int segment, int iters, int sms,
+                           cudaStream_t st) {
+  const GramSplit sp = gram_split(p.ntiles, p.n_c, sms);
+  cudaError_t e = cudaFuncSetAttribute(pi_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramSmem);
+  if (e != cudaSuccess) return e;
+  pi_gram_kernel<<<sp.ctas, 256, kGramSmem, st>>>(p, sms);
+  if (p.rank <= 4) pi_iterate_kernel<4><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters, sp.ctas, sms);
+  else if (p.rank <= 8) pi_iterate_kernel<8><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters, sp.ctas, sms);
+  else pi_iterate_kernel<16><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters, sp.ctas, sms);
+  count_launches(2);
+  return cudaGetLastError();
+}
+
+}  // namespace gear

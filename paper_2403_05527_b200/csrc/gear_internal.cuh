@@ -45,6 +45,8 @@ struct PiArgs {
   unsigned char* arena;
   float* R;             // [ntiles][n_c][128]
   unsigned int* Rmax;   // [ntiles] bit pattern of the tile's largest |R|
+  float* Gpart;         // partials of R^T R, [CTA + tile][128][128] (gear_gram.cu)
+  int* status;          // the cache's status word
   float* Bcur;          // [ntiles][128][16]
   float* Bp;            // [ntiles][nchunk][128][16]
   float* A0;            // [ntiles][n_c][16]
@@ -67,9 +69,15 @@ struct CompressJob {
   unsigned long long seed;
   int segment_index;
   int iters;
+  int sms;
+  int* status;
 };
 
-size_t compress_workspace_bytes(int nbh, int n_c, int rank, int csr_k = -1);
+size_t compress_workspace_bytes(int nbh, int n_c, int rank, int sms, int csr_k = -1);
+// R^T R of every tile, then everything of Algorithm 2 that runs on it: leaves the last loop's factor in p.Bcur
+size_t pi_gram_workspace_bytes(int ntiles, int n_c, int sms);
+cudaError_t launch_pi_gram(const PiArgs& p, const float* B0, unsigned long long seed, int segment, int iters, int sms,
+                           cudaStream_t st);
 // whole-tile path for short segments (one launch): usable when compress_tile_fits()
 bool compress_tile_fits(int T, int n_c, int rank);
 cudaError_t compress_tile(const CompressJob& job, int BH, cudaStream_t st);

@@ -1,0 +1,55 @@
+"""Long segments: the loops of Algorithm 2 on R^T R.  Sizes where the work split of the Gram kernel can go wrong (a last
+block of 16 rows, fewer blocks than CTAs, ranges that end inside a tile), every factor width, and loop counts."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,H,n,bits,group,rank,iters", [
+    (1, 1, 144, 2, 16, 4, 3),       # three blocks per tile, the last one with 16 rows; one range for both tiles
+    (1, 1, 160, 4, 32, 16, 3),      # rank 16, last block of 32 rows
+    (1, 3, 1088, 2, 64, 8, 3),      # 17 blocks per tile: ranges end inside tiles
+    (2, 5, 576, 2, 64, 5, 1),       # a single loop: B0 itself is orthonormalised
+    (1, 2, 2048, 4, 64, 1, 12),     # many loops: the factor is rescaled on the way
+    (1, 2, 256, 2, 128, 3, 2),
+])
+def test_factors_match_the_oracle(B, H, n, bits, group, rank, iters):
+    from tests.gear_harness import Pair
+    p = Pair(14, B, H, H, bits, group, 2.0, max(group, 16), min(rank, max(group, 16)), n + 128, r_max=rank, iters=iters)
+    try:
+        p.compress(n, rank)
+        # 22 bits of every operand, sums over n rows: 1e-5 is what the shapes above show at most away from close
+        # singular values; the oracle's own bound on A B^T is 1e-3
+        p.check_segment(0)
+        p.check_attention()
+    finally:
+        p.close()
+
+
+def test_residuals_of_zeros_and_of_rank_one():
+    """Entries on the quantization grid leave no residual (factors zero); a column off the grid leaves a residual of rank
+    one, of which a rank-4 fit must reproduce exactly that and invent nothing."""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+    from tests.gear_harness import Pair
+    p = Pair(15, 1, 1, 1, 2, 64, 0.0, 64, 4, 1024)
+    try:
+        gen = np.random.default_rng(1)
+        k16 = gen.permuted(np.tile(np.array([0.0, 1.0, 2.0, 3.0], np.float16), (1, 1, 256, 32)), axis=2)
+        k16[0, 0, 2::3, 7] = 1.25
+        k16[0, 0, 0::64], k16[0, 0, 1::64] = 0.0, 3.0        # every key group spans the grid exactly
+        v16 = np.tile(np.arange(4, dtype=np.float16), (1, 1, 256, 32))
+        b0 = gen.standard_normal((1, 1, 2, 128, 4)).astype(np.float32)
+        p.oracle.compress(k16, v16, 4, b0)
+        G.gear_compress(p.cache, None, torch.from_numpy(k16).cuda(), torch.from_numpy(v16).cuda(), 256, 4,
+                        torch.from_numpy(b0).cuda())
+        p.check_segment(0)
+        ab = {s: G.gear_export(p.cache, 0, s + "_A_FP32", 1, 1)[0, 0] @ G.gear_export(p.cache, 0, s + "_B_FP32", 1, 1)[0, 0].T
+              for s in "KV"}
+        assert np.array_equal(ab["V"], np.zeros((256, 128)))
+        assert np.array_equal(np.delete(ab["K"], 7, axis=1), np.zeros((256, 127)))
+        # 22-bit operands and fp32 sums of at most 86 equal terms
+        assert np.abs(ab["K"][:, 7] - np.where(k16[0, 0, :, 7] == 1.25, 0.25, 0.0)).max() <= 0.25 * 2.0 ** -20
+    finally:
+        p.close()
