@@ -773,53 +773,62 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// transpose of an 8 x 8 tile of 16-bit elements held one row pair per lane (the ldmatrix distribution)
-__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
-  uint32_t d;
-  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
-  return d;
-}
-// x -> (head, remainder) packed in one register, head in the low half
-__device__ __forceinline__ void split_pair_hl(float x, uint32_t& hl) {
-  const __half h = __float2half_rn(x);
-  const __half l = __float2half_rn(x - __half2float(h));
-  const __half2 v = __halves2half2(h, l);
-  hl = *reinterpret_cast<const uint32_t*>(&v);
-}
-
 constexpr int kChunkRows = 512;
 constexpr int kPassWarps = 4;
+constexpr int kPassPitch = kHeadDim * 4 + 16;    // bytes per residual row in shared memory (the lanes' 128-bit reads of two rows hit different banks)
+constexpr int kPassStage = 16 * kPassPitch;      // the 16 rows a warp takes at a time
+constexpr int kPassStages = 2;
+constexpr int kPassSmem = kPassWarps * kPassStages * kPassStage;
+constexpr int kRtaParts = 4;
 
-// The last loop's pass over the residual: the rows a = R b (A0, stored), this chunk's part of R^T a, and of a^T a.  The loops
-// before it run on R^T R alone (gear_gram.cu).  The orthonormalising factor W comes from pi_finish_kernel, and since
-// R^T (A0 W) = (R^T A0) W, with W only 16 x 16, R is not read again.
+// The last loop's pass over the residual: the rows A0 = R b, stored, and this chunk's part of A0^T A0.  The loops before it
+// run on R^T R alone (gear_gram.cu), which also gives R^T A0 = (R^T R) b, so this is the only product of the residual
+// itself.  The orthonormalising factor W comes from pi_finish_kernel, and R^T (A0 W) = (R^T A0) W.
 //
-// Both products run on the tensor cores (mma.sync.m16n8k16, fp16 operands, fp32 accumulation) with every fp32
-// operand cut into an fp16 head and an fp16 remainder, the four cross products summed in fp32: 22 bits of each
-// operand survive.  Powers of two bring the operands into fp16's range first (R by the tile's largest magnitude, each
-// column of b by its own, a by the bound that follows) and are divided out of the results, so the scaling itself is
-// exact.  A warp owns 16 rows at a time.  A lane loads, for rows gid and gid + 8, the four channels 16c + 4t .. + 3 of
-// each 16-channel step c as one 128-bit load; since a contraction does not care about the order of its index, these
-// four channels serve as the step's k indices 2t, 2t+1, 2t+8, 2t+9 of the A fragment.  For R^T a the same registers,
-// transposed 8 x 8 by movmatrix, are the A fragment of R^T (rows: channels 4j, 4j+1 | 4j+2, 4j+3 of the step).
-// NT = 8-column tiles of n per CTA: one (four rank columns; three CTAs per SM) or two (eight columns, the residual is
-// converted once for both; two CTAs per SM).
+// Bound: the fp32 residual from HBM.  The product runs on the tensor cores (mma.sync.m16n8k16, fp16 operands, fp32
+// accumulation; n is the rank, too narrow for a tile of its own in tensor memory) with every fp32 operand cut into an
+// fp16 head and an fp16 remainder, the four cross products summed in fp32: 22 bits of each operand survive.  Powers of two
+// bring the operands into fp16's range first (R by the tile's largest magnitude, each column of b by its own) and are
+// divided out of the results, so the scaling itself is exact.  A warp owns 16 rows at a time; they come through a ring of
+// its own in shared memory (bulk copies of a row each), because rows loaded into registers leave nothing in flight
+// during the products.  A lane reads, for rows gid and gid + 8, the four channels 16c + 4t .. + 3 of each 16-channel step c
+// as one 128-bit load; since a contraction does not care about the order of its index, these four channels serve as the
+// step's k indices 2t, 2t+1, 2t+8, 2t+9 of the A fragment.  NT = 8-column tiles of n: four rank columns (head and
+// remainder each) per tile.
 template <int NT>
-__global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kernel(PiArgs p) {
-  constexpr int RP = 4 * NT;                       // rank columns per CTA: each gives a (head, remainder) column pair of n
-  __shared__ float red[kHeadDim * RP];             // cross-warp sum, accumulated warp by warp
+__global__ void __launch_bounds__(kPassWarps * 32, 3) pi_pass_kernel(PiArgs p) {
+  constexpr int RP = 4 * NT;                       // rank columns: each gives a (head, remainder) column pair of n
+  constexpr bool kGram = NT <= 2;                  // A0^T A0 here (in registers), else by pi_gram2_kernel
   __shared__ __align__(16) __half bsplit[2 * RP][kHeadDim];   // [2 rho + (0: head, 1: remainder)][channel]
   __shared__ float colmax[kPassWarps][RP];
-  __shared__ float gred[kPassWarps][RP][RP];        // Gram partials of the rows a
-  // grid (rank column groups, chunks, tiles): the CTAs that read the same chunk of R are neighbours in launch order,
-  // so all but the first find it in L2
-  const int tile = blockIdx.z, chunk = blockIdx.y;
+  __shared__ float gred[kGram ? kPassWarps : 1][RP][RP];
+  __shared__ uint64_t full[kPassWarps][kPassStages];
+  extern __shared__ __align__(128) unsigned char ring_all[];
+  const int tile = blockIdx.y, chunk = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, t = lane & 3;
   const int row0 = chunk * kChunkRows;
   const int row1 = min(p.n_c, row0 + kChunkRows);
-  const int rho0 = blockIdx.x * RP;                // this CTA's rank columns [rho0, rho0 + RP)
   const float* R = p.R + (size_t)tile * p.n_c * kHeadDim;
-  float* A0 = p.A0 + (size_t)tile * p.n_c * kMaxRank + rho0;
+  float* A0 = p.A0 + (size_t)tile * p.n_c * RP;
+
+  // ---- the warp's ring: rows [rb, rb + 16) of its it-th group go to stage it % kPassStages
+  unsigned char* ring = ring_all + warp * kPassStages * kPassStage;
+  if (lane == 0) {
+#pragma unroll
+    for (int s = 0; s < kPassStages; ++s) bar_init(&full[warp][s]);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+  auto request = [&](int rb, int s) {
+    const int rows = min(16, row1 - rb);
+    if (rows <= 0) return;
+    __syncwarp();                                  // every lane is done with the stage
+    if (lane == 0) bar_expect(&full[warp][s], rows * kHeadDim * 4);
+    __syncwarp();
+    if (lane < rows) bulk_copy(ring + s * kPassStage + lane * kPassPitch, R + (size_t)(rb + lane) * kHeadDim, kHeadDim * 4, &full[warp][s]);
+  };
+#pragma unroll
+  for (int s = 0; s < kPassStages; ++s) request(row0 + (s * kPassWarps + warp) * 16, s);
 
   // ---- the scaled, split factor columns
   const int er = pow2_exponent(__uint_as_float(p.Rmax[tile]));
@@ -830,10 +839,8 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
     float bj[RP];
 #pragma unroll
     for (int r = 0; r < RP; ++r) {
-      bj[r] = p.Bcur[((size_t)tile * kHeadDim + j) * kMaxRank + rho0 + r];
-      float m = fabsf(bj[r]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      bj[r] = p.Bcur[((size_t)tile * kHeadDim + j) * kMaxRank + r];
+      const float m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(bj[r]))));
       if (lane == 0) colmax[warp][r] = m;
     }
     __syncthreads();
@@ -848,7 +855,6 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
       bsplit[2 * r][j] = h;
       bsplit[2 * r + 1][j] = __float2half_rn(v - __half2float(h));
     }
-    for (int i = threadIdx.x; i < kHeadDim * RP; i += blockDim.x) red[i] = 0.f;
     __syncthreads();
   }
   // B fragments of a = R b: column n = gid of tile nt is (rho = 4 nt + gid / 2, head | remainder), k as described above
@@ -860,70 +866,64 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
       const uint2 v = *reinterpret_cast<const uint2*>(&bsplit[8 * nt + gid][16 * c + 4 * t]);
       bf[c][nt][0] = v.x; bf[c][nt][1] = v.y;
     }
-  // The columns of a = R b have a norm of at most one (b carries that scaling), so a 2^14 fits fp16 and entries down to
-  // 2^-18 keep a remainder of full length
-  float inv_a[NT], scale_a[NT];                    // back to a for column rho = 4 nt + t, and to a 2^14
-  const float inv_acc = exp2_int(er - 14);         // back to R^T a
+  float inv_a[NT];                                 // back to a for column rho = 4 nt + t
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) {
     int ebt = eb[4 * nt];
 #pragma unroll
     for (int q = 1; q < 4; ++q) ebt = t == q ? eb[4 * nt + q] : ebt;
     inv_a[nt] = exp2_int(er + ebt);
-    scale_a[nt] = exp2_int(er + ebt + 14);
   }
+  float gram[kGram ? NT : 1][kGram ? RP : 1];      // gram[nt][v]: row rho = 4 nt + t of A0^T A0, column v
+#pragma unroll
+  for (int nt = 0; nt < (kGram ? NT : 1); ++nt)
+#pragma unroll
+    for (int v = 0; v < (kGram ? RP : 1); ++v) gram[nt][v] = 0.f;
 
-  // Where this CTA holds every rank column, the Gram matrix of the rows a is summed here, so that A0 is not read again for
-  // it.  gram[nt][v]: row rho = 4 nt + t of the matrix, column v.
-  const bool with_gram = gridDim.x == 1;
-  float gram[NT][RP];
-#pragma unroll
-  for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-    for (int v = 0; v < RP; ++v) gram[nt][v] = 0.f;
-
-  float acc[8][NT][4];    // R^T a: [step c][tile][(channel 4 gid/2 + gid%2 of the step | the same + 2) x (head, remainder)]
-#pragma unroll
-  for (int c = 0; c < 8; ++c)
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) acc[c][nt][i] = 0.f;
-
+  int stage = 0;
+  uint32_t parity = 0;
   for (int rb = row0 + warp * 16; rb < row1; rb += kPassWarps * 16) {
     const int ra = rb + gid, rc = rb + gid + 8;
     const bool va = ra < row1, vc = rc < row1;
-    float4 xa[8], xc[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      xa[c] = va ? *reinterpret_cast<const float4*>(R + (size_t)ra * kHeadDim + 16 * c + 4 * t) : make_float4(0.f, 0.f, 0.f, 0.f);
-      xc[c] = vc ? *reinterpret_cast<const float4*>(R + (size_t)rc * kHeadDim + 16 * c + 4 * t) : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (!bar_wait(&full[warp][stage], parity)) {   // gave up: report, let the later copies land (bounded), leave the loop
+      if (lane == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
+      for (int s = 0; s < kPassStages - 1; ++s) {
+        rb += kPassWarps * 16;
+        if (++stage == kPassStages) { stage = 0; parity ^= 1; }
+        if (rb < row1) bar_wait(&full[warp][stage], parity);
+      }
+      break;
     }
-    uint32_t fh[8][4], fl[8][4];
+    const float4* xa = reinterpret_cast<const float4*>(ring + stage * kPassStage + gid * kPassPitch) + t;
+    const float4* xc = reinterpret_cast<const float4*>(ring + stage * kPassStage + (gid + 8) * kPassPitch) + t;
     float d[NT][4];
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) d[nt][0] = d[nt][1] = d[nt][2] = d[nt][3] = 0.f;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
-      split_pair(xa[c].x * sr, xa[c].y * sr, fh[c][0], fl[c][0]);
-      split_pair(xc[c].x * sr, xc[c].y * sr, fh[c][1], fl[c][1]);
-      split_pair(xa[c].z * sr, xa[c].w * sr, fh[c][2], fl[c][2]);
-      split_pair(xc[c].z * sr, xc[c].w * sr, fh[c][3], fl[c][3]);
+      const float4 a = va ? xa[4 * c] : make_float4(0.f, 0.f, 0.f, 0.f), b = vc ? xc[4 * c] : make_float4(0.f, 0.f, 0.f, 0.f);
+      uint32_t fh[4], fl[4];
+      split_pair(a.x * sr, a.y * sr, fh[0], fl[0]);
+      split_pair(b.x * sr, b.y * sr, fh[1], fl[1]);
+      split_pair(a.z * sr, a.w * sr, fh[2], fl[2]);
+      split_pair(b.z * sr, b.w * sr, fh[3], fl[3]);
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
-        mma16816(d[nt], fh[c], bf[c][nt][0], bf[c][nt][1]);
-        mma16816(d[nt], fl[c], bf[c][nt][0], bf[c][nt][1]);
+        mma16816(d[nt], fh, bf[c][nt][0], bf[c][nt][1]);
+        mma16816(d[nt], fl, bf[c][nt][0], bf[c][nt][1]);
       }
     }
-    // B fragment of R^T a: k = row, n = (rho, head | remainder): the 8 x 8 tiles [row][2 rho + part], transposed
-    uint32_t ab[NT][2];
-    if (with_gram) {
-      float mine[2][NT];                            // a[row gid | gid + 8][rho 4 nt + t]; rows past the chunk are zero
+    request(rb + kPassStages * kPassWarps * 16, stage);
+    if (++stage == kPassStages) { stage = 0; parity ^= 1; }
+    float mine[2][NT];                             // a[row gid | gid + 8][rho 4 nt + t]; rows past the chunk are zero
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        mine[0][nt] = (d[nt][0] + d[nt][1]) * inv_a[nt];
-        mine[1][nt] = (d[nt][2] + d[nt][3]) * inv_a[nt];
-      }
+    for (int nt = 0; nt < NT; ++nt) {
+      mine[0][nt] = (d[nt][0] + d[nt][1]) * inv_a[nt];
+      mine[1][nt] = (d[nt][2] + d[nt][3]) * inv_a[nt];
+      if (va) A0[(size_t)ra * RP + 4 * nt + t] = mine[0][nt];
+      if (vc) A0[(size_t)rc * RP + 4 * nt + t] = mine[1][nt];
+    }
+    if (kGram) {
 #pragma unroll
       for (int half = 0; half < 2; ++half)
 #pragma unroll
@@ -932,94 +932,91 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 1 ? 3 : 2) pi_pass_kern
           for (int tv = 0; tv < 4; ++tv) {
             const float other = __shfl_sync(0xffffffffu, mine[half][nv], (lane & ~3) | tv);   // a[row][4 nv + tv]
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) gram[nt][4 * nv + tv] = fmaf(mine[half][nt], other, gram[nt][4 * nv + tv]);
+            for (int nt = 0; nt < NT; ++nt)
+              gram[kGram ? nt : 0][kGram ? 4 * nv + tv : 0] = fmaf(mine[half][nt], other, gram[kGram ? nt : 0][kGram ? 4 * nv + tv : 0]);
           }
     }
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      const float a_lo_rows = d[nt][0] + d[nt][1], a_hi_rows = d[nt][2] + d[nt][3];   // a[row gid | gid + 8][rho 4 nt + t], scaled
-      if (va) A0[(size_t)ra * kMaxRank + 4 * nt + t] = a_lo_rows * inv_a[nt];
-      if (vc) A0[(size_t)rc * kMaxRank + 4 * nt + t] = a_hi_rows * inv_a[nt];
-      uint32_t m0, m1;
-      split_pair_hl(a_lo_rows * scale_a[nt], m0);
-      split_pair_hl(a_hi_rows * scale_a[nt], m1);
-      ab[nt][0] = movmatrix_trans(m0);
-      ab[nt][1] = movmatrix_trans(m1);
-    }
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      uint32_t th[4], tl[4];
-      th[0] = movmatrix_trans(fh[c][0]); th[1] = movmatrix_trans(fh[c][2]);
-      th[2] = movmatrix_trans(fh[c][1]); th[3] = movmatrix_trans(fh[c][3]);
-      tl[0] = movmatrix_trans(fl[c][0]); tl[1] = movmatrix_trans(fl[c][2]);
-      tl[2] = movmatrix_trans(fl[c][1]); tl[3] = movmatrix_trans(fl[c][3]);
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        mma16816(acc[c][nt], th, ab[nt][0], ab[nt][1]);
-        mma16816(acc[c][nt], tl, ab[nt][0], ab[nt][1]);
-      }
-    }
   }
-  if (with_gram) {      // rows of the warp (over gid), then the warps, in a fixed order
+  if (kGram) {                                     // rows of the warp (over gid), then the warps, in a fixed order
 #pragma unroll
-    for (int nt = 0; nt < NT; ++nt)
+    for (int nt = 0; nt < (kGram ? NT : 1); ++nt)
 #pragma unroll
-      for (int v = 0; v < RP; ++v) {
+      for (int v = 0; v < (kGram ? RP : 1); ++v) {
         float g = gram[nt][v];
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-        if (gid == 0) gred[warp][4 * nt + t][v] = g;
+        if (gid == 0) gred[kGram ? warp : 0][4 * nt + t][v] = g;
       }
     __syncthreads();
-    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-      const int u = i / kMaxRank, v = i % kMaxRank;
+    for (int i = threadIdx.x; i < RP * RP; i += blockDim.x) {
+      const int u = i / RP, v = i % RP;
       float g = 0.f;
-      if (u < RP && v < RP)
-        for (int w = 0; w < kPassWarps; ++w) g += gred[w][u][v];
-      p.Gp[((size_t)tile * p.nchunk + chunk) * 256 + i] = g;
+      for (int w = 0; w < kPassWarps; ++w) g += gred[kGram ? w : 0][u][v];
+      p.Gp[((size_t)tile * p.nchunk + chunk) * 256 + u * kMaxRank + v] = g;
     }
   }
-  // combine the warps of this block in a fixed order, write the chunk's partial
-  for (int w = 0; w < kPassWarps; ++w) {
-    if (warp == w) {
+}
+
+// R^T A0 from the residual itself, for tiles whose factor columns differ so much in norm that (R^T R) b would lose digits
+// of the small ones (pi_iterate_kernel sets the flag; most residuals have no such tile, and the CTAs leave at once).  One
+// channel per thread; kRtaParts CTAs per tile, each with a contiguous share of the rows.
+__global__ void __launch_bounds__(kHeadDim) pi_rta_kernel(PiArgs p) {
+  constexpr int kRows = 32;
+  __shared__ float a[kRows * kMaxRank];
+  const int tile = blockIdx.y, part = blockIdx.x, j = threadIdx.x;
+  if (!p.ill[tile]) return;
+  const int RP = p.a0_pitch;
+  const int row0 = (int)((long long)part * p.n_c / kRtaParts), row1 = (int)((long long)(part + 1) * p.n_c / kRtaParts);
+  const float* R = p.R + (size_t)tile * p.n_c * kHeadDim + j;
+  const float* A0 = p.A0 + (size_t)tile * p.n_c * RP;
+  float b[kMaxRank];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const int ch = 16 * c + 4 * (gid >> 1) + (gid & 1);
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          red[ch * RP + 4 * nt + t] += (acc[c][nt][0] + acc[c][nt][1]) * inv_acc;
-          red[(ch + 2) * RP + 4 * nt + t] += (acc[c][nt][2] + acc[c][nt][3]) * inv_acc;
-        }
-      }
-    }
+  for (int q = 0; q < kMaxRank; ++q) b[q] = 0.f;
+  for (int r0 = row0; r0 < row1; r0 += kRows) {
+    const int rows = min(kRows, row1 - r0);
     __syncthreads();
+    for (int i = j; i < rows * RP; i += kHeadDim) a[(i / RP) * kMaxRank + i % RP] = A0[(size_t)r0 * RP + i];
+    __syncthreads();
+    for (int i = 0; i < rows; ++i) {
+      const float x = R[(size_t)(r0 + i) * kHeadDim];
+#pragma unroll
+      for (int q = 0; q < kMaxRank; ++q)
+        if (q < RP) b[q] = fmaf(x, a[i * kMaxRank + q], b[q]);
+    }
   }
-  for (int i = threadIdx.x; i < kHeadDim * RP; i += blockDim.x)
-    p.Bp[(((size_t)tile * p.nchunk + chunk) * kHeadDim + i / RP) * kMaxRank + rho0 + i % RP] = red[i];
+  float* out = p.Bp + (((size_t)tile * kRtaParts + part) * kHeadDim + j) * kMaxRank;
+#pragma unroll
+  for (int q = 0; q < kMaxRank; ++q) out[q] = q < RP ? b[q] : 0.f;
 }
 
 // The stored A = A0 W (W = U^-1 of A0's Cholesky factor): one thread per row.  Keys: a row is r_pad
 // consecutive fp16 of its slab; values: the slab is transposed ([r_pad][16 tokens]), so the threads of a slab fill
 // 32 contiguous bytes per rank index.  fp32 copy on request.
+template <int RP>
 __global__ void __launch_bounds__(256) pi_store_a_kernel(PiArgs p) {
-  __shared__ float Wm[kMaxRank * kMaxRank];
+  __shared__ __align__(16) float Wm[RP][RP];
   const int tile = blockIdx.y;
-  for (int i = threadIdx.x; i < kMaxRank * kMaxRank; i += blockDim.x) Wm[i] = p.W[(size_t)tile * 256 + i];
+  for (int i = threadIdx.x; i < RP * RP; i += blockDim.x) Wm[i / RP][i % RP] = p.W[(size_t)tile * 256 + (i / RP) * kMaxRank + i % RP];
   __syncthreads();
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= p.n_c) return;
   const SegDesc& sd = p.seg;
   const int r = sd.rank;
-  const float* a0p = p.A0 + ((size_t)tile * p.n_c + row) * kMaxRank;
-  float a0[kMaxRank], a[kMaxRank];
+  const float4* a0p = reinterpret_cast<const float4*>(p.A0 + ((size_t)tile * p.n_c + row) * RP);
+  float a0[RP], a[kMaxRank];
 #pragma unroll
-  for (int q = 0; q < kMaxRank; ++q) a0[q] = q < r ? a0p[q] : 0.f;
+  for (int q = 0; q < RP / 4; ++q) {               // columns past the rank are zero (the factor's are)
+    const float4 v = a0p[q];
+    a0[4 * q] = v.x; a0[4 * q + 1] = v.y; a0[4 * q + 2] = v.z; a0[4 * q + 3] = v.w;
+  }
 #pragma unroll
   for (int c = 0; c < kMaxRank; ++c) {
     float v = 0.f;
+    if (c < RP) {
 #pragma unroll
-    for (int q = 0; q < kMaxRank; ++q)
-      if (q < r && c < r) v = fmaf(a0[q], Wm[q * kMaxRank + c], v);
+      for (int q = 0; q < RP; ++q)
+        if (q <= c) v = fmaf(a0[q], Wm[q][c < RP ? c : 0], v);         // W is upper triangular
+    }
     a[c] = v;
   }
   const int bhl = tile >> 1, side = tile & 1;
@@ -1045,7 +1042,7 @@ __global__ void __launch_bounds__(256) pi_store_a_kernel(PiArgs p) {
   }
 }
 
-// One CTA per tile: the chunk partials of A0^T A0 and R^T A0 are summed (fixed order), W = U^-1 of the Gram matrix's
+// One CTA per tile: the chunk partials of A0^T A0 are summed (fixed order), W = U^-1 of the Gram matrix's
 // Cholesky factor orthonormalises A0 (its columns are nearly orthonormal already, see pi_iterate_kernel) and the final
 // factor B = (R^T A0) W is stored as fp16 ([r_pad][128] for keys, [128][r_pad] for values).
 template <int RP>
@@ -1062,9 +1059,10 @@ __global__ void __launch_bounds__(kHeadDim) pi_finish_kernel(PiArgs p) {
   float b[RP];
 #pragma unroll
   for (int q = 0; q < RP; ++q) b[q] = 0.f;
-  const float4* bp = reinterpret_cast<const float4*>(p.Bp + ((size_t)tile * p.nchunk * kHeadDim + j) * kMaxRank);
-#pragma unroll 4
-  for (int c = 0; c < p.nchunk; ++c)
+  const bool ill = p.ill[tile] != 0;               // R^T A0: from pi_rta_kernel's partials, else (R^T R) b
+  const float4* bp = reinterpret_cast<const float4*>(ill ? p.Bp + ((size_t)tile * kRtaParts * kHeadDim + j) * kMaxRank
+                                                         : p.Bg + ((size_t)tile * kHeadDim + j) * kMaxRank);
+  for (int c = 0; c < (ill ? kRtaParts : 1); ++c)
 #pragma unroll
     for (int q = 0; q < RP / 4; ++q) {
       const float4 v = bp[(size_t)c * (kHeadDim * kMaxRank / 4) + q];
@@ -1094,14 +1092,14 @@ __global__ void __launch_bounds__(kHeadDim) pi_finish_kernel(PiArgs p) {
   }
 }
 
-// Gram partials of A0 for ranks whose columns are spread over two CTAs of the pass: one thread per row.
+// Gram partials of A0 for ranks above 8 (the pass has no registers left for them): one thread per row.
 __global__ void __launch_bounds__(256) pi_gram2_kernel(PiArgs p) {
   __shared__ float rows[8][32][kMaxRank + 1];
   __shared__ float red[8][256];
   const int tile = blockIdx.y, chunk = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = p.rank;
   const int row0 = chunk * kChunkRows, row1 = min(p.n_c, row0 + kChunkRows);
-  const float* A0 = p.A0 + (size_t)tile * p.n_c * kMaxRank;
+  const float* A0 = p.A0 + (size_t)tile * p.n_c * p.a0_pitch;
   float g[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) g[i] = 0.f;
@@ -1109,7 +1107,7 @@ __global__ void __launch_bounds__(256) pi_gram2_kernel(PiArgs p) {
     const int row = base + lane;
 #pragma unroll
     for (int q = 0; q < kMaxRank; ++q)
-      if (q < r) rows[warp][lane][q] = row < row1 ? A0[(size_t)row * kMaxRank + q] : 0.f;   // uniform: only the rank's columns exist
+      if (q < r) rows[warp][lane][q] = row < row1 ? A0[(size_t)row * p.a0_pitch + q] : 0.f;   // uniform: only the rank's columns exist
     __syncwarp();
     // entry (u, v) of the Gram matrix, u, v < r: pair number i * 32 + lane, so that a small rank takes one round
 #pragma unroll
@@ -1559,12 +1557,16 @@ static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, cudaSt
   return cudaGetLastError();
 }
 
-static void launch_pass(const PiArgs& p, cudaStream_t st) {
-  // Four or eight rank columns per CTA; rank 16 is spread over two CTAs that read the same chunk of R one after the
-  // other (the second finds it in L2).
-  if (p.rank <= 4) pi_pass_kernel<1><<<dim3(1, p.nchunk, p.ntiles), kPassWarps * 32, 0, st>>>(p);
-  else pi_pass_kernel<2><<<dim3(p.rank <= 8 ? 1 : 2, p.nchunk, p.ntiles), kPassWarps * 32, 0, st>>>(p);
+static cudaError_t launch_pass(const PiArgs& p, cudaStream_t st) {
+  auto launch = [&](auto kern) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassSmem);
+    if (e == cudaSuccess) kern<<<dim3(p.nchunk, p.ntiles), kPassWarps * 32, kPassSmem, st>>>(p);
+    return e;
+  };
+  return p.rank <= 4 ? launch(pi_pass_kernel<1>) : p.rank <= 8 ? launch(pi_pass_kernel<2>) : launch(pi_pass_kernel<4>);
 }
+
+static int a0_columns(int rank) { return rank <= 4 ? 4 : (rank <= 8 ? 8 : kMaxRank); }   // of the A0 rows in the workspace
 
 // bytes of the power iteration's part of the workspace (a multiple of 256)
 static size_t pi_workspace_bytes(int nbh, int n_c, int rank, int sms) {
@@ -1575,11 +1577,12 @@ static size_t pi_workspace_bytes(int nbh, int n_c, int rank, int sms) {
   b += ntiles * n_c * kHeadDim * 4;               // R
   b += pi_gram_workspace_bytes((int)ntiles, n_c, sms);   // Gpart
   b += ntiles * kHeadDim * kMaxRank * 4;          // Bcur
-  b += ntiles * nchunk * kHeadDim * kMaxRank * 4; // Bp
-  b += ntiles * n_c * kMaxRank * 4;               // A0
+  b += ntiles * kHeadDim * kMaxRank * 4;          // Bg
+  b += ntiles * kRtaParts * kHeadDim * kMaxRank * 4;   // Bp
+  b += ntiles * n_c * a0_columns(rank) * 4;       // A0
   b += ntiles * nchunk * 256 * 4;                 // Gp
   b += ntiles * 256 * 4;                          // W
-  b += ntiles * 4;                                // Rmax
+  b += ntiles * 8;                                // Rmax, ill
   return (b + 1024 + 255) / 256 * 256;
 }
 
@@ -1596,18 +1599,20 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
   PiArgs pa;
   pa.seg = sd; pa.arena = job.arena; pa.bh0 = bh0; pa.ntiles = (int)ntiles; pa.n_c = sd.n_c; pa.rank = sd.rank;
   pa.nchunk = nchunk;
-  pa.status = job.status;
-  pa.R = nullptr; pa.Rmax = nullptr; pa.Gpart = nullptr; pa.Bcur = nullptr; pa.Bp = nullptr; pa.A0 = nullptr; pa.Gp = nullptr; pa.W = nullptr;
+  pa.status = job.status; pa.a0_pitch = a0_columns(sd.rank);
+  pa.R = nullptr; pa.Rmax = nullptr; pa.Gpart = nullptr; pa.Bcur = nullptr; pa.Bp = nullptr; pa.Bg = nullptr; pa.ill = nullptr; pa.A0 = nullptr; pa.Gp = nullptr; pa.W = nullptr;
   pa.dbgA = job.dbgA; pa.dbgB = job.dbgB;
   if (sd.rank > 0) {
     pa.R = wsf;       wsf += ntiles * sd.n_c * kHeadDim;
     pa.Gpart = wsf;   wsf += pi_gram_workspace_bytes((int)ntiles, sd.n_c, job.sms) / 4;
     pa.Bcur = wsf;    wsf += ntiles * kHeadDim * kMaxRank;
-    pa.Bp = wsf;      wsf += ntiles * nchunk * kHeadDim * kMaxRank;
-    pa.A0 = wsf;      wsf += ntiles * sd.n_c * kMaxRank;
+    pa.Bg = wsf;      wsf += ntiles * kHeadDim * kMaxRank;
+    pa.Bp = wsf;      wsf += ntiles * kRtaParts * kHeadDim * kMaxRank;
+    pa.A0 = wsf;      wsf += ntiles * sd.n_c * a0_columns(sd.rank);
     pa.Gp = wsf;      wsf += ntiles * nchunk * 256;
     pa.W = wsf;       wsf += ntiles * 256;
     pa.Rmax = reinterpret_cast<unsigned int*>(wsf);
+    pa.ill = reinterpret_cast<int*>(wsf) + ntiles;
     if (cudaMemsetAsync(pa.Rmax, 0, ntiles * 4, st) != cudaSuccess) return cudaGetLastError();
   }
   CompressArgs ca;
@@ -1631,13 +1636,18 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
   if (sd.rank == 0) return cudaSuccess;
   e = launch_pi_gram(pa, job.B0, job.seed, job.segment_index, job.iters, job.sms, st);   // the loops, B <- Q(B), its scaling
   if (e != cudaSuccess) return e;
-  launch_pass(pa, st);                                              // A0 = R B, R^T A0; for ranks up to 8 also A0^T A0
+  e = launch_pass(pa, st);                                          // A0 = R B; for ranks up to 8 also A0^T A0
+  if (e != cudaSuccess) return e;
+  pi_rta_kernel<<<dim3(kRtaParts, (int)ntiles), kHeadDim, 0, st>>>(pa);                  // R^T A0 of ill-conditioned tiles
   if (sd.rank > 8) pi_gram2_kernel<<<dim3(nchunk, (int)ntiles), 256, 0, st>>>(pa);
   if (sd.rank <= 4) pi_finish_kernel<4><<<(int)ntiles, kHeadDim, 0, st>>>(pa);           // W, B
   else if (sd.rank <= 8) pi_finish_kernel<8><<<(int)ntiles, kHeadDim, 0, st>>>(pa);
   else pi_finish_kernel<16><<<(int)ntiles, kHeadDim, 0, st>>>(pa);
-  pi_store_a_kernel<<<dim3((sd.n_c + 255) / 256, (int)ntiles), 256, 0, st>>>(pa);        // A = A0 W
-  count_launches(sd.rank > 8 ? 4 : 3);
+  const dim3 sgrid((sd.n_c + 255) / 256, (int)ntiles);                                   // A = A0 W
+  if (sd.rank <= 4) pi_store_a_kernel<4><<<sgrid, 256, 0, st>>>(pa);
+  else if (sd.rank <= 8) pi_store_a_kernel<8><<<sgrid, 256, 0, st>>>(pa);
+  else pi_store_a_kernel<16><<<sgrid, 256, 0, st>>>(pa);
+  count_launches(sd.rank > 8 ? 5 : 4);
   return cudaGetLastError();
 }
 

@@ -10,26 +10,8 @@
 
 namespace gear {
 
-// ------------------------------------------------------------------ tcgen05 / mbarrier helpers
+// ------------------------------------------------------------------ tcgen05 helpers
 namespace {
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void bar_init(uint64_t* b) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(b)) : "memory");
-}
-// bounded: false when the phase did not complete within the limit
-__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
-  uint32_t ok = 0;
-#pragma unroll 1
-  for (int i = 0; i < kDecodeSpinLimit && !ok; ++i)
-    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(ok) : "r"(smem_addr(b)), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* b) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(b)), "r"(bytes) : "memory");
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(dst)),
-               "l"(src), "r"(bytes), "r"(smem_addr(b)) : "memory");
-}
 __device__ __forceinline__ void umma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
@@ -52,13 +34,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t addr) {
 }  // namespace
 
 // ------------------------------------------------------------------ G = R^T R
-// Work: the 64-row blocks of all tiles, one after the other, cut into equal contiguous ranges, one per CTA (two CTAs per
+// Work: the 32-row blocks of all tiles, one after the other, cut into equal contiguous ranges, one per CTA (two CTAs per
 // SM); a CTA leaves one partial G per tile it touches.  Partial number = CTA + tile, which is different for all of them.
-constexpr int kGramRows = 64;
+constexpr int kGramRows = 32;
+constexpr int kGramStages = 4;                                      // blocks in flight or being converted
 constexpr int kGramStage = kGramRows * kHeadDim * 4;                // fp32 rows as they lie in memory
 constexpr int kGramOperand = kGramRows * kHeadDim * 2;              // fp16 heads or remainders of a block
-constexpr int kGramSmem = 1024 + 2 * kGramOperand + 2 * kGramStage;
-constexpr int kGramMinBlocks = 4;                                   // a partial is 64 KB, a block 32 KB: at least 256 rows per CTA
+constexpr int kGramSmem = 1024 + 4 * kGramOperand + kGramStages * kGramStage;   // heads and remainders, two buffers
+constexpr int kGramMinBlocks = 8;                                   // a partial is 64 KB, a block 16 KB: at least 256 rows per CTA
 
 struct GramSplit { int nb; long long blocks; int ctas; };
 static __host__ __device__ inline GramSplit gram_split(int ntiles, int n_c, int sms) {
@@ -73,28 +56,31 @@ size_t pi_gram_workspace_bytes(int ntiles, int n_c, int sms) {
   return (size_t)(gram_split(ntiles, n_c, sms).ctas + ntiles) * kHeadDim * kHeadDim * 4;
 }
 
-// Bound: the fp32 residual from HBM, once (32 KB per block; the products of a block take 12 tcgen05.mma of 128 x 128 x 16,
-// a third of the time its bytes take).  Every fp32 entry becomes an fp16 head and an fp16 remainder after exact
-// power-of-two scaling by the tile's largest magnitude; head x head, head x remainder and remainder x head are summed in
-// fp32, so 22 bits of each operand count.  The rows of a block lie in shared memory as they come ([token][channel]), which
-// is the MN-major layout for both operands: G[i][j] = sum over tokens (K) of R[k][i] R[k][j].
+// Bound: the fp32 residual from HBM, once, with the shared memory close behind (a block crosses it as fp32 twice, as fp16
+// operands once, and the products read their operands from there).  Every fp32 entry becomes an fp16 head h and an fp16
+// remainder l after exact power-of-two scaling by the tile's largest magnitude; h h, h l and l h are summed in fp32, so 22
+// bits of each operand count.  One tcgen05.mma of 128 x 256 x 16 takes h^T [h | l]: 12 KB of operands per step instead of
+// the 24 KB of three 128 x 128 products, l h being the transpose of h l.  The rows of a block lie in shared memory as they
+// come ([token][channel]), which is the MN-major layout for both operands.  Blocks of 32 rows keep four of them in flight
+// per CTA and the operands double, so that the conversion of a block runs beside the products of the one before.
 __global__ void __launch_bounds__(256, 2) pi_gram_kernel(PiArgs p, int sms) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ uint64_t full[2], mma_done;
+  __shared__ uint64_t full[kGramStages], mma_done[2];
   __shared__ uint32_t tmem_slot;
   unsigned char* smem = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
-  unsigned char* op_hi = smem;                                      // [2 halves of the channels][8-token groups][8][128 B], 128B swizzle
-  unsigned char* op_lo = smem + kGramOperand;
-  unsigned char* stage = smem + 2 * kGramOperand;
+  // operand buffer b: heads at 2 b, remainders at 2 b + 1 (in units of kGramOperand); each [2 halves of the channels]
+  // [8-token groups][8][128 B], 128B swizzle
+  unsigned char* stage = smem + 4 * kGramOperand;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const GramSplit sp = gram_split(p.ntiles, p.n_c, sms);
   const long long f0 = blockIdx.x * sp.blocks / gridDim.x, f1 = (blockIdx.x + 1LL) * sp.blocks / gridDim.x;
   if (tid == 0) {
-    bar_init(&full[0]); bar_init(&full[1]); bar_init(&mma_done);
+    for (uint64_t& b : full) bar_init(&b);
+    bar_init(&mma_done[0]); bar_init(&mma_done[1]);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 128;" ::"r"(smem_addr(&tmem_slot)) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_addr(&tmem_slot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -102,33 +88,44 @@ __global__ void __launch_bounds__(256, 2) pi_gram_kernel(PiArgs p, int sms) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
 
-  auto rows_of = [&](long long f) { return min(kGramRows, p.n_c - (int)(f % sp.nb) * kGramRows); };
-  auto request = [&](long long f) {                                 // thread 0: block f into its stage
-    const int s = (int)(f - f0) & 1;
-    const long long tile = f / sp.nb;
-    const float* src = p.R + ((size_t)tile * p.n_c + (size_t)(f % sp.nb) * kGramRows) * kHeadDim;
-    bulk_load(stage + s * kGramStage, src, (uint32_t)rows_of(f) * kHeadDim * 4, &full[s]);
+  // (tile, block) of the block being worked on and, thread 0, of the next one to request; 64-bit divisions would cost more
+  // than the products of a block
+  const int count = (int)(f1 - f0);
+  int tile = (int)(f0 / sp.nb), blk = (int)(f0 - (long long)tile * sp.nb);
+  int q_it = 0, q_tile = tile, q_blk = blk;
+  auto request_next = [&]() {
+    const int s = q_it % kGramStages;
+    const float* src = p.R + ((size_t)q_tile * p.n_c + (size_t)q_blk * kGramRows) * kHeadDim;
+    const uint32_t bytes = (uint32_t)min(kGramRows, p.n_c - q_blk * kGramRows) * kHeadDim * 4;
+    bar_expect(&full[s], bytes);
+    bulk_copy(stage + s * kGramStage, src, bytes, &full[s]);
+    ++q_it;
+    if (++q_blk == sp.nb) { q_blk = 0; ++q_tile; }
   };
-  if (tid == 0) {
-    request(f0);
-    if (f0 + 1 < f1) request(f0 + 1);
-  }
-  // descriptors: 128B swizzle, 64-channel halves 8 KB apart (leading), 8-token groups 1 KB apart (stride)
+  if (tid == 0)
+    for (int s = 0; s < kGramStages && s < count; ++s) request_next();
+  // descriptors: 128B swizzle, 64-channel halves 4 KB apart (leading), 8-token groups 1 KB apart (stride)
   constexpr uint64_t kDesc = ((uint64_t)(kGramOperand / 2 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
-  // fp32 accumulator, fp16 operands, both MN-major, N = 128, M = 128
-  constexpr uint32_t kIdesc = (1u << 4) | (1u << 15) | (1u << 16) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-  const uint64_t d_hi = kDesc | (smem_addr(op_hi) >> 4), d_lo = kDesc | (smem_addr(op_lo) >> 4);
+  // (the remainders follow the heads, so the N = 256 operand has the same strides); fp32 accumulator, fp16 operands, both
+  // MN-major, N = 256, M = 128
+  constexpr uint32_t kIdesc = (1u << 4) | (1u << 15) | (1u << 16) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
 
   bool ok = true;
+  // products of block i complete mma_done[i & 1]; the buffer is written again two blocks later
   uint32_t mma_waits = 0, mma_issued = 0;
+  auto products_up_to = [&](uint32_t count) {
+    for (; mma_waits < count; ++mma_waits) ok = bar_wait(&mma_done[mma_waits & 1u], (mma_waits >> 1) & 1u) && ok;
+  };
   float sr = 0.f;
   bool fresh = true;                                                // the accumulator holds nothing of this tile yet
-  long long f = f0;
-  for (; f < f1; ++f) {
-    const int s = (int)(f - f0) & 1, tile = (int)(f / sp.nb), rows = rows_of(f);
-    if (f == f0 || f % sp.nb == 0) sr = exp2_int(-pow2_exponent(__uint_as_float(p.Rmax[tile])));
-    ok = bar_wait(&full[s], (uint32_t)((f - f0) >> 1) & 1u) && ok;
-    while (mma_waits < mma_issued) ok = bar_wait(&mma_done, mma_waits++ & 1u) && ok;   // the operands of the block before are free
+  int it = 0;
+  for (; it < count; ++it) {
+    const int s = it % kGramStages, rows = min(kGramRows, p.n_c - blk * kGramRows);
+    unsigned char* op_hi = smem + (it & 1) * 2 * kGramOperand;
+    unsigned char* op_lo = op_hi + kGramOperand;
+    if (it == 0 || blk == 0) sr = exp2_int(-pow2_exponent(__uint_as_float(p.Rmax[tile])));
+    ok = bar_wait(&full[s], (uint32_t)(it / kGramStages) & 1u) && ok;
+    if (it >= 2) products_up_to((uint32_t)it - 1u);                          // this operand buffer is free again
     const float4* src = reinterpret_cast<const float4*>(stage + s * kGramStage);
 #pragma unroll
     for (int j = 0; j < kGramRows * 32 / 256; ++j) {
@@ -147,41 +144,60 @@ __global__ void __launch_bounds__(256, 2) pi_gram_kernel(PiArgs p, int sms) {
     ++mma_issued;
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint64_t d_hi = kDesc | (smem_addr(op_hi) >> 4);
 #pragma unroll
       for (int k = 0; k < kGramRows / 16; ++k) {
-        const uint64_t ah = d_hi + k * (2048 >> 4), al = d_lo + k * (2048 >> 4);
-        umma_f16(tmem, ah, ah, kIdesc, (fresh && k == 0) ? 0u : 1u);
-        umma_f16(tmem, ah, al, kIdesc, 1u);
-        umma_f16(tmem, al, ah, kIdesc, 1u);
+        const uint64_t op = d_hi + k * (2048 >> 4);
+        umma_f16(tmem, op, op, kIdesc, (fresh && k == 0) ? 0u : 1u);
       }
-      umma_commit(&mma_done);
-      if (f + 2 < f1) request(f + 2);
+      umma_commit(&mma_done[it & 1]);
+      if (q_it < count) request_next();
     }
     fresh = false;
-    if (f + 1 == f1 || (f + 1) % sp.nb == 0) {                      // last block of the tile in this range: leave the partial
-      while (mma_waits < mma_issued) ok = bar_wait(&mma_done, mma_waits++ & 1u) && ok;
-      if (__syncthreads_or(!ok)) { ok = false; ++f; break; }
+    if (it + 1 == count || blk + 1 == sp.nb) {                      // last block of the tile in this range: leave the partial
+      products_up_to(mma_issued);
+      if (__syncthreads_or(!ok)) { ok = false; ++it; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // G is symmetric: column c of the accumulator row i goes to row c, so that a warp writes 128 consecutive bytes
-      float* out = p.Gpart + (size_t)(blockIdx.x + tile) * kHeadDim * kHeadDim + (warp & 3) * 32 + lane;
-#pragma unroll
+      // columns 0..127 of accumulator row i are h h, 128..255 h l.  First (h h + h l)[i][c] goes to row c of the partial (h h
+      // is symmetric), so that a warp writes 128 consecutive bytes; then h l[i][c] is added to row i, column c
+      float* part = p.Gpart + (size_t)(blockIdx.x + tile) * kHeadDim * kHeadDim;
+      const int i = (warp & 3) * 32 + lane;
+      const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+#pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         const int c0 = (warp >> 2) * 64 + h * 32;
-        uint32_t v[32];
-        tmem_ld32(v, tmem + ((uint32_t)((warp & 3) * 32) << 16) + c0);
+        uint32_t v[32], w[32];
+        tmem_ld32(v, lanes + c0);
+        tmem_ld32(w, lanes + 128 + c0);
 #pragma unroll
-        for (int c = 0; c < 32; ++c) out[(size_t)(c0 + c) * kHeadDim] = __uint_as_float(v[c]);
+        for (int c = 0; c < 32; ++c) part[(size_t)(c0 + c) * kHeadDim + i] = __uint_as_float(v[c]) + __uint_as_float(w[c]);
+      }
+      __syncthreads();
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        const int c0 = (warp >> 2) * 64 + h * 32;
+        uint32_t w[32];
+        tmem_ld32(w, lanes + 128 + c0);
+        float4* row = reinterpret_cast<float4*>(part + (size_t)i * kHeadDim + c0);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          float4 g = __ldcg(row + c);
+          g.x += __uint_as_float(w[4 * c]); g.y += __uint_as_float(w[4 * c + 1]);
+          g.z += __uint_as_float(w[4 * c + 2]); g.w += __uint_as_float(w[4 * c + 3]);
+          row[c] = g;
+        }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       fresh = true;
     }
+    if (++blk == sp.nb) { blk = 0; ++tile; }
   }
   if (!ok && tid == 0) {                                            // gave up (all threads): report, let the copies in flight land (bounded)
     atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
-    for (long long g = f; g < f1 && g < f + 2; ++g) bar_wait(&full[(int)(g - f0) & 1], (uint32_t)((g - f0) >> 1) & 1u);
+    for (; it < q_it; ++it) bar_wait(&full[it % kGramStages], (uint32_t)(it / kGramStages) & 1u);
   }
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem) : "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
 }
 
 // ------------------------------------------------------------------ the loops on G
@@ -324,21 +340,26 @@ __global__ void __launch_bounds__(256) pi_iterate_kernel(PiArgs p, const float* 
     if (lane == 0) Gm[u][v] = s;
   }
   __syncthreads();
-  if (warp == 0) warp_chol_inverse<RP, true>(&Gm[0][0], &Wm[0][0], RP + 1, r, lane);
+  if (warp == 0) {
+    const bool small = warp_chol_inverse<RP, true>(&Gm[0][0], &Wm[0][0], RP + 1, r, lane);
+    if (lane == 0) p.ill[tile] = small;
+  }
   __syncthreads();
-  if (half == 0) {
-    // G was summed over R 2^-er, so the columns of R (B W) would have norm 2^er
-    const float down = exp2_int(-pow2_exponent(__uint_as_float(p.Rmax[tile])));
-    float* out = p.Bcur + ((size_t)tile * kHeadDim + i) * kMaxRank;
+  {
+    // half 0: b = Q(B) W; half 1: (R^T R) b = G Q(B) W.  G was summed over R 2^-er, so the columns of R b would have norm 2^er
+    const float (*m)[RP] = half == 0 ? Bs : Cs;
+    const int er = pow2_exponent(__uint_as_float(p.Rmax[tile]));
+    const float sc = exp2_int(half == 0 ? -er : er);
+    float* out = (half == 0 ? p.Bcur : p.Bg) + ((size_t)tile * kHeadDim + i) * kMaxRank;
 #pragma unroll
     for (int rho = 0; rho < kMaxRank; ++rho) {
       float v = 0.f;
       if (rho < RP && rho < r) {
 #pragma unroll
         for (int q = 0; q < RP; ++q)
-          if (q <= rho && q < r) v = fmaf(Bs[i][q], Wm[q][rho < RP ? rho : 0], v);
+          if (q <= rho && q < r) v = fmaf(m[i][q], Wm[q][rho < RP ? rho : 0], v);
       }
-      out[rho] = v * down;
+      out[rho] = v * sc;
     }
   }
 }

@@ -48,13 +48,16 @@ struct PiArgs {
   float* Gpart;         // partials of R^T R, [CTA + tile][128][128] (gear_gram.cu)
   int* status;          // the cache's status word
   float* Bcur;          // [ntiles][128][16]
-  float* Bp;            // [ntiles][nchunk][128][16]
-  float* A0;            // [ntiles][n_c][16]
+  float* Bg;            // [ntiles][128][16]: (R^T R) Bcur = R^T A0
+  float* Bp;            // [ntiles][parts][128][16]: R^T A0 summed from the residual (tiles with `ill` set)
+  int* ill;             // [ntiles]
+  float* A0;            // [ntiles][n_c][a0_pitch]
   float* Gp;            // [ntiles][nchunk][256]
   float* W;             // [ntiles][256]
   float* dbgA;          // fp32 copies for export, whole segment: [BH][2][n_c][rank] / [BH][2][128][rank]
   float* dbgB;
   int bh0, ntiles, n_c, rank, nchunk;
+  int a0_pitch;         // 4, 8 or 16 columns, zero past the rank
 };
 
 struct CompressJob {

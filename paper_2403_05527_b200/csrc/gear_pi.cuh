@@ -3,9 +3,33 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
-#include "gear_layout.cuh"
+#include "gear_internal.cuh"
 
 namespace gear {
+
+// ------------------------------------------------------------------ bulk copies and barriers
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void bar_init(uint64_t* b) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(b)) : "memory");
+}
+// bounded: false when the phase did not complete within the limit
+__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
+  uint32_t ok = 0;
+#pragma unroll 1
+  for (int i = 0; i < kDecodeSpinLimit && !ok; ++i)
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(smem_addr(b)), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void bar_expect(uint64_t* b, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(b)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* b) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(dst)),
+               "l"(src), "r"(bytes), "r"(smem_addr(b)) : "memory");
+}
+
+// ------------------------------------------------------------------ numbers
 
 // floor(log2 |x|) for a finite x > 0 (0 for x == 0): the power of two that brings x into [1, 2)
 __device__ __forceinline__ int pow2_exponent(float x) { return x > 0.f ? ilogbf(x) : 0; }
@@ -44,18 +68,19 @@ __device__ __forceinline__ float start_value(unsigned long long seed, int segmen
 // FLOOR = true (scaling a factor that has not been computed yet): a pivot below 1e-6 of the trace is rounding of G as much
 // as it is the column, so the column is scaled by that floor and nothing is eliminated with it; FLOOR = false (columns of
 // norm about one, or shorter where the floor was used): a column below 1e-6, i.e. below 1e-12 of the trace of the
-// unscaled factor, is zeroed.
+// unscaled factor, is zeroed.  Returns whether a pivot lies below a thousandth of the largest diagonal entry.
 template <int RP, bool FLOOR>
-__device__ __forceinline__ void warp_chol_inverse(const float* G, float* W, int pitch, int r, int lane) {
+__device__ __forceinline__ bool warp_chol_inverse(const float* G, float* W, int pitch, int r, int lane) {
   float u[RP], x[RP];
   const int c = lane < RP ? lane : 0;
 #pragma unroll
   for (int k = 0; k < RP; ++k) u[k] = lane < r && k < r ? G[k * pitch + c] : 0.f;
-  float low = 1e-6f;
-  if (FLOOR) {
-    float diag = 0.f;
+  float low = 1e-6f, diag = 0.f;
 #pragma unroll
-    for (int k = 0; k < RP; ++k) diag = lane == k ? u[k] : diag;
+  for (int k = 0; k < RP; ++k) diag = lane == k ? u[k] : diag;
+  const float dmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(diag, 0.f))));
+  bool small = false;
+  if (FLOOR) {
     low = 1e-6f * warp_sum(diag);
     if (!(low > 0.f)) low = 1.f;                   // a residual of zeros: no scaling
   }
@@ -63,6 +88,7 @@ __device__ __forceinline__ void warp_chol_inverse(const float* G, float* W, int 
   for (int j = 0; j < RP; ++j) {
     const float d = __shfl_sync(0xffffffffu, u[j], j);
     const bool good = d > low;
+    small = small || (j < r && d < 1e-3f * dmax);
     const float ujj = j >= r ? 0.f : (good ? sqrtf(d) : (FLOOR ? sqrtf(low) : 0.f));
     const float ujc = lane == j ? ujj : (lane > j && good ? u[j] / ujj : 0.f);
     u[j] = ujc;
@@ -82,6 +108,7 @@ __device__ __forceinline__ void warp_chol_inverse(const float* G, float* W, int 
     for (int k = 0; k < RP; ++k) W[k * pitch + lane] = x[k];
   }
   __syncwarp();
+  return small;
 }
 
 }  // namespace gear

@@ -53,3 +53,33 @@ def test_residuals_of_zeros_and_of_rank_one():
         assert np.abs(ab["K"][:, 7] - np.where(k16[0, 0, :, 7] == 1.25, 0.25, 0.0)).max() <= 0.25 * 2.0 ** -20
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("rank", [2, 8, 16])
+def test_tiles_whose_singular_values_span_decades(rank):
+    """A few channels 60 times as large as the others: the factor columns differ so much in norm that R^T A0 is taken from
+    the residual instead of from R^T R.  Two loops: each one squares the ratio of the directions, and past that the fp32
+    iterates of Algorithm 2 hold nothing of the small ones.  (The oracle's bound on A B^T is relative to its largest
+    entry; the last assertion looks at the small directions by themselves.)"""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+    from tests.gear_harness import Pair
+    p = Pair(16, 1, 1, 1, 4, 64, 2.0, 64, 4, 1024, r_max=16, iters=2)
+    try:
+        gen = np.random.default_rng(rank)
+        x = gen.standard_normal((1, 1, 320, 128))
+        x[..., :rank // 2] *= 60.0
+        k16, v16 = x.astype(np.float16), gen.standard_normal((1, 1, 320, 128)).astype(np.float16)
+        b0 = gen.standard_normal((1, 1, 2, 128, rank)).astype(np.float32)
+        p.oracle.compress(k16, v16, rank, b0)
+        G.gear_compress(p.cache, None, torch.from_numpy(k16).cuda(), torch.from_numpy(v16).cuda(), 320, rank,
+                        torch.from_numpy(b0).cuda())
+        p.check_segment(0)
+        a, b = (G.gear_export(p.cache, 0, w, 1, 1)[0, 0].astype(np.float64) for w in ("K_A_FP32", "K_B_FP32"))
+        assert np.abs(a.T @ a - np.eye(rank)).max() <= 1e-5
+        t = p.oracle.segments[0]["K"][0][0]
+        got, ref = a @ b.T, t["A"] @ t["B"].T
+        small = slice(rank // 2, 128)            # fp32 rounding of the large directions in B: 60^2 * 2^-22, a thousandth
+        assert np.abs(got[:, small] - ref[:, small]).max() <= 5e-3 * np.abs(ref[:, small]).max()
+    finally:
+        p.close()
