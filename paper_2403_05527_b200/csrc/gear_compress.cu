@@ -1600,11 +1600,12 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
   pa.seg = sd; pa.arena = job.arena; pa.bh0 = bh0; pa.ntiles = (int)ntiles; pa.n_c = sd.n_c; pa.rank = sd.rank;
   pa.nchunk = nchunk;
   pa.status = job.status; pa.a0_pitch = a0_columns(sd.rank);
-  pa.R = nullptr; pa.Rmax = nullptr; pa.Gpart = nullptr; pa.Bcur = nullptr; pa.Bp = nullptr; pa.Bg = nullptr; pa.ill = nullptr; pa.A0 = nullptr; pa.Gp = nullptr; pa.W = nullptr;
+  pa.R = nullptr; pa.Rmax = nullptr; pa.Gpart = nullptr; pa.G = nullptr; pa.Bcur = nullptr; pa.Bp = nullptr; pa.Bg = nullptr; pa.ill = nullptr; pa.A0 = nullptr; pa.Gp = nullptr; pa.W = nullptr;
   pa.dbgA = job.dbgA; pa.dbgB = job.dbgB;
   if (sd.rank > 0) {
     pa.R = wsf;       wsf += ntiles * sd.n_c * kHeadDim;
-    pa.Gpart = wsf;   wsf += pi_gram_workspace_bytes((int)ntiles, sd.n_c, job.sms) / 4;
+    pa.G = wsf;       pa.Gpart = wsf + ntiles * kHeadDim * kHeadDim;
+    wsf += pi_gram_workspace_bytes((int)ntiles, sd.n_c, job.sms) / 4;
     pa.Bcur = wsf;    wsf += ntiles * kHeadDim * kMaxRank;
     pa.Bg = wsf;      wsf += ntiles * kHeadDim * kMaxRank;
     pa.Bp = wsf;      wsf += ntiles * kRtaParts * kHeadDim * kMaxRank;

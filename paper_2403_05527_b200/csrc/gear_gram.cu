@@ -41,7 +41,8 @@ constexpr int kGramStages = 4;                                      // blocks in
 constexpr int kGramStage = kGramRows * kHeadDim * 4;                // fp32 rows as they lie in memory
 constexpr int kGramOperand = kGramRows * kHeadDim * 2;              // fp16 heads or remainders of a block
 constexpr int kGramSmem = 1024 + 4 * kGramOperand + kGramStages * kGramStage;   // heads and remainders, two buffers
-constexpr int kGramMinBlocks = 8;                                   // a partial is 64 KB, a block 16 KB: at least 256 rows per CTA
+constexpr int kGramMinBlocks = 8;                                   // a partial is 128 KB, a block 16 KB: at least 256 rows per CTA
+constexpr int kGramPartial = 2 * kHeadDim * kHeadDim;               // floats: two planes
 
 struct GramSplit { int nb; long long blocks; int ctas; };
 static __host__ __device__ inline GramSplit gram_split(int ntiles, int n_c, int sms) {
@@ -53,7 +54,7 @@ static __host__ __device__ inline GramSplit gram_split(int ntiles, int n_c, int 
   return s;
 }
 size_t pi_gram_workspace_bytes(int ntiles, int n_c, int sms) {
-  return (size_t)(gram_split(ntiles, n_c, sms).ctas + ntiles) * kHeadDim * kHeadDim * 4;
+  return (size_t)(gram_split(ntiles, n_c, sms).ctas + ntiles) * kGramPartial * 4 + (size_t)ntiles * kHeadDim * kHeadDim * 4;
 }
 
 // Bound: the fp32 residual from HBM, once, with the shared memory close behind (a block crosses it as fp32 twice, as fp16
@@ -63,9 +64,14 @@ size_t pi_gram_workspace_bytes(int ntiles, int n_c, int sms) {
 // the 24 KB of three 128 x 128 products, l h being the transpose of h l.  The rows of a block lie in shared memory as they
 // come ([token][channel]), which is the MN-major layout for both operands.  Blocks of 32 rows keep four of them in flight
 // per CTA and the operands double, so that the conversion of a block runs beside the products of the one before.
-__global__ void __launch_bounds__(256, 2) pi_gram_kernel(PiArgs p, int sms) {
+// Eight warps convert, a ninth requests the copies and issues the products; they meet at mbarriers only, so a warp that is
+// done with its part of a block goes on to the next one.
+constexpr int kGramWarps = 8;
+__global__ void __launch_bounds__(kGramWarps * 32 + 32, 2) pi_gram_kernel(PiArgs p, int sms) {
   extern __shared__ unsigned char smem_raw[];
-  __shared__ uint64_t full[kGramStages], mma_done[2];
+  // full: the copy of a stage has landed; ready: every converting warp is done with a block (its operands are written, its
+  // stage is read); mma_done: the products of a block are complete (its operand buffer is free, the accumulator current)
+  __shared__ uint64_t full[kGramStages], ready[2], mma_done[2];
   __shared__ uint32_t tmem_slot;
   unsigned char* smem = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
   // operand buffer b: heads at 2 b, remainders at 2 b + 1 (in units of kGramOperand); each [2 halves of the channels]
@@ -76,10 +82,11 @@ __global__ void __launch_bounds__(256, 2) pi_gram_kernel(PiArgs p, int sms) {
   const long long f0 = blockIdx.x * sp.blocks / gridDim.x, f1 = (blockIdx.x + 1LL) * sp.blocks / gridDim.x;
   if (tid == 0) {
     for (uint64_t& b : full) bar_init(&b);
-    bar_init(&mma_done[0]); bar_init(&mma_done[1]);
+    for (uint64_t& b : mma_done) bar_init(&b);
+    for (uint64_t& b : ready) bar_init(&b, kGramWarps);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {
+  if (warp == kGramWarps) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_addr(&tmem_slot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -87,117 +94,127 @@ __global__ void __launch_bounds__(256, 2) pi_gram_kernel(PiArgs p, int sms) {
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
-
-  // (tile, block) of the block being worked on and, thread 0, of the next one to request; 64-bit divisions would cost more
-  // than the products of a block
   const int count = (int)(f1 - f0);
-  int tile = (int)(f0 / sp.nb), blk = (int)(f0 - (long long)tile * sp.nb);
-  int q_it = 0, q_tile = tile, q_blk = blk;
-  auto request_next = [&]() {
-    const int s = q_it % kGramStages;
-    const float* src = p.R + ((size_t)q_tile * p.n_c + (size_t)q_blk * kGramRows) * kHeadDim;
-    const uint32_t bytes = (uint32_t)min(kGramRows, p.n_c - q_blk * kGramRows) * kHeadDim * 4;
-    bar_expect(&full[s], bytes);
-    bulk_copy(stage + s * kGramStage, src, bytes, &full[s]);
-    ++q_it;
-    if (++q_blk == sp.nb) { q_blk = 0; ++q_tile; }
-  };
-  if (tid == 0)
-    for (int s = 0; s < kGramStages && s < count; ++s) request_next();
-  // descriptors: 128B swizzle, 64-channel halves 4 KB apart (leading), 8-token groups 1 KB apart (stride)
-  constexpr uint64_t kDesc = ((uint64_t)(kGramOperand / 2 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
-  // (the remainders follow the heads, so the N = 256 operand has the same strides); fp32 accumulator, fp16 operands, both
-  // MN-major, N = 256, M = 128
-  constexpr uint32_t kIdesc = (1u << 4) | (1u << 15) | (1u << 16) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
+  int tile = (int)(f0 / sp.nb), blk = (int)(f0 - (long long)tile * sp.nb);    // 64-bit divisions only here
+  bool ok = true;                                                   // a wait gave up: go on without waiting, every loop still ends
 
-  bool ok = true;
-  // products of block i complete mma_done[i & 1]; the buffer is written again two blocks later
-  uint32_t mma_waits = 0, mma_issued = 0;
-  auto products_up_to = [&](uint32_t count) {
-    for (; mma_waits < count; ++mma_waits) ok = bar_wait(&mma_done[mma_waits & 1u], (mma_waits >> 1) & 1u) && ok;
-  };
-  float sr = 0.f;
-  bool fresh = true;                                                // the accumulator holds nothing of this tile yet
-  int it = 0;
-  for (; it < count; ++it) {
-    const int s = it % kGramStages, rows = min(kGramRows, p.n_c - blk * kGramRows);
-    unsigned char* op_hi = smem + (it & 1) * 2 * kGramOperand;
-    unsigned char* op_lo = op_hi + kGramOperand;
-    if (it == 0 || blk == 0) sr = exp2_int(-pow2_exponent(__uint_as_float(p.Rmax[tile])));
-    ok = bar_wait(&full[s], (uint32_t)(it / kGramStages) & 1u) && ok;
-    if (it >= 2) products_up_to((uint32_t)it - 1u);                          // this operand buffer is free again
-    const float4* src = reinterpret_cast<const float4*>(stage + s * kGramStage);
+  if (warp == kGramWarps) {
+    if (lane == 0) {
+      // descriptors: 128B swizzle, 64-channel halves 4 KB apart (leading), 8-token groups 1 KB apart (stride); the remainders
+      // follow the heads, so the N = 256 operand has the same strides; fp32 accumulator, fp16 operands, both MN-major
+      constexpr uint64_t kDesc = ((uint64_t)(kGramOperand / 2 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+      constexpr uint32_t kIdesc = (1u << 4) | (1u << 15) | (1u << 16) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
+      int q_it = 0, q_tile = tile, q_blk = blk;
+      auto request_next = [&]() {
+        const int s = q_it % kGramStages;
+        const float* src = p.R + ((size_t)q_tile * p.n_c + (size_t)q_blk * kGramRows) * kHeadDim;
+        const uint32_t bytes = (uint32_t)min(kGramRows, p.n_c - q_blk * kGramRows) * kHeadDim * 4;
+        bar_expect(&full[s], bytes);
+        bulk_copy(stage + s * kGramStage, src, bytes, &full[s]);
+        ++q_it;
+        if (++q_blk == sp.nb) { q_blk = 0; ++q_tile; }
+      };
+      for (int s = 0; s < kGramStages && s < count; ++s) request_next();
+      for (int it = 0; it < count; ++it) {
+        ok = ok && bar_wait(&ready[it & 1], (uint32_t)(it >> 1) & 1u);
+        if (ok) {
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t op = kDesc | (smem_addr(smem + (it & 1) * 2 * kGramOperand) >> 4);
 #pragma unroll
-    for (int j = 0; j < kGramRows * 32 / 256; ++j) {
-      const int i = tid + 256 * j, row = i >> 5, q = i & 31;        // four channels of a row
-      const float4 v = row < rows ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-      uint32_t h0, l0, h1, l1;
-      split_pair(v.x * sr, v.y * sr, h0, l0);
-      split_pair(v.z * sr, v.w * sr, h1, l1);
-      const int at = (q >> 4) * (kGramOperand / 2) + (row >> 3) * 1024 + (row & 7) * 128 + ((((q & 15) >> 1) ^ (row & 7)) << 4) + (q & 1) * 8;
-      *reinterpret_cast<uint2*>(op_hi + at) = make_uint2(h0, h1);
-      *reinterpret_cast<uint2*>(op_lo + at) = make_uint2(l0, l1);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    if (__syncthreads_or(!ok)) { ok = false; break; }
-    ++mma_issued;
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t d_hi = kDesc | (smem_addr(op_hi) >> 4);
-#pragma unroll
-      for (int k = 0; k < kGramRows / 16; ++k) {
-        const uint64_t op = d_hi + k * (2048 >> 4);
-        umma_f16(tmem, op, op, kIdesc, (fresh && k == 0) ? 0u : 1u);
-      }
-      umma_commit(&mma_done[it & 1]);
-      if (q_it < count) request_next();
-    }
-    fresh = false;
-    if (it + 1 == count || blk + 1 == sp.nb) {                      // last block of the tile in this range: leave the partial
-      products_up_to(mma_issued);
-      if (__syncthreads_or(!ok)) { ok = false; ++it; break; }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // columns 0..127 of accumulator row i are h h, 128..255 h l.  First (h h + h l)[i][c] goes to row c of the partial (h h
-      // is symmetric), so that a warp writes 128 consecutive bytes; then h l[i][c] is added to row i, column c
-      float* part = p.Gpart + (size_t)(blockIdx.x + tile) * kHeadDim * kHeadDim;
-      const int i = (warp & 3) * 32 + lane;
-      const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-#pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
-        const int c0 = (warp >> 2) * 64 + h * 32;
-        uint32_t v[32], w[32];
-        tmem_ld32(v, lanes + c0);
-        tmem_ld32(w, lanes + 128 + c0);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) part[(size_t)(c0 + c) * kHeadDim + i] = __uint_as_float(v[c]) + __uint_as_float(w[c]);
-      }
-      __syncthreads();
-#pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
-        const int c0 = (warp >> 2) * 64 + h * 32;
-        uint32_t w[32];
-        tmem_ld32(w, lanes + 128 + c0);
-        float4* row = reinterpret_cast<float4*>(part + (size_t)i * kHeadDim + c0);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          float4 g = __ldcg(row + c);
-          g.x += __uint_as_float(w[4 * c]); g.y += __uint_as_float(w[4 * c + 1]);
-          g.z += __uint_as_float(w[4 * c + 2]); g.w += __uint_as_float(w[4 * c + 3]);
-          row[c] = g;
+          for (int k = 0; k < kGramRows / 16; ++k)
+            umma_f16(tmem, op + k * (2048 >> 4), op + k * (2048 >> 4), kIdesc, ((it == 0 || blk == 0) && k == 0) ? 0u : 1u);
+          umma_commit(&mma_done[it & 1]);
+          if (q_it < count) request_next();
         }
+        if (++blk == sp.nb) blk = 0;
       }
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      fresh = true;
+      if (!ok) {
+        atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
+        for (int it = max(0, q_it - kGramStages); it < q_it; ++it)  // let the copies in flight land (bounded)
+          bar_wait(&full[it % kGramStages], (uint32_t)(it / kGramStages) & 1u);
+      }
     }
-    if (++blk == sp.nb) { blk = 0; ++tile; }
+  } else {
+    float sr = 0.f;
+    for (int it = 0; it < count; ++it) {
+      const int s = it % kGramStages, rows = min(kGramRows, p.n_c - blk * kGramRows);
+      unsigned char* op_hi = smem + (it & 1) * 2 * kGramOperand;
+      unsigned char* op_lo = op_hi + kGramOperand;
+      if (it == 0 || blk == 0) sr = exp2_int(-pow2_exponent(__uint_as_float(p.Rmax[tile])));
+      ok = ok && bar_wait(&full[s], (uint32_t)(it / kGramStages) & 1u);
+      if (it >= 2) ok = ok && bar_wait(&mma_done[it & 1], (uint32_t)((it - 2) >> 1) & 1u);    // this operand buffer is free again
+      const float4* src = reinterpret_cast<const float4*>(stage + s * kGramStage);
+#pragma unroll
+      for (int j = 0; j < kGramRows / kGramWarps; ++j) {
+        const int row = warp + kGramWarps * j, q = lane;            // a row per warp, four channels per lane
+        const float4 v = row < rows ? src[row * 32 + q] : make_float4(0.f, 0.f, 0.f, 0.f);
+        uint32_t h0, l0, h1, l1;
+        split_pair(v.x * sr, v.y * sr, h0, l0);
+        split_pair(v.z * sr, v.w * sr, h1, l1);
+        const int at = (q >> 4) * (kGramOperand / 2) + (row >> 3) * 1024 + (row & 7) * 128 + ((((q & 15) >> 1) ^ (row & 7)) << 4) + (q & 1) * 8;
+        *reinterpret_cast<uint2*>(op_hi + at) = make_uint2(h0, h1);
+        *reinterpret_cast<uint2*>(op_lo + at) = make_uint2(l0, l1);
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) bar_arrive(&ready[it & 1]);
+      if (it + 1 == count || blk + 1 == sp.nb) {                    // last block of the tile in this range: leave the partial
+        ok = ok && bar_wait(&mma_done[it & 1], (uint32_t)(it >> 1) & 1u);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        __syncwarp();
+        // columns 0..127 of accumulator row i are h h, 128..255 h l; plane 0 of the partial gets (h h + h l)[i][c] in row c
+        // (h h is symmetric), plane 1 h l[i][c] in row c: a warp writes 128 consecutive bytes.  The transpose of h l is
+        // taken where the partials are summed (adding it here costs a second trip to L2: 41 us of 220 at 512 tiles)
+        float* part = p.Gpart + (size_t)(blockIdx.x + tile) * kGramPartial + (warp & 3) * 32 + lane;
+        const uint32_t lanes = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          const int c0 = (warp >> 2) * 64 + h * 32;
+          uint32_t v[32], w[32];
+          tmem_ld32(v, lanes + c0);
+          tmem_ld32(w, lanes + 128 + c0);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) {
+            part[(size_t)(c0 + c) * kHeadDim] = __uint_as_float(v[c]) + __uint_as_float(w[c]);
+            part[(size_t)(kHeadDim + c0 + c) * kHeadDim] = __uint_as_float(w[c]);
+          }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      }
+      if (++blk == sp.nb) { blk = 0; ++tile; }
+    }
+    if (!ok && lane == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
   }
-  if (!ok && tid == 0) {                                            // gave up (all threads): report, let the copies in flight land (bounded)
-    atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
-    for (; it < q_it; ++it) bar_wait(&full[it % kGramStages], (uint32_t)(it / kGramStages) & 1u);
-  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
+  if (warp == kGramWarps) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
+}
+
+// G of every tile from its partials (fixed order): 8 rows per CTA, thread i sums column i.  Plane 0 is read by rows, of plane
+// 1 (the transpose is wanted) the thread takes one 32-byte sector of row i.  Few tiles have many partials each (one
+// per CTA of the Gram kernel); 16 CTAs per tile keep their sum short.  Bound: the partials, from L2.
+constexpr int kSumRows = 8;
+__global__ void __launch_bounds__(kHeadDim) pi_gram_sum_kernel(PiArgs p, int gram_ctas, int sms) {
+  const int tile = blockIdx.y, k0 = blockIdx.x * kSumRows, i = threadIdx.x;
+  const GramSplit sp = gram_split(p.ntiles, p.n_c, sms);
+  const long long NW = gram_ctas, b0 = (long long)tile * sp.nb, b1 = b0 + sp.nb;
+  const int w0 = (int)(((b0 + 1) * NW + sp.blocks - 1) / sp.blocks - 1), w1 = (int)((b1 * NW + sp.blocks - 1) / sp.blocks - 1);
+  float g[kSumRows];
+#pragma unroll
+  for (int k = 0; k < kSumRows; ++k) g[k] = 0.f;
+  const float* src = p.Gpart + (size_t)(w0 + tile) * kGramPartial;
+#pragma unroll 2
+  for (int w = w0; w <= w1; ++w, src += kGramPartial) {
+    const float4* hl = reinterpret_cast<const float4*>(src + (size_t)(kHeadDim + i) * kHeadDim + k0);
+    const float4 a = __ldcg(hl), b = __ldcg(hl + 1);
+#pragma unroll
+    for (int k = 0; k < kSumRows; ++k) g[k] += __ldcg(src + (size_t)(k0 + k) * kHeadDim + i);
+    g[0] += a.x; g[1] += a.y; g[2] += a.z; g[3] += a.w;
+    g[4] += b.x; g[5] += b.y; g[6] += b.z; g[7] += b.w;
+  }
+#pragma unroll
+  for (int k = 0; k < kSumRows; ++k) p.G[((size_t)tile * kHeadDim + k0 + k) * kHeadDim + i] = g[k];
 }
 
 // ------------------------------------------------------------------ the loops on G
@@ -206,10 +223,10 @@ __global__ void __launch_bounds__(256, 2) pi_gram_kernel(PiArgs p, int sms) {
 //   B <- Q(B), classical Gram-Schmidt with each projection taken twice, one warp;
 //   G0 = B^T G B is the Gram matrix of A0 = R B up to rounding: U^-1 of its Cholesky factor, folded into B, makes the
 //   columns of R B nearly orthonormal before they are computed, so one explicit round of CholeskyQR is enough after.
-// Bound: latency of the chain (partials from L2, products, Gram-Schmidt, Cholesky); r^2 and 128 r work per step.
+// Bound: latency of the chain (G from L2, products, Gram-Schmidt, Cholesky); r^2 and 128 r work per step.
 template <int RP>
 __global__ void __launch_bounds__(256) pi_iterate_kernel(PiArgs p, const float* B0, unsigned long long seed, int segment,
-                                                         int iters, int gram_ctas, int sms) {
+                                                         int iters) {
   __shared__ __align__(16) float Bs[kHeadDim][RP];
   __shared__ __align__(16) float Cs[kHeadDim][RP];
   __shared__ float Gm[RP][RP + 1], Wm[RP][RP + 1];
@@ -218,16 +235,9 @@ __global__ void __launch_bounds__(256) pi_iterate_kernel(PiArgs p, const float* 
   const int r = p.rank;
   float g[64];
   {
-    const GramSplit sp = gram_split(p.ntiles, p.n_c, sms);
-    const long long NW = gram_ctas, b0 = (long long)tile * sp.nb, b1 = b0 + sp.nb;
-    const long long w0 = ((b0 + 1) * NW + sp.blocks - 1) / sp.blocks - 1, w1 = (b1 * NW + sp.blocks - 1) / sp.blocks - 1;
+    const float* src = p.G + ((size_t)tile * kHeadDim + half * 64) * kHeadDim + i;
 #pragma unroll
-    for (int k = 0; k < 64; ++k) g[k] = 0.f;
-    for (long long w = w0; w <= w1; ++w) {
-      const float* src = p.Gpart + (size_t)(w + tile) * kHeadDim * kHeadDim + (size_t)(half * 64) * kHeadDim + i;
-#pragma unroll
-      for (int k = 0; k < 64; ++k) g[k] += __ldcg(src + k * kHeadDim);
-    }
+    for (int k = 0; k < 64; ++k) g[k] = __ldcg(src + (size_t)k * kHeadDim);
   }
   if (half == 0) {
     const size_t gtile = (size_t)p.bh0 * 2 + tile;
@@ -369,11 +379,12 @@ cudaError_t launch_pi_gram(const PiArgs& p, const float* B0, unsigned long long 
   const GramSplit sp = gram_split(p.ntiles, p.n_c, sms);
   cudaError_t e = cudaFuncSetAttribute(pi_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramSmem);
   if (e != cudaSuccess) return e;
-  pi_gram_kernel<<<sp.ctas, 256, kGramSmem, st>>>(p, sms);
-  if (p.rank <= 4) pi_iterate_kernel<4><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters, sp.ctas, sms);
-  else if (p.rank <= 8) pi_iterate_kernel<8><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters, sp.ctas, sms);
-  else pi_iterate_kernel<16><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters, sp.ctas, sms);
-  count_launches(2);
+  pi_gram_kernel<<<sp.ctas, kGramWarps * 32 + 32, kGramSmem, st>>>(p, sms);
+  pi_gram_sum_kernel<<<dim3(kHeadDim / kSumRows, p.ntiles), kHeadDim, 0, st>>>(p, sp.ctas, sms);
+  if (p.rank <= 4) pi_iterate_kernel<4><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters);
+  else if (p.rank <= 8) pi_iterate_kernel<8><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters);
+  else pi_iterate_kernel<16><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters);
+  count_launches(3);
   return cudaGetLastError();
 }
 

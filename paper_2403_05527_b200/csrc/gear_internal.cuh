@@ -45,7 +45,8 @@ struct PiArgs {
   unsigned char* arena;
   float* R;             // [ntiles][n_c][128]
   unsigned int* Rmax;   // [ntiles] bit pattern of the tile's largest |R|
-  float* Gpart;         // partials of R^T R, [CTA + tile][128][128] (gear_gram.cu)
+  float* Gpart;         // partials of R^T R, [CTA + tile][2][128][128] (gear_gram.cu)
+  float* G;             // [ntiles][128][128]: R^T R (of R scaled by the tile's power of two)
   int* status;          // the cache's status word
   float* Bcur;          // [ntiles][128][16]
   float* Bg;            // [ntiles][128][16]: (R^T R) Bcur = R^T A0

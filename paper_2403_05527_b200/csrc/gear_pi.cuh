@@ -9,8 +9,11 @@ namespace gear {
 
 // ------------------------------------------------------------------ bulk copies and barriers
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void bar_init(uint64_t* b) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(b)) : "memory");
+__device__ __forceinline__ void bar_init(uint64_t* b, int count = 1) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint64_t* b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(b)) : "memory");
 }
 // bounded: false when the phase did not complete within the limit
 __device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
