@@ -173,7 +173,7 @@ struct gear_cache {
   int* blk2seg; int blk_cap;                             // segment index of every compressed block
   void* buf_k; void* buf_v;                              // [BH][n_b][128] fp16
   unsigned char* flush_ws; size_t flush_ws_bytes;
-  float* partial; size_t partial_bytes; int max_parts;
+  float* partial; size_t partial_bytes;
   int* tickets; int* status;                             // one block; zeroed on the caller's stream by the first call (scratch_clean)
   bool scratch_clean;
   void* stage_q; float* stage_out; float* stage_b0;      // for the *_host calls: query; result for pageable destinations; B0
@@ -298,6 +298,17 @@ static bool scratch_zeroed(gear_cache* c, cudaStream_t st) {
   return true;
 }
 
+// Partial results of a launch for G query rows per kv head: slots per unit (a unit's share of the launch's CTAs, the first and
+// the last of which may be shared with its neighbours), and the bytes of all slots.
+static int partial_slots(const gear_cache* c, int G) {
+  const size_t units = (size_t)c->cc.BH * decode_passes(G);
+  const size_t ctas = (size_t)c->sm_count * (G == 1 ? 32 : kRowsCtasPerSm);
+  return (int)(ctas / units + 3);
+}
+static size_t partial_bytes_for(const gear_cache* c, int G) {
+  return (size_t)c->cc.BH * decode_passes(G) * partial_slots(c, G) * (size_t)decode_heads_per_pass(G) * kPartRow * 4;
+}
+
 #define GEAR_TRY_ALLOC(ptr, bytes)                                                   \
   do {                                                                               \
     *reinterpret_cast<void**>(&(ptr)) = c->mem.get(bytes);                           \
@@ -376,13 +387,15 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
   // decode scratch: one partial per (unit, warp touching it); upper bound of warps in a launch
   // scratch for the largest group of query rows a call may bring: G query heads x max_queries rows per kv head
   c->max_queries = cfg->max_queries > 1 ? (int)cfg->max_queries : 1;
-  const int hp = decode_heads_per_pass(c->G * c->max_queries);
-  const int passes = decode_passes(c->G * c->max_queries);
-  c->units_alloc = (int)(BH * passes);
-  const size_t units = BH * passes;
-  const size_t nw_max = (size_t)c->sm_count * 32;        // one warp per CTA, at most 32 CTAs per SM
-  c->max_parts = (int)(nw_max / units + 3);
-  c->partial_bytes = units * c->max_parts * (size_t)hp * kPartRow * 4;
+  const int Gs[2] = {c->G, c->G * c->max_queries};
+  c->units_alloc = 0; c->partial_bytes = 0;
+  for (int G : Gs) {
+    const size_t n = partial_bytes_for(c, G);
+    if (n > c->partial_bytes) c->partial_bytes = n;
+    const int un = (int)(BH * decode_passes(G));
+    if (un > c->units_alloc) c->units_alloc = un;
+  }
+  const size_t units = (size_t)c->units_alloc;
   GEAR_TRY_ALLOC(c->partial, c->partial_bytes);
   GEAR_TRY_ALLOC(c->tickets, (units + 1) * 4);
   c->status = c->tickets + units;
@@ -552,9 +565,12 @@ static gear_status plan_decode(gear_cache* c, int Gq) {
     if (s.bfac_bytes > max_bfac) max_bfac = s.bfac_bytes;
     if ((s.T + 31) / 32 * 32 > max_T) max_T = (s.T + 31) / 32 * 32;
   }
-  if (!decode_plan(c->cc.bits, Gq, c->cc.ngv, max_k, max_v, max_bfac, max_T, kDecodeSmemBudget, warps_cap, &c->plan))
+  if (Gq == 1 ? !decode_plan(c->cc.bits, Gq, c->cc.ngv, max_k, max_v, max_bfac, max_T, kDecodeSmemBudget, warps_cap, &c->plan)
+              : !rows_plan(Gq, c->cc.ngv, max_k, max_v, max_bfac, max_T, &c->plan))
     return GEAR_ERR_SHAPE;
-  const int occ = decode_occupancy(c->cc.bits, Gq, c->cc.ngv, c->plan.wide, (size_t)c->plan.ws.total);
+  int occ = Gq == 1 ? decode_occupancy(c->cc.bits, Gq, c->cc.ngv, c->plan.wide, (size_t)c->plan.ws.total)
+                    : rows_occupancy(c->plan, c->cc.bits, c->cc.ngv);
+  if (Gq > 1 && occ > kRowsCtasPerSm) occ = kRowsCtasPerSm;      // what the partial slots are for
   if (occ < 1) return GEAR_ERR_CUDA;
   c->plan_occ = occ;
   c->plan_key = key;
@@ -581,15 +597,13 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
     const unsigned long long call = next_call_number((cudaStream_t)stream);
     a.early_reads = c->written && c->write_stream == (cudaStream_t)stream && call >= c->write_call + 2 ? 1 : 0;
   }
-  // one warp per CTA; never more warps than blocks of work
+  // never more CTAs than blocks of work
   const int passes = decode_passes(Gq);
   if ((long long)c->cc.BH * passes > c->units_alloc) return GEAR_ERR_CAPACITY;
-  // partial slots per unit for this call's unit count (the scratch was sized for the most units: fewer units get more
-  // slots each out of the same memory)
-  a.max_parts = (int)((size_t)c->sm_count * 32 / ((size_t)c->cc.BH * passes) + 3);
-  if ((size_t)c->cc.BH * passes * a.max_parts * decode_heads_per_pass(Gq) * kPartRow * 4 > c->partial_bytes)
-    return GEAR_ERR_CAPACITY;
-  const long long work = (long long)c->cc.BH * passes * (c->n_blocks_c + (c->buf_len + 15) / 16);
+  a.max_parts = partial_slots(c, Gq);
+  if (partial_bytes_for(c, Gq) > c->partial_bytes) return GEAR_ERR_CAPACITY;
+  const int buf_block = Gq == 1 ? 16 : kRowsBufBlock;
+  const long long work = (long long)c->cc.BH * passes * (c->n_blocks_c + (c->buf_len + buf_block - 1) / buf_block);
   long long grid = (long long)c->sm_count * c->plan_occ;
   if (grid > work) grid = work;
   // With few blocks per warp, a warp that runs from one unit into the next pays a second prologue and epilogue and
@@ -621,7 +635,7 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
       grid = start;                                                     // = units * pb + ua
     }
   }
-  if (launch_decode(a, (int)grid, (cudaStream_t)stream) != cudaSuccess) {
+  if ((Gq == 1 ? launch_decode(a, (int)grid, (cudaStream_t)stream) : launch_rows(a, (int)grid, (cudaStream_t)stream)) != cudaSuccess) {
     cudaGetLastError();
     return GEAR_ERR_CUDA;
   }

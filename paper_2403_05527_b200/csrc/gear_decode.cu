@@ -34,17 +34,12 @@
 
 #include <type_traits>
 
-#include "gear_internal.cuh"
+#include "gear_decode.cuh"
 
 namespace gear {
 
-constexpr int kBufPitch = 272;                  // bytes per fp16 row of a buffer slab in shared memory
 constexpr int kBufItem = kSlab * kBufPitch;     // one slab of key rows or of value rows
 constexpr int kCsrAhead = 6;                    // outlier-list entries per lane requested one block ahead (per-vector keys)
-constexpr int kFragKRow = 40;                   // 32-bit words per (head, limb) row of the key B-operand staging area
-constexpr int kTokLimit = 16384;                // tokens a value accumulator takes before it is folded (int32 headroom)
-constexpr float kMagic = 12582912.0f;           // 1.5 * 2^23: x + kMagic carries rint(x) in its low mantissa bits, |x| < 2^22
-constexpr uint32_t kMagicBits = 0x4B400000u;
 // 32-bit words per fp16 B-fragment row set.  A row set holds, for every column that carries a query head (hi, lo) and
 // every lane column t, two registers; with one head only two of the eight columns exist and the lanes of the other
 // columns read those (their results are never used).  Padded against bank conflicts.
@@ -52,111 +47,11 @@ __host__ __device__ constexpr int frag_row_words(int hp) { return hp == 1 ? 24 :
 
 static_assert(sizeof(SegDesc) <= 128 && sizeof(SegDesc) % 4 == 0, "descriptor copy assumes <= 32 words");
 
-// ------------------------------------------------------------------ PTX helpers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(uint64_t* b, int count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* b) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(b))
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok)
-      : "r"(smem_u32(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait: gives up after `limit` polls and reports through `status`.
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, int limit, int* status) {
-#pragma unroll 1
-  for (int i = 0; i < limit; ++i)
-    if (mbar_try(b, parity)) return true;
-  atomicExch(status, -7 /* GEAR_ERR_TIMEOUT */);
-  return false;
-}
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// d = a * b (no accumulator input)
-__device__ __forceinline__ void mma16816_z(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  const float z = 0.f;
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
-      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(z));
-}
-// integer product: A unsigned bytes (codes in place), B signed bytes (limbs), 32-bit sums
-__device__ __forceinline__ void imma16832(int (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(smem_u32(p)));
-}
-__device__ __forceinline__ uint32_t h2_as_u32(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }
-__device__ __forceinline__ __half2 u32_as_h2(uint32_t u) { return *reinterpret_cast<__half2*>(&u); }
-
-// mask of field j of every byte of a word of packed codes
-template <int BITS>
-__host__ __device__ constexpr uint32_t field_mask(int j) {
-  return BITS == 2 ? (0x03030303u << (2 * j)) : (0x0F0F0F0Fu << (4 * j));
-}
-// Signed base-256 digits of a 32-bit integer y, |y| < 2^31 - 2^23: byte l of the result, read as a signed byte, is
-// digit l, and sum digit_l * 256^l = y.
-__device__ __forceinline__ uint32_t balanced_digits(uint32_t y) { return (y + 0x80808080u) ^ 0x80808080u; }
-
-// fp32 pair -> half2 of the high parts and half2 of the rounding remainders
-__device__ __forceinline__ void split_hi_lo(float x0, float x1, uint32_t& hi, uint32_t& lo) {
-  const __half2 h = __floats2half2_rn(x0, x1);
-  hi = h2_as_u32(h);
-  lo = h2_as_u32(__floats2half2_rn(x0 - __low2float(h), x1 - __high2float(h)));
-}
-
-// maximum over the warp in one instruction
-__device__ __forceinline__ float warp_max(float x) {
-  float r;
-  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ uint32_t warp_max_u32(uint32_t x) { return __reduce_max_sync(0xffffffffu, x); }
-__device__ __forceinline__ int float_exponent(float x) { return (int)((__float_as_uint(x) >> 23) & 0xFFu) - 127; }
-// 2^x for x <= 0 (scores minus a maximum): one instruction, relative error about 2^-22, flushes tiny results to zero
-__device__ __forceinline__ float exp2_fast(float x) {
-  float r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-// 2^e for |e| <= 120
-__device__ __forceinline__ float pow2i(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
-__device__ __forceinline__ int clamp60(int e) { return max(-60, min(60, e)); }
-
 // ------------------------------------------------------------------ shared memory plan (per warp)
 bool decode_plan(int bits, int heads, int ngv, int max_kpart, int max_vpart, int max_bfac, int max_T, size_t smem_budget,
                  int warps_cap, DecodeArgs* a) {
   (void)bits;
-  const int HP = decode_heads_per_pass(heads);
+  const int HP = fp16_heads_per_pass(heads);
   const int frs = frag_row_words(HP);
   const int bregion = round_up(max_bfac / 2, 16);
   int part = max_kpart > max_vpart ? max_kpart : max_vpart;
@@ -211,48 +106,6 @@ bool decode_plan(int bits, int heads, int ngv, int max_kpart, int max_vpart, int
 }
 
 // ------------------------------------------------------------------ block shapes
-// The work on a block depends on its shape: tokens T, outliers per key group, padded rank, outliers per value
-// group.  The shapes of the usual configurations are compile-time constants (every offset inside the record becomes
-// an immediate and the loops unroll); any other segment runs through the same code with run-time values.
-struct DynShape {                      // values read from the segment descriptor
-  static constexpr bool kDyn = true, kCsr = true;     // kCsr: the segment may keep its key outliers in a list
-  static constexpr int T = 0, k2k = 0, r_pad = 0, k2v = 0, unroll = 1;
-  static constexpr int off_kscale = 0, off_koval = 0, off_koidx = 0, off_kcodes = 0, off_ak = 0, off_av = 0, off_vscale = 0,
-                       off_voval = 0, off_voidx = 0;
-};
-template <int BITS, int NGV, int T_, int KK, int RP, int KV, bool CSR = false>
-struct StaticShape {                   // mirrors layout_segment(); checked against it on the host (static_shape_id)
-  static constexpr bool kDyn = false, kCsr = CSR;
-  static constexpr int T = T_, k2k = 2 * KK, r_pad = RP, k2v = 2 * KV, unroll = 2;
-  static constexpr int nslab = T_ / kSlab, slab_codes = kSlab * kHeadDim * BITS / 8, nchunk = (T_ + 31) / 32;
-  static constexpr int off_kscale = kRecHeader;
-  static constexpr int off_koval = off_kscale + kHeadDim * 4;
-  static constexpr int off_koidx = off_koval + kHeadDim * 2 * KK * 2;
-  static constexpr int off_kcodes = off_koidx + (kHeadDim * 2 * KK + 15) / 16 * 16;
-  static constexpr int off_ak = off_kcodes + nslab * slab_codes;
-  static constexpr int off_vpart = off_ak + (nslab * kSlab * RP * 2 + 15) / 16 * 16;
-  // value part, relative to its start
-  static constexpr int off_av = nchunk * 2 * slab_codes;
-  static constexpr int off_vscale = off_av + (nslab * kSlab * RP * 2 + 15) / 16 * 16;
-  static constexpr int off_voval = off_vscale + T_ * NGV * 4;
-  static constexpr int off_voidx = off_voval + (T_ * NGV * 2 * KV * 2 + 15) / 16 * 16;
-  static constexpr int rec_bytes = off_vpart + off_voidx + (T_ * NGV * 2 * KV + 15) / 16 * 16;
-  static bool matches(const SegDesc& s, const CacheConst& c) {
-    return c.bits == BITS && c.ngv == NGV && c.k_v == KV && s.T == T_ && s.k_k == KK && s.r_pad == RP &&
-           (s.csr_base16 != 0) == CSR &&
-           s.off_kscale == off_kscale && s.off_koval == off_koval && s.off_koidx == off_koidx &&
-           s.off_kcodes == off_kcodes && s.off_ak == off_ak && s.off_vpart == off_vpart &&
-           s.off_vcodes == off_vpart && s.off_av == off_vpart + off_av && s.off_vscale == off_vpart + off_vscale &&
-           s.off_voval == off_vpart + off_voval && s.off_voidx == off_vpart + off_voidx && s.rec_bytes == rec_bytes;
-  }
-};
-// static shapes by id (0 = none).  Two value groups per token (g = 64): ids 1, 2; one group (g = 128): ids 3, 4.
-template <int BITS> using ShapeA1 = StaticShape<BITS, 2, 64, 1, 4, 1>;     // g 64, s <= 3 %, rank 3..4
-template <int BITS> using ShapeA2 = StaticShape<BITS, 2, 64, 1, 8, 1>;     // g 64, rank 5..8
-template <int BITS> using ShapeB1 = StaticShape<BITS, 1, 128, 2, 4, 2>;    // g 128 prefill blocks
-template <int BITS> using ShapeB2 = StaticShape<BITS, 1, 64, 1, 4, 2>;     // g 128, flushed 64-token buffers
-template <int BITS> using ShapeP1 = StaticShape<BITS, 1, 64, 0, 4, 2, true>;   // per-vector keys (outlier list), rank 3..4
-
 int static_shape_id(const SegDesc& s, const CacheConst& c) {
   if (ShapeA1<2>::matches(s, c) || ShapeA1<4>::matches(s, c)) return 1;
   if (ShapeA2<2>::matches(s, c) || ShapeA2<4>::matches(s, c)) return 2;
@@ -263,7 +116,8 @@ int static_shape_id(const SegDesc& s, const CacheConst& c) {
 }
 
 // ------------------------------------------------------------------ the kernel
-// HEADS = query heads handled per pass: 1 (multi-head attention) or 4 (grouped queries; a pass may hold fewer).
+// HEADS = query heads handled per pass: 1, or 4 for grouped queries over an fp16 cache (a pass may hold fewer); compressed
+// caches with several query rows per kv head take gear_decode_rows_kernel.
 // MINB = resident warps per SM the registers are budgeted for: 16 (128 registers) or 12 (168 registers: about a tenth
 // fewer instructions, for long streams where twelve warps are enough) with one head per pass, 8 with four.
 template <int BITS, int HEADS, int NGV, int MINB>
@@ -483,7 +337,7 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
     };
 
     // ==================================================================== compressed blocks
-    if (blk_lo < c_hi) {
+    if (HEADS == 1 && blk_lo < c_hi) {
       int O[8][NT][4];                                   // value sums: tile (16 channels) x column tile, 32-bit integers
       float U[4], cm[HP][NGV];
       uint32_t bw[NT][2];                                // low-rank key term: B operand (q B_K) of the current segment
@@ -682,36 +536,13 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
                 row[3 * kFragKRow] = __byte_perm(p01h, p23h, 0x7632);
 
                 float c = fmaf(qv[0], zr4[0], fmaf(qv[1], zr4[1], fmaf(qv[2], zr4[2], qv[3] * zr4[3])));   // this lane's part
-                if (HP != 4) {
 #pragma unroll
-                  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-                }
+                for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
                 const int sexp = clamp60(21 - qexp_s[h] - ed);
                 const float Sx = pow2i(sexp);
                 qS[h][0] = qv[0] * Sx; qS[h][1] = qv[1] * Sx; qS[h][2] = qv[2] * Sx; qS[h][3] = qv[3] * Sx;
                 c_zero[h] = c; sexp_k[h] = sexp;
               }
-            }
-            if (HP == 4) {            // c_zero of four heads: sums over the warp
-              // four sums at once: two exchange steps halve what a lane carries, a butterfly finishes the one value left
-              // (head 2 * bit4 + bit3 of the lane), four broadcasts hand the sums back: 10 shuffles instead of 20
-              float s0 = c_zero[0], s1 = c_zero[1 % HP];
-              {
-                const bool up = (lane & 16) != 0;
-                const float send0 = up ? c_zero[0] : c_zero[2 % HP], keep0 = up ? c_zero[2 % HP] : c_zero[0];
-                const float send1 = up ? c_zero[1 % HP] : c_zero[3 % HP], keep1 = up ? c_zero[3 % HP] : c_zero[1 % HP];
-                s0 = keep0 + __shfl_xor_sync(0xffffffffu, send0, 16);
-                s1 = keep1 + __shfl_xor_sync(0xffffffffu, send1, 16);
-              }
-              {
-                const bool up = (lane & 8) != 0;
-                const float send = up ? s0 : s1, keep = up ? s1 : s0;
-                s0 = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-              }
-#pragma unroll
-              for (int o = 4; o > 0; o >>= 1) s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-#pragma unroll
-              for (int h = 0; h < HP; ++h) c_zero[h] = __shfl_sync(0xffffffffu, s0, 8 * h);
             }
             // what turns this lane's integer sums of column tile nt into scores: the inverse fixed-point scale of the
             // head it serves, the weight of the highest field, and 2^16 for the high limb pair
@@ -891,12 +722,21 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
           // ---------------- softmax over the block, the B operands of the value products and the sparse value term in
           //                  one pass over this lane's token pairs (pairs lane, lane + 32), probabilities in registers
           constexpr int NPR = S::kDyn ? 2 : (S::T > 64 ? S::T / 64 : 1);
+          // The integer value sums carry the scale 2^eV_cur, which a block keeps when p * scale * 2^eV_cur stays below 2^22 at
+          // p = 1 and is no more than three bits short of it (precision).  What is left of those bits is room for the
+          // running maximum to lag behind: it is moved, and everything summed so far scaled, only when a score exceeds it
+          // by more than that, because the integers have to be folded into the fp32 copy then.  (Every second or third
+          // block of a short range raises the maximum by a little.)
+          const int need = clamp60(21 - float_exponent(smax_v));
+          const bool exp_bad = eV_cur > need || eV_cur < need - 3;
+          const int eV_new = exp_bad ? need - kLag : eV_cur;
+          const float room = (float)(need - eV_new);
           float2 sc[HP][NPR];
-          float alpha[HP], m_new[HP];
+          float alpha[HP], m_new[HP], lag[HP];
           bool grew = false;
 #pragma unroll
           for (int h = 0; h < HP; ++h) {
-            alpha[h] = 1.f; m_new[h] = 0.f;
+            alpha[h] = 1.f; m_new[h] = 0.f; lag[h] = 1.f;
             if (h < HC) {
               const float Sik = pow2i(-sexp_k[h]);
               float mx = -INFINITY;
@@ -918,21 +758,19 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
                 mx = fmaxf(mx, fmaxf(v.x, v.y));
               }
               mx = warp_max(mx);
-              m_new[h] = fmaxf(m_run[h], mx);
-              if (m_new[h] > m_run[h]) {                    // warp-uniform
-                alpha[h] = exp2f(m_run[h] - m_new[h]);
-                m_run[h] = m_new[h];
+              if (mx > m_run[h] + room) {                   // warp-uniform
+                alpha[h] = exp2f(m_run[h] - mx);
+                m_run[h] = mx;
                 grew = true;
               }
+              m_new[h] = m_run[h];
+              // the sparse value term's fixed point is set for probabilities of one at most: the block's own maximum
+              lag[h] = pow2i(-max(0, (int)ceilf(mx - m_new[h])));
             }
           }
-          // The integer value sums carry the scale 2^eV_cur.  They are folded into the fp32 copy when the running
-          // maximum grew (everything so far shrinks by alpha), when this block's scales do not fit that exponent (too
-          // large: overflow of the 22-bit image; more than three bits too small: precision), or when the 32-bit range
-          // nears its end.
+          // The integers are folded into the fp32 copy when the maximum moved (everything so far shrinks by alpha), when this
+          // block's scales do not fit their exponent, or when the 32-bit range nears its end.
           {
-            const int need = clamp60(21 - float_exponent(smax_v));      // p <= 1: p * scale * 2^need < 2^22
-            const bool exp_bad = eV_cur > need || eV_cur < need - 3;
             const bool conv = tok_acc > 0 && (grew || exp_bad || tok_acc + T > kTokLimit);
             if (conv) {
               fold_O(alpha);
@@ -954,7 +792,7 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
 #pragma unroll
                 for (int g = 0; g < NGV; ++g) cm[h][g] *= alpha[h];
             }
-            if (tok_acc == 0 && exp_bad) eV_cur = need;
+            eV_cur = eV_new;                    // a change comes with a fold (or with empty sums)
             tok_acc += T;
           }
           const float Sv = pow2i(eV_cur);
@@ -1025,7 +863,7 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
                   const float d = (val - __high2float(z[e2][g])) * Sx;
 #pragma unroll
                   for (int h = 0; h < HP; ++h)
-                    if (h < HC) atomicAdd(&corr_v[h * kHeadDim + g * GV + idx], __float2int_rn(p[h][e2] * d));
+                    if (h < HC) atomicAdd(&corr_v[h * kHeadDim + g * GV + idx], __float2int_rn(p[h][e2] * lag[h] * d));
                 };
                 if (NGV * k2v == 4) {
                   const uint2 ov = reinterpret_cast<const uint2*>(vp + o_voval)[tk];
@@ -1109,10 +947,10 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
 
           // ---------------- sparse value term: the fixed-point sums of this block join the fp32 copy
           if (k2v > 0) {
-            const float Si = 1.0f / Sx;
 #pragma unroll
             for (int h = 0; h < HP; ++h) {
               if (h < HC) {
+                const float Si = 1.0f / (Sx * lag[h]);
                 int4* cv = reinterpret_cast<int4*>(corr_v + h * kHeadDim) + lane;
                 float4* oc = reinterpret_cast<float4*>(ocorr + h * kHeadDim) + lane;
                 const int4 v = *cv;
@@ -1453,11 +1291,12 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
 // ------------------------------------------------------------------ host side
 template <class Fn>
 static bool with_decode_kernel(int bits, int heads, int ngv, int wide, Fn fn) {
-  const int hp = decode_heads_per_pass(heads);
+  const int hp = fp16_heads_per_pass(heads);
   const int minb = hp == 1 ? (wide ? 12 : 16) : 8;
 #define GEAR_DEC_CASE(B, N, V, M) \
   if (bits == B && hp == N && ngv == V && minb == M) { fn(gear_decode_kernel<B, N, V, M>); return true; }
-#define GEAR_DEC_HEADS(B, V) GEAR_DEC_CASE(B, 1, V, 16) GEAR_DEC_CASE(B, 1, V, 12) GEAR_DEC_CASE(B, 4, V, 8)
+#define GEAR_DEC_HEADS(B, V) GEAR_DEC_CASE(B, 1, V, 16) GEAR_DEC_CASE(B, 1, V, 12)
+  GEAR_DEC_CASE(2, 4, 1, 8)          // four heads: fp16 caches only (compressed ones take gear_decode_rows_kernel)
   GEAR_DEC_HEADS(2, 1) GEAR_DEC_HEADS(2, 2) GEAR_DEC_HEADS(2, 4) GEAR_DEC_HEADS(2, 8)
   GEAR_DEC_HEADS(4, 1) GEAR_DEC_HEADS(4, 2) GEAR_DEC_HEADS(4, 4) GEAR_DEC_HEADS(4, 8)
 #undef GEAR_DEC_HEADS

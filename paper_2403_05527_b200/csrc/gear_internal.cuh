@@ -108,6 +108,9 @@ struct WarpSmem {      // byte offsets of a warp's (= a CTA's) shared-memory reg
   int fragv_stride;    // words per row of the value B-operand staging area
   int fragp;           // byte offset of the fp16 probability fragments inside the xr region
 };
+struct RowsSmem {      // the same of a CTA of gear_decode_rows_kernel
+  int sdc, qs, qf, xk, fragv, fragp, ps, corr_k, corr_v, fold, usum, wl, scal, bars, ring, total;
+};
 struct DecodeArgs {
   const unsigned char* arena;
   const SegDesc* table;
@@ -135,12 +138,13 @@ struct DecodeArgs {
   int stage_bytes;            // bytes of one ring stage
   int bregion;                // bytes at the front of a stage reserved for one B factor
   int max_T;                  // largest block length over the segments
-  int hpa;                    // query heads per pass (1 or 4)
+  int hpa;                    // query rows per pass
   int spin_limit;             // polls a consumer spends on one ring stage before it gives up
   int test_dead_wait;         // test only: wait once on a barrier that nothing completes, with a short limit
   int wide;                   // one head per pass: use the kernel built for twelve resident warps (more registers)
   int early_reads;            // the cache's data was last written at least two launches back on this stream (see the kernel)
   WarpSmem ws;
+  RowsSmem rows;
   float scale_log2;           // softmax scale * log2(e)
 };
 cudaError_t launch_decode(const DecodeArgs& a, int grid, cudaStream_t st);
@@ -150,11 +154,22 @@ bool decode_plan(int bits, int heads, int ngv, int max_kpart, int max_vpart, int
                  int warps_cap, DecodeArgs* a);
 int decode_occupancy(int bits, int heads, int ngv, int wide, size_t smem);
 int static_shape_id(const SegDesc& s, const CacheConst& c);
-// query heads one pass of the kernel takes for G query heads per kv head, and the number of passes
-inline int decode_heads_per_pass(int G) { return G == 1 ? 1 : 4; }
+// query rows one pass over the cache takes for G rows per kv head, and the number of passes
+inline int decode_heads_per_pass(int G) { return G == 1 ? 1 : (G <= 4 ? 4 : 8); }
 inline int decode_passes(int G) { return (G + decode_heads_per_pass(G) - 1) / decode_heads_per_pass(G); }
+// several rows per pass (gear_decode_rows.cuh): warps of a CTA, CTAs per SM that registers and shared memory are planned for
+constexpr int kRowsWarps = 4;
+constexpr int kRowsCtasPerSm = 4;
+constexpr int kRowsBufBlock = 32;      // buffer tokens per block of work there (one row per pass: a slab)
+bool rows_plan(int heads, int ngv, int max_kpart, int max_vpart, int max_bfac, int max_T, DecodeArgs* a);
+int rows_occupancy(const DecodeArgs& a, int bits, int ngv);
+cudaError_t launch_rows(const DecodeArgs& a, int grid, cudaStream_t st);
+// the fp16-cache kernel takes one or four query heads per pass
+inline int fp16_heads_per_pass(int G) { return G == 1 ? 1 : 4; }
+inline int fp16_passes(int G) { return (G + fp16_heads_per_pass(G) - 1) / fp16_heads_per_pass(G); }
 constexpr int kDecodeSmemBudget = 227 * 1024;    // shared memory of an SM that a launch may spread over its warps
-constexpr int kDecodeSpinLimit = 4000000;
+constexpr unsigned int kWaitHintNs = 20000;       // longest suspension of one poll of a barrier
+constexpr int kDecodeSpinLimit = 200000;          // polls before a wait gives up: four seconds at most
 
 // fp16-cache attention
 cudaError_t launch_fp16_attn(const void* K, const void* V, const void* q, float* out, int batch, int n_q_heads,

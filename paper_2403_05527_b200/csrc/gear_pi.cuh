@@ -20,8 +20,8 @@ __device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
   uint32_t ok = 0;
 #pragma unroll 1
   for (int i = 0; i < kDecodeSpinLimit && !ok; ++i)
-    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(ok) : "r"(smem_addr(b)), "r"(parity) : "memory");
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(smem_addr(b)), "r"(parity), "r"(kWaitHintNs) : "memory");
   return ok != 0;
 }
 __device__ __forceinline__ void bar_expect(uint64_t* b, uint32_t bytes) {
