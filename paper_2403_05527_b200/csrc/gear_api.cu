@@ -192,8 +192,8 @@ struct gear_cache {
   DecodeArgs plan;
   int test_dead_wait;            // gear_test_dead_wait: the next decode calls wait on a barrier nothing completes
   int max_queries, units_alloc;  // query rows per head the scratch was sized for; units of that size
-  // the last call that wrote the cache (records, descriptors, buffer rows): its stream and its number on that stream
-  cudaStream_t write_stream; unsigned long long write_call; bool written;
+  // the last calls that wrote the segments (records, descriptors) and the buffer rows: stream and number on that stream
+  struct LastWrite { cudaStream_t stream; unsigned long long call; bool any; } seg_write, buf_write;
 };
 
 static int outlier_count(float s_pct, int len) {
@@ -330,7 +330,7 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
     c->mem.alloc = g_alloc; c->mem.free = g_free; c->mem.ctx = g_alloc_ctx;
   }
   c->test_dead_wait = 0;
-  c->write_stream = nullptr; c->write_call = 0; c->written = false;
+  c->seg_write = {nullptr, 0, false}; c->buf_write = {nullptr, 0, false};
   c->arena = nullptr; c->dbg = nullptr; c->table_dev = nullptr; c->blk2seg = nullptr; c->buf_k = c->buf_v = nullptr; c->flush_ws = nullptr;
   c->partial = nullptr; c->tickets = nullptr; c->status = nullptr;
   c->scratch_clean = false;
@@ -484,7 +484,7 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
   c->n_compressed += n;
   c->n_blocks_c += sd.nblk;
   c->plan_key = -1;
-  c->write_stream = st; c->write_call = next_call_number(st); c->written = true;
+  c->seg_write = {st, next_call_number(st), true};
   return GEAR_OK;
 }
 
@@ -529,7 +529,7 @@ static gear_status push_rows(gear_cache* c, const void* k_new, const void* v_new
     return GEAR_ERR_CUDA;
   }
   c->buf_len += 1;
-  c->write_stream = st; c->write_call = next_call_number(st); c->written = true;
+  c->buf_write = {st, next_call_number(st), true};
   if (c->buf_len < n_b) return GEAR_OK;
   gear_status s = compress_segment(c, c->buf_k, c->buf_v, n_b, c->cfg.rank_flush, B0_flush, true, st);
   if (s != GEAR_OK) { c->buf_len -= 1; return s; }
@@ -595,7 +595,9 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
   a.test_dead_wait = c->test_dead_wait;
   {
     const unsigned long long call = next_call_number((cudaStream_t)stream);
-    a.early_reads = c->written && c->write_stream == (cudaStream_t)stream && call >= c->write_call + 2 ? 1 : 0;
+    auto long_ago = [&](const gear_cache::LastWrite& w) { return w.stream == (cudaStream_t)stream && call >= w.call + 2; };
+    a.early_reads = c->seg_write.any && long_ago(c->seg_write) ? 1 : 0;
+    a.early_buf = !c->buf_write.any || long_ago(c->buf_write) ? 1 : 0;
   }
   // never more CTAs than blocks of work
   const int passes = decode_passes(Gq);
@@ -606,12 +608,31 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
   const long long work = (long long)c->cc.BH * passes * (c->n_blocks_c + (c->buf_len + buf_block - 1) / buf_block);
   long long grid = (long long)c->sm_count * c->plan_occ;
   if (grid > work) grid = work;
+  // Ranges of one or two blocks: a warp's partial result, its ticket and the merge of up to 64 partials then take as long as
+  // the blocks themselves (8 of 15 us for one sequence of 3800 tokens and 32 heads).  Several warps of a unit share a CTA
+  // and join in shared memory instead, if that leaves nobody more blocks than one warp per CTA would: the fewest CTAs per
+  // unit (one needs no ticket at all), then the fewest warps.
+  if (Gq == 1 && !c->plan.wide) {
+    const long long units = c->cc.BH, nb = work / units;
+    const long long p1 = grid / units > 1 ? (grid / units < nb ? grid / units : nb) : 1;
+    const long long len = (nb + p1 - 1) / p1;
+    long long best = 0;
+    int best_w = 0;
+    if (len <= 2 && nb > 1)
+      for (int w = 2; w <= 16 && w <= c->plan_occ; ++w) {
+        const long long slots = (long long)c->sm_count * (c->plan_occ / w);
+        const long long need = (nb + len * w - 1) / (len * w);            // CTAs per unit for ranges of `len` blocks
+        if (need * units > slots || need >= a.max_parts) continue;
+        if (best_w == 0 || need < best) { best = need; best_w = w; }
+      }
+    if (best_w) { a.cta_warps = best_w; a.unit_ctas = (int)best; grid = best * units; }
+  }
   // With few blocks per warp, a warp that runs from one unit into the next pays a second prologue and epilogue and
   // finishes last.  When every unit gets at least six warps, cut each unit into ranges of its own instead: the first
   // units into one range more than the others so that every resident warp has work, and order the CTAs by the length
   // of their range, longest first (the hardware dispatches them in index order, and the oldest warps of an SM
   // finish first).  Otherwise (many blocks per warp) cut the flat space evenly.
-  {
+  if (a.unit_ctas == 0) {
     const long long units = (long long)c->cc.BH * passes, nb = work / units;
     const long long pb = grid / units, ua = grid - pb * units;         // ua units get pb + 1 ranges
     if (pb >= 6 && pb + 1 <= nb && pb + 1 < a.max_parts) {

@@ -93,12 +93,12 @@ bool decode_plan(int bits, int heads, int ngv, int max_kpart, int max_vpart, int
     long long ns = (per - w.ring) / stage;
     if (ns < 2) continue;
     if (ns > kMaxStages) ns = kMaxStages;
-    w.total = w.ring + (int)ns * stage;
+    w.total = round_up(w.ring + (int)ns * stage, 16);
     // a cap below what the registers allow is enforced through the shared-memory request
     if (capped && warps == warps_cap) w.total = (int)(per & ~15LL);
     a->aligned = 0;
     a->nstage = (int)ns; a->stage_bytes = stage; a->bregion = bregion; a->max_T = max_T; a->hpa = HP; a->ws = w;
-    a->spin_limit = kDecodeSpinLimit; a->test_dead_wait = 0;
+    a->spin_limit = kDecodeSpinLimit; a->test_dead_wait = 0; a->early_reads = 0; a->early_buf = 0; a->cta_warps = 1; a->unit_ctas = 0;
     a->wide = (HP == 1 && warps <= 12) ? 1 : 0;          // twelve warps or fewer: the 168-register build
     return true;
   }
@@ -120,8 +120,9 @@ int static_shape_id(const SegDesc& s, const CacheConst& c) {
 // caches with several query rows per kv head take gear_decode_rows_kernel.
 // MINB = resident warps per SM the registers are budgeted for: 16 (128 registers) or 12 (168 registers: about a tenth
 // fewer instructions, for long streams where twelve warps are enough) with one head per pass, 8 with four.
-template <int BITS, int HEADS, int NGV, int MINB>
-__global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_constant__ DecodeArgs a) {
+// JOIN: up to sixteen warps of one unit per CTA, joined in shared memory at the end (short ranges of few units).
+template <int BITS, int HEADS, int NGV, int MINB, bool JOIN>
+__global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_kernel(const __grid_constant__ DecodeArgs a) {
   constexpr int HP = HEADS;
   constexpr int NT = HP == 1 ? 1 : 2;             // 8-column tiles of the integer B operands: four limb columns per head
   constexpr int F = 8 / BITS;                     // code fields per byte
@@ -132,9 +133,10 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
   constexpr int kFragStride = frag_row_words(HP);
   constexpr int CMASK = HP == 1 ? 1 : 7;          // fp16 fragment columns that exist, as a mask on the lane's column
   constexpr int WLS = HP == 1 ? 1 : 8;            // row stride of the small factor exchange buffer wl[16][heads]
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem_all[];
 
-  const int lane = threadIdx.x, gid = lane >> 2, t = lane & 3;
+  const int lane = JOIN ? threadIdx.x & 31 : threadIdx.x, gid = lane >> 2, t = lane & 3, wrp = JOIN ? threadIdx.x >> 5 : 0;
+  unsigned char* smem = smem_all + wrp * a.ws.total;
   const int G = a.group_heads;
   const int passes = (G + HP - 1) / HP;
   const int maxT = a.max_T;
@@ -174,7 +176,15 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
   const int NB = a.n_blocks_c + nbuf_blocks;
   int n_left, u, blk_lo;                        // blocks left for this warp, current unit, first block in it
   int part = 0, parts_u = 0;                    // unit-aligned split: this warp's range inside its unit, ranges of the unit
-  if (a.aligned) {
+  if (JOIN) {
+    const int W = blockDim.x >> 5;
+    u = blockIdx.x / a.unit_ctas;
+    part = (blockIdx.x % a.unit_ctas) * W + wrp;
+    parts_u = a.unit_ctas * W;                                      // may exceed NB: the last warps have no block
+    const int base = NB / parts_u, rem = NB - base * parts_u;
+    blk_lo = part * base + min(part, rem);
+    n_left = base + (part < rem ? 1 : 0);
+  } else if (a.aligned) {
     int k = 0;
     while (k < 3 && (int)blockIdx.x >= a.cls_start[k + 1]) ++k;
     const int idx = blockIdx.x - a.cls_start[k];
@@ -198,10 +208,11 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
   // kernel before it on the stream: it waits (griddepcontrol.wait) until that kernel has completed and its writes
   // are visible.  Only after its own wait does a decode kernel let its dependents start, so whoever starts early
   // knows that everything two launches back is complete.  When the host has seen another launch of the library on
-  // this stream since the cache was last written (early_reads), the first copies of the ring -- descriptors,
-  // records and buffer rows, none of them written by the kernel right before this one -- are requested before the
-  // wait, so that they travel while that kernel drains; the query and everything else is read after it.
-  if (!a.early_reads) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // this stream since the records (early_reads) and the buffer rows (early_buf: the kernel in front is the push of a
+  // decoding step) were last written, the first copies of the ring -- descriptors, records, buffer rows -- are requested
+  // before the wait, so that they travel while that kernel drains; the query and everything else is read after it.
+  const bool early = early_start(a, NS, blk_lo, n_left);
+  if (!early) asm volatile("griddepcontrol.wait;" ::: "memory");
 
   auto load_desc = [&](SegDesc* dst, int blk) {
     const int* src = reinterpret_cast<const int*>(a.table + a.blk2seg[blk]);
@@ -266,7 +277,7 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
     }
   };
   for (int s = 0; s < NS; ++s) issue();
-  if (a.early_reads) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (early) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   int c_stage = 0, c_par = 0, c_seg_lo = 0, c_seg_hi = 0, c_shape = 0;
@@ -286,7 +297,51 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
     issue();
   };
 
+  // the partials of a unit, all written and visible -> its output rows
+  auto merge = [&](int unit, int row0, int rows, int n_parts) {
+      const float* pb = a.partial + (size_t)unit * a.max_parts * (HP * kPartRow);
+      const size_t pstride = (size_t)HP * kPartRow;
+      for (int h = 0; h < rows; ++h) {
+        // Chunks of up to 16 partials: every load of a chunk (lane i: max and denominator of partial i; all lanes: their
+        // four channels of every partial) is issued before anything is used, so a chunk costs one round trip to L2.
+        float M = -INFINITY, den = 0.f, n0 = 0.f, n1 = 0.f, n2 = 0.f, n3 = 0.f;
+        for (int base = 0; base < n_parts; base += 16) {
+          const int cnt = min(16, n_parts - base);
+          const float* ph = pb + (size_t)base * pstride + h * kPartRow;
+          float mi = -INFINITY, li = 0.f;
+          if (lane < cnt) { mi = __ldcg(ph + lane * pstride + 128); li = __ldcg(ph + lane * pstride + 129); }
+          float4 v[16];
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            v[j] = j < cnt ? __ldcg(reinterpret_cast<const float4*>(ph + j * pstride) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
+          float cm_ = mi;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) cm_ = fmaxf(cm_, __shfl_xor_sync(0xffffffffu, cm_, o));
+          const float Mn = fmaxf(M, cm_);
+          const float resc = M == -INFINITY ? 0.f : exp2f(M - Mn);
+          const float wgt = mi == -INFINITY ? 0.f : exp2f(mi - Mn);
+          float dsum = wgt * li;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
+          den = fmaf(den, resc, dsum);
+          n0 *= resc; n1 *= resc; n2 *= resc; n3 *= resc;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const float wj = __shfl_sync(0xffffffffu, wgt, j);
+            n0 = fmaf(wj, v[j].x, n0); n1 = fmaf(wj, v[j].y, n1); n2 = fmaf(wj, v[j].z, n2); n3 = fmaf(wj, v[j].w, n3);
+          }
+          M = Mn;
+        }
+        const float inv = 1.0f / den;
+        *reinterpret_cast<float4*>(a.out + (size_t)(row0 + h) * kHeadDim + lane * 4) =
+            make_float4(n0 * inv, n1 * inv, n2 * inv, n3 * inv);
+      }
+  };
+
   // ---- loop over the units this warp touches
+  const int unit0 = u;
+  float* ml_s = reinterpret_cast<float*>(qexp_s + HP);          // [2] maximum and denominator of the warp's range (JOIN)
+  if (JOIN && lane == 0) { ml_s[0] = -INFINITY; ml_s[1] = 0.f; }
   while (n_left > 0 && alive) {
     const int blk_hi = min(NB, blk_lo + n_left);
     const int c_hi = min(blk_hi, a.n_blocks_c);          // end of the compressed blocks of this range
@@ -1199,6 +1254,13 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
     }
     if (!alive) break;
 
+    if (JOIN) {                                // the whole range lies in one unit: joined with the other warps' below
+      float l = l_run[0];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      if (lane == 0) { ml_s[0] = m_run[0]; ml_s[1] = l; }
+      break;
+    }
     // ---------------- partial result of this unit: (m, l, o) per head
     int n_parts, slot;
     if (a.aligned) {
@@ -1236,48 +1298,54 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
     last = __shfl_sync(0xffffffffu, last, 0);
     __syncwarp();
     if (last) {
-      const float* pb = a.partial + (size_t)u * a.max_parts * (HP * kPartRow);
-      const size_t pstride = (size_t)HP * kPartRow;
-      for (int h = 0; h < HPu; ++h) {
-        // Chunks of up to 16 partials: every load of a chunk (lane i: max and denominator of partial i; all lanes: their
-        // four channels of every partial) is issued before anything is used, so a chunk costs one round trip to L2.
-        float M = -INFINITY, den = 0.f, n0 = 0.f, n1 = 0.f, n2 = 0.f, n3 = 0.f;
-        for (int base = 0; base < n_parts; base += 16) {
-          const int cnt = min(16, n_parts - base);
-          const float* ph = pb + (size_t)base * pstride + h * kPartRow;
-          float mi = -INFINITY, li = 0.f;
-          if (lane < cnt) { mi = __ldcg(ph + lane * pstride + 128); li = __ldcg(ph + lane * pstride + 129); }
-          float4 v[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j)
-            v[j] = j < cnt ? __ldcg(reinterpret_cast<const float4*>(ph + j * pstride) + lane) : make_float4(0.f, 0.f, 0.f, 0.f);
-          float cm_ = mi;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) cm_ = fmaxf(cm_, __shfl_xor_sync(0xffffffffu, cm_, o));
-          const float Mn = fmaxf(M, cm_);
-          const float resc = M == -INFINITY ? 0.f : exp2f(M - Mn);
-          const float wgt = mi == -INFINITY ? 0.f : exp2f(mi - Mn);
-          float dsum = wgt * li;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-          den = fmaf(den, resc, dsum);
-          n0 *= resc; n1 *= resc; n2 *= resc; n3 *= resc;
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float wj = __shfl_sync(0xffffffffu, wgt, j);
-            n0 = fmaf(wj, v[j].x, n0); n1 = fmaf(wj, v[j].y, n1); n2 = fmaf(wj, v[j].z, n2); n3 = fmaf(wj, v[j].w, n3);
-          }
-          M = Mn;
-        }
-        const float inv = 1.0f / den;
-        *reinterpret_cast<float4*>(a.out + (size_t)(hq0 + h) * kHeadDim + lane * 4) =
-            make_float4(n0 * inv, n1 * inv, n2 * inv, n3 * inv);
-      }
+      merge(u, hq0, HPu, n_parts);
       if (lane == 0) a.tickets[u] = 0;
     }
     n_left -= blk_hi - blk_lo;
     blk_lo = 0;
     ++u;
+  }
+  if (JOIN) {
+    // Join the warps of the CTA: thread i takes channel i.  The result is the unit's output, or one partial of it for the
+    // CTA that takes the last ticket.
+    __syncthreads();
+    const int W = blockDim.x >> 5, hq0 = unit0 * G;              // one head per pass: the unit is its query head
+    const int off_ml = a.ws.misc + HP * 4;
+    float* part_base = a.partial + ((size_t)unit0 * a.max_parts + blockIdx.x % a.unit_ctas) * kPartRow;
+    for (int ch = threadIdx.x; ch < kHeadDim; ch += blockDim.x) {
+      float M = -INFINITY, den = 0.f, acc = 0.f;
+      for (int w = 0; w < W; ++w) M = fmaxf(M, reinterpret_cast<const float*>(smem_all + w * a.ws.total + off_ml)[0]);
+      for (int w = 0; w < W; ++w) {
+        const float* ml = reinterpret_cast<const float*>(smem_all + w * a.ws.total + off_ml);
+        if (ml[0] == -INFINITY) continue;                        // no block: its output row was never set
+        const float wgt = exp2f(ml[0] - M);
+        den = fmaf(wgt, ml[1], den);
+        acc = fmaf(wgt, reinterpret_cast<const float*>(smem_all + w * a.ws.total + a.ws.ocorr)[ch], acc);
+      }
+      if (a.unit_ctas == 1) {
+        a.out[(size_t)hq0 * kHeadDim + ch] = acc * (1.0f / den);
+      } else {
+        part_base[ch] = acc;
+        if (ch == 0) { part_base[128] = M; part_base[129] = den; }
+      }
+    }
+    if (a.unit_ctas > 1) {
+      __syncthreads();
+      if (wrp == 0) {
+        int last = 0;
+        if (lane == 0) {
+          int old;
+          asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(old) : "l"(a.tickets + unit0) : "memory");
+          last = old == a.unit_ctas - 1;
+        }
+        last = __shfl_sync(0xffffffffu, last, 0);
+        __syncwarp();
+        if (last) {
+          merge(unit0, hq0, 1, a.unit_ctas);
+          if (lane == 0) a.tickets[unit0] = 0;
+        }
+      }
+    }
   }
   // a warp that gave up still has copies in flight: let them land (bounded) before leaving
   if (!alive) {
@@ -1290,13 +1358,13 @@ __global__ void __launch_bounds__(32, MINB) gear_decode_kernel(const __grid_cons
 
 // ------------------------------------------------------------------ host side
 template <class Fn>
-static bool with_decode_kernel(int bits, int heads, int ngv, int wide, Fn fn) {
+static bool with_decode_kernel(int bits, int heads, int ngv, int wide, bool join, Fn fn) {
   const int hp = fp16_heads_per_pass(heads);
   const int minb = hp == 1 ? (wide ? 12 : 16) : 8;
-#define GEAR_DEC_CASE(B, N, V, M) \
-  if (bits == B && hp == N && ngv == V && minb == M) { fn(gear_decode_kernel<B, N, V, M>); return true; }
-#define GEAR_DEC_HEADS(B, V) GEAR_DEC_CASE(B, 1, V, 16) GEAR_DEC_CASE(B, 1, V, 12)
-  GEAR_DEC_CASE(2, 4, 1, 8)          // four heads: fp16 caches only (compressed ones take gear_decode_rows_kernel)
+#define GEAR_DEC_CASE(B, N, V, M, J) \
+  if (bits == B && hp == N && ngv == V && minb == M && join == J) { fn(gear_decode_kernel<B, N, V, M, J>); return true; }
+#define GEAR_DEC_HEADS(B, V) GEAR_DEC_CASE(B, 1, V, 16, false) GEAR_DEC_CASE(B, 1, V, 16, true) GEAR_DEC_CASE(B, 1, V, 12, false)
+  GEAR_DEC_CASE(2, 4, 1, 8, false)   // four heads: fp16 caches only (compressed ones take gear_decode_rows_kernel)
   GEAR_DEC_HEADS(2, 1) GEAR_DEC_HEADS(2, 2) GEAR_DEC_HEADS(2, 4) GEAR_DEC_HEADS(2, 8)
   GEAR_DEC_HEADS(4, 1) GEAR_DEC_HEADS(4, 2) GEAR_DEC_HEADS(4, 4) GEAR_DEC_HEADS(4, 8)
 #undef GEAR_DEC_HEADS
@@ -1307,13 +1375,13 @@ static bool with_decode_kernel(int bits, int heads, int ngv, int wide, Fn fn) {
 cudaError_t launch_decode(const DecodeArgs& a, int grid, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   const size_t smem = (size_t)a.ws.total;
-  const bool ok = with_decode_kernel(a.cc.bits, a.group_heads, a.cc.ngv, a.wide, [&](auto kern) {
+  const bool ok = with_decode_kernel(a.cc.bits, a.group_heads, a.cc.ngv, a.wide, a.unit_ctas > 0, [&](auto kern) {
     // Programmatic dependent launch: the CTAs of this launch may become resident while the kernel before it on the
     // stream drains (the kernel below announces that at once, and waits for its predecessor before its first read of
     // global memory), so that back-to-back decode calls do not pay the launch ramp one after the other.
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(32); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(32 * a.cta_warps); cfg.dynamicSmemBytes = smem * a.cta_warps; cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1328,7 +1396,11 @@ cudaError_t launch_decode(const DecodeArgs& a, int grid, cudaStream_t st) {
 int decode_occupancy(int bits, int heads, int ngv, int wide, size_t smem) {
   int occ = 0;
   cudaError_t e = cudaErrorInvalidValue;
-  with_decode_kernel(bits, heads, ngv, wide, [&](auto kern) {
+  if (!wide && fp16_heads_per_pass(heads) == 1)       // the joining form may follow from the same plan
+    with_decode_kernel(bits, heads, ngv, wide, true, [&](auto kern) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecodeSmemBudget);
+    });
+  with_decode_kernel(bits, heads, ngv, wide, false, [&](auto kern) {
     // every launch is planned first, through here: the kernel may then ask for any amount (the plans of different caches
     // differ), and the launches themselves need no attribute call
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecodeSmemBudget);

@@ -161,4 +161,10 @@ template <int BITS> using ShapeB1 = StaticShape<BITS, 1, 128, 2, 4, 2>;    // g 
 template <int BITS> using ShapeB2 = StaticShape<BITS, 1, 64, 1, 4, 2>;     // g 128, flushed 64-token buffers
 template <int BITS> using ShapeP1 = StaticShape<BITS, 1, 64, 0, 4, 2, true>;   // per-vector keys (outlier list), rank 3..4
 
+// Whether the first copies of a ring of `stages` items may be requested before the wait for the kernel in front: none of
+// them may read what that kernel can have written.
+__device__ __forceinline__ bool early_start(const DecodeArgs& a, int stages, int blk_lo, int n_left) {
+  return a.early_reads && (a.early_buf || blk_lo + min(n_left, (stages + 1) / 2) <= a.n_blocks_c);
+}
+
 }  // namespace gear

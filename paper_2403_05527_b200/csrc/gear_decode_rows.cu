@@ -40,7 +40,7 @@ bool rows_plan(int heads, int ngv, int max_kpart, int max_vpart, int max_bfac, i
     w.total = w.ring + (int)ns * stage;
     a->aligned = 0;
     a->nstage = (int)ns; a->stage_bytes = stage; a->bregion = bregion; a->max_T = max_T; a->hpa = hp; a->rows = w;
-    a->spin_limit = kDecodeSpinLimit; a->test_dead_wait = 0; a->wide = 0;
+    a->spin_limit = kDecodeSpinLimit; a->test_dead_wait = 0; a->early_reads = 0; a->early_buf = 0; a->wide = 0;
     return true;
   }
   return false;

@@ -107,7 +107,8 @@ __global__ void __launch_bounds__(kRowsWarps * 32, kRowsCtasPerSm) gear_decode_r
     blk_lo = (int)(f0 - (long long)u * NB);
   }
   // programmatic dependent launch: see gear_decode_kernel
-  if (!a.early_reads) asm volatile("griddepcontrol.wait;" ::: "memory");
+  const bool early = early_start(a, NS, blk_lo, n_left);
+  if (!early) asm volatile("griddepcontrol.wait;" ::: "memory");
 
   // ---- producer (warp 0): two items per block, issued in order into the ring
   int p_left = n_left, p_blk = blk_lo, p_share_lo = blk_lo, p_half = 0, p_stage = 0;
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(kRowsWarps * 32, kRowsCtasPerSm) gear_decode_r
     }
   };
   for (int s = 0; s < NS; ++s) issue();
-  if (a.early_reads) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (early) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   int c_stage = 0, c_par = 0, n_used = 0, c_seg_lo = 0, c_seg_hi = 0, c_shape = 0;

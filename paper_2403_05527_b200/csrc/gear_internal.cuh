@@ -134,6 +134,8 @@ struct DecodeArgs {
   // aligned == 0: the flat (unit, block) space is cut into gridDim.x equal ranges.
   int aligned, units_a, parts_a, parts_b;
   int cls_start[5], cls_u0[4], cls_n[4], cls_p0[4];
+  // Short ranges of few units (unit_ctas > 0): cta_warps warps per CTA, unit_ctas CTAs per unit, joined in shared memory.
+  int cta_warps, unit_ctas;
   int nstage;                 // ring stages (<= kMaxStages)
   int stage_bytes;            // bytes of one ring stage
   int bregion;                // bytes at the front of a stage reserved for one B factor
@@ -142,7 +144,8 @@ struct DecodeArgs {
   int spin_limit;             // polls a consumer spends on one ring stage before it gives up
   int test_dead_wait;         // test only: wait once on a barrier that nothing completes, with a short limit
   int wide;                   // one head per pass: use the kernel built for twelve resident warps (more registers)
-  int early_reads;            // the cache's data was last written at least two launches back on this stream (see the kernel)
+  int early_reads;            // the segments were last written at least two launches back on this stream (see the kernel)
+  int early_buf;              // so were the buffer rows
   WarpSmem ws;
   RowsSmem rows;
   float scale_log2;           // softmax scale * log2(e)
