@@ -277,230 +277,292 @@ __global__ void __launch_bounds__(128) quant_pack_kernel(CompressArgs p) {
 // leaves only the codes in shared memory, one byte each, transposed so that the packing step fetches the four codes
 // of an output byte row with one 32-bit load.  Every code, scale, outlier and residual is bit-identical to
 // quant_pack_kernel: the operations on a group are the same binary32 sequence.
+//
+// Bound: instruction issue (about thirty instructions per pair of entries), with the residual's bytes not far behind.  CTAs
+// are persistent and the block after the one being worked on comes into shared memory by a bulk copy, so that no warp
+// waits for a load it has just issued; the entries' arithmetic runs on pairs (f32x2); a value group reads and writes its
+// own 32-byte sectors (256-bit stores), so the residual takes no way through shared memory.  Against one CTA per block,
+// scalar arithmetic and a residual staged through shared memory (2 bits, 8 x 32 heads x 4096): keys 181 -> 153 us, values
+// 261 -> 168 us; 4 bits, 16 x 40 heads x 8192: 469 -> 415 and 652 -> 434 us.
 // ---------------------------------------------------------------------------
 constexpr int kFastLen = 64;
 constexpr int kCodePitchK = kHeadDim + 4;   // bytes per token row of the key codes  [token][channel]
 constexpr int kCodePitchV = kFastLen + 4;   // bytes per channel row of the value codes [channel][token]
+// 128 registers, no spills.  Five or six CTAs (96 or 80 registers) are slower on both sides: keys 153 -> 166 -> 196 us, values
+// 168 -> 169 -> 171 us (the first size above).
+constexpr int kFastCtasPerSm = 4;
+constexpr int kFast2KeyCtasPerSm = 3;       // a channel's 128 tokens in registers: at four CTAs they spill (240 -> 204 us)
 
-// Value side, shared-memory staging (a thread's 64 channels are contiguous in memory, so direct accesses of a warp
-// would touch 32 lines each): the fp16 tile comes in with coalesced loads, the fp32 residual tile leaves the same way.
-// Row (c, token) of the fp16 tile holds the 64 channels of group c; rows are 36 words apart and the second group
-// starts 16 words late, rows of the residual tile are 164 words with group 1 at word 80: both make the 128-bit
-// accesses of a quarter warp (four tokens x two groups) hit 32 different banks.
-constexpr int kStageRowWords = 36, kStageGroupSkew = 16;
-constexpr int kResPitch = 164, kResGroup = 80;
-constexpr int kFastSmemV = kFastLen * kResPitch * 4;     // the residual tile; the fp16 tile lives in it first
+// pairs of binary32 operations, each rounded like the scalar one
+struct F32x2 { unsigned long long v; };
+__device__ __forceinline__ F32x2 pack2(float x, float y) {
+  F32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(F32x2 a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 add2(F32x2 a, F32x2 b) { F32x2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ F32x2 mul2(F32x2 a, F32x2 b) { F32x2 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v)); return r; }
+__device__ __forceinline__ F32x2 fma2(F32x2 a, F32x2 b, F32x2 c) {
+  F32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ void store8(float* dst, const float2 (&r)[4]) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(r[0].x), "f"(r[0].y), "f"(r[1].x),
+               "f"(r[1].y), "f"(r[2].x), "f"(r[2].y), "f"(r[3].x), "f"(r[3].y) : "memory");
+}
+
+// Eq. 2 for a pair of entries of one group: t = (x - min) * inv, code = round-to-nearest-even of t by adding 1.5 * 2^23 (the
+// low byte of the sum), residual x - (code * step + min).  Kept entries have t >= 0; t can exceed the top level where the
+// step is subnormal in fp16.  The filtered entries come out as anything and are cleared by the caller.
+struct PairQuant {
+  F32x2 neg_min, inv, neg_step;
+  float levels;
+  __device__ __forceinline__ PairQuant(float mn, float invs, float d, float levels_)
+      : neg_min(pack2(-mn, -mn)), inv(pack2(invs, invs)), neg_step(pack2(-d, -d)), levels(levels_) {}
+  __device__ __forceinline__ float2 operator()(float2 x, unsigned int& c0, unsigned int& c1) const {
+    const F32x2 round = pack2(12582912.0f, 12582912.0f), unround = pack2(-12582912.0f, -12582912.0f);
+    const F32x2 x2 = pack2(x.x, x.y);
+    // The bound between the product and the sum also keeps the compiler from contracting the two packed operations into one
+    // fused one, which would not round the product: the two results differ where a value lies half way between two codes.
+    float2 t = unpack2(mul2(add2(x2, neg_min), inv));
+    t.x = fminf(t.x, levels); t.y = fminf(t.y, levels);
+    const F32x2 y2 = add2(pack2(t.x, t.y), round);
+    const float2 y = unpack2(y2);
+    c0 = __float_as_uint(y.x); c1 = __float_as_uint(y.y);            // the code is the low byte
+    return unpack2(add2(x2, fma2(add2(y2, unround), neg_step, neg_min)));
+  }
+};
+
+// The blocks that a persistent CTA works on, one after the other through one buffer in shared memory: the copy of the next
+// block is requested as soon as every thread is done with the present one.
+struct BlockFeed {
+  unsigned char* tile; uint64_t* full;
+  const __half* X; int n_c, nblk, T, total;
+  uint32_t parity;
+  __device__ __forceinline__ void request(int item) const {
+    const int bhl = item / nblk, blk = item - bhl * nblk;
+    bar_expect(full, T * kHeadDim * 2);
+    bulk_copy(tile, X + ((size_t)bhl * n_c + (size_t)blk * T) * kHeadDim, T * kHeadDim * 2, full);
+  }
+};
 
 template <int BITS, int SIDE>
-__global__ void __launch_bounds__(128) quant_fast_kernel(CompressArgs p) {
+__global__ void __launch_bounds__(128, kFastCtasPerSm) quant_fast_kernel(CompressArgs p, int nbh) {
   constexpr int L = kFastLen, F = 8 / BITS;
   constexpr int side = SIDE;
-  extern __shared__ __align__(16) unsigned char stage_raw[];    // value side only
+  __shared__ __align__(128) unsigned char tile[L * kHeadDim * 2];
   __shared__ __align__(16) unsigned char codes[SIDE == 0 ? L * kCodePitchK : kHeadDim * kCodePitchV];
+  __shared__ uint64_t full;
   __shared__ unsigned int dmax_bits, smax_bits, rmax_bits;
   const SegDesc& sd = p.seg;
-  const int bhl = blockIdx.y, blk = blockIdx.x, tid = threadIdx.x;
-  if (tid == 0) { dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u; }
+  const int tid = threadIdx.x;
+  BlockFeed feed{tile, &full, side == 0 ? p.K : p.V, sd.n_c, sd.nblk, L, sd.nblk * nbh, 0u};
+  if (tid == 0) {
+    dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;
+    bar_init(&full);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if ((int)blockIdx.x < feed.total) feed.request(blockIdx.x);
+  }
   __syncthreads();
-  const __half* X = (side == 0 ? p.K : p.V) + ((size_t)bhl * sd.n_c + (size_t)blk * L) * kHeadDim;
-  float* R = p.R ? p.R + (((size_t)bhl * 2 + side) * sd.n_c + (size_t)blk * L) * kHeadDim : nullptr;
-  unsigned char* rec = p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride + sd.bfac_bytes +
-                       (size_t)blk * sd.rec_bytes;
-  // element e of this thread's group sits at X[first + e * step]
-  const int first = side == 0 ? tid : (tid >> 1) * kHeadDim + (tid & 1) * L;
-  const int step = side == 0 ? kHeadDim : 1;
-  float* rs = reinterpret_cast<float*>(stage_raw);
+  const __half* group = reinterpret_cast<const __half*>(tile) + (side == 0 ? tid : tid * L);   // entry e: group[e * step]
+  constexpr int step = SIDE == 0 ? kHeadDim : 1;
+  const int rot = SIDE == 0 ? 0 : tid & 7;        // values: a thread starts with another 16-byte piece than its neighbours
 
-  // the group as 32 packed pairs (entries 2q, 2q + 1)
-  __half2 xp[L / 2];
-  if (side == 0) {
+  for (int item = blockIdx.x; item < feed.total; item += gridDim.x) {
+    const int bhl = item / sd.nblk, blk = item - bhl * sd.nblk;
+    const bool ok = bar_wait(&full, feed.parity);
+    feed.parity ^= 1u;
+    float* R = p.R ? p.R + (((size_t)bhl * 2 + side) * sd.n_c + (size_t)blk * L) * kHeadDim : nullptr;
+    unsigned char* rec = p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride + sd.bfac_bytes +
+                         (size_t)blk * sd.rec_bytes;
+
+    // the group as 32 packed pairs: keys entries 2q, 2q + 1; values the same, in pieces of eight entries from piece `rot` on
+    __half2 xp[L / 2];
+    if (side == 0) {
 #pragma unroll
-    for (int q = 0; q < L / 2; ++q) xp[q] = __halves2half2(X[first + (2 * q) * kHeadDim], X[first + (2 * q + 1) * kHeadDim]);
-  } else {
-    uint4* xs = reinterpret_cast<uint4*>(stage_raw);
-    for (int i = tid; i < L * 16; i += 128) {           // 16-byte pieces of the tile, in memory order
-      const int tok = i >> 4, c = (i >> 3) & 1, q = i & 7;
-      xs[(((c * L + tok) * kStageRowWords + c * kStageGroupSkew) >> 2) + q] = reinterpret_cast<const uint4*>(X)[i];
-    }
-    __syncthreads();
-    const int tok = tid >> 1, c = tid & 1;
-    const uint4* src = xs + (((c * L + tok) * kStageRowWords + c * kStageGroupSkew) >> 2);
+      for (int q = 0; q < L / 2; ++q) xp[q] = __halves2half2(group[(2 * q) * step], group[(2 * q + 1) * step]);
+    } else {
+      const uint4* src = reinterpret_cast<const uint4*>(group);
 #pragma unroll
-    for (int q = 0; q < L / 8; ++q) {
-      const uint4 v = src[q];
-      xp[4 * q] = *reinterpret_cast<const __half2*>(&v.x);
-      xp[4 * q + 1] = *reinterpret_cast<const __half2*>(&v.y);
-      xp[4 * q + 2] = *reinterpret_cast<const __half2*>(&v.z);
-      xp[4 * q + 3] = *reinterpret_cast<const __half2*>(&v.w);
-    }
-    __syncthreads();                                     // the residual tile takes the place of the fp16 tile
-  }
-  // Filter_s (Eq. 4), one entry per side: the largest and the smallest entry leave the group, the second largest and
-  // second smallest instances bound what is kept.  Comparisons of fp16 values are exact in fp16, so the search runs on
-  // the packed pairs: even and odd entries keep their own two largest / smallest and are merged at the end.
-  float max1, max2, min1, min2;
-  {
-    const __half2 ninf = __float2half2_rn(-INFINITY), pinf = __float2half2_rn(INFINITY);
-    __half2 M1 = ninf, M2 = ninf, m1 = pinf, m2 = pinf;
-#pragma unroll
-    for (int q = 0; q < L / 2; ++q) {
-      M2 = __hmax2(M2, __hmin2(xp[q], M1));
-      M1 = __hmax2(M1, xp[q]);
-      m2 = __hmin2(m2, __hmax2(xp[q], m1));
-      m1 = __hmin2(m1, xp[q]);
-    }
-    const float2 fM1 = __half22float2(M1), fM2 = __half22float2(M2), fm1 = __half22float2(m1), fm2 = __half22float2(m2);
-    max1 = fmaxf(fM1.x, fM1.y);
-    max2 = fmaxf(fminf(fM1.x, fM1.y), fmaxf(fM2.x, fM2.y));
-    min1 = fminf(fm1.x, fm1.y);
-    min2 = fminf(fmaxf(fm1.x, fm1.y), fminf(fm2.x, fm2.y));
-  }
-  // first index of the maximum and of the minimum (ties go to the lower index): one mask bit per entry
-  int imax, imin;
-  {
-    const __half2 vM = __float2half2_rn(max1), vm = __float2half2_rn(min1);
-    unsigned int a0 = 0u, a1 = 0u, b0 = 0u, b1 = 0u;   // bit q of a half word: pair q (a0, b0) or pair 16 + q (a1, b1)
-#pragma unroll
-    for (int q = 0; q < L / 2; ++q) {
-      const unsigned int bit = 0x00010001u << (q & 15);
-      const unsigned int eM = __heq2_mask(xp[q], vM) & bit, em = __heq2_mask(xp[q], vm) & bit;
-      if (q < 16) { a0 |= eM; b0 |= em; } else { a1 |= eM; b1 |= em; }
-    }
-    auto first_set = [](unsigned int lo16, unsigned int hi16) {
-      const unsigned int even = __byte_perm(lo16, hi16, 0x5410);   // bit q: entry 2 q
-      const unsigned int odd = __byte_perm(lo16, hi16, 0x7632);    // bit q: entry 2 q + 1
-      const int fe = even ? 2 * (__ffs((int)even) - 1) : L;
-      const int fo = odd ? 2 * (__ffs((int)odd) - 1) + 1 : L;
-      return min(fe, fo);
-    };
-    imax = first_set(a0, a1);
-    imin = first_set(b0, b1);
-  }
-  if (imin == imax) imin = 1;               // all entries equal: the bottom entry is the next index
-  const float mn = min2, mx = max2;
-  // Eq. 2 on the kept entries: binary32, one rounding per operation
-  const float levels = (float)((1 << BITS) - 1);
-  const float range = __fsub_rn(mx, mn);
-  const float d32 = __fdiv_rn(range, levels);
-  const __half d16 = __float2half_rn(d32);
-  const float d = __half2float(d16);
-  const float inv = d != 0.f ? __fdiv_rn(1.0f, d) : 0.f;
-  // Codes and residuals are computed for every entry as if it were kept; the two filtered entries are cleared
-  // afterwards.  round-to-nearest-even of the clamped quotient by adding 1.5 * 2^23: the code is the low byte of the sum.
-  constexpr float kRound = 12582912.0f;
-  auto quantize = [&](float x, unsigned int& code) {
-    const float t = __fmul_rn(__fsub_rn(x, mn), inv);
-    const float y = __fadd_rn(fminf(fmaxf(t, 0.f), levels), kRound);
-    code = __float_as_uint(y) & 0xFFu;
-    return x - fmaf(__fsub_rn(y, kRound), d, mn);
-  };
-  if (side == 0) {
-#pragma unroll
-    for (int q = 0; q < L / 2; ++q) {
-      const float2 f = __half22float2(xp[q]);
-      unsigned int c0, c1;
-      const float r0 = quantize(f.x, c0), r1 = quantize(f.y, c1);
-      codes[(2 * q) * kCodePitchK + tid] = (unsigned char)c0;
-      codes[(2 * q + 1) * kCodePitchK + tid] = (unsigned char)c1;
-      if (R != nullptr) {
-        R[(2 * q) * kHeadDim + tid] = r0;
-        R[(2 * q + 1) * kHeadDim + tid] = r1;
+      for (int q = 0; q < L / 8; ++q) {
+        const uint4 v = src[(q + rot) & 7];
+        xp[4 * q] = *reinterpret_cast<const __half2*>(&v.x);
+        xp[4 * q + 1] = *reinterpret_cast<const __half2*>(&v.y);
+        xp[4 * q + 2] = *reinterpret_cast<const __half2*>(&v.z);
+        xp[4 * q + 3] = *reinterpret_cast<const __half2*>(&v.w);
       }
     }
-    codes[imax * kCodePitchK + tid] = 0;
-    codes[imin * kCodePitchK + tid] = 0;
-    if (R != nullptr) {
-      R[imax * kHeadDim + tid] = 0.f;
-      R[imin * kHeadDim + tid] = 0.f;
-    }
-  } else {
-    const int tok = tid >> 1, c0 = (tid & 1) * L;
-    float* rrow = rs + tok * kResPitch + (tid & 1) * kResGroup;
+    // Filter_s (Eq. 4), one entry per side: the largest and the smallest entry leave the group, the second largest and
+    // second smallest instances bound what is kept.  Comparisons of fp16 values are exact in fp16, so the search runs on
+    // the packed pairs: even and odd entries keep their own two largest / smallest and are merged at the end.
+    float max1, max2, min1, min2;
+    {
+      const __half2 ninf = __float2half2_rn(-INFINITY), pinf = __float2half2_rn(INFINITY);
+      __half2 M1 = ninf, M2 = ninf, m1 = pinf, m2 = pinf;
 #pragma unroll
-    for (int q = 0; q < L / 4; ++q) {
-      const float2 f0 = __half22float2(xp[2 * q]), f1 = __half22float2(xp[2 * q + 1]);
-      unsigned int k0, k1, k2, k3;
-      const float4 rr = make_float4(quantize(f0.x, k0), quantize(f0.y, k1), quantize(f1.x, k2), quantize(f1.y, k3));
-      codes[(c0 + 4 * q) * kCodePitchV + tok] = (unsigned char)k0;
-      codes[(c0 + 4 * q + 1) * kCodePitchV + tok] = (unsigned char)k1;
-      codes[(c0 + 4 * q + 2) * kCodePitchV + tok] = (unsigned char)k2;
-      codes[(c0 + 4 * q + 3) * kCodePitchV + tok] = (unsigned char)k3;
-      *reinterpret_cast<float4*>(rrow + 4 * q) = rr;
+      for (int q = 0; q < L / 2; ++q) {
+        M2 = __hmax2(M2, __hmin2(xp[q], M1));
+        M1 = __hmax2(M1, xp[q]);
+        m2 = __hmin2(m2, __hmax2(xp[q], m1));
+        m1 = __hmin2(m1, xp[q]);
+      }
+      const float2 fM1 = __half22float2(M1), fM2 = __half22float2(M2), fm1 = __half22float2(m1), fm2 = __half22float2(m2);
+      max1 = fmaxf(fM1.x, fM1.y);
+      max2 = fmaxf(fminf(fM1.x, fM1.y), fmaxf(fM2.x, fM2.y));
+      min1 = fminf(fm1.x, fm1.y);
+      min2 = fminf(fmaxf(fm1.x, fm1.y), fminf(fm2.x, fm2.y));
     }
-    codes[(c0 + imax) * kCodePitchV + tok] = 0;
-    codes[(c0 + imin) * kCodePitchV + tok] = 0;
-    rrow[imax] = 0.f;
-    rrow[imin] = 0.f;
-  }
-  // A bound on the group's residuals instead of their maximum (it only picks the power of two the power iteration
-  // scales by): half a step for a kept entry, the whole range if the step rounded to zero, plus the rounding of the
-  // dequantised value
-  float rmax = (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
-  // the group's scale, zero point and its two outliers (in-group index ascending)
-  {
-    const __half vmax = X[first + imax * step], vmin = X[first + imin * step];
-    const bool max_first = imax < imin;
-    const __half2 ov = max_first ? __halves2half2(vmax, vmin) : __halves2half2(vmin, vmax);
-    const uchar2 oi = max_first ? make_uchar2((unsigned char)imax, (unsigned char)imin)
-                                : make_uchar2((unsigned char)imin, (unsigned char)imax);
-    reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_koval : sd.off_voval))[tid] = ov;
-    reinterpret_cast<uchar2*>(rec + (side == 0 ? sd.off_koidx : sd.off_voidx))[tid] = oi;
-    reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_kscale : sd.off_vscale))[tid] =
-        __halves2half2(d16, __float2half_rn(mn));
-    float dm = fmaxf(fabsf(__half2float(vmax) - mn), fabsf(__half2float(vmin) - mn));
-    float sm = d;
+    // first index of the maximum and of the minimum (ties go to the lower index): one mask bit per entry
+    int imax, imin;
+    {
+      const __half2 vM = __float2half2_rn(max1), vm = __float2half2_rn(min1);
+      unsigned int a0 = 0u, a1 = 0u, b0 = 0u, b1 = 0u;   // bit q of a half word: pair q (a0, b0) or pair 16 + q (a1, b1)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      dm = fmaxf(dm, __shfl_xor_sync(0xffffffffu, dm, o));
-      sm = fmaxf(sm, __shfl_xor_sync(0xffffffffu, sm, o));
-      rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+      for (int q = 0; q < L / 2; ++q) {
+        const unsigned int bit = 0x00010001u << (q & 15);
+        const unsigned int eM = __heq2_mask(xp[q], vM) & bit, em = __heq2_mask(xp[q], vm) & bit;
+        if (q < 16) { a0 |= eM; b0 |= em; } else { a1 |= eM; b1 |= em; }
+      }
+      auto first_set = [&](unsigned int lo16, unsigned int hi16) {
+        // bit q: entry 2 q / 2 q + 1 (values: the pieces back in order)
+        const unsigned int even = __funnelshift_l(__byte_perm(lo16, hi16, 0x5410), __byte_perm(lo16, hi16, 0x5410), 4 * rot);
+        const unsigned int odd = __funnelshift_l(__byte_perm(lo16, hi16, 0x7632), __byte_perm(lo16, hi16, 0x7632), 4 * rot);
+        const int fe = even ? 2 * (__ffs((int)even) - 1) : L;
+        const int fo = odd ? 2 * (__ffs((int)odd) - 1) + 1 : L;
+        return min(fe, fo);
+      };
+      imax = first_set(a0, a1);
+      imin = first_set(b0, b1);
     }
-    if ((tid & 31) == 0) {                   // non-negative floats order like their bit patterns
-      atomicMax(&dmax_bits, __float_as_uint(dm));
-      atomicMax(&smax_bits, __float_as_uint(sm));
-      atomicMax(&rmax_bits, __float_as_uint(rmax));
+    if (imin == imax) imin = 1;               // all entries equal: the bottom entry is the next index
+    const float mn = min2, mx = max2;
+    // Eq. 2 on the kept entries: binary32, one rounding per operation
+    const float levels = (float)((1 << BITS) - 1);
+    const float range = __fsub_rn(mx, mn);
+    const float d32 = __fdiv_rn(range, levels);
+    const __half d16 = __float2half_rn(d32);
+    const float d = __half2float(d16);
+    const float inv = d != 0.f ? __fdiv_rn(1.0f, d) : 0.f;
+    const __half vmax = group[imax * step], vmin = group[imin * step];
+    if (__syncthreads_or(!ok)) {              // every thread has read the block
+      if (tid == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
+      break;
     }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    reinterpret_cast<float*>(rec)[side] = __uint_as_float(dmax_bits);
-    reinterpret_cast<float*>(rec)[2 + side] = __uint_as_float(smax_bits);
-    if (R != nullptr) atomicMax(p.Rmax + bhl * 2 + side, rmax_bits);
-  }
-  if (side == 1 && R != nullptr) {
-    for (int i = tid; i < L * 32; i += 128) {            // 16-byte pieces of the residual tile, in memory order
-      const int tok = i >> 5, c = (i >> 4) & 1, q = i & 15;
-      reinterpret_cast<float4*>(R)[i] = *reinterpret_cast<const float4*>(rs + tok * kResPitch + c * kResGroup + 4 * q);
-    }
-  }
-  // pack the codes into mma-fragment order (code_coord_k / code_coord_v): the four codes of a byte row are neighbours
-  // in shared memory, a field of the word is one 32-bit load shifted into place
-  unsigned int* dst = reinterpret_cast<unsigned int*>(rec + (side == 0 ? sd.off_kcodes : sd.off_vcodes));
-  if (side == 0) {
-    constexpr int kWords = kSlab * kHeadDim * BITS / 32;            // words per slab
-    for (int li = tid; li < (L / kSlab) * kWords; li += 128) {
-      const int slab = li / kWords, wl = li % kWords;
-      const int w = wl & 3, lane = (wl >> 2) & 31, tau = wl >> 7;
-      const int tok = slab * kSlab + (lane >> 2) + 8 * (w & 1);
-      const int ch = 32 * F * tau + 16 * (w >> 1) + 4 * (lane & 3);
-      unsigned int word = 0;
+    if (tid == 0 && item + (int)gridDim.x < feed.total) feed.request(item + gridDim.x);
+    // Codes and residuals are computed for every entry as if it were kept; the two filtered entries are cleared afterwards.
+    const PairQuant quantize(mn, inv, d, levels);
+    if (side == 0) {
 #pragma unroll
-      for (int j = 0; j < F; ++j)
-        word |= *reinterpret_cast<const unsigned int*>(&codes[tok * kCodePitchK + ch + 32 * j]) << (BITS * j);
-      dst[li] = word;
-    }
-  } else {
-    constexpr int kWords = 32 * kHeadDim * BITS / 32;               // words per 32-token chunk
-    for (int li = tid; li < (L / 32) * kWords; li += 128) {
-      const int chunk = li / kWords, wl = li % kWords;
-      const int w = wl & 3, lane = (wl >> 2) & 31, tau = wl >> 7;
-      const int ch = 16 * F * tau + (lane >> 2) + 8 * (w & 1);
-      const int tok = chunk * 32 + 16 * (w >> 1) + 4 * (lane & 3);
-      unsigned int word = 0;
+      for (int q = 0; q < L / 2; ++q) {
+        unsigned int c0, c1;
+        const float2 r = quantize(__half22float2(xp[q]), c0, c1);
+        codes[(2 * q) * kCodePitchK + tid] = (unsigned char)c0;
+        codes[(2 * q + 1) * kCodePitchK + tid] = (unsigned char)c1;
+        if (R != nullptr) {
+          R[(2 * q) * kHeadDim + tid] = r.x;
+          R[(2 * q + 1) * kHeadDim + tid] = r.y;
+        }
+      }
+      codes[imax * kCodePitchK + tid] = 0;
+      codes[imin * kCodePitchK + tid] = 0;
+      if (R != nullptr) {
+        R[imax * kHeadDim + tid] = 0.f;
+        R[imin * kHeadDim + tid] = 0.f;
+      }
+    } else {
+      const int tok = tid >> 1;
+      unsigned char* mine = codes + (tid & 1) * L * kCodePitchV + tok;
 #pragma unroll
-      for (int j = 0; j < F; ++j)
-        word |= *reinterpret_cast<const unsigned int*>(&codes[(ch + 16 * j) * kCodePitchV + tok]) << (BITS * j);
-      dst[li] = word;
+      for (int q = 0; q < L / 8; ++q) {
+        const int piece = (q + rot) & 7;
+        unsigned char* cp = mine + piece * 8 * kCodePitchV;
+        float2 r[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          unsigned int c0, c1;
+          r[k] = quantize(__half22float2(xp[4 * q + k]), c0, c1);
+          cp[(2 * k) * kCodePitchV] = (unsigned char)c0;
+          cp[(2 * k + 1) * kCodePitchV] = (unsigned char)c1;
+        }
+        if (R != nullptr) store8(R + tid * L + piece * 8, r);
+      }
+      mine[imax * kCodePitchV] = 0;
+      mine[imin * kCodePitchV] = 0;
+      if (R != nullptr) {
+        R[tid * L + imax] = 0.f;
+        R[tid * L + imin] = 0.f;
+      }
+    }
+    // A bound on the group's residuals instead of their maximum (it only picks the power of two the power iteration
+    // scales by): half a step for a kept entry, the whole range if the step rounded to zero, plus the rounding of the
+    // dequantised value
+    float rmax = (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
+    // the group's scale, zero point and its two outliers (in-group index ascending)
+    {
+      const bool max_first = imax < imin;
+      const __half2 ov = max_first ? __halves2half2(vmax, vmin) : __halves2half2(vmin, vmax);
+      const uchar2 oi = max_first ? make_uchar2((unsigned char)imax, (unsigned char)imin)
+                                  : make_uchar2((unsigned char)imin, (unsigned char)imax);
+      reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_koval : sd.off_voval))[tid] = ov;
+      reinterpret_cast<uchar2*>(rec + (side == 0 ? sd.off_koidx : sd.off_voidx))[tid] = oi;
+      reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_kscale : sd.off_vscale))[tid] =
+          __halves2half2(d16, __float2half_rn(mn));
+      float dm = fmaxf(fabsf(__half2float(vmax) - mn), fabsf(__half2float(vmin) - mn));
+      float sm = d;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        dm = fmaxf(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+        sm = fmaxf(sm, __shfl_xor_sync(0xffffffffu, sm, o));
+        rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+      }
+      if ((tid & 31) == 0) {                   // non-negative floats order like their bit patterns
+        atomicMax(&dmax_bits, __float_as_uint(dm));
+        atomicMax(&smax_bits, __float_as_uint(sm));
+        atomicMax(&rmax_bits, __float_as_uint(rmax));
+      }
+    }
+    __syncthreads();
+    if (tid == 0) {
+      reinterpret_cast<float*>(rec)[side] = __uint_as_float(dmax_bits);
+      reinterpret_cast<float*>(rec)[2 + side] = __uint_as_float(smax_bits);
+      if (R != nullptr) atomicMax(p.Rmax + bhl * 2 + side, rmax_bits);
+      dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;       // the next updates come behind the next block's first barrier
+    }
+    // pack the codes into mma-fragment order (code_coord_k / code_coord_v): the four codes of a byte row are neighbours
+    // in shared memory, a field of the word is one 32-bit load shifted into place
+    unsigned int* dst = reinterpret_cast<unsigned int*>(rec + (side == 0 ? sd.off_kcodes : sd.off_vcodes));
+    if (side == 0) {
+      constexpr int kWords = kSlab * kHeadDim * BITS / 32;            // words per slab
+      for (int li = tid; li < (L / kSlab) * kWords; li += 128) {
+        const int slab = li / kWords, wl = li % kWords;
+        const int w = wl & 3, lane = (wl >> 2) & 31, tau = wl >> 7;
+        const int tok = slab * kSlab + (lane >> 2) + 8 * (w & 1);
+        const int ch = 32 * F * tau + 16 * (w >> 1) + 4 * (lane & 3);
+        unsigned int word = 0;
+#pragma unroll
+        for (int j = 0; j < F; ++j)
+          word |= *reinterpret_cast<const unsigned int*>(&codes[tok * kCodePitchK + ch + 32 * j]) << (BITS * j);
+        dst[li] = word;
+      }
+    } else {
+      constexpr int kWords = 32 * kHeadDim * BITS / 32;               // words per 32-token chunk
+      for (int li = tid; li < (L / 32) * kWords; li += 128) {
+        const int chunk = li / kWords, wl = li % kWords;
+        const int w = wl & 3, lane = (wl >> 2) & 31, tau = wl >> 7;
+        const int ch = 16 * F * tau + (lane >> 2) + 8 * (w & 1);
+        const int tok = chunk * 32 + 16 * (w >> 1) + 4 * (lane & 3);
+        unsigned int word = 0;
+#pragma unroll
+        for (int j = 0; j < F; ++j)
+          word |= *reinterpret_cast<const unsigned int*>(&codes[(ch + 16 * j) * kCodePitchV + tok]) << (BITS * j);
+        dst[li] = word;
+      }
     }
   }
 }
@@ -511,7 +573,8 @@ __global__ void __launch_bounds__(128) quant_fast_kernel(CompressArgs p) {
 // and three smallest instances; the halves are merged; the entries above / equal to the second largest instance (and
 // below / equal to the second smallest) are found as bit masks, which give the two filtered entries per side in
 // (value, index) order.  A group in which the two sides would share an entry (nearly constant groups) takes the
-// general routine instead.  Same binary32 sequence per entry as everywhere else.
+// general routine instead.  Same binary32 sequence per entry as everywhere else.  Bound and layout as above (2 bits, 4 x 8
+// heads x 32768: keys 279 -> 204 us, values 290 -> 184 us).
 // ---------------------------------------------------------------------------
 constexpr int kFast2Len = 128;
 constexpr int kCodePitch2 = kFast2Len + 4;
@@ -550,213 +613,237 @@ __device__ __forceinline__ void top3_of6(float (&v)[6], float (&out)[3]) {
 }
 
 template <int BITS, int SIDE>
-__global__ void __launch_bounds__(128) quant_fast2_kernel(CompressArgs p) {
+__global__ void __launch_bounds__(128, SIDE == 0 ? kFast2KeyCtasPerSm : kFastCtasPerSm) quant_fast2_kernel(CompressArgs p, int nbh) {
   constexpr int L = kFast2Len, F = 8 / BITS;
+  extern __shared__ __align__(128) unsigned char tile[];            // the block's T x 128 fp16 entries
   __shared__ __align__(16) unsigned char codes[L * kCodePitch2];    // keys [token][channel], values [channel][token]
+  __shared__ uint64_t full;
   __shared__ unsigned int dmax_bits, smax_bits, rmax_bits;
   const SegDesc& sd = p.seg;
   const int T = sd.T;                               // keys: 128; values: tokens (= groups) of the block
-  const int bhl = blockIdx.y, blk = blockIdx.x, tid = threadIdx.x;
-  if (tid == 0) { dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u; }
+  const int tid = threadIdx.x;
+  BlockFeed feed{tile, &full, SIDE == 0 ? p.K : p.V, sd.n_c, sd.nblk, T, sd.nblk * nbh, 0u};
+  if (tid == 0) {
+    dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;
+    bar_init(&full);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if ((int)blockIdx.x < feed.total) feed.request(blockIdx.x);
+  }
   __syncthreads();
-  const __half* X = (SIDE == 0 ? p.K : p.V) + ((size_t)bhl * sd.n_c + (size_t)blk * T) * kHeadDim;
-  float* R = p.R ? p.R + (((size_t)bhl * 2 + SIDE) * sd.n_c + (size_t)blk * T) * kHeadDim : nullptr;
-  unsigned char* rec = p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride + sd.bfac_bytes +
-                       (size_t)blk * sd.rec_bytes;
   const int first = SIDE == 0 ? tid : tid * kHeadDim;      // element e of the group: X[first + e * step]
-  const int step = SIDE == 0 ? kHeadDim : 1;
+  constexpr int step = SIDE == 0 ? kHeadDim : 1;
+  const __half* group = reinterpret_cast<const __half*>(tile) + first;
+  const int rot = SIDE == 0 ? 0 : tid & 7;        // values: a thread starts with another 16-byte piece than its neighbours
   // where code / residual of element e go
   auto code_at = [&](int e) -> unsigned char& { return codes[e * kCodePitch2 + tid]; };   // row: token (keys) / channel (values)
   const bool active = SIDE == 0 || tid < T;
 
-  if (active) {
+  for (int item = blockIdx.x; item < feed.total; item += gridDim.x) {
+    const int bhl = item / sd.nblk, blk = item - bhl * sd.nblk;
+    const bool ok = bar_wait(&full, feed.parity);
+    feed.parity ^= 1u;
+    const __half* X = (SIDE == 0 ? p.K : p.V) + ((size_t)bhl * sd.n_c + (size_t)blk * T) * kHeadDim;
+    float* R = p.R ? p.R + (((size_t)bhl * 2 + SIDE) * sd.n_c + (size_t)blk * T) * kHeadDim : nullptr;
+    unsigned char* rec = p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride + sd.bfac_bytes +
+                         (size_t)blk * sd.rec_bytes;
     __half2 xp[L / 2];
-    if (SIDE == 0) {
-#pragma unroll
-      for (int q = 0; q < L / 2; ++q) xp[q] = __halves2half2(X[first + (2 * q) * kHeadDim], X[first + (2 * q + 1) * kHeadDim]);
-    } else {
-      const uint4* src = reinterpret_cast<const uint4*>(X + first);
-#pragma unroll
-      for (int q = 0; q < L / 8; ++q) {
-        const uint4 v = src[q];
-        xp[4 * q] = *reinterpret_cast<const __half2*>(&v.x);
-        xp[4 * q + 1] = *reinterpret_cast<const __half2*>(&v.y);
-        xp[4 * q + 2] = *reinterpret_cast<const __half2*>(&v.z);
-        xp[4 * q + 3] = *reinterpret_cast<const __half2*>(&v.w);
-      }
-    }
-    // the three largest / smallest instances of the even and of the odd entries, then of all
+    int it[2] = {0, 0}, ib[2] = {0, 0};
     float top[3], bot[3];
-    {
-      const __half2 ninf = __float2half2_rn(-INFINITY), pinf = __float2half2_rn(INFINITY);
-      __half2 M1 = ninf, M2 = ninf, M3 = ninf, m1 = pinf, m2 = pinf, m3 = pinf;
-#pragma unroll
-      for (int q = 0; q < L / 2; ++q) {
-        const __half2 t = __hmin2(xp[q], M1);
-        M1 = __hmax2(M1, xp[q]);
-        const __half2 u = __hmin2(t, M2);
-        M2 = __hmax2(M2, t);
-        M3 = __hmax2(M3, u);
-        const __half2 tb = __hmax2(xp[q], m1);
-        m1 = __hmin2(m1, xp[q]);
-        const __half2 ub = __hmax2(tb, m2);
-        m2 = __hmin2(m2, tb);
-        m3 = __hmin2(m3, ub);
-      }
-      float v[6] = {__low2float(M1), __low2float(M2), __low2float(M3), __high2float(M1), __high2float(M2), __high2float(M3)};
-      top3_of6(v, top);
-      float w[6] = {-__low2float(m1), -__low2float(m2), -__low2float(m3), -__high2float(m1), -__high2float(m2), -__high2float(m3)};
-      top3_of6(w, bot);
-      bot[0] = -bot[0]; bot[1] = -bot[1]; bot[2] = -bot[2];
-    }
-    // entries above / equal to the second largest instance, below / equal to the second smallest
-    int it[2], ib[2];
-    {
-      const __half2 vT = __float2half2_rn(top[1]), vB = __float2half2_rn(bot[1]);
-      unsigned int gt[4] = {0u, 0u, 0u, 0u}, et[4] = {0u, 0u, 0u, 0u}, lt[4] = {0u, 0u, 0u, 0u}, eb[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-      for (int q = 0; q < L / 2; ++q) {
-        const unsigned int bit = 0x00010001u << (q & 15);
-        gt[q >> 4] |= __hgt2_mask(xp[q], vT) & bit;
-        et[q >> 4] |= __heq2_mask(xp[q], vT) & bit;
-        lt[q >> 4] |= __hlt2_mask(xp[q], vB) & bit;
-        eb[q >> 4] |= __heq2_mask(xp[q], vB) & bit;
-      }
-      unsigned long long ge, go, ee, eo;
-      masks_of(gt, ge, go); masks_of(et, ee, eo);
-      it[0] = take_first(ge, go);                      // the one entry above the second largest instance, if any
-      if (it[0] >= L) it[0] = take_first(ee, eo);
-      it[1] = take_first(ee, eo);
-      masks_of(lt, ge, go); masks_of(eb, ee, eo);
-      ib[0] = take_first(ge, go);
-      if (ib[0] >= L) ib[0] = take_first(ee, eo);
-      ib[1] = take_first(ee, eo);
-    }
-    const bool shared_entry = it[0] == ib[0] || it[0] == ib[1] || it[1] == ib[0] || it[1] == ib[1];
-    const float levels = (float)((1 << BITS) - 1);
-    float d, mn, dm, rmax;
-    __half d16;
-    unsigned char* orec_v = rec + (SIDE == 0 ? sd.off_koval : sd.off_voval) + tid * 8;
-    unsigned char* orec_i = rec + (SIDE == 0 ? sd.off_koidx : sd.off_voidx) + tid * 4;
-    if (!shared_entry) {
-      mn = bot[2];
-      const float mx = top[2];
-      // Eq. 2 on the kept entries: binary32, one rounding per operation
-      const float range = __fsub_rn(mx, mn);
-      const float d32 = __fdiv_rn(range, levels);
-      d16 = __float2half_rn(d32);
-      d = __half2float(d16);
-      const float inv = d != 0.f ? __fdiv_rn(1.0f, d) : 0.f;
-      constexpr float kRound = 12582912.0f;
-      auto quantize = [&](float x, unsigned int& code) {
-        const float t = __fmul_rn(__fsub_rn(x, mn), inv);
-        const float y = __fadd_rn(fminf(fmaxf(t, 0.f), levels), kRound);
-        code = __float_as_uint(y) & 0xFFu;
-        return x - fmaf(__fsub_rn(y, kRound), d, mn);
-      };
+    unsigned short ov[4];
+    int oi[4] = {0, 0, 0, 0};
+    if (active) {
       if (SIDE == 0) {
 #pragma unroll
-        for (int q = 0; q < L / 2; ++q) {
-          const float2 f = __half22float2(xp[q]);
-          unsigned int c0, c1;
-          const float r0 = quantize(f.x, c0), r1 = quantize(f.y, c1);
-          code_at(2 * q) = (unsigned char)c0;
-          code_at(2 * q + 1) = (unsigned char)c1;
-          if (R != nullptr) {
-            R[(2 * q) * kHeadDim + tid] = r0;
-            R[(2 * q + 1) * kHeadDim + tid] = r1;
-          }
-        }
+        for (int q = 0; q < L / 2; ++q) xp[q] = __halves2half2(group[(2 * q) * step], group[(2 * q + 1) * step]);
       } else {
+        const uint4* src = reinterpret_cast<const uint4*>(group);
 #pragma unroll
-        for (int q = 0; q < L / 4; ++q) {
-          const float2 f0 = __half22float2(xp[2 * q]), f1 = __half22float2(xp[2 * q + 1]);
-          unsigned int k0, k1, k2, k3;
-          const float4 rr = make_float4(quantize(f0.x, k0), quantize(f0.y, k1), quantize(f1.x, k2), quantize(f1.y, k3));
-          code_at(4 * q) = (unsigned char)k0;
-          code_at(4 * q + 1) = (unsigned char)k1;
-          code_at(4 * q + 2) = (unsigned char)k2;
-          code_at(4 * q + 3) = (unsigned char)k3;
-          if (R != nullptr) *reinterpret_cast<float4*>(R + first + 4 * q) = rr;
+        for (int q = 0; q < L / 8; ++q) {
+          const uint4 v = src[(q + rot) & 15];
+          xp[4 * q] = *reinterpret_cast<const __half2*>(&v.x);
+          xp[4 * q + 1] = *reinterpret_cast<const __half2*>(&v.y);
+          xp[4 * q + 2] = *reinterpret_cast<const __half2*>(&v.z);
+          xp[4 * q + 3] = *reinterpret_cast<const __half2*>(&v.w);
         }
       }
-      // the four filtered entries: cleared, and stored in-group index ascending
-      int oi[4] = {it[0], it[1], ib[0], ib[1]};
+      // the three largest / smallest instances of the even and of the odd entries, then of all
+      {
+        const __half2 ninf = __float2half2_rn(-INFINITY), pinf = __float2half2_rn(INFINITY);
+        __half2 M1 = ninf, M2 = ninf, M3 = ninf, m1 = pinf, m2 = pinf, m3 = pinf;
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        code_at(oi[a]) = 0;
-        if (R != nullptr) R[SIDE == 0 ? oi[a] * kHeadDim + tid : first + oi[a]] = 0.f;
+        for (int q = 0; q < L / 2; ++q) {
+          const __half2 t = __hmin2(xp[q], M1);
+          M1 = __hmax2(M1, xp[q]);
+          const __half2 u = __hmin2(t, M2);
+          M2 = __hmax2(M2, t);
+          M3 = __hmax2(M3, u);
+          const __half2 tb = __hmax2(xp[q], m1);
+          m1 = __hmin2(m1, xp[q]);
+          const __half2 ub = __hmax2(tb, m2);
+          m2 = __hmin2(m2, tb);
+          m3 = __hmin2(m3, ub);
+        }
+        float v[6] = {__low2float(M1), __low2float(M2), __low2float(M3), __high2float(M1), __high2float(M2), __high2float(M3)};
+        top3_of6(v, top);
+        float w[6] = {-__low2float(m1), -__low2float(m2), -__low2float(m3), -__high2float(m1), -__high2float(m2), -__high2float(m3)};
+        top3_of6(w, bot);
+        bot[0] = -bot[0]; bot[1] = -bot[1]; bot[2] = -bot[2];
       }
+      // entries above / equal to the second largest instance, below / equal to the second smallest
+      {
+        const __half2 vT = __float2half2_rn(top[1]), vB = __float2half2_rn(bot[1]);
+        unsigned int gt[4] = {0u, 0u, 0u, 0u}, et[4] = {0u, 0u, 0u, 0u}, lt[4] = {0u, 0u, 0u, 0u}, eb[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int q = 0; q < L / 2; ++q) {
+          const unsigned int bit = 0x00010001u << (q & 15);
+          gt[q >> 4] |= __hgt2_mask(xp[q], vT) & bit;
+          et[q >> 4] |= __heq2_mask(xp[q], vT) & bit;
+          lt[q >> 4] |= __hlt2_mask(xp[q], vB) & bit;
+          eb[q >> 4] |= __heq2_mask(xp[q], vB) & bit;
+        }
+        unsigned long long ge, go, ee, eo;
+        auto in_order = [&](unsigned long long m) {            // values: the pieces back in order
+          return SIDE == 0 || rot == 0 ? m : (m << (4 * rot)) | (m >> (64 - 4 * rot));
+        };
+        auto masks = [&](const unsigned int (&acc)[4], unsigned long long& even, unsigned long long& odd) {
+          masks_of(acc, even, odd);
+          even = in_order(even); odd = in_order(odd);
+        };
+        masks(gt, ge, go); masks(et, ee, eo);
+        it[0] = take_first(ge, go);                      // the one entry above the second largest instance, if any
+        if (it[0] >= L) it[0] = take_first(ee, eo);
+        it[1] = take_first(ee, eo);
+        masks(lt, ge, go); masks(eb, ee, eo);
+        ib[0] = take_first(ge, go);
+        if (ib[0] >= L) ib[0] = take_first(ee, eo);
+        ib[1] = take_first(ee, eo);
+      }
+      // the four filtered entries, in-group index ascending
+      oi[0] = it[0]; oi[1] = it[1]; oi[2] = ib[0]; oi[3] = ib[1];
       auto order = [&](int a, int b) { if (oi[a] > oi[b]) { const int t = oi[a]; oi[a] = oi[b]; oi[b] = t; } };
       order(0, 1); order(2, 3); order(0, 2); order(1, 3); order(1, 2);
-      unsigned short ov[4];
-      dm = 0.f;
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const __half h = X[first + oi[a] * step];
-        ov[a] = __half_as_ushort(h);
-        dm = fmaxf(dm, fabsf(__half2float(h) - mn));
+      for (int a = 0; a < 4; ++a) ov[a] = __half_as_ushort(group[min(oi[a], L - 1) * step]);
+    }
+    if (__syncthreads_or(!ok)) {                    // every thread has read the block
+      if (tid == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
+      break;
+    }
+    if (tid == 0 && item + (int)gridDim.x < feed.total) feed.request(item + gridDim.x);
+    if (active) {
+      const bool shared_entry = it[0] == ib[0] || it[0] == ib[1] || it[1] == ib[0] || it[1] == ib[1];
+      const float levels = (float)((1 << BITS) - 1);
+      float d, mn, dm, rmax;
+      __half d16;
+      unsigned char* orec_v = rec + (SIDE == 0 ? sd.off_koval : sd.off_voval) + tid * 8;
+      unsigned char* orec_i = rec + (SIDE == 0 ? sd.off_koidx : sd.off_voidx) + tid * 4;
+      if (!shared_entry) {
+        mn = bot[2];
+        const float mx = top[2];
+        // Eq. 2 on the kept entries: binary32, one rounding per operation
+        const float range = __fsub_rn(mx, mn);
+        const float d32 = __fdiv_rn(range, levels);
+        d16 = __float2half_rn(d32);
+        d = __half2float(d16);
+        const float inv = d != 0.f ? __fdiv_rn(1.0f, d) : 0.f;
+        const PairQuant quantize(mn, inv, d, levels);
+        if (SIDE == 0) {
+#pragma unroll
+          for (int q = 0; q < L / 2; ++q) {
+            unsigned int c0, c1;
+            const float2 r = quantize(__half22float2(xp[q]), c0, c1);
+            code_at(2 * q) = (unsigned char)c0;
+            code_at(2 * q + 1) = (unsigned char)c1;
+            if (R != nullptr) {
+              R[(2 * q) * kHeadDim + tid] = r.x;
+              R[(2 * q + 1) * kHeadDim + tid] = r.y;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < L / 8; ++q) {
+            const int piece = (q + rot) & 15;
+            float2 r[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              unsigned int c0, c1;
+              r[k] = quantize(__half22float2(xp[4 * q + k]), c0, c1);
+              code_at(8 * piece + 2 * k) = (unsigned char)c0;
+              code_at(8 * piece + 2 * k + 1) = (unsigned char)c1;
+            }
+            if (R != nullptr) store8(R + first + 8 * piece, r);
+          }
+        }
+        // the filtered entries: cleared and stored
+        dm = 0.f;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          code_at(oi[a]) = 0;
+          if (R != nullptr) R[SIDE == 0 ? oi[a] * kHeadDim + tid : first + oi[a]] = 0.f;
+          dm = fmaxf(dm, fabsf(__half2float(__ushort_as_half(ov[a])) - mn));
+        }
+        *reinterpret_cast<uint2*>(orec_v) = make_uint2(ov[0] | ((unsigned int)ov[1] << 16), ov[2] | ((unsigned int)ov[3] << 16));
+        *reinterpret_cast<unsigned int*>(orec_i) = (unsigned int)oi[0] | ((unsigned int)oi[1] << 8) |
+                                                   ((unsigned int)oi[2] << 16) | ((unsigned int)oi[3] << 24);
+        rmax = (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
+      } else {
+        rmax = 0.f;
+        GroupResult g = process_group<BITS, 2>(
+            L, 2, [&](int e) { return __half2float(X[first + e * step]); },
+            [&](int e, int code, float r) {
+              code_at(e) = (unsigned char)code;
+              if (R != nullptr) R[SIDE == 0 ? e * kHeadDim + tid : first + e] = r;
+              rmax = fmaxf(rmax, fabsf(r));
+            },
+            [&](int slot, int idx, float v) {
+              reinterpret_cast<__half*>(orec_v)[slot] = __float2half_rn(v);
+              orec_i[slot] = (unsigned char)idx;
+            });
+        d16 = g.scale;
+        d = __half2float(d16);
+        mn = __half2float(g.zero);
+        dm = g.dmax;
       }
-      *reinterpret_cast<uint2*>(orec_v) = make_uint2(ov[0] | ((unsigned int)ov[1] << 16), ov[2] | ((unsigned int)ov[3] << 16));
-      *reinterpret_cast<unsigned int*>(orec_i) = (unsigned int)oi[0] | ((unsigned int)oi[1] << 8) |
-                                                 ((unsigned int)oi[2] << 16) | ((unsigned int)oi[3] << 24);
-      rmax = (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
+      reinterpret_cast<__half2*>(rec + (SIDE == 0 ? sd.off_kscale : sd.off_vscale))[tid] = __halves2half2(d16, __float2half_rn(mn));
+      atomicMax(&dmax_bits, __float_as_uint(dm));       // non-negative floats order like their bit patterns
+      atomicMax(&smax_bits, __float_as_uint(d));
+      atomicMax(&rmax_bits, __float_as_uint(rmax));
+    }
+    __syncthreads();
+    if (tid == 0) {
+      reinterpret_cast<float*>(rec)[SIDE] = __uint_as_float(dmax_bits);
+      reinterpret_cast<float*>(rec)[2 + SIDE] = __uint_as_float(smax_bits);
+      if (R != nullptr) atomicMax(p.Rmax + bhl * 2 + SIDE, rmax_bits);
+      dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;       // the next updates come behind the next block's first barrier
+    }
+    // pack the codes into mma-fragment order (code_coord_k / code_coord_v), one 32-bit load per field
+    unsigned int* dst = reinterpret_cast<unsigned int*>(rec + (SIDE == 0 ? sd.off_kcodes : sd.off_vcodes));
+    if (SIDE == 0) {
+      constexpr int kWords = kSlab * kHeadDim * BITS / 32;            // words per slab
+      for (int li = tid; li < (L / kSlab) * kWords; li += 128) {
+        const int slab = li / kWords, wl = li % kWords;
+        const int w = wl & 3, lane = (wl >> 2) & 31, tau = wl >> 7;
+        const int tok = slab * kSlab + (lane >> 2) + 8 * (w & 1);
+        const int ch = 32 * F * tau + 16 * (w >> 1) + 4 * (lane & 3);
+        unsigned int word = 0;
+#pragma unroll
+        for (int j = 0; j < F; ++j)
+          word |= *reinterpret_cast<const unsigned int*>(&codes[tok * kCodePitch2 + ch + 32 * j]) << (BITS * j);
+        dst[li] = word;
+      }
     } else {
-      rmax = 0.f;
-      GroupResult g = process_group<BITS, 2>(
-          L, 2, [&](int e) { return __half2float(X[first + e * step]); },
-          [&](int e, int code, float r) {
-            code_at(e) = (unsigned char)code;
-            if (R != nullptr) R[SIDE == 0 ? e * kHeadDim + tid : first + e] = r;
-            rmax = fmaxf(rmax, fabsf(r));
-          },
-          [&](int slot, int idx, float v) {
-            reinterpret_cast<__half*>(orec_v)[slot] = __float2half_rn(v);
-            orec_i[slot] = (unsigned char)idx;
-          });
-      d16 = g.scale;
-      d = __half2float(d16);
-      mn = __half2float(g.zero);
-      dm = g.dmax;
-    }
-    reinterpret_cast<__half2*>(rec + (SIDE == 0 ? sd.off_kscale : sd.off_vscale))[tid] = __halves2half2(d16, __float2half_rn(mn));
-    atomicMax(&dmax_bits, __float_as_uint(dm));       // non-negative floats order like their bit patterns
-    atomicMax(&smax_bits, __float_as_uint(d));
-    atomicMax(&rmax_bits, __float_as_uint(rmax));
-  }
-  __syncthreads();
-  if (tid == 0) {
-    reinterpret_cast<float*>(rec)[SIDE] = __uint_as_float(dmax_bits);
-    reinterpret_cast<float*>(rec)[2 + SIDE] = __uint_as_float(smax_bits);
-    if (R != nullptr) atomicMax(p.Rmax + bhl * 2 + SIDE, rmax_bits);
-  }
-  // pack the codes into mma-fragment order (code_coord_k / code_coord_v), one 32-bit load per field
-  unsigned int* dst = reinterpret_cast<unsigned int*>(rec + (SIDE == 0 ? sd.off_kcodes : sd.off_vcodes));
-  if (SIDE == 0) {
-    constexpr int kWords = kSlab * kHeadDim * BITS / 32;            // words per slab
-    for (int li = tid; li < (L / kSlab) * kWords; li += 128) {
-      const int slab = li / kWords, wl = li % kWords;
-      const int w = wl & 3, lane = (wl >> 2) & 31, tau = wl >> 7;
-      const int tok = slab * kSlab + (lane >> 2) + 8 * (w & 1);
-      const int ch = 32 * F * tau + 16 * (w >> 1) + 4 * (lane & 3);
-      unsigned int word = 0;
+      constexpr int kWords = 32 * kHeadDim * BITS / 32;               // words per 32-token chunk
+      for (int li = tid; li < (T / 32) * kWords; li += 128) {
+        const int chunk = li / kWords, wl = li % kWords;
+        const int w = wl & 3, lane = (wl >> 2) & 31, tau = wl >> 7;
+        const int ch = 16 * F * tau + (lane >> 2) + 8 * (w & 1);
+        const int tok = chunk * 32 + 16 * (w >> 1) + 4 * (lane & 3);
+        unsigned int word = 0;
 #pragma unroll
-      for (int j = 0; j < F; ++j)
-        word |= *reinterpret_cast<const unsigned int*>(&codes[tok * kCodePitch2 + ch + 32 * j]) << (BITS * j);
-      dst[li] = word;
-    }
-  } else {
-    constexpr int kWords = 32 * kHeadDim * BITS / 32;               // words per 32-token chunk
-    for (int li = tid; li < (T / 32) * kWords; li += 128) {
-      const int chunk = li / kWords, wl = li % kWords;
-      const int w = wl & 3, lane = (wl >> 2) & 31, tau = wl >> 7;
-      const int ch = 16 * F * tau + (lane >> 2) + 8 * (w & 1);
-      const int tok = chunk * 32 + 16 * (w >> 1) + 4 * (lane & 3);
-      unsigned int word = 0;
-#pragma unroll
-      for (int j = 0; j < F; ++j)
-        word |= *reinterpret_cast<const unsigned int*>(&codes[(ch + 16 * j) * kCodePitch2 + tok]) << (BITS * j);
-      dst[li] = word;
+        for (int j = 0; j < F; ++j)
+          word |= *reinterpret_cast<const unsigned int*>(&codes[(ch + 16 * j) * kCodePitch2 + tok]) << (BITS * j);
+        dst[li] = word;
+      }
     }
   }
 }
@@ -1517,7 +1604,7 @@ __global__ void __launch_bounds__(256) push_kernel(PushArgs p) {
 // Filter / Quant / pack / residual of a long segment: per side, the register-resident kernel that fits the group
 // shape, else the general one.  side0 = 1: the value side only.  Returns the number of launches through *launches.
 template <int BITS>
-static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, cudaStream_t st, int* launches) {
+static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, int sms, cudaStream_t st, int* launches) {
   const int T = a.seg.T;
   const size_t smem = round_up(T * kXPitch * 2, 16) + (size_t)T * kRPitch * 4;
   const dim3 grid(a.seg.nblk, nbh, 1);
@@ -1526,17 +1613,21 @@ static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, cudaSt
   for (int side = first_side; side < 2; ++side) {
     const int len = side == 0 ? T : a.cc.g_v, k = side == 0 ? a.seg.k_k : a.cc.k_v;
     cudaError_t e = cudaSuccess;
+    const long long items = (long long)a.seg.nblk * nbh;
+    const long long room = (long long)(len == kFast2Len && side == 0 ? kFast2KeyCtasPerSm : kFastCtasPerSm) * sms;
+    const int ctas = (int)(items < room ? items : room);
     if (T == kFastLen && len == kFastLen && k == 1) {
-      if (side == 0) {
-        quant_fast_kernel<BITS, 0><<<grid, 128, 0, st>>>(a);
-      } else {
-        e = cudaFuncSetAttribute(quant_fast_kernel<BITS, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFastSmemV);
-        if (e != cudaSuccess) return e;
-        quant_fast_kernel<BITS, 1><<<grid, 128, kFastSmemV, st>>>(a);
-      }
+      if (side == 0) quant_fast_kernel<BITS, 0><<<ctas, 128, 0, st>>>(a, nbh);
+      else quant_fast_kernel<BITS, 1><<<ctas, 128, 0, st>>>(a, nbh);
     } else if (len == kFast2Len && k == 2 && T % 32 == 0 && T <= kFast2Len) {
-      if (side == 0) quant_fast2_kernel<BITS, 0><<<grid, 128, 0, st>>>(a);
-      else quant_fast2_kernel<BITS, 1><<<grid, 128, 0, st>>>(a);
+      const int tile = T * kHeadDim * 2;
+      auto launch = [&](auto kern) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFast2Len * kHeadDim * 2);
+        if (e == cudaSuccess) kern<<<ctas, 128, tile, st>>>(a, nbh);
+      };
+      if (side == 0) launch(quant_fast2_kernel<BITS, 0>);
+      else launch(quant_fast2_kernel<BITS, 1>);
+      if (e != cudaSuccess) return e;
     } else {
       a.side0 = side;
 #define GEAR_LAUNCH_Q(KM)                                                                                   \
@@ -1620,12 +1711,12 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
   ca.seg = sd; ca.cc = job.cc; ca.arena = job.arena; ca.bh0 = bh0;
   ca.K = job.K + (size_t)bh0 * sd.n_c * kHeadDim;
   ca.V = job.V + (size_t)bh0 * sd.n_c * kHeadDim;
-  ca.R = pa.R; ca.Rmax = pa.Rmax;
+  ca.R = pa.R; ca.Rmax = pa.Rmax; ca.status = job.status;
   const int kneed = sd.k_k > job.cc.k_v ? sd.k_k : job.cc.k_v;
   const bool per_vector = sd.csr_base16 != 0;          // keys: one group per channel over the whole segment
   ca.side0 = per_vector ? 1 : 0;
   int n_quant = 0;
-  cudaError_t e = job.cc.bits == 2 ? launch_quant<2>(ca, nbh, kneed, st, &n_quant) : launch_quant<4>(ca, nbh, kneed, st, &n_quant);
+  cudaError_t e = job.cc.bits == 2 ? launch_quant<2>(ca, nbh, kneed, job.sms, st, &n_quant) : launch_quant<4>(ca, nbh, kneed, job.sms, st, &n_quant);
   if (e != cudaSuccess) return e;
   count_launches(n_quant);
   if (per_vector) {

@@ -22,6 +22,7 @@ struct CompressArgs {
   unsigned int* Rmax;   // [nbh][2] bit patterns of max |R| per tile (zeroed before the launch), with R
   int bh0;              // first (batch, head) of the range, for addressing the records
   int side0;            // first side the launch covers (blockIdx.z + side0: 0 keys, 1 values)
+  int* status;          // the cache's status word
 };
 
 // Key side of a segment with per-vector grouping (gear_kcvt.cu)
