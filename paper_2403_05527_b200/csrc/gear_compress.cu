@@ -271,9 +271,9 @@ __global__ void __launch_bounds__(128) quant_pack_kernel(CompressArgs p) {
 }
 
 // ---------------------------------------------------------------------------
-// The same step for the common shape -- blocks of 64 tokens, value groups of 64 channels, one outlier per side and
-// group (s <= 3.1 %) -- with the group in registers: a thread owns one group (keys: a channel's 64 tokens, read as a
-// column; values: 64 consecutive channels of a token), walks it in fully unrolled loops, stores the residual itself and
+// The same step for groups of L = 32, 64 or 128 entries with at most one outlier per side (64 at s <= 3.1 %, 128 at s <= 1.5 %)
+// with the group in registers: a thread owns one group (keys: a channel's L tokens, read as a column of a block of L tokens;
+// values: L consecutive channels of a token; a block has 128 groups), walks it in fully unrolled loops, stores the residual itself and
 // leaves only the codes in shared memory, one byte each, transposed so that the packing step fetches the four codes
 // of an output byte row with one 32-bit load.  Every code, scale, outlier and residual is bit-identical to
 // quant_pack_kernel: the operations on a group are the same binary32 sequence.
@@ -283,15 +283,17 @@ __global__ void __launch_bounds__(128) quant_pack_kernel(CompressArgs p) {
 // waits for a load it has just issued; the entries' arithmetic runs on pairs (f32x2); a value group reads and writes its
 // own 32-byte sectors (256-bit stores), so the residual takes no way through shared memory.  Against one CTA per block,
 // scalar arithmetic and a residual staged through shared memory (2 bits, 8 x 32 heads x 4096): keys 181 -> 153 us, values
-// 261 -> 168 us; 4 bits, 16 x 40 heads x 8192: 469 -> 415 and 652 -> 434 us.
+// 261 -> 168 us; 4 bits, 16 x 40 heads x 8192: 469 -> 415 and 652 -> 434 us.  Against quant_pack_kernel (8 x 32 heads x 4096,
+// keys / values): groups of 32 283 / 298 -> 165 / 175 us, of 64 without outliers 266 / 299 -> 150 / 159, of 128 with one
+// outlier 581 / 604 -> 172 / 169, without 441 / 480 -> 146 / 162, values of per-vector keys 517 -> 209.
 // ---------------------------------------------------------------------------
-constexpr int kFastLen = 64;
 constexpr int kCodePitchK = kHeadDim + 4;   // bytes per token row of the key codes  [token][channel]
-constexpr int kCodePitchV = kFastLen + 4;   // bytes per channel row of the value codes [channel][token]
-// 128 registers, no spills.  Five or six CTAs (96 or 80 registers) are slower on both sides: keys 153 -> 166 -> 196 us, values
-// 168 -> 169 -> 171 us (the first size above).
-constexpr int kFastCtasPerSm = 4;
-constexpr int kFast2KeyCtasPerSm = 3;       // a channel's 128 tokens in registers: at four CTAs they spill (240 -> 204 us)
+// CTAs per SM.  L = 64 (128 registers): five or six are slower, keys 153 -> 166 -> 196 us, values 168 -> 169 -> 171 (8 x 32 heads
+// x 4096).  Columns of 128 tokens spill at four (240 us against 204 with two outliers, 4 x 8 heads x 32768).  L = 32: five,
+// six and eight are alike.
+__host__ __device__ constexpr int fast_ctas_per_sm(int side, int len) {
+  return len == 32 ? 6 : len == kHeadDim && side == 0 ? 3 : 4;
+}
 
 // pairs of binary32 operations, each rounded like the scalar one
 struct F32x2 { unsigned long long v; };
@@ -352,17 +354,34 @@ struct BlockFeed {
   }
 };
 
-template <int BITS, int SIDE>
-__global__ void __launch_bounds__(128, kFastCtasPerSm) quant_fast_kernel(CompressArgs p, int nbh) {
-  constexpr int L = kFastLen, F = 8 / BITS;
-  constexpr int side = SIDE;
-  __shared__ __align__(128) unsigned char tile[L * kHeadDim * 2];
+// Entry of the first set bit of L mask bits: bit t of the low / high half of word w stands for entry 2 (16 w + t) / that + 1 of
+// a group whose pairs are rotated by `turn` (a multiple of four).  An entry of the group also if no bit is set (all NaN).
+template <int L>
+__device__ __forceinline__ int first_set(const unsigned int (&m)[4], int turn) {
+  auto first = [&](unsigned int sel) {
+    const unsigned int lo = __byte_perm(m[0], m[L == 32 ? 0 : 1], sel);            // 32 entries: their 16 bits twice
+    if (L <= 64) return __ffs((int)__funnelshift_l(lo, lo, turn)) - 1;
+    const unsigned int hi = __byte_perm(m[2], m[3], sel);
+    const unsigned int l = __funnelshift_l(hi, lo, turn), h = __funnelshift_l(lo, hi, turn);
+    return l ? __ffs((int)l) - 1 : h ? 32 + __ffs((int)h) - 1 : -1;
+  };
+  const int even = first(0x5410), odd = first(0x7632);
+  return min(L - 1, min(even < 0 ? L : 2 * even, odd < 0 ? L : 2 * odd + 1));
+}
+
+template <int BITS, int SIDE, int L, int K>
+__global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_kernel(CompressArgs p, int nbh) {
+  constexpr int F = 8 / BITS, side = SIDE, kGroups = kHeadDim / L, kPieces = L / 8;
+  constexpr int kCodePitchV = L + 4;               // bytes per channel row of the value codes [channel][token]
+  extern __shared__ __align__(128) unsigned char tile[];            // the block's T x 128 fp16 entries
   __shared__ __align__(16) unsigned char codes[SIDE == 0 ? L * kCodePitchK : kHeadDim * kCodePitchV];
   __shared__ uint64_t full;
   __shared__ unsigned int dmax_bits, smax_bits, rmax_bits;
   const SegDesc& sd = p.seg;
   const int tid = threadIdx.x;
-  BlockFeed feed{tile, &full, side == 0 ? p.K : p.V, sd.n_c, sd.nblk, L, sd.nblk * nbh, 0u};
+  const int T = SIDE == 1 && L == kHeadDim ? sd.T : L;              // tokens of a block; values: 128 / L groups each
+  const bool active = L < kHeadDim || SIDE == 0 || tid < T;         // a thread per group
+  BlockFeed feed{tile, &full, side == 0 ? p.K : p.V, sd.n_c, sd.nblk, T, sd.nblk * nbh, 0u};
   if (tid == 0) {
     dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;
     bar_init(&full);
@@ -372,17 +391,18 @@ __global__ void __launch_bounds__(128, kFastCtasPerSm) quant_fast_kernel(Compres
   __syncthreads();
   const __half* group = reinterpret_cast<const __half*>(tile) + (side == 0 ? tid : tid * L);   // entry e: group[e * step]
   constexpr int step = SIDE == 0 ? kHeadDim : 1;
-  const int rot = SIDE == 0 ? 0 : tid & 7;        // values: a thread starts with another 16-byte piece than its neighbours
+  // values: a thread starts with another 16-byte piece than the neighbours whose groups lie in the same banks
+  const int rot = SIDE == 0 ? 0 : L == 32 ? (tid >> 1) & 3 : tid & 7;
 
   for (int item = blockIdx.x; item < feed.total; item += gridDim.x) {
     const int bhl = item / sd.nblk, blk = item - bhl * sd.nblk;
     const bool ok = bar_wait(&full, feed.parity);
     feed.parity ^= 1u;
-    float* R = p.R ? p.R + (((size_t)bhl * 2 + side) * sd.n_c + (size_t)blk * L) * kHeadDim : nullptr;
+    float* R = p.R ? p.R + (((size_t)bhl * 2 + side) * sd.n_c + (size_t)blk * T) * kHeadDim : nullptr;
     unsigned char* rec = p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride + sd.bfac_bytes +
                          (size_t)blk * sd.rec_bytes;
 
-    // the group as 32 packed pairs: keys entries 2q, 2q + 1; values the same, in pieces of eight entries from piece `rot` on
+    // the group as packed pairs: keys entries 2q, 2q + 1; values the same, in pieces of eight entries from piece `rot` on
     __half2 xp[L / 2];
     if (side == 0) {
 #pragma unroll
@@ -390,8 +410,8 @@ __global__ void __launch_bounds__(128, kFastCtasPerSm) quant_fast_kernel(Compres
     } else {
       const uint4* src = reinterpret_cast<const uint4*>(group);
 #pragma unroll
-      for (int q = 0; q < L / 8; ++q) {
-        const uint4 v = src[(q + rot) & 7];
+      for (int q = 0; q < kPieces; ++q) {
+        const uint4 v = active ? src[(q + rot) & (kPieces - 1)] : make_uint4(0u, 0u, 0u, 0u);
         xp[4 * q] = *reinterpret_cast<const __half2*>(&v.x);
         xp[4 * q + 1] = *reinterpret_cast<const __half2*>(&v.y);
         xp[4 * q + 2] = *reinterpret_cast<const __half2*>(&v.z);
@@ -399,49 +419,42 @@ __global__ void __launch_bounds__(128, kFastCtasPerSm) quant_fast_kernel(Compres
       }
     }
     // Filter_s (Eq. 4), one entry per side: the largest and the smallest entry leave the group, the second largest and
-    // second smallest instances bound what is kept.  Comparisons of fp16 values are exact in fp16, so the search runs on
-    // the packed pairs: even and odd entries keep their own two largest / smallest and are merged at the end.
-    float max1, max2, min1, min2;
+    // second smallest instances bound what is kept (no outliers: the largest and the smallest).  Comparisons of fp16 values
+    // are exact in fp16, so the search runs on the packed pairs: even and odd entries keep their own two largest / smallest
+    // and are merged at the end.
+    float mx, mn;
+    int imax = 0, imin = 1;
     {
       const __half2 ninf = __float2half2_rn(-INFINITY), pinf = __float2half2_rn(INFINITY);
       __half2 M1 = ninf, M2 = ninf, m1 = pinf, m2 = pinf;
 #pragma unroll
       for (int q = 0; q < L / 2; ++q) {
-        M2 = __hmax2(M2, __hmin2(xp[q], M1));
+        if (K == 1) {
+          M2 = __hmax2(M2, __hmin2(xp[q], M1));
+          m2 = __hmin2(m2, __hmax2(xp[q], m1));
+        }
         M1 = __hmax2(M1, xp[q]);
-        m2 = __hmin2(m2, __hmax2(xp[q], m1));
         m1 = __hmin2(m1, xp[q]);
       }
       const float2 fM1 = __half22float2(M1), fM2 = __half22float2(M2), fm1 = __half22float2(m1), fm2 = __half22float2(m2);
-      max1 = fmaxf(fM1.x, fM1.y);
-      max2 = fmaxf(fminf(fM1.x, fM1.y), fmaxf(fM2.x, fM2.y));
-      min1 = fminf(fm1.x, fm1.y);
-      min2 = fminf(fmaxf(fm1.x, fm1.y), fminf(fm2.x, fm2.y));
-    }
-    // first index of the maximum and of the minimum (ties go to the lower index): one mask bit per entry
-    int imax, imin;
-    {
-      const __half2 vM = __float2half2_rn(max1), vm = __float2half2_rn(min1);
-      unsigned int a0 = 0u, a1 = 0u, b0 = 0u, b1 = 0u;   // bit q of a half word: pair q (a0, b0) or pair 16 + q (a1, b1)
+      const float max1 = fmaxf(fM1.x, fM1.y), min1 = fminf(fm1.x, fm1.y);
+      mx = K == 0 ? max1 : fmaxf(fminf(fM1.x, fM1.y), fmaxf(fM2.x, fM2.y));
+      mn = K == 0 ? min1 : fminf(fmaxf(fm1.x, fm1.y), fminf(fm2.x, fm2.y));
+      // first index of the maximum and of the minimum (ties go to the lower index): one mask bit per entry
+      if (K == 1) {
+        const __half2 vM = __float2half2_rn(max1), vm = __float2half2_rn(min1);
+        unsigned int a[4] = {0u, 0u, 0u, 0u}, b[4] = {0u, 0u, 0u, 0u};   // bit t of a half of word w: pair 16 w + t
 #pragma unroll
-      for (int q = 0; q < L / 2; ++q) {
-        const unsigned int bit = 0x00010001u << (q & 15);
-        const unsigned int eM = __heq2_mask(xp[q], vM) & bit, em = __heq2_mask(xp[q], vm) & bit;
-        if (q < 16) { a0 |= eM; b0 |= em; } else { a1 |= eM; b1 |= em; }
+        for (int q = 0; q < L / 2; ++q) {
+          const unsigned int bit = 0x00010001u << (q & 15);
+          a[q >> 4] |= __heq2_mask(xp[q], vM) & bit;
+          b[q >> 4] |= __heq2_mask(xp[q], vm) & bit;
+        }
+        imax = first_set<L>(a, 4 * rot);
+        imin = first_set<L>(b, 4 * rot);
+        if (imin == imax) imin = 1;           // all entries equal: the bottom entry is the next index
       }
-      auto first_set = [&](unsigned int lo16, unsigned int hi16) {
-        // bit q: entry 2 q / 2 q + 1 (values: the pieces back in order)
-        const unsigned int even = __funnelshift_l(__byte_perm(lo16, hi16, 0x5410), __byte_perm(lo16, hi16, 0x5410), 4 * rot);
-        const unsigned int odd = __funnelshift_l(__byte_perm(lo16, hi16, 0x7632), __byte_perm(lo16, hi16, 0x7632), 4 * rot);
-        const int fe = even ? 2 * (__ffs((int)even) - 1) : L;
-        const int fo = odd ? 2 * (__ffs((int)odd) - 1) + 1 : L;
-        return min(fe, fo);
-      };
-      imax = first_set(a0, a1);
-      imin = first_set(b0, b1);
     }
-    if (imin == imax) imin = 1;               // all entries equal: the bottom entry is the next index
-    const float mn = min2, mx = max2;
     // Eq. 2 on the kept entries: binary32, one rounding per operation
     const float levels = (float)((1 << BITS) - 1);
     const float range = __fsub_rn(mx, mn);
@@ -449,7 +462,8 @@ __global__ void __launch_bounds__(128, kFastCtasPerSm) quant_fast_kernel(Compres
     const __half d16 = __float2half_rn(d32);
     const float d = __half2float(d16);
     const float inv = d != 0.f ? __fdiv_rn(1.0f, d) : 0.f;
-    const __half vmax = group[imax * step], vmin = group[imin * step];
+    __half vmax = __ushort_as_half(0), vmin = vmax;
+    if (K == 1 && active) { vmax = group[imax * step]; vmin = group[imin * step]; }
     if (__syncthreads_or(!ok)) {              // every thread has read the block
       if (tid == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
       break;
@@ -469,18 +483,20 @@ __global__ void __launch_bounds__(128, kFastCtasPerSm) quant_fast_kernel(Compres
           R[(2 * q + 1) * kHeadDim + tid] = r.y;
         }
       }
-      codes[imax * kCodePitchK + tid] = 0;
-      codes[imin * kCodePitchK + tid] = 0;
-      if (R != nullptr) {
-        R[imax * kHeadDim + tid] = 0.f;
-        R[imin * kHeadDim + tid] = 0.f;
+      if (K == 1) {
+        codes[imax * kCodePitchK + tid] = 0;
+        codes[imin * kCodePitchK + tid] = 0;
+        if (R != nullptr) {
+          R[imax * kHeadDim + tid] = 0.f;
+          R[imin * kHeadDim + tid] = 0.f;
+        }
       }
-    } else {
-      const int tok = tid >> 1;
-      unsigned char* mine = codes + (tid & 1) * L * kCodePitchV + tok;
+    } else if (active) {
+      const int tok = tid / kGroups;
+      unsigned char* mine = codes + (tid % kGroups) * L * kCodePitchV + tok;
 #pragma unroll
-      for (int q = 0; q < L / 8; ++q) {
-        const int piece = (q + rot) & 7;
+      for (int q = 0; q < kPieces; ++q) {
+        const int piece = (q + rot) & (kPieces - 1);
         unsigned char* cp = mine + piece * 8 * kCodePitchV;
         float2 r[4];
 #pragma unroll
@@ -492,29 +508,35 @@ __global__ void __launch_bounds__(128, kFastCtasPerSm) quant_fast_kernel(Compres
         }
         if (R != nullptr) store8(R + tid * L + piece * 8, r);
       }
-      mine[imax * kCodePitchV] = 0;
-      mine[imin * kCodePitchV] = 0;
-      if (R != nullptr) {
-        R[tid * L + imax] = 0.f;
-        R[tid * L + imin] = 0.f;
+      if (K == 1) {
+        mine[imax * kCodePitchV] = 0;
+        mine[imin * kCodePitchV] = 0;
+        if (R != nullptr) {
+          R[tid * L + imax] = 0.f;
+          R[tid * L + imin] = 0.f;
+        }
       }
     }
     // A bound on the group's residuals instead of their maximum (it only picks the power of two the power iteration
     // scales by): half a step for a kept entry, the whole range if the step rounded to zero, plus the rounding of the
     // dequantised value
-    float rmax = (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
+    float rmax = active ? (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx)) : 0.f;
     // the group's scale, zero point and its two outliers (in-group index ascending)
     {
-      const bool max_first = imax < imin;
-      const __half2 ov = max_first ? __halves2half2(vmax, vmin) : __halves2half2(vmin, vmax);
-      const uchar2 oi = max_first ? make_uchar2((unsigned char)imax, (unsigned char)imin)
-                                  : make_uchar2((unsigned char)imin, (unsigned char)imax);
-      reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_koval : sd.off_voval))[tid] = ov;
-      reinterpret_cast<uchar2*>(rec + (side == 0 ? sd.off_koidx : sd.off_voidx))[tid] = oi;
-      reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_kscale : sd.off_vscale))[tid] =
-          __halves2half2(d16, __float2half_rn(mn));
-      float dm = fmaxf(fabsf(__half2float(vmax) - mn), fabsf(__half2float(vmin) - mn));
-      float sm = d;
+      if (K == 1 && active) {
+        const bool max_first = imax < imin;
+        const __half2 ov = max_first ? __halves2half2(vmax, vmin) : __halves2half2(vmin, vmax);
+        const uchar2 oi = max_first ? make_uchar2((unsigned char)imax, (unsigned char)imin)
+                                    : make_uchar2((unsigned char)imin, (unsigned char)imax);
+        reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_koval : sd.off_voval))[tid] = ov;
+        reinterpret_cast<uchar2*>(rec + (side == 0 ? sd.off_koidx : sd.off_voidx))[tid] = oi;
+      }
+      if (active) {
+        reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_kscale : sd.off_vscale))[tid] =
+            __halves2half2(d16, __float2half_rn(mn));
+      }
+      float dm = K == 1 && active ? fmaxf(fabsf(__half2float(vmax) - mn), fabsf(__half2float(vmin) - mn)) : 0.f;
+      float sm = active ? d : 0.f;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         dm = fmaxf(dm, __shfl_xor_sync(0xffffffffu, dm, o));
@@ -552,7 +574,7 @@ __global__ void __launch_bounds__(128, kFastCtasPerSm) quant_fast_kernel(Compres
       }
     } else {
       constexpr int kWords = 32 * kHeadDim * BITS / 32;               // words per 32-token chunk
-      for (int li = tid; li < (L / 32) * kWords; li += 128) {
+      for (int li = tid; li < (T / 32) * kWords; li += 128) {
         const int chunk = li / kWords, wl = li % kWords;
         const int w = wl & 3, lane = (wl >> 2) & 31, tau = wl >> 7;
         const int ch = 16 * F * tau + (lane >> 2) + 8 * (w & 1);
@@ -613,7 +635,7 @@ __device__ __forceinline__ void top3_of6(float (&v)[6], float (&out)[3]) {
 }
 
 template <int BITS, int SIDE>
-__global__ void __launch_bounds__(128, SIDE == 0 ? kFast2KeyCtasPerSm : kFastCtasPerSm) quant_fast2_kernel(CompressArgs p, int nbh) {
+__global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_fast2_kernel(CompressArgs p, int nbh) {
   constexpr int L = kFast2Len, F = 8 / BITS;
   extern __shared__ __align__(128) unsigned char tile[];            // the block's T x 128 fp16 entries
   __shared__ __align__(16) unsigned char codes[L * kCodePitch2];    // keys [token][channel], values [channel][token]
@@ -1614,20 +1636,26 @@ static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, int sm
     const int len = side == 0 ? T : a.cc.g_v, k = side == 0 ? a.seg.k_k : a.cc.k_v;
     cudaError_t e = cudaSuccess;
     const long long items = (long long)a.seg.nblk * nbh;
-    const long long room = (long long)(len == kFast2Len && side == 0 ? kFast2KeyCtasPerSm : kFastCtasPerSm) * sms;
+    // a thread per group of 32, 64 or 128 entries (values of 128: one per token, whole 32-token chunks of codes)
+    const bool shape = len == kHeadDim && side == 1 ? T % 32 == 0 && T <= kHeadDim : T == len;
+    const long long room = (long long)fast_ctas_per_sm(side, len) * sms;
     const int ctas = (int)(items < room ? items : room);
-    if (T == kFastLen && len == kFastLen && k == 1) {
-      if (side == 0) quant_fast_kernel<BITS, 0><<<ctas, 128, 0, st>>>(a, nbh);
-      else quant_fast_kernel<BITS, 1><<<ctas, 128, 0, st>>>(a, nbh);
-    } else if (len == kFast2Len && k == 2 && T % 32 == 0 && T <= kFast2Len) {
+    auto launch = [&](auto kern) {
       const int tile = T * kHeadDim * 2;
-      auto launch = [&](auto kern) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFast2Len * kHeadDim * 2);
-        if (e == cudaSuccess) kern<<<ctas, 128, tile, st>>>(a, nbh);
-      };
-      if (side == 0) launch(quant_fast2_kernel<BITS, 0>);
-      else launch(quant_fast2_kernel<BITS, 1>);
-      if (e != cudaSuccess) return e;
+      if (len == kHeadDim) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadDim * kHeadDim * 2);
+      if (e == cudaSuccess) kern<<<ctas, 128, tile, st>>>(a, nbh);
+    };
+#define GEAR_LAUNCH_FAST(LEN, K) \
+  if (side == 0) launch(quant_fast_kernel<BITS, 0, LEN, K>); else launch(quant_fast_kernel<BITS, 1, LEN, K>);
+    if (shape && len == 32 && k == 0) { GEAR_LAUNCH_FAST(32, 0) }
+    else if (shape && len == 32 && k == 1) { GEAR_LAUNCH_FAST(32, 1) }
+    else if (shape && len == 64 && k == 0) { GEAR_LAUNCH_FAST(64, 0) }
+    else if (shape && len == 64 && k == 1) { GEAR_LAUNCH_FAST(64, 1) }
+    else if (shape && len == 128 && k == 0) { GEAR_LAUNCH_FAST(128, 0) }
+    else if (shape && len == 128 && k == 1) { GEAR_LAUNCH_FAST(128, 1) }
+    else if (shape && len == 128 && k == 2) {
+      if (side == 0) launch(quant_fast2_kernel<BITS, 0>); else launch(quant_fast2_kernel<BITS, 1>);
+#undef GEAR_LAUNCH_FAST
     } else {
       a.side0 = side;
 #define GEAR_LAUNCH_Q(KM)                                                                                   \
@@ -1643,6 +1671,7 @@ static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, int sm
       else GEAR_LAUNCH_Q(8)
 #undef GEAR_LAUNCH_Q
     }
+    if (e != cudaSuccess) return e;
     *launches += 1;
   }
   return cudaGetLastError();

@@ -1,4 +1,4 @@
-"""Quantization of groups of 64 and 128 by CTAs that take one block after the other: more blocks than the device holds
+"""Quantization of groups of 32, 64 and 128 by CTAs that take one block after the other: more blocks than the device holds
 CTAs for, a single block, and values that lie half way between two codes."""
 import numpy as np
 import pytest
@@ -6,20 +6,25 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("bits,group,H,n,rank", [
-    (2, 64, 11, 4096, 1),      # 704 blocks per side
-    (4, 64, 11, 4096, 0),      # the same without a residual
-    (4, 128, 6, 16384, 1),     # 768 blocks per side
-    (2, 128, 1, 128, 1),       # one block
-    (4, 64, 1, 64, 1),
+@pytest.mark.parametrize("bits,group,s_pct,H,n,rank", [
+    (2, 64, 2.0, 11, 4096, 1),      # one outlier per side and group; 704 blocks per side
+    (4, 64, 2.0, 11, 4096, 0),      # the same without a residual
+    (4, 128, 2.0, 6, 16384, 1),     # two outliers; 768 blocks per side
+    (2, 128, 2.0, 1, 128, 1),       # one block
+    (4, 64, 2.0, 1, 64, 1),
+    (2, 64, 0.0, 3, 1024, 1),       # no outliers
+    (4, 32, 2.0, 13, 4096, 1),      # groups of 32; 1664 blocks per side
+    (2, 32, 0.0, 1, 32, 1),
+    (2, 128, 1.0, 2, 1024, 1),      # groups of 128 with one outlier
+    (4, 128, 0.0, 5, 512, 1),
 ])
-def test_blocks_and_ties(bits, group, H, n, rank):
+def test_blocks_and_ties(bits, group, s_pct, H, n, rank):
     """A grid of 1.5 under a step of 3: x / 3 is not exact in binary32, and the rounded product is half way between two codes
     where the exact one is not.  Codes, scales and outliers have to be the oracle's bit for bit."""
     import torch
     from paper_2403_05527_b200 import binding as G, synth
     from tests.gear_harness import Pair
-    p = Pair(16, 1, H, H, bits, group, 2.0, 64, 1, n + 128, r_max=1, iters=1)
+    p = Pair(16, 1, H, H, bits, group, s_pct, 64, 1, n + 128, r_max=1, iters=1)
     try:
         top = 3 * (2 ** bits - 1)
         gen = np.random.default_rng(n + bits)
@@ -34,3 +39,26 @@ def test_blocks_and_ties(bits, group, H, n, rank):
         p.check_segment(0)
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("s_pct", [0.0, 1.0])
+@pytest.mark.parametrize("kind", ["equal", "one peak"])
+def test_flat_groups(kind, s_pct):
+    """Groups whose entries are all equal (the bottom outlier is the next index), or equal but for one on each side."""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+    from tests.gear_harness import Pair
+    for group in (32, 64, 128):
+        p = Pair(16, 1, 1, 1, 2, group, s_pct, 64, 0, 512)
+        try:
+            x = np.full((1, 1, 2 * group, 128), 1.25, np.float16)
+            if kind == "one peak":
+                x[0, 0, 5::group, :] = 9.0
+                x[0, 0, :, 7::group] = -9.0
+            p.oracle.compress(x, x, 0, np.zeros((1, 1, 2, 128, 0), np.float32))
+            xd = torch.from_numpy(x).cuda()
+            G.gear_compress(p.cache, None, xd, xd, 2 * group, 0, None)
+            torch.cuda.synchronize()
+            p.check_segment(0)
+        finally:
+            p.close()
