@@ -141,3 +141,24 @@ def test_capacity_of_the_arena_is_an_error_not_a_fault():
         assert G.gear_last_device_status(cache) == 0
     finally:
         G.gear_free(cache)
+
+
+@pytest.mark.parametrize("n,s", [(192, 2.0), (4096, 4.0), (4096, 2.0), (8192, 5.0), (4160, 2.0)])
+def test_selection_of_the_outliers(pair_factory, n, s):
+    """Counts of outliers on both sides of the select kernel's limits (one or two extremes per lane, the histograms), and
+    channels whose extremes all lie with few lanes, that are sorted, rounded to few values or zeros of both signs."""
+    import torch
+    from paper_2403_05527_b200 import binding as G, synth
+    k16, v16 = synth.make_kv(9, 1, 1, n, 128)
+    t = np.arange(n)
+    k16[0, 0, t % 256 < 8, 3] += np.float16(40.0)          # a lane's eight neighbours, every 256 tokens
+    k16[0, 0, t % 256 < 8, 3] *= (1 + t[t % 256 < 8] / n).astype(np.float16)
+    k16[0, 0, :, 4] = np.sort(k16[0, 0, :, 4])
+    k16[0, 0, :, 5] = np.sort(k16[0, 0, :, 5])[::-1]
+    k16[0, 0, :, 6] = np.round(k16[0, 0, :, 6] * 4) / 4    # ties at both thresholds
+    k16[0, 0, :, 7] = np.sign(k16[0, 0, :, 7]) * np.float16(0.0) + (t == 11) - (t == 12)
+    p = pair_factory(9, 1, 1, 1, 4, 0, s, 64, 0, n + 64, r_max=0)
+    p.oracle.compress(k16, v16, 0, None)
+    G.gear_compress(p.cache, None, torch.from_numpy(k16).to(p.dev), torch.from_numpy(v16).to(p.dev), n, 0, None)
+    torch.cuda.synchronize()
+    p.check_segment(0)
