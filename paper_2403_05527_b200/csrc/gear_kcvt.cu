@@ -17,6 +17,7 @@ namespace gear {
 
 constexpr int kSelChannels = 8;     // channels per CTA of the select kernel, one per warp
 constexpr int kBlockTok = 64;       // tokens per record block of such a segment
+constexpr int kListAhead = 16;      // list entries that a thread of the list kernel loads at once
 
 // Two fp16 values <-> two 16-bit keys with the order of the values; -0 and +0 share a key.
 __device__ __forceinline__ unsigned int order_keys(unsigned int h2) {
@@ -220,6 +221,10 @@ __device__ __forceinline__ bool select_channel(unsigned short* keys, int n, int 
   return true;
 }
 
+// Bound: shared-memory and load / store pipes (rows of the CTA's eight channels are 16 to 32 bytes of a line each), with the
+// residual's bytes behind them; two histogram levels over all entries and residuals staged in shared memory made it 1145 us at 8 x 32
+// heads x 4096, 4 bits, s = 2 %, now 517 (2 x 32 x 8192: 911 -> 309).  Two warps per channel, one for either side, come to the same
+// (523 and 275 us, but 83 -> 99 at 4 x 32 x 1024).
 template <int BITS>
 __global__ void __launch_bounds__(kSelChannels * 32, 2) kcvt_select_kernel(KcvtArgs p) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -364,6 +369,8 @@ __global__ void __launch_bounds__(kSelChannels * 32, 2) kcvt_select_kernel(KcvtA
 
 // One CTA per (batch, head): the per-channel outlier lists (token ascending) become per-block lists, and every
 // block record gets its header fields of the key side and the channels' (scale, zero).
+// Bound: latency; a channel's list is walked by one thread, so its entries are loaded sixteen at a time (8 x 32 heads x 4096
+// 57 -> 36 us).
 __global__ void __launch_bounds__(256) kcvt_list_kernel(KcvtArgs p) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   const SegDesc& sd = p.seg;
@@ -379,7 +386,14 @@ __global__ void __launch_bounds__(256) kcvt_list_kernel(KcvtArgs p) {
   const unsigned int* olist = p.olist + (size_t)bhl * kHeadDim * k2;
   const __half2* sz = p.sz + (size_t)bhl * kHeadDim;
   if (tid < kHeadDim) {
-    for (int e = 0; e < k2; ++e) cnt[((olist[tid * k2 + e] & 0xFFFFu) / kBlockTok) * kHeadDim + tid] += 1u;
+    for (int e0 = 0; e0 < k2; e0 += kListAhead) {
+      unsigned int w[kListAhead];
+#pragma unroll
+      for (int i = 0; i < kListAhead; ++i) w[i] = e0 + i < k2 ? olist[tid * k2 + e0 + i] : 0u;
+#pragma unroll
+      for (int i = 0; i < kListAhead; ++i)
+        if (e0 + i < k2) cnt[((w[i] & 0xFFFFu) / kBlockTok) * kHeadDim + tid] += 1u;
+    }
     atomicMax(&smax_bits, __float_as_uint(__low2float(sz[tid])));      // scales are non-negative
   }
   __syncthreads();
@@ -402,15 +416,22 @@ __global__ void __launch_bounds__(256) kcvt_list_kernel(KcvtArgs p) {
   if (tid < kHeadDim) {
     const float zero = __high2float(sz[tid]);
     int prev_blk = -1, run = 0;
-    for (int e = 0; e < k2; ++e) {
-      const unsigned int w = olist[tid * k2 + e];
-      const int tok = (int)(w & 0xFFFFu), blk = tok / kBlockTok;
-      run = blk == prev_blk ? run + 1 : 0;
-      prev_blk = blk;
-      g_ent[off[blk] + cnt[blk * kHeadDim + tid] + run] =
-          (unsigned int)(tok - blk * kBlockTok) | ((unsigned int)tid << 8) | (w & 0xFFFF0000u);
-      const float v = __half2float(__ushort_as_half((unsigned short)(w >> 16)));
-      atomicMax(&dmax[blk], __float_as_uint(fabsf(v - zero)));
+    for (int e0 = 0; e0 < k2; e0 += kListAhead) {
+      unsigned int ws[kListAhead];
+#pragma unroll
+      for (int i = 0; i < kListAhead; ++i) ws[i] = e0 + i < k2 ? olist[tid * k2 + e0 + i] : 0u;
+#pragma unroll
+      for (int i = 0; i < kListAhead; ++i) {
+        if (e0 + i >= k2) break;
+        const unsigned int w = ws[i];
+        const int tok = (int)(w & 0xFFFFu), blk = tok / kBlockTok;
+        run = blk == prev_blk ? run + 1 : 0;
+        prev_blk = blk;
+        g_ent[off[blk] + cnt[blk * kHeadDim + tid] + run] =
+            (unsigned int)(tok - blk * kBlockTok) | ((unsigned int)tid << 8) | (w & 0xFFFF0000u);
+        const float v = __half2float(__ushort_as_half((unsigned short)(w >> 16)));
+        atomicMax(&dmax[blk], __float_as_uint(fabsf(v - zero)));
+      }
     }
   }
   __syncthreads();
