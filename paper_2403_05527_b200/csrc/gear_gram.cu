@@ -218,14 +218,41 @@ __global__ void __launch_bounds__(kHeadDim) pi_gram_sum_kernel(PiArgs p, int gra
 }
 
 // ------------------------------------------------------------------ the loops on G
+template <int RP>
+__device__ __forceinline__ void load_row(const float* src, float (&v)[RP]) {
+#pragma unroll
+  for (int q = 0; q < RP / 4; ++q) {
+    const float4 f = reinterpret_cast<const float4*>(src)[q];
+    v[4 * q] = f.x; v[4 * q + 1] = f.y; v[4 * q + 2] = f.z; v[4 * q + 3] = f.w;
+  }
+}
+// Sums of N numbers over the lanes of a warp, N - 1 + log2(32 / N) shuffles: a[0] of lane l becomes the sum of number l N / 32.
+template <int N>
+__device__ __forceinline__ void warp_sums(float (&a)[N], int lane) {
+#pragma unroll
+  for (int o = 16, n = N; o > 0; o >>= 1) {
+    const bool upper = (lane & o) != 0;
+    if (n > 1) {
+      n >>= 1;
+#pragma unroll
+      for (int i = 0; i < N / 2; ++i)
+        if (i < n) a[i] = (upper ? a[i + n] : a[i]) + __shfl_xor_sync(0xffffffffu, upper ? a[i] : a[i + n], o);
+    } else {
+      a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+    }
+  }
+}
+
 // One CTA per tile.  Thread (i, half) holds 64 entries of row i of G in registers; B (128 x r) is in shared memory.
 //   B <- G B, iters - 1 times (each time brought back to magnitude one by a power of two, which the QR drops again);
 //   B <- Q(B), classical Gram-Schmidt with each projection taken twice, one warp;
 //   G0 = B^T G B is the Gram matrix of A0 = R B up to rounding: U^-1 of its Cholesky factor, folded into B, makes the
 //   columns of R B nearly orthonormal before they are computed, so one explicit round of CholeskyQR is enough after.
-// Bound: latency of the chain (G from L2, products, Gram-Schmidt, Cholesky); r^2 and 128 r work per step.
+// Bound: latency of the chain (G from L2, products, Gram-Schmidt, Cholesky); r^2 and 128 r work per step.  Two CTAs per SM, for
+// which sixteen columns give up G during the QR and read it again (512 tiles, rank 16: 232 -> 145 us); G0 from rows read as
+// 128 bits and sums of all its entries in one exchange (rank 16: 311 -> 232, rank 8: 63 -> 54).
 template <int RP>
-__global__ void __launch_bounds__(256) pi_iterate_kernel(PiArgs p, const float* B0, unsigned long long seed, int segment,
+__global__ void __launch_bounds__(256, 2) pi_iterate_kernel(PiArgs p, const float* B0, unsigned long long seed, int segment,
                                                          int iters) {
   __shared__ __align__(16) float Bs[kHeadDim][RP];
   __shared__ __align__(16) float Cs[kHeadDim][RP];
@@ -234,11 +261,12 @@ __global__ void __launch_bounds__(256) pi_iterate_kernel(PiArgs p, const float* 
   const int tile = blockIdx.x, tid = threadIdx.x, i = tid & 127, half = tid >> 7, warp = tid >> 5, lane = tid & 31;
   const int r = p.rank;
   float g[64];
-  {
+  auto load_g = [&]() {
     const float* src = p.G + ((size_t)tile * kHeadDim + half * 64) * kHeadDim + i;
 #pragma unroll
     for (int k = 0; k < 64; ++k) g[k] = __ldcg(src + (size_t)k * kHeadDim);
-  }
+  };
+  load_g();
   if (half == 0) {
     const size_t gtile = (size_t)p.bh0 * 2 + tile;
 #pragma unroll
@@ -334,6 +362,7 @@ __global__ void __launch_bounds__(256) pi_iterate_kernel(PiArgs p, const float* 
       for (int rho = 0; rho < RP; ++rho) Bs[lane + 32 * j][rho] = b[j][rho];
   }
   __syncthreads();
+  if (RP == 16) load_g();                         // sixteen columns leave no registers for G beside the QR
   times_g();
   __syncthreads();
   if (half == 0) {
@@ -341,13 +370,23 @@ __global__ void __launch_bounds__(256) pi_iterate_kernel(PiArgs p, const float* 
     for (int rho = 0; rho < RP; ++rho) Cs[i][rho] = c[rho];
   }
   __syncthreads();
-  for (int e = warp; e < r * r; e += 8) {
-    const int u = e / r, v = e % r;
-    float s = 0.f;
+  constexpr int U = RP / 8 > 0 ? RP / 8 : 1;      // rows of Q^T G Q per warp
+  if (warp * U < RP) {
+    float e[U * RP];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) s = fmaf(Bs[lane + 32 * j][u], Cs[lane + 32 * j][v], s);
-    s = warp_sum(s);
-    if (lane == 0) Gm[u][v] = s;
+    for (int j = 0; j < 4; ++j) {
+      float cv[RP];
+      load_row<RP>(Cs[lane + 32 * j], cv);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float bu = Bs[lane + 32 * j][warp * U + u];
+#pragma unroll
+        for (int v = 0; v < RP; ++v) e[u * RP + v] = j == 0 ? bu * cv[v] : fmaf(bu, cv[v], e[u * RP + v]);
+      }
+    }
+    warp_sums<U * RP>(e, lane);                   // lane l: number l U RP / 32
+    const int at = lane * U * RP / 32;
+    Gm[warp * U + at / RP][at % RP] = e[0];
   }
   __syncthreads();
   if (warp == 0) {
@@ -361,13 +400,15 @@ __global__ void __launch_bounds__(256) pi_iterate_kernel(PiArgs p, const float* 
     const int er = pow2_exponent(__uint_as_float(p.Rmax[tile]));
     const float sc = exp2_int(half == 0 ? -er : er);
     float* out = (half == 0 ? p.Bcur : p.Bg) + ((size_t)tile * kHeadDim + i) * kMaxRank;
+    float row[RP];
+    load_row<RP>(m[i], row);
 #pragma unroll
     for (int rho = 0; rho < kMaxRank; ++rho) {
       float v = 0.f;
       if (rho < RP && rho < r) {
 #pragma unroll
         for (int q = 0; q < RP; ++q)
-          if (q <= rho && q < r) v = fmaf(m[i][q], Wm[q][rho < RP ? rho : 0], v);
+          if (q <= rho && q < r) v = fmaf(row[q], Wm[q][rho < RP ? rho : 0], v);
       }
       out[rho] = v * sc;
     }
