@@ -384,15 +384,14 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
     c->dbg_used = 0;
     GEAR_TRY_ALLOC(c->dbg, c->dbg_bytes);
   }
-  // decode scratch: one partial per (unit, warp touching it); upper bound of warps in a launch
-  // scratch for the largest group of query rows a call may bring: G query heads x max_queries rows per kv head
+  // decode scratch: one partial per (unit, warp touching it), for every count of query rows that a call may bring.  The bytes
+  // do not grow with the count (more units leave fewer slots to each), so the largest count alone would not do.
   c->max_queries = cfg->max_queries > 1 ? (int)cfg->max_queries : 1;
-  const int Gs[2] = {c->G, c->G * c->max_queries};
   c->units_alloc = 0; c->partial_bytes = 0;
-  for (int G : Gs) {
-    const size_t n = partial_bytes_for(c, G);
+  for (int nq = 1; nq <= c->max_queries; ++nq) {
+    const size_t n = partial_bytes_for(c, c->G * nq);
     if (n > c->partial_bytes) c->partial_bytes = n;
-    const int un = (int)(BH * decode_passes(G));
+    const int un = (int)(BH * decode_passes(c->G * nq));
     if (un > c->units_alloc) c->units_alloc = un;
   }
   const size_t units = (size_t)c->units_alloc;

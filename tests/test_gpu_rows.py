@@ -59,3 +59,27 @@ def test_scores_that_keep_growing():
             assert max(rel_max(got[0, h], ref[0, h]) for h in range(hq)) <= 4e-5
         finally:
             p.close()
+
+
+@pytest.mark.parametrize("batch,hq,hkv,most", [(3, 32, 8, 10), (16, 32, 8, 10), (4, 64, 8, 7), (2, 5, 5, 12)])
+def test_every_row_count_up_to_the_cache_s_own(batch, hq, hkv, most):
+    """The scratch for partial results does not grow with the row count: seven or eight positions of the first shape need
+    more of it than nine or ten.  Every count is taken, and its rows are those of the largest call."""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+    gen = torch.Generator(device="cuda").manual_seed(batch)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").half()   # noqa: E731
+    k, v, q = draw(batch, hkv, 192, 128), draw(batch, hkv, 192, 128), draw(batch, hq, most, 128)
+    cache = G.gear_compress(None, G.make_config(batch, hq, hkv, 2, 64, 2.0, 64, 4, 256, seed=1, max_queries=most), k, v, 192, 4)
+    try:
+        want = torch.empty(q.shape, device="cuda")
+        G.gear_decode_attn_multi(cache, q, want, most)
+        for rows in range(1, most):
+            got = torch.full((batch, hq, rows, 128), float("nan"), device="cuda")
+            G.gear_decode_attn_multi(cache, q[:, :, :rows].contiguous(), got, rows)
+            # the same arithmetic per row (one row per kv head: another kernel's), split over other ranges of blocks
+            err = (got - want[:, :, :rows]).abs().amax(-1) / want[:, :, :rows].abs().amax(-1)
+            assert err.max().item() <= 4e-5, rows
+        assert G.gear_last_device_status(cache) == 0
+    finally:
+        G.gear_free(cache)
