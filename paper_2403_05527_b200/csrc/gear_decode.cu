@@ -10,13 +10,13 @@
 // (cp.async.bulk + mbarrier), so that the copies of the next items run while the
 // warp works on the current one.
 //
-// Codes meet the query on the integer tensor cores (mma.sync.m16n8k32, u8 x s8,
-// s32 accumulation).  A packed word becomes fragment registers of the A operand
+// Codes meet the query on the integer tensor cores (mma.sync.m16n8k32, u8 x s8
+// for keys, u8 x u8 for values, s32 accumulation).  A packed word becomes fragment registers of the A operand
 // with one AND per register: a b-bit field left where it sits in its byte is the
 // code times a power of two, which the B operand (keys) or the output row
 // (values) absorbs.  The B operand is a block-wide fixed-point image of
 // q * scale (keys, per channel) or p * scale (values, per token and group), cut
-// into signed base-256 digits ("limbs"), one column per limb: integer products
+// into base-256 digits ("limbs"; signed for keys), one column per limb: integer products
 // are exact, so the result does not depend on any order of summation.  Key
 // scores leave the integers once per 16-token slab; value sums stay in 32-bit
 // integers across blocks and are folded into an fp32 copy in shared memory only
@@ -777,12 +777,12 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
           // ---------------- softmax over the block, the B operands of the value products and the sparse value term in
           //                  one pass over this lane's token pairs (pairs lane, lane + 32), probabilities in registers
           constexpr int NPR = S::kDyn ? 2 : (S::T > 64 ? S::T / 64 : 1);
-          // The integer value sums carry the scale 2^eV_cur, which a block keeps when p * scale * 2^eV_cur stays below 2^22 at
+          // The integer value sums carry the scale 2^eV_cur, which a block keeps when p * scale * 2^eV_cur stays below 2^23 at
           // p = 1 and is no more than three bits short of it (precision).  What is left of those bits is room for the
           // running maximum to lag behind: it is moved, and everything summed so far scaled, only when a score exceeds it
           // by more than that, because the integers have to be folded into the fp32 copy then.  (Every second or third
           // block of a short range raises the maximum by a little.)
-          const int need = clamp60(21 - float_exponent(smax_v));
+          const int need = clamp60(22 - float_exponent(smax_v));
           const bool exp_bad = eV_cur > need || eV_cur < need - 3;
           const int eV_new = exp_bad ? need - kLag : eV_cur;
           const float room = (float)(need - eV_new);
@@ -900,8 +900,8 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
                 }
 #pragma unroll
                 for (int g = 0; g < NGV; ++g) {
-                  const uint32_t y0 = balanced_digits(__float_as_uint(fmaf(p0 * __low2float(z[0][g]), Sv, kMagic)) - kMagicBits);
-                  const uint32_t y1 = balanced_digits(__float_as_uint(fmaf(p1 * __low2float(z[1][g]), Sv, kMagic)) - kMagicBits);
+                  const uint32_t y0 = __float_as_uint(fmaf(p0 * __low2float(z[0][g]), Sv, kMagicV));
+                  const uint32_t y1 = __float_as_uint(fmaf(p1 * __low2float(z[1][g]), Sv, kMagicV));
                   unsigned char* rowb = fragVb + ((g * HP + h) * 4) * RS * 4 + vboff;
                   *reinterpret_cast<unsigned short*>(rowb) = (unsigned short)__byte_perm(y0, y1, 0x0040);
                   *reinterpret_cast<unsigned short*>(rowb + RS * 4) = (unsigned short)__byte_perm(y0, y1, 0x0051);
@@ -971,7 +971,7 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
                   const int mt = F * tau + j, g = (mt * 16) / GV;
                   const uint32_t af[4] = {w.x & m, w.y & m, w.z & m, w.w & m};
 #pragma unroll
-                  for (int nt = 0; nt < NT; ++nt) imma16832(O[mt][nt], af, bV[g][nt][0], bV[g][nt][1]);
+                  for (int nt = 0; nt < NT; ++nt) imma16832_u(O[mt][nt], af, bV[g][nt][0], bV[g][nt][1]);
                 }
               }
               cwp += VT * 32;

@@ -12,9 +12,15 @@ namespace gear {
 constexpr int kBufPitch = 272;                  // bytes per fp16 row of a buffer slab in shared memory
 constexpr int kFragKRow = 40;                   // 32-bit words per (head, limb) row of the key B-operand staging area
 constexpr int kTokLimit = 16384;                // tokens a value accumulator takes before it is folded (int32 headroom)
-constexpr int kLag = 2;                         // bits of the value fixed point kept free for a lagging running maximum
+// Bits of the value fixed point kept free for a lagging running maximum: the one that its unsigned digits have more than the
+// signed ones of the keys, so that a probability of one keeps 22 bits.  (With two, 20 bits are left, and a value is up to
+// 9e-5 off where a block holds one large score and many that are 2^-18 to 2^-22 of it; without the lag batch 8 x 32 heads
+// x 4096, 2 bits, takes 157.3 instead of 155.5 us for four layers.)
+constexpr int kLag = 1;
 constexpr float kMagic = 12582912.0f;           // 1.5 * 2^23: x + kMagic carries rint(x) in its low mantissa bits, |x| < 2^22
 constexpr uint32_t kMagicBits = 0x4B400000u;
+constexpr float kMagicV = 8388608.0f;           // 2^23: the same for 0 <= x < 2^23; the low three bytes of the sum are the digits of rint(x)
+
 
 // ------------------------------------------------------------------ PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -64,10 +70,17 @@ __device__ __forceinline__ void mma16816_z(float (&d)[4], const uint32_t (&a)[4]
       : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(z));
 }
-// integer product: A unsigned bytes (codes in place), B signed bytes (limbs), 32-bit sums
+// integer products: A unsigned bytes (codes in place), B signed (imma16832, keys) or unsigned bytes (imma16832_u, values),
+// 32-bit sums
 __device__ __forceinline__ void imma16832(int (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void imma16832_u(int (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k32.row.col.s32.u8.u8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -89,10 +102,6 @@ template <int BITS>
 __host__ __device__ constexpr uint32_t field_mask(int j) {
   return BITS == 2 ? (0x03030303u << (2 * j)) : (0x0F0F0F0Fu << (4 * j));
 }
-// Signed base-256 digits of a 32-bit integer y, |y| < 2^31 - 2^23: byte l of the result, read as a signed byte, is
-// digit l, and sum digit_l * 256^l = y.
-__device__ __forceinline__ uint32_t balanced_digits(uint32_t y) { return (y + 0x80808080u) ^ 0x80808080u; }
-
 // fp32 pair -> half2 of the high parts and half2 of the rounding remainders
 __device__ __forceinline__ void split_hi_lo(float x0, float x1, uint32_t& hi, uint32_t& lo) {
   const __half2 h = __floats2half2_rn(x0, x1);

@@ -556,11 +556,11 @@ __global__ void __launch_bounds__(kRowsWarps * 32, kRowsCtasPerSm) gear_decode_r
           unsigned char* stV = acquire();
           const unsigned char* vp = stV + a.bregion;
           // The integer value sums carry the scale 2^eV_cur, which this block keeps when p * scale * 2^eV_cur stays below
-          // 2^22 at p = 1 and is no more than three bits short of it.  What is left of those bits is room for the
+          // 2^23 at p = 1 and is no more than three bits short of it.  What is left of those bits is room for the
           // running maximum to lag behind: a row's maximum is moved (and everything summed so far scaled) only when
           // a score exceeds it by more than that, because the integers have to be folded then (a row's maximum grows in
           // every other block of a range otherwise, and a block has several rows).
-          const int need = clamp60(21 - float_exponent(smax_v));
+          const int need = clamp60(22 - float_exponent(smax_v));
           const bool exp_bad = eV_cur > need || eV_cur < need - 3;
           const int eV_new = exp_bad ? need - kLag : eV_cur;
           const float room = (float)(need - eV_new);                      // p <= 2^room
@@ -635,8 +635,8 @@ __global__ void __launch_bounds__(kRowsWarps * 32, kRowsCtasPerSm) gear_decode_r
 #pragma unroll
                 for (int g = 0; g < NGV; ++g) {
                   const __half2 z0 = vsz[tp * NGV + g], z1 = vsz[(tp + 1) * NGV + g];
-                  const uint32_t y0 = balanced_digits(__float_as_uint(fmaf(p0 * __low2float(z0), Sv, kMagic)) - kMagicBits);
-                  const uint32_t y1 = balanced_digits(__float_as_uint(fmaf(p1 * __low2float(z1), Sv, kMagic)) - kMagicBits);
+                  const uint32_t y0 = __float_as_uint(fmaf(p0 * __low2float(z0), Sv, kMagicV));
+                  const uint32_t y1 = __float_as_uint(fmaf(p1 * __low2float(z1), Sv, kMagicV));
                   const int go = g * NTV * 8 * RS * 4 + vboff;
                   *reinterpret_cast<unsigned short*>(rows01 + go) = (unsigned short)__byte_perm(y0, y1, 0x0040);
                   *reinterpret_cast<unsigned short*>(rows01 + RS * 4 + go) = (unsigned short)__byte_perm(y0, y1, 0x0051);
@@ -716,7 +716,7 @@ __global__ void __launch_bounds__(kRowsWarps * 32, kRowsCtasPerSm) gear_decode_r
                 const uint32_t m = m0 << (BITS * ((mt0 + i) % F));
                 const uint32_t af[4] = {w.x & m, w.y & m, w.z & m, w.w & m};
 #pragma unroll
-                for (int n = 0; n < NTV; ++n) imma16832(O[i][n], af, bV[n].x, bV[n].y);
+                for (int n = 0; n < NTV; ++n) imma16832_u(O[i][n], af, bV[n].x, bV[n].y);
               }
             }
             if (r_pad > 0) {                      // low-rank value term, first product: U = A_V^T p, the warp's slabs

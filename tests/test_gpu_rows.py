@@ -83,3 +83,35 @@ def test_every_row_count_up_to_the_cache_s_own(batch, hq, hkv, most):
         assert G.gear_last_device_status(cache) == 0
     finally:
         G.gear_free(cache)
+
+
+@pytest.mark.parametrize("bits", [2, 4])
+@pytest.mark.parametrize("hq", [1, 4, 8])
+def test_small_probabilities_beside_a_large_one(hq, bits):
+    """In every block one token holds nearly all of the probability and the others 2^-21 of it, which is one or two units of
+    the value fixed point: 22 bits at a probability of one, so an entry of the output is off by at most half a unit per code
+    (and fp32 rounding), whatever the maximum may lag by."""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+    from tests.gear_harness import Pair
+    p = Pair(18, 1, hq, 1, bits, 64, 0.0, 64, 0, 1024, keep_fp32=False)
+    try:
+        n, levels = 512, 2 ** bits - 1
+        gen = np.random.default_rng(bits)
+        k16 = np.zeros((1, 1, n, 128), np.float16)
+        k16[0, 0, ::64, 0] = 21.1 / (8.0 / np.sqrt(128.0) * np.log2(np.e))          # the others score 21.1 bits less
+        v16 = gen.uniform(0.0, levels, (1, 1, n, 128)).astype(np.float16)
+        q = np.zeros((1, hq, 128), np.float16)
+        q[..., 0] = 8.0
+        p.oracle.compress(k16, v16, 0, np.zeros((1, 1, 2, 128, 0), np.float32))
+        tile = p.oracle.segments[0]["V"][0][0]
+        assert (0.5 <= tile["scale"]).all() and (tile["scale"] < 1.0).all()        # the exponent that fixes the unit
+        G.gear_compress(p.cache, None, torch.from_numpy(k16).cuda(), torch.from_numpy(v16).cuda(), n, 0)
+        out = torch.empty((1, hq, 128), device="cuda")
+        G.gear_decode_attn(p.cache, torch.from_numpy(q).cuda(), out)
+        got, ref = out.cpu().numpy().astype(np.float64)[0], p.oracle.decode_attn(q, None)[0]
+        unit = 2.0 ** -22                                # of a scale below one
+        bound = tile["codes"].sum(0) * (unit / 2) / (n // 64) + 2.0 ** -20 * np.abs(ref)
+        assert (np.abs(got - ref) <= bound).all(), (np.abs(got - ref) / bound).max()
+    finally:
+        p.close()
