@@ -7,22 +7,28 @@
 #include <atomic>
 #include <mutex>
 #include <new>
-#include <unordered_map>
 #include <vector>
 
 #include "../../include/gear.h"
+#include "gear_call_order.h"
 #include "gear_internal.cuh"
 
 using namespace gear;
 
 static std::atomic<unsigned long long> g_launches{0};
-// Calls of the library that launch kernels, numbered per stream: a decode call may request its first copies before
-// it waits for the kernel in front of it only if that kernel cannot be the one that last wrote the cache.
-static std::mutex g_seq_mutex;
-static std::unordered_map<cudaStream_t, unsigned long long> g_stream_seq;
-static unsigned long long next_call_number(cudaStream_t st) {
-  std::lock_guard<std::mutex> lock(g_seq_mutex);
-  return ++g_stream_seq[st];
+static CallOrder g_order;
+static CallOrder::Key order_key(cudaStream_t st) {
+  CallOrder::Key k = {(uint64_t)(uintptr_t)st, 0, 0, st != cudaStreamPerThread};    // one handle, a stream per thread
+  if (st == cudaStreamLegacy) k.stream = 0;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  unsigned long long id = 0;
+  if ((k.stream == 0 && cudaGetDevice(&k.device) != cudaSuccess) || cudaStreamGetCaptureInfo(st, &capture, &id) != cudaSuccess) {
+    cudaGetLastError();
+    k.ordered = false;
+  }
+  if (capture == cudaStreamCaptureStatusActive) k.capture = id;
+  if (capture == cudaStreamCaptureStatusInvalidated) k.ordered = false;
+  return k;
 }
 
 void gear::count_launches(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
@@ -192,8 +198,7 @@ struct gear_cache {
   DecodeArgs plan;
   int test_dead_wait;            // gear_test_dead_wait: the next decode calls wait on a barrier nothing completes
   int max_queries, units_alloc;  // query rows per head the scratch was sized for; units of that size
-  // the last calls that wrote the segments (records, descriptors) and the buffer rows: stream and number on that stream
-  struct LastWrite { cudaStream_t stream; unsigned long long call; bool any; } seg_write, buf_write;
+  CallOrder::Write seg_write, buf_write;   // the last calls that wrote the segments (records, descriptors) and the buffer rows
 };
 
 static int outlier_count(float s_pct, int len) {
@@ -330,7 +335,6 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
     c->mem.alloc = g_alloc; c->mem.free = g_free; c->mem.ctx = g_alloc_ctx;
   }
   c->test_dead_wait = 0;
-  c->seg_write = {nullptr, 0, false}; c->buf_write = {nullptr, 0, false};
   c->arena = nullptr; c->dbg = nullptr; c->table_dev = nullptr; c->blk2seg = nullptr; c->buf_k = c->buf_v = nullptr; c->flush_ws = nullptr;
   c->partial = nullptr; c->tickets = nullptr; c->status = nullptr;
   c->scratch_clean = false;
@@ -443,6 +447,8 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
   job.seed = c->cfg.seed; job.segment_index = (int)c->segs.size(); job.iters = c->cfg.power_iters;
   job.sms = c->sm_count; job.status = c->status;
 
+  const CallOrder::Key key = order_key(st);
+  const uint64_t begun = g_order.begin();
   cudaError_t e = cudaSuccess;
   if (!scratch_zeroed(c, st)) return GEAR_ERR_CUDA;
   if (sd.T % 16) {     // the last slab of every block is partly empty: its codes, factor rows and scales read as zero
@@ -483,7 +489,8 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
   c->n_compressed += n;
   c->n_blocks_c += sd.nblk;
   c->plan_key = -1;
-  c->seg_write = {st, next_call_number(st), true};
+  g_order.queued(key, begun);
+  c->seg_write = g_order.written(key);
   return GEAR_OK;
 }
 
@@ -523,12 +530,15 @@ static gear_status push_rows(gear_cache* c, const void* k_new, const void* v_new
   a.buf_k = (__half*)c->buf_k; a.buf_v = (__half*)c->buf_v; a.k_new = (const __half*)k_new; a.v_new = (const __half*)v_new;
   a.q_src = (const __half*)q_src; a.q_dst = (__half*)c->stage_q; a.q_pieces = q_src ? (int)(host_query_bytes(c) / 16) : 0;
   a.BH = c->cc.BH; a.n_b = n_b; a.slot = c->buf_len; a.host_src = host_src ? 1 : 0;
+  const CallOrder::Key key = order_key(st);
+  const uint64_t begun = g_order.begin();
   if (launch_push(a, st) != cudaSuccess) {
     cudaGetLastError();
     return GEAR_ERR_CUDA;
   }
+  g_order.queued(key, begun);
+  c->buf_write = g_order.written(key);
   c->buf_len += 1;
-  c->buf_write = {st, next_call_number(st), true};
   if (c->buf_len < n_b) return GEAR_OK;
   gear_status s = compress_segment(c, c->buf_k, c->buf_v, n_b, c->cfg.rank_flush, B0_flush, true, st);
   if (s != GEAR_OK) { c->buf_len -= 1; return s; }
@@ -592,12 +602,10 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
   const float sc = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)kHeadDim);
   a.scale_log2 = sc * 1.4426950408889634f;
   a.test_dead_wait = c->test_dead_wait;
-  {
-    const unsigned long long call = next_call_number((cudaStream_t)stream);
-    auto long_ago = [&](const gear_cache::LastWrite& w) { return w.stream == (cudaStream_t)stream && call >= w.call + 2; };
-    a.early_reads = c->seg_write.any && long_ago(c->seg_write) ? 1 : 0;
-    a.early_buf = !c->buf_write.any || long_ago(c->buf_write) ? 1 : 0;
-  }
+  const CallOrder::Key key = order_key((cudaStream_t)stream);
+  const uint64_t begun = g_order.begin();
+  a.early_reads = g_order.another_since(key, c->seg_write) ? 1 : 0;
+  a.early_buf = c->buf_write.number == 0 || g_order.another_since(key, c->buf_write) ? 1 : 0;
   // never more CTAs than blocks of work
   const int passes = decode_passes(Gq);
   if ((long long)c->cc.BH * passes > c->units_alloc) return GEAR_ERR_CAPACITY;
@@ -659,6 +667,7 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
     cudaGetLastError();
     return GEAR_ERR_CUDA;
   }
+  g_order.queued(key, begun);
   return GEAR_OK;
 }
 
