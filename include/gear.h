@@ -56,7 +56,11 @@ enum {
 /* Device memory of the caches.  By default gear_create uses cudaMalloc / cudaFree.  A caller that owns the
  * device heap installs its own pair here (process-wide; NULL, NULL restores the default): alloc returns a
  * device pointer aligned to 256 bytes or NULL, which gear_create reports as GEAR_ERR_ALLOC after handing back
- * what it had taken.  A cache frees through the pair it was created with. */
+ * what it had taken.  A cache frees through the pair it was created with.
+ * Neither gear_create nor gear_free waits for work on the default stream (stream NULL): a pair must hand out and take
+ * back the memory of a cache that is used there in the order of that stream, as a pool of that stream does.  For a cache
+ * that is used on any other stream the pair may belong to whatever stream: the first call that writes such a cache
+ * waits until the device is idle, and so does gear_free before it hands memory back. */
 typedef void* (*gear_alloc_fn)(size_t bytes, void* ctx);
 typedef void (*gear_free_fn)(void* ptr, void* ctx);
 
@@ -99,8 +103,8 @@ typedef struct gear_cache gear_cache;   /* opaque */
 gear_status gear_set_allocator(gear_alloc_fn alloc_fn, gear_free_fn free_fn, void* ctx);
 
 /* Create an empty cache (no segment, empty buffer) on the current device.
- * Allocates all the device memory the cache will ever use, without waiting for the device; the pinned host memory of the
- * *_host calls is made by the first of them.  *cache must be NULL. */
+ * Allocates all the device memory the cache will ever use, without waiting for the device (see gear_set_allocator); the
+ * pinned host memory of the *_host calls is made by the first of them.  *cache must be NULL. */
 gear_status gear_create(gear_cache** cache, const gear_config* cfg);
 
 /* Algorithm 1, prefill body, applied to a block of n tokens: for X in {K, V}
@@ -149,7 +153,8 @@ gear_status gear_decode_attn(gear_cache* cache, const void* q, float* out,
 gear_status gear_decode_attn_multi(gear_cache* cache, const void* q, float* out, int32_t n_queries,
                                    float softmax_scale, void* stream);
 
-/* Release the cache and everything it owns.  NULL is allowed. */
+/* Release the cache and everything it owns.  NULL is allowed.  Work queued on the cache may still be running: memory from
+ * cudaMalloc is given back when that work is done, memory of the caller's allocator as gear_set_allocator says. */
 void gear_free(gear_cache* cache);
 
 /* gear_compress takes its transient workspace (the residual of the block being compressed, up to 3 GB)

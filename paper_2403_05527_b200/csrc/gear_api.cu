@@ -182,6 +182,7 @@ struct gear_cache {
   float* partial; size_t partial_bytes;
   int* tickets; int* status;                             // one block; zeroed on the caller's stream by the first call (scratch_clean)
   bool scratch_clean;
+  bool off_default;              // some call went to another stream than the default one
   void* stage_q; float* stage_out; float* stage_b0;      // for the *_host calls: query; result for pageable destinations; B0
   // The *_host calls copy the caller's rows and query into a slot of a pinned ring, from which the push kernel reads them
   // itself: no copy engine and no second stream, hence no event waits between the kernels of a step.  A slot is filled
@@ -260,6 +261,9 @@ extern "C" void gear_free(gear_cache* c) {
   // kernels queued by the host-buffer calls still read the ring and write the caller's memory
   if (c->host_last >= 0) cudaEventSynchronize(c->host.ev[c->host_last]);
   const DeviceAllocator& m = c->mem;
+  // A pool may hand the memory to work of its own stream at once.  Off the default stream nothing says that this is the stream
+  // of the kernels that are still queued here.
+  if (m.free && c->off_default && cudaDeviceSynchronize() != cudaSuccess) cudaGetLastError();
   m.put(c->arena); m.put(c->dbg); m.put(c->table_dev); m.put(c->buf_k);
   m.put(c->flush_ws); m.put(c->partial); m.put(c->tickets);
   m.put(c->stage_q); m.put(c->stage_b0);
@@ -294,10 +298,21 @@ static gear_status host_slot_failed(gear_cache* c, int slot, cudaStream_t st, ge
   return s;
 }
 
+static bool note_stream(gear_cache* c, cudaStream_t st) {                 // whether it is another stream than the default one
+  const bool off = st != nullptr && st != cudaStreamLegacy;
+  c->off_default = c->off_default || off;
+  return off;
+}
+
 // The merge counters and the status word start at zero on the stream of the first call that writes the cache, so that
-// creating one neither waits for the device nor orders itself against other streams.
+// creating one does not wait for the device.  Off the default stream memory of the caller's allocator may still be in use by
+// work of the stream that the allocator belongs to: wait for that once.
 static bool scratch_zeroed(gear_cache* c, cudaStream_t st) {
   if (c->scratch_clean) return true;
+  if (note_stream(c, st) && c->mem.alloc && order_key(st).capture == 0 && cudaDeviceSynchronize() != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
   if (cudaMemsetAsync(c->tickets, 0, ((size_t)c->units_alloc + 1) * 4, st) != cudaSuccess) { cudaGetLastError(); return false; }
   c->scratch_clean = true;
   return true;
@@ -338,6 +353,7 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
   c->arena = nullptr; c->dbg = nullptr; c->table_dev = nullptr; c->blk2seg = nullptr; c->buf_k = c->buf_v = nullptr; c->flush_ws = nullptr;
   c->partial = nullptr; c->tickets = nullptr; c->status = nullptr;
   c->scratch_clean = false;
+  c->off_default = false;
   c->stage_q = nullptr; c->stage_out = nullptr; c->stage_b0 = nullptr;
   memset(&c->host, 0, sizeof(c->host));
   for (bool& u : c->host_used) u = false;
@@ -450,6 +466,7 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
   const CallOrder::Key key = order_key(st);
   const uint64_t begun = g_order.begin();
   cudaError_t e = cudaSuccess;
+  note_stream(c, st);
   if (!scratch_zeroed(c, st)) return GEAR_ERR_CUDA;
   if (sd.T % 16) {     // the last slab of every block is partly empty: its codes, factor rows and scales read as zero
     if (cudaMemsetAsync(c->arena + sd.seg_base, 0, need, st) != cudaSuccess) { cudaGetLastError(); return GEAR_ERR_CUDA; }
@@ -525,6 +542,7 @@ static gear_status push_rows(gear_cache* c, const void* k_new, const void* v_new
   if (c->buf_len + 1 == n_b) {     // this push will flush: make sure the segment fits before touching anything
     if (c->n_compressed + n_b > c->cfg.max_tokens || (int)c->segs.size() >= c->table_cap) return GEAR_ERR_CAPACITY;
   }
+  note_stream(c, st);
   if (!scratch_zeroed(c, st)) return GEAR_ERR_CUDA;
   PushArgs a;
   a.buf_k = (__half*)c->buf_k; a.buf_v = (__half*)c->buf_v; a.k_new = (const __half*)k_new; a.v_new = (const __half*)v_new;
@@ -591,6 +609,7 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
   if (!c || !q || !out) return GEAR_ERR_ARG;
   if (((uintptr_t)q | (uintptr_t)out) & 15) return GEAR_ERR_ALIGN;
   if (c->n_compressed == 0 && c->buf_len == 0) return GEAR_ERR_STATE;
+  note_stream(c, (cudaStream_t)stream);
   gear_status s = plan_decode(c, Gq);
   if (s != GEAR_OK) return s;
   DecodeArgs a = c->plan;
@@ -741,6 +760,7 @@ static gear_status decode_host(gear_cache* c, const void* q_host, float* out_hos
   gear_status s = host_slot(c, &mem, &slot);
   if (s != GEAR_OK) return s;
   memcpy(mem, q_host, host_query_bytes(c));
+  note_stream(c, st);
   PushArgs a;
   memset(&a, 0, sizeof(a));
   a.q_src = (const __half*)mem; a.q_dst = (__half*)c->stage_q; a.q_pieces = (int)(host_query_bytes(c) / 16); a.host_src = 1;

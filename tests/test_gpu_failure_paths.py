@@ -96,3 +96,51 @@ def test_injected_allocation_failure_is_reported_and_nothing_leaks():
         G.gear_set_allocator(None, None)
     cache = G.gear_create(cfg)                      # the default allocator is back
     G.gear_free(cache)
+
+
+@pytest.mark.parametrize("use", ["segments", "rows", "host"])
+def test_an_allocator_of_another_stream_meets_no_running_work(use):
+    """Memory of a pool whose blocks belong to one stream, for a cache that is used on another: it is not written before what
+    that stream had queued is done, and not handed back while the cache's own work runs."""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+
+    held, idle_at_free = {}, []
+    side = torch.cuda.Stream()
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    k, v = (torch.randn((1, 2, 192, 128), generator=gen, device="cuda").half() for _ in range(2))
+    rows, q = torch.randn((2, 1, 2, 128), device="cuda").half(), torch.randn((1, 4, 128), device="cuda").half()
+    q_host, out = q.cpu(), torch.empty((1, 4, 128), device="cuda")
+    out_host = torch.empty((1, 4, 128)).pin_memory()
+    torch.cuda.synchronize()
+
+    def alloc(nbytes, _ctx):
+        t = torch.empty(max(int(nbytes), 1), dtype=torch.uint8, device="cuda:0")
+        held[t.data_ptr()] = t
+        return t.data_ptr()
+
+    def free(ptr, _ctx):
+        idle_at_free.append(side.query())
+        del held[ptr]
+
+    a_cb, f_cb = G.ALLOC_FN(alloc), G.FREE_FN(free)
+    cfg = G.make_config(1, 4, 2, 2, 64, 2.0, 64, 4, 512)
+    G.gear_set_allocator(a_cb, f_cb)
+    try:
+        cache = G.gear_create(cfg)
+        torch.cuda._sleep(20_000_000)                   # ten milliseconds of the pool's stream
+        if use == "segments":
+            G.gear_compress(cache, None, k, v, 192, 4, stream=side.cuda_stream)
+        else:
+            G.gear_append_buffer(cache, rows[0], rows[1], stream=side.cuda_stream)
+        assert torch.cuda.default_stream().query()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(20_000_000)
+        if use == "host":
+            G.gear_decode_attn_host_async(cache, q_host, out_host, stream=side.cuda_stream)
+        else:
+            G.gear_decode_attn(cache, q, out, stream=side.cuda_stream)
+        G.gear_free(cache)
+        assert idle_at_free and all(idle_at_free) and not held
+    finally:
+        G.gear_set_allocator(None, None)
