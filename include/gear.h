@@ -12,7 +12,9 @@
  *    borrowed for the duration of the work enqueued on `stream`; the library
  *    never frees or keeps them.  All tensors are contiguous, row-major.
  *  - The library owns a gear_cache (one per layer): all of its device memory
- *    is allocated when the cache is created and released by gear_free.
+ *    is allocated when the cache is created and released by gear_free.  The
+ *    transient workspace of a compression is not part of it (see
+ *    gear_release_workspace).
  *  - Calls enqueue work on `stream` (a cudaStream_t passed as void*) and return
  *    without synchronising, except where stated (the *_host variants,
  *    gear_export, gear_last_device_status).
@@ -159,7 +161,8 @@ void gear_free(gear_cache* cache);
 
 /* gear_compress takes its transient workspace (the residual of the block being compressed, up to 3 GB)
  * from a stream-ordered pool that the library keeps per device, so that repeated calls do not go back
- * to the driver; the pinned rows of the *_host calls (64 MB at most) are kept the same way when a cache is freed.
+ * to the driver, and so does a push that compresses a buffer of more than 128 tokens (GEAR_ERR_ALLOC where the pool cannot
+ * give it; the row is then not counted); the pinned rows of the *_host calls (64 MB at most) are kept the same way when a cache is freed.
  * This call synchronises the current device and returns both kinds of memory to the driver. */
 gear_status gear_release_workspace(void);
 

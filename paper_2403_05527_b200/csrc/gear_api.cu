@@ -178,7 +178,6 @@ struct gear_cache {
   SegDesc* table_dev; int table_cap;
   int* blk2seg; int blk_cap;                             // segment index of every compressed block
   void* buf_k; void* buf_v;                              // [BH][n_b][128] fp16
-  unsigned char* flush_ws; size_t flush_ws_bytes;
   float* partial; size_t partial_bytes;
   int* tickets; int* status;                             // one block; zeroed on the caller's stream by the first call (scratch_clean)
   bool scratch_clean;
@@ -265,8 +264,8 @@ extern "C" void gear_free(gear_cache* c) {
   // of the kernels that are still queued here.
   if (m.free && c->off_default && cudaDeviceSynchronize() != cudaSuccess) cudaGetLastError();
   m.put(c->arena); m.put(c->dbg); m.put(c->table_dev); m.put(c->buf_k);
-  m.put(c->flush_ws); m.put(c->partial); m.put(c->tickets);
-  m.put(c->stage_q); m.put(c->stage_b0);
+  m.put(c->partial); m.put(c->tickets);
+  m.put(c->stage_q); m.put(c->stage_out); m.put(c->stage_b0);
   host_block_put(c->host);
   delete c;
 }
@@ -350,7 +349,7 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
     c->mem.alloc = g_alloc; c->mem.free = g_free; c->mem.ctx = g_alloc_ctx;
   }
   c->test_dead_wait = 0;
-  c->arena = nullptr; c->dbg = nullptr; c->table_dev = nullptr; c->blk2seg = nullptr; c->buf_k = c->buf_v = nullptr; c->flush_ws = nullptr;
+  c->arena = nullptr; c->dbg = nullptr; c->table_dev = nullptr; c->blk2seg = nullptr; c->buf_k = c->buf_v = nullptr;
   c->partial = nullptr; c->tickets = nullptr; c->status = nullptr;
   c->scratch_clean = false;
   c->off_default = false;
@@ -395,9 +394,6 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
   c->blk2seg = reinterpret_cast<int*>(c->table_dev + c->table_cap);
   GEAR_TRY_ALLOC(c->buf_k, 2 * BH * n_b * kHeadDim * 2);
   c->buf_v = reinterpret_cast<__half*>(c->buf_k) + BH * n_b * kHeadDim;
-  c->flush_ws_bytes = compress_tile_fits(sf.T, n_b, cfg->rank_flush)      // flushed in one launch without a workspace
-                          ? 256 : compress_workspace_bytes((int)BH, n_b, cfg->rank_flush, c->sm_count);
-  GEAR_TRY_ALLOC(c->flush_ws, c->flush_ws_bytes);
   if (cfg->flags & GEAR_FLAG_KEEP_FP32_FACTORS) {
     const size_t rm = cfg->rank_max > 0 ? cfg->rank_max : 1;
     c->dbg_bytes = (BH * 2 * (size_t)cfg->max_tokens * rm + BH * 2 * kHeadDim * rm * (size_t)c->table_cap) * 4;
@@ -419,8 +415,8 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
   GEAR_TRY_ALLOC(c->tickets, (units + 1) * 4);
   c->status = c->tickets + units;
   const size_t q_bytes = host_query_bytes(c);
-  GEAR_TRY_ALLOC(c->stage_q, 3 * q_bytes);                                // the query (fp16), then a result (fp32)
-  c->stage_out = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(c->stage_q) + q_bytes);
+  GEAR_TRY_ALLOC(c->stage_q, q_bytes);
+  GEAR_TRY_ALLOC(c->stage_out, 2 * q_bytes);
   GEAR_TRY_ALLOC(c->stage_b0, BH * 2 * kHeadDim * (size_t)(cfg->rank_flush > 0 ? cfg->rank_flush : 1) * 4);
   *out = c;
   return GEAR_OK;
@@ -428,7 +424,7 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
 
 // Append one compressed segment built from K, V [BH][n][128] on the device.
 static gear_status compress_segment(gear_cache* c, const void* K, const void* V, int n, int rank, const float* B0,
-                                    bool is_flush, cudaStream_t st) {
+                                    cudaStream_t st) {
   if ((int)c->segs.size() >= c->table_cap) return GEAR_ERR_CAPACITY;
   if (c->n_compressed + n > c->cfg.max_tokens) return GEAR_ERR_CAPACITY;
   SegDesc sd = shape_segment(c, n, rank);
@@ -474,10 +470,10 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
   }
   if (!per_vector && compress_tile_fits(sd.T, sd.n_c, sd.rank)) {
     e = compress_tile(job, c->cc.BH, st);              // short segment: one launch, residual in shared memory
-  } else if (is_flush) {
-    e = compress_range(job, 0, c->cc.BH, c->flush_ws, st);
   } else {
-    // bounded transient workspace, (batch, head) pairs processed in ranges
+    // Bounded transient workspace, (batch, head) pairs processed in ranges.  Flushes of buffers too long for one launch take it
+    // from the pool like prompts: held by every cache it was 235 MB for 256 pairs of 256 tokens at rank 4, 7.5 GB for 32 layers.
+    // (Kept small by ranges instead, 88 MB, such a flush took 350 us and not 235, of 64 pairs 365 and not 110.)
     const int csr_k = per_vector ? sd.csr_k : -1;
     const size_t budget = (size_t)3 << 30;
     auto bytes_of = [&](int nbh) { return compress_workspace_bytes(nbh, n, rank, c->sm_count, csr_k); };
@@ -530,7 +526,7 @@ extern "C" gear_status gear_compress(gear_cache** cache, const gear_config* cfg,
   }
   gear_cache* c = *cache;
   if (c->buf_len != 0) return GEAR_ERR_STATE;
-  st = compress_segment(c, K, V, (int)n, rank, B0, false, (cudaStream_t)stream);
+  st = compress_segment(c, K, V, (int)n, rank, B0, (cudaStream_t)stream);
   if (st != GEAR_OK && created) { gear_free(c); *cache = nullptr; }
   return st;
 }
@@ -558,7 +554,7 @@ static gear_status push_rows(gear_cache* c, const void* k_new, const void* v_new
   c->buf_write = g_order.written(key);
   c->buf_len += 1;
   if (c->buf_len < n_b) return GEAR_OK;
-  gear_status s = compress_segment(c, c->buf_k, c->buf_v, n_b, c->cfg.rank_flush, B0_flush, true, st);
+  gear_status s = compress_segment(c, c->buf_k, c->buf_v, n_b, c->cfg.rank_flush, B0_flush, st);
   if (s != GEAR_OK) { c->buf_len -= 1; return s; }
   c->buf_len = 0;
   return GEAR_FLUSHED;
@@ -941,7 +937,7 @@ extern "C" gear_status gear_cache_bytes(const gear_cache* c, gear_bytes* out) {
   }
   out->buffer = BH * 2 * (long long)c->buf_len * d * 2;
   out->stored_total += out->buffer;
-  out->alloc_total = (long long)(c->arena_bytes + c->dbg_bytes + c->flush_ws_bytes + c->partial_bytes +
+  out->alloc_total = (long long)(c->arena_bytes + c->dbg_bytes + c->partial_bytes +
                                  2 * (size_t)BH * c->cfg.buffer_cap * d * 2 + sizeof(SegDesc) * (size_t)c->table_cap);
   return GEAR_OK;
 }

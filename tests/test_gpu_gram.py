@@ -83,3 +83,45 @@ def test_tiles_whose_singular_values_span_decades(rank):
         assert np.abs(got[:, small] - ref[:, small]).max() <= 5e-3 * np.abs(ref[:, small]).max()
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("batch,hkv,group,nb,rank", [
+    (1, 2, 64, 256, 4),
+    (2, 32, 64, 256, 4),
+    (1, 9, 128, 1024, 16),
+    (1, 3, 32, 160, 6),             # 160 tokens: the last 32-row block of a tile is its fifth
+])
+def test_flush_of_a_long_buffer(batch, hkv, group, nb, rank):
+    """Buffers above 128 tokens are compressed like a prompt.  The workspace of that is not the cache's: what it holds does not
+    depend on the rank that flushes use, but for the factors themselves."""
+    import torch
+    from paper_2403_05527_b200 import binding as G, synth
+    from tests.gear_harness import Pair
+    total = lambda r: alloc(G.make_config(batch, hkv, hkv, 4, group, 2.0, nb, r, 2 * nb, rank_max=16))   # noqa: E731
+
+    def alloc(cfg):
+        c = G.gear_create(cfg)
+        n = G.gear_cache_bytes(c).alloc_total
+        G.gear_free(c)
+        return n
+    assert total(rank) - total(0) <= batch * hkv * 3 * 2 * 128 * 16 * 2        # B of the flushed segments
+    p = Pair(14, batch, hkv, hkv, 4, group, 2.0, nb, rank, 2 * nb)
+    try:
+        ks, vs = synth.make_appended(14, batch, hkv, 128, nb)
+        b0 = synth.make_b0(14, batch, hkv, 128, rank)
+        p.oracle.compress(np.stack(list(ks), 2), np.stack(list(vs), 2), rank, b0)
+        kd, vd, b0d = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (ks, vs, b0))
+        launches = []
+        for i in range(nb):
+            before = G.gear_kernel_launches()
+            flushed = G.gear_append_buffer(p.cache, kd[i], vd[i], b0d)
+            assert (flushed == G.GEAR_FLUSHED) == (i == nb - 1)
+            launches.append(G.gear_kernel_launches() - before)
+        assert set(launches[:-1]) == {1}
+        # the push, two of Filter / Quant, three on R^T R, four or five after, the descriptor: not the one-launch path
+        assert launches[-1] == (12 if rank > 8 else 11)
+        torch.cuda.synchronize()
+        p.check_segment(0)
+        p.check_attention()
+    finally:
+        p.close()
