@@ -633,7 +633,15 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
   // Ranges of one or two blocks: a warp's partial result, its ticket and the merge of up to 64 partials then take as long as
   // the blocks themselves (8 of 15 us for one sequence of 3800 tokens and 32 heads).  Several warps of a unit share a CTA
   // and join in shared memory instead, if that leaves nobody more blocks than one warp per CTA would: the fewest CTAs per
-  // unit (one needs no ticket at all), then the fewest warps.
+  // unit (one needs no ticket at all), then the fewest warps.  Warps of a CTA wait for one another and for one SM, so with
+  // idle SMs about (little work) that has to be worth it.  Where the lines lie (2 bits, groups of 64, rank 4; us without and
+  // with):
+  //   one CTA per unit       up to ten warps always (8 heads of 10 blocks 7.85 / 7.34), more from 400 blocks of work on
+  //                          (8 heads of 14 blocks 7.85 / 8.36, 64 heads 9.81 / 8.70)
+  //   several CTAs           of four to eight warps (one head of 66 blocks: 10.55 / 10.5 with 2 or 14, 8.85 with 8); few
+  //                          partials only where there is much work, because their merge is short (one head of 26 blocks
+  //                          8.36 / 8.50, of 34 8.87 / 8.53, 16 heads of 18 9.20 / 9.01, of 14 8.28 / 9.04); not where a
+  //                          few SMs would get a second CTA (32 heads of 34 blocks: 160 CTAs 11.25, 192 10.55)
   if (Gq == 1 && !c->plan.wide) {
     const long long units = c->cc.BH, nb = work / units;
     const long long p1 = grid / units > 1 ? (grid / units < nb ? grid / units : nb) : 1;
@@ -645,6 +653,9 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
         const long long slots = (long long)c->sm_count * (c->plan_occ / w);
         const long long need = (nb + len * w - 1) / (len * w);            // CTAs per unit for ranges of `len` blocks
         if (need * units > slots || need >= a.max_parts) continue;
+        if (need == 1 ? w > 10 && work < 400
+                      : w < 4 || w > 8 || (nb <= 32 && work < 200) || (nb <= 16 && work < 400) ||
+                            (need * units > c->sm_count && 4 * need * units < 5 * c->sm_count)) continue;
         if (best_w == 0 || need < best) { best = need; best_w = w; }
       }
     if (best_w) { a.cta_warps = best_w; a.unit_ctas = (int)best; grid = best * units; }
