@@ -150,8 +150,8 @@ gear_status gear_decode_attn(gear_cache* cache, const void* q, float* out,
  * cache, as in speculative or chunked decoding): every row attends to every cached token, no mask among the rows.
  *   q     device fp16 [batch, n_q_heads, n_queries, head_dim];  out device fp32, same shape.
  *   n_queries  1 .. cfg.max_queries.
- * The rows of a kv head share each read of its compressed blocks eight at a time (four, where there are no more):
- * G * n_queries rows take ceil(G * n_queries / 8) passes over the cache. */
+ * The rows of a kv head share each read of its compressed blocks four at a time, or eight where the cache is long
+ * enough: G * n_queries rows take a quarter or an eighth as many passes over the cache, rounded up. */
 gear_status gear_decode_attn_multi(gear_cache* cache, const void* q, float* out, int32_t n_queries,
                                    float softmax_scale, void* stream);
 

@@ -317,15 +317,27 @@ static bool scratch_zeroed(gear_cache* c, cudaStream_t st) {
   return true;
 }
 
-// Partial results of a launch for G query rows per kv head: slots per unit (a unit's share of the launch's CTAs, the first and
-// the last of which may be shared with its neighbours), and the bytes of all slots.
-static int partial_slots(const gear_cache* c, int G) {
-  const size_t units = (size_t)c->cc.BH * decode_passes(G);
+// Query rows per pass over the cache for G rows per kv head and `nb` blocks.  Eight rows share what a block costs once, but a
+// block then takes longer and there are half as many: that pays where the CTAs have long ranges and the last pass is more than
+// half full.  Blocks per CTA (of 592) when eight rows go together, and the time of fours over that of eights (5 to 32 rows,
+// groups of 64 and 128, 2 and 4 bits): below 2 0.48 to 1.04, 6 to 8 0.87 to 1.06, 10 to 12 0.98 to 1.12, above 12 1.03 to 1.15;
+// with the last pass half empty 1.02 at most.  16 rows, 2 bits, groups of 64, 4096 tokens, us for fours and eights: 8 heads 18.9 / 27.1, 16
+// 28.8 / 32.6, 32 51.7 / 50.5, 128 166.6 / 153.7; 12 rows, 32 heads x 16384 124 / 148.
+static int rows_per_pass(const gear_cache* c, int G, long long nb) {
+  if (G <= 4) return G == 1 ? 1 : 4;
+  if (decode_passes(G, 4) % 2) return 4;
+  return c->cc.BH * nb * decode_passes(G, 8) >= 10LL * c->sm_count * kRowsCtasPerSm ? 8 : 4;
+}
+
+// Partial results of a launch for G query rows per kv head, hp at a time: slots per unit (a unit's share of the launch's CTAs,
+// the first and the last of which may be shared with its neighbours), and the bytes of all slots.
+static int partial_slots(const gear_cache* c, int G, int hp) {
+  const size_t units = (size_t)c->cc.BH * decode_passes(G, hp);
   const size_t ctas = (size_t)c->sm_count * (G == 1 ? 32 : kRowsCtasPerSm);
   return (int)(ctas / units + 3);
 }
-static size_t partial_bytes_for(const gear_cache* c, int G) {
-  return (size_t)c->cc.BH * decode_passes(G) * partial_slots(c, G) * (size_t)decode_heads_per_pass(G) * kPartRow * 4;
+static size_t partial_bytes_for(const gear_cache* c, int G, int hp) {
+  return (size_t)c->cc.BH * decode_passes(G, hp) * partial_slots(c, G, hp) * (size_t)hp * kPartRow * 4;
 }
 
 #define GEAR_TRY_ALLOC(ptr, bytes)                                                   \
@@ -400,15 +412,19 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
     c->dbg_used = 0;
     GEAR_TRY_ALLOC(c->dbg, c->dbg_bytes);
   }
-  // decode scratch: one partial per (unit, warp touching it), for every count of query rows that a call may bring.  The bytes
-  // do not grow with the count (more units leave fewer slots to each), so the largest count alone would not do.
+  // decode scratch: one partial per (unit, warp touching it), for every count of query rows that a call may bring and the rows
+  // per pass it may take.  The bytes do not grow with the count (more units leave fewer slots to each), so the largest count
+  // alone would not do.
   c->max_queries = cfg->max_queries > 1 ? (int)cfg->max_queries : 1;
   c->units_alloc = 0; c->partial_bytes = 0;
   for (int nq = 1; nq <= c->max_queries; ++nq) {
-    const size_t n = partial_bytes_for(c, c->G * nq);
-    if (n > c->partial_bytes) c->partial_bytes = n;
-    const int un = (int)(BH * decode_passes(c->G * nq));
-    if (un > c->units_alloc) c->units_alloc = un;
+    const int G = c->G * nq;
+    for (int hp = G == 1 ? 1 : 4; hp <= (G > 4 ? 8 : G == 1 ? 1 : 4); hp += 4) {
+      const size_t n = partial_bytes_for(c, G, hp);
+      if (n > c->partial_bytes) c->partial_bytes = n;
+      const int un = (int)(BH * decode_passes(G, hp));
+      if (un > c->units_alloc) c->units_alloc = un;
+    }
   }
   const size_t units = (size_t)c->units_alloc;
   GEAR_TRY_ALLOC(c->partial, c->partial_bytes);
@@ -567,7 +583,7 @@ extern "C" gear_status gear_append_buffer(gear_cache* c, const void* k_new, cons
   return push_rows(c, k_new, v_new, nullptr, false, B0_flush, (cudaStream_t)stream);
 }
 
-static gear_status plan_decode(gear_cache* c, int Gq) {
+static gear_status plan_decode(gear_cache* c, int Gq, int hp) {
   // One-head passes: with four warps per scheduler the warps of a scheduler slow one another down by more than
   // the fourth warp adds (measured: 3 warps finish 0.85 blocks per microsecond and scheduler, 4 warps 0.79), so
   // long streams run with twelve resident warps.  Short streams (few blocks per warp) keep sixteen: there the
@@ -579,7 +595,7 @@ static gear_status plan_decode(gear_cache* c, int Gq) {
   }
   // everything else the plan depends on is fixed by the segments: a push that does not flush keeps it (asking the driver
   // for the occupancy again costs a microsecond and a half per decoding step)
-  const long long key = ((long long)c->segs.size() * 4096 + Gq) * 2 + (warps_cap ? 1 : 0);
+  const long long key = ((long long)c->segs.size() * 4096 + Gq) * 2 + (warps_cap || hp == 8 ? 1 : 0);
   if (c->plan_key == key) return GEAR_OK;
   int max_k = 0, max_v = 0, max_bfac = 0, max_T = 16;
   for (const SegDesc& s : c->segs) {
@@ -589,7 +605,7 @@ static gear_status plan_decode(gear_cache* c, int Gq) {
     if ((s.T + 31) / 32 * 32 > max_T) max_T = (s.T + 31) / 32 * 32;
   }
   if (Gq == 1 ? !decode_plan(c->cc.bits, Gq, c->cc.ngv, max_k, max_v, max_bfac, max_T, kDecodeSmemBudget, warps_cap, &c->plan)
-              : !rows_plan(Gq, c->cc.ngv, max_k, max_v, max_bfac, max_T, &c->plan))
+              : !rows_plan(hp, c->cc.ngv, max_k, max_v, max_bfac, max_T, &c->plan))
     return GEAR_ERR_SHAPE;
   int occ = Gq == 1 ? decode_occupancy(c->cc.bits, Gq, c->cc.ngv, c->plan.wide, (size_t)c->plan.ws.total)
                     : rows_occupancy(c->plan, c->cc.bits, c->cc.ngv);
@@ -606,7 +622,10 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
   if (((uintptr_t)q | (uintptr_t)out) & 15) return GEAR_ERR_ALIGN;
   if (c->n_compressed == 0 && c->buf_len == 0) return GEAR_ERR_STATE;
   note_stream(c, (cudaStream_t)stream);
-  gear_status s = plan_decode(c, Gq);
+  const int buf_block = Gq == 1 ? 16 : kRowsBufBlock;
+  const long long nblocks = c->n_blocks_c + (c->buf_len + buf_block - 1) / buf_block;
+  const int hp = rows_per_pass(c, Gq, nblocks), passes = decode_passes(Gq, hp);
+  gear_status s = plan_decode(c, Gq, hp);
   if (s != GEAR_OK) return s;
   DecodeArgs a = c->plan;
   a.arena = c->arena; a.table = c->table_dev; a.blk2seg = c->blk2seg;
@@ -622,12 +641,10 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
   a.early_reads = g_order.another_since(key, c->seg_write) ? 1 : 0;
   a.early_buf = c->buf_write.number == 0 || g_order.another_since(key, c->buf_write) ? 1 : 0;
   // never more CTAs than blocks of work
-  const int passes = decode_passes(Gq);
   if ((long long)c->cc.BH * passes > c->units_alloc) return GEAR_ERR_CAPACITY;
-  a.max_parts = partial_slots(c, Gq);
-  if (partial_bytes_for(c, Gq) > c->partial_bytes) return GEAR_ERR_CAPACITY;
-  const int buf_block = Gq == 1 ? 16 : kRowsBufBlock;
-  const long long work = (long long)c->cc.BH * passes * (c->n_blocks_c + (c->buf_len + buf_block - 1) / buf_block);
+  a.max_parts = partial_slots(c, Gq, hp);
+  if (partial_bytes_for(c, Gq, hp) > c->partial_bytes) return GEAR_ERR_CAPACITY;
+  const long long work = (long long)c->cc.BH * passes * nblocks;
   long long grid = (long long)c->sm_count * c->plan_occ;
   if (grid > work) grid = work;
   // Ranges of one or two blocks: a warp's partial result, its ticket and the merge of up to 64 partials then take as long as

@@ -6,8 +6,8 @@
 namespace gear {
 
 // ------------------------------------------------------------------ shared memory plan (per CTA)
-bool rows_plan(int heads, int ngv, int max_kpart, int max_vpart, int max_bfac, int max_T, DecodeArgs* a) {
-  const int hp = decode_heads_per_pass(heads), nw = kRowsWarps;
+bool rows_plan(int hp, int ngv, int max_kpart, int max_vpart, int max_bfac, int max_T, DecodeArgs* a) {
+  const int nw = kRowsWarps;
   const int bregion = round_up(max_bfac / 2, 16);
   int stage = bregion + (max_kpart > max_vpart ? max_kpart : max_vpart);
   if (stage < kRowsBufItem) stage = kRowsBufItem;

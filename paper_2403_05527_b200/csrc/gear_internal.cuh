@@ -158,14 +158,13 @@ bool decode_plan(int bits, int heads, int ngv, int max_kpart, int max_vpart, int
                  int warps_cap, DecodeArgs* a);
 int decode_occupancy(int bits, int heads, int ngv, int wide, size_t smem);
 int static_shape_id(const SegDesc& s, const CacheConst& c);
-// query rows one pass over the cache takes for G rows per kv head, and the number of passes
-inline int decode_heads_per_pass(int G) { return G == 1 ? 1 : (G <= 4 ? 4 : 8); }
-inline int decode_passes(int G) { return (G + decode_heads_per_pass(G) - 1) / decode_heads_per_pass(G); }
+// passes over the cache that G query rows per kv head take, hp rows (1, 4 or 8) at a time
+inline int decode_passes(int G, int hp) { return (G + hp - 1) / hp; }
 // several rows per pass (gear_decode_rows.cuh): warps of a CTA, CTAs per SM that registers and shared memory are planned for
 constexpr int kRowsWarps = 4;
 constexpr int kRowsCtasPerSm = 4;
 constexpr int kRowsBufBlock = 32;      // buffer tokens per block of work there (one row per pass: a slab)
-bool rows_plan(int heads, int ngv, int max_kpart, int max_vpart, int max_bfac, int max_T, DecodeArgs* a);
+bool rows_plan(int hp, int ngv, int max_kpart, int max_vpart, int max_bfac, int max_T, DecodeArgs* a);
 int rows_occupancy(const DecodeArgs& a, int bits, int ngv);
 cudaError_t launch_rows(const DecodeArgs& a, int grid, cudaStream_t st);
 // the fp16-cache kernel takes one or four query heads per pass

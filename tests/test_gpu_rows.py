@@ -115,3 +115,47 @@ def test_small_probabilities_beside_a_large_one(hq, bits):
         assert (np.abs(got - ref) <= bound).all(), (np.abs(got - ref) / bound).max()
     finally:
         p.close()
+
+
+@pytest.mark.parametrize("hkv,bits,group,s,rank,n,rows", [
+    (32, 2, 64, 2.0, 4, 5888, 16),       # every block shape the kernel is built for, eight rows at a time ...
+    (32, 4, 64, 2.0, 8, 4096, 24),
+    (24, 2, 128, 2.0, 4, 16384, 15),     # the last pass with seven rows
+    (32, 4, 128, 2.0, 4, 8192, 29),      # ... and five
+    (32, 4, 0, 2.0, 4, 6144, 16),
+    (48, 2, 32, 0.0, 0, 4096, 7),
+    (24, 4, 16, 6.0, 2, 4096, 16),
+    (32, 2, 64, 2.0, 4, 5888, 12),       # a last pass of four: fours although the cache is long
+])
+def test_rows_in_eights_against_rows_in_fours(hkv, bits, group, s, rank, n, rows):
+    """Long caches take eight rows per pass.  Each row has to be what it is in a call of four rows, before and after the cache
+    grows over the line (a prompt of an eighth, the rest behind it)."""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+    gen = torch.Generator(device="cuda").manual_seed(rows)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").half()   # noqa: E731
+    nb = 64 if group != 0 else 20
+    cfg = G.make_config(1, hkv, hkv, bits, group, s, nb, min(rank, nb), n + nb, rank_max=max(rank, 0), seed=1, max_queries=rows)
+    k, v, q = draw(1, hkv, n, 128), draw(1, hkv, n, 128), draw(1, hkv, rows, 128)
+    cache = G.gear_create(cfg)
+    try:
+        first = n // 8 // 128 * 128
+        for lo, hi in ((0, first), (first, n)):
+            G.gear_compress(cache, None, k[:, :, lo:hi].contiguous(), v[:, :, lo:hi].contiguous(), hi - lo, rank)
+            if hi == n:
+                for _ in range(7):
+                    G.gear_append_buffer(cache, draw(1, hkv, 128), draw(1, hkv, 128))
+            got = torch.full(q.shape, float("nan"), device="cuda")
+            G.gear_decode_attn_multi(cache, q, got, rows)
+            for r0 in range(0, rows, 4):
+                part = q[:, :, r0:r0 + 4].contiguous()
+                want = torch.empty(part.shape, device="cuda")
+                if part.shape[2] > 1:
+                    G.gear_decode_attn_multi(cache, part, want, part.shape[2])
+                else:
+                    G.gear_decode_attn(cache, part, want)
+                err = (got[:, :, r0:r0 + 4] - want).abs().amax(-1) / want.abs().amax(-1)
+                assert err.max().item() <= 8e-5          # twice what a kernel's own arithmetic may be off
+        assert G.gear_last_device_status(cache) == 0
+    finally:
+        G.gear_free(cache)
