@@ -417,8 +417,23 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
     const __half d16 = __float2half_rn(d32);
     const float d = __half2float(d16);
     const float inv = d != 0.f ? __fdiv_rn(1.0f, d) : 0.f;
+    // The group's scale, zero point and its two outliers (in-group index ascending), ahead of the barrier: the next block's copy is
+    // requested behind it and does not wait for loads from this one that are still on their way, so everything loaded has to
+    // be used before it.  The two stores depend on all of it.
     __half vmax = __ushort_as_half(0), vmin = vmax;
-    if (K == 1 && active) { vmax = group[imax * step]; vmin = group[imin * step]; }
+    if (active) {
+      if (K == 1) {
+        vmax = group[imax * step];
+        vmin = group[imin * step];
+        const bool max_first = imax < imin;
+        const __half2 ov = max_first ? __halves2half2(vmax, vmin) : __halves2half2(vmin, vmax);
+        const uchar2 oi = max_first ? make_uchar2((unsigned char)imax, (unsigned char)imin)
+                                    : make_uchar2((unsigned char)imin, (unsigned char)imax);
+        reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_koval : sd.off_voval))[tid] = ov;
+        reinterpret_cast<uchar2*>(rec + (side == 0 ? sd.off_koidx : sd.off_voidx))[tid] = oi;
+      }
+      reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_kscale : sd.off_vscale))[tid] = __halves2half2(d16, __float2half_rn(mn));
+    }
     if (__syncthreads_or(!ok)) {              // every thread has read the block
       if (tid == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
       break;
@@ -476,20 +491,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
     // scales by): half a step for a kept entry, the whole range if the step rounded to zero, plus the rounding of the
     // dequantised value
     float rmax = active ? (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx)) : 0.f;
-    // the group's scale, zero point and its two outliers (in-group index ascending)
     {
-      if (K == 1 && active) {
-        const bool max_first = imax < imin;
-        const __half2 ov = max_first ? __halves2half2(vmax, vmin) : __halves2half2(vmin, vmax);
-        const uchar2 oi = max_first ? make_uchar2((unsigned char)imax, (unsigned char)imin)
-                                    : make_uchar2((unsigned char)imin, (unsigned char)imax);
-        reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_koval : sd.off_voval))[tid] = ov;
-        reinterpret_cast<uchar2*>(rec + (side == 0 ? sd.off_koidx : sd.off_voidx))[tid] = oi;
-      }
-      if (active) {
-        reinterpret_cast<__half2*>(rec + (side == 0 ? sd.off_kscale : sd.off_vscale))[tid] =
-            __halves2half2(d16, __float2half_rn(mn));
-      }
       float dm = K == 1 && active ? fmaxf(fabsf(__half2float(vmax) - mn), fabsf(__half2float(vmin) - mn)) : 0.f;
       float sm = active ? d : 0.f;
 #pragma unroll
@@ -623,6 +625,8 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
     float* R = p.R ? p.R + (((size_t)bhl * 2 + SIDE) * sd.n_c + (size_t)blk * T) * kHeadDim : nullptr;
     unsigned char* rec = p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride + sd.bfac_bytes +
                          (size_t)blk * sd.rec_bytes;
+    unsigned char* orec_v = rec + (SIDE == 0 ? sd.off_koval : sd.off_voval) + tid * 8;
+    unsigned char* orec_i = rec + (SIDE == 0 ? sd.off_koidx : sd.off_voidx) + tid * 4;
     __half2 xp[L / 2];
     int it[2] = {0, 0}, ib[2] = {0, 0};
     float top[3], bot[3];
@@ -701,6 +705,11 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
       order(0, 1); order(2, 3); order(0, 2); order(1, 3); order(1, 2);
 #pragma unroll
       for (int a = 0; a < 4; ++a) ov[a] = __half_as_ushort(group[min(oi[a], L - 1) * step]);
+      // stored ahead of the barrier, so that all loads from the block have returned (see quant_fast_kernel); a group that takes
+      // the general routine below overwrites them
+      *reinterpret_cast<uint2*>(orec_v) = make_uint2(ov[0] | ((unsigned int)ov[1] << 16), ov[2] | ((unsigned int)ov[3] << 16));
+      *reinterpret_cast<unsigned int*>(orec_i) = (unsigned int)oi[0] | ((unsigned int)oi[1] << 8) |
+                                                 ((unsigned int)oi[2] << 16) | ((unsigned int)oi[3] << 24);
     }
     if (__syncthreads_or(!ok)) {                    // every thread has read the block
       if (tid == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
@@ -712,8 +721,6 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
       const float levels = (float)((1 << BITS) - 1);
       float d, mn, dm, rmax;
       __half d16;
-      unsigned char* orec_v = rec + (SIDE == 0 ? sd.off_koval : sd.off_voval) + tid * 8;
-      unsigned char* orec_i = rec + (SIDE == 0 ? sd.off_koidx : sd.off_voidx) + tid * 4;
       if (!shared_entry) {
         mn = bot[2];
         const float mx = top[2];
@@ -751,7 +758,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
             if (R != nullptr) store8(R + first + 8 * piece, r);
           }
         }
-        // the filtered entries: cleared and stored
+        // the filtered entries: cleared
         dm = 0.f;
 #pragma unroll
         for (int a = 0; a < 4; ++a) {
@@ -759,9 +766,6 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
           if (R != nullptr) R[SIDE == 0 ? oi[a] * kHeadDim + tid : first + oi[a]] = 0.f;
           dm = fmaxf(dm, fabsf(__half2float(__ushort_as_half(ov[a])) - mn));
         }
-        *reinterpret_cast<uint2*>(orec_v) = make_uint2(ov[0] | ((unsigned int)ov[1] << 16), ov[2] | ((unsigned int)ov[3] << 16));
-        *reinterpret_cast<unsigned int*>(orec_i) = (unsigned int)oi[0] | ((unsigned int)oi[1] << 8) |
-                                                   ((unsigned int)oi[2] << 16) | ((unsigned int)oi[3] << 24);
         rmax = (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
       } else {
         rmax = 0.f;
@@ -977,7 +981,7 @@ __global__ void __launch_bounds__(kPassWarps * 32, 3) pi_pass_kernel(PiArgs p) {
         mma16816(d[nt], fl, bf[c][nt][0], bf[c][nt][1]);
       }
     }
-    request(rb + kPassStages * kPassWarps * 16, stage);
+    const int used = stage;
     if (++stage == kPassStages) { stage = 0; parity ^= 1; }
     float mine[2][NT];                             // a[row gid | gid + 8][rho 4 nt + t]; rows past the chunk are zero
 #pragma unroll
@@ -987,6 +991,7 @@ __global__ void __launch_bounds__(kPassWarps * 32, 3) pi_pass_kernel(PiArgs p) {
       if (va) A0[(size_t)ra * RP + 4 * nt + t] = mine[0][nt];
       if (vc) A0[(size_t)rc * RP + 4 * nt + t] = mine[1][nt];
     }
+    request(rb + kPassStages * kPassWarps * 16, used);             // behind stores that need every load from the stage
     if (kGram) {
 #pragma unroll
       for (int half = 0; half < 2; ++half)
