@@ -90,6 +90,20 @@ class Pair:
                             err = rel_max(got, ref)
                             assert err <= tol, f"{side} low-rank reconstruction seg {si} b{b} h{h}{suffix}: {err:.2e}"
 
+    def with_stored_factors(self):
+        """The oracle's cache with the library's fp16 factors in the place of its own: what the attention kernels read."""
+        import copy
+        stored = copy.deepcopy(self.oracle)
+        for si, seg in enumerate(stored.segments):
+            if not seg["rank"]:
+                continue
+            for side in ("K", "V"):
+                a, bm = (G.gear_export(self.cache, si, f"{side}_{w}", self.B, self.Hkv).astype(np.float64) for w in "AB")
+                for b in range(self.B):
+                    for h in range(self.Hkv):
+                        seg[side][b][h]["A"], seg[side][b][h]["B"] = a[b, h], bm[b, h]
+        return stored
+
     def check_attention(self, extra=0, tol=TOL, scale=0.0):
         t = self.torch
         q = synth.make_query(self.cid, self.B, self.Hq, 128, extra=extra)

@@ -1,5 +1,6 @@
 """Quantization of groups of 32, 64 and 128 by CTAs that take one block after the other: more blocks than the device holds
-CTAs for, a single block, and values that lie half way between two codes."""
+CTAs for, few blocks, and values that lie half way between two codes.  Segments of more than 128 tokens: shorter ones are
+compressed by another kernel, in one launch."""
 import numpy as np
 import pytest
 
@@ -10,11 +11,11 @@ pytestmark = pytest.mark.gpu
     (2, 64, 2.0, 11, 4096, 1),      # one outlier per side and group; 704 blocks per side
     (4, 64, 2.0, 11, 4096, 0),      # the same without a residual
     (4, 128, 2.0, 6, 16384, 1),     # two outliers; 768 blocks per side
-    (2, 128, 2.0, 1, 128, 1),       # one block
-    (4, 64, 2.0, 1, 64, 1),
+    (2, 128, 2.0, 1, 256, 1),       # few blocks
+    (4, 64, 2.0, 1, 192, 1),
     (2, 64, 0.0, 3, 1024, 1),       # no outliers
     (4, 32, 2.0, 13, 4096, 1),      # groups of 32; 1664 blocks per side
-    (2, 32, 0.0, 1, 32, 1),
+    (2, 32, 0.0, 1, 160, 1),
     (2, 128, 1.0, 2, 1024, 1),      # groups of 128 with one outlier
     (4, 128, 0.0, 5, 512, 1),
 ])
@@ -33,8 +34,10 @@ def test_blocks_and_ties(bits, group, s_pct, H, n, rank):
             x[..., :3], x[..., 3:6] = 0.0, float(top)       # the group spans 0 .. top also without its outliers
         b0 = synth.make_b0(16, 1, H, 128, rank)
         p.oracle.compress(k16, v16, rank, b0)
+        before = G.gear_kernel_launches()
         G.gear_compress(p.cache, None, torch.from_numpy(k16).cuda(), torch.from_numpy(v16).cuda(), n, rank,
                         torch.from_numpy(np.ascontiguousarray(b0)).cuda() if rank else None)
+        assert G.gear_kernel_launches() - before == (10 if rank else 3)      # a launch per side, seven for the rank, the descriptor
         torch.cuda.synchronize()
         p.check_segment(0)
     finally:
@@ -51,13 +54,16 @@ def test_flat_groups(kind, s_pct):
     for group in (32, 64, 128):
         p = Pair(16, 1, 1, 1, 2, group, s_pct, 64, 0, 512)
         try:
-            x = np.full((1, 1, 2 * group, 128), 1.25, np.float16)
+            n = 256                                       # more than 128: a launch per side and the descriptor
+            x = np.full((1, 1, n, 128), 1.25, np.float16)
             if kind == "one peak":
                 x[0, 0, 5::group, :] = 9.0
                 x[0, 0, :, 7::group] = -9.0
             p.oracle.compress(x, x, 0, np.zeros((1, 1, 2, 128, 0), np.float32))
             xd = torch.from_numpy(x).cuda()
-            G.gear_compress(p.cache, None, xd, xd, 2 * group, 0, None)
+            before = G.gear_kernel_launches()
+            G.gear_compress(p.cache, None, xd, xd, n, 0, None)
+            assert G.gear_kernel_launches() - before == 3
             torch.cuda.synchronize()
             p.check_segment(0)
         finally:
