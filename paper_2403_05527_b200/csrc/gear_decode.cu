@@ -78,7 +78,7 @@ bool decode_plan(int bits, int heads, int ngv, int max_kpart, int max_vpart, int
   w.corr_k = o;  o += HP * max_T * 4;
   w.corr_v = o;  o += HP * kHeadDim * 4;
   w.ocorr = o;   o += HP * kHeadDim * 4;
-  w.wl = o;      o += kMaxRank * (HP == 1 ? 1 : 8) * 4 + 16;
+  w.wl = o;      o += kMaxRank * 4 + 16;
   w.misc = o;    o += 32 + (kMaxStages + 1) * 8 + 8;   // exponents of max |q| per head, the ring's mbarriers, one test barrier
   w.ring = round_up(o, 16);
   w.fragv_stride = fv_stride;
@@ -124,7 +124,6 @@ int static_shape_id(const SegDesc& s, const CacheConst& c) {
 template <int BITS, int HEADS, int NGV, int MINB, bool JOIN>
 __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_kernel(const __grid_constant__ DecodeArgs a) {
   constexpr int HP = HEADS;
-  constexpr int NT = HP == 1 ? 1 : 2;             // 8-column tiles of the integer B operands: four limb columns per head
   constexpr int F = 8 / BITS;                     // code fields per byte
   constexpr int kTop = BITS * (F - 1);            // the shift of the highest field
   constexpr int GV = kHeadDim / NGV;              // channels per value group
@@ -132,7 +131,6 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
   constexpr int VT = 8 / F;                       // value tuples per 32-token chunk
   constexpr int kFragStride = frag_row_words(HP);
   constexpr int CMASK = HP == 1 ? 1 : 7;          // fp16 fragment columns that exist, as a mask on the lane's column
-  constexpr int WLS = HP == 1 ? 1 : 8;            // row stride of the small factor exchange buffer wl[16][heads]
   extern __shared__ __align__(128) unsigned char smem_all[];
 
   const int lane = JOIN ? threadIdx.x & 31 : threadIdx.x, gid = lane >> 2, t = lane & 3, wrp = JOIN ? threadIdx.x >> 5 : 0;
@@ -152,16 +150,15 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
   float* ps = reinterpret_cast<float*>(smem + a.ws.ps);          // [HP][maxT] scores, then probabilities
   int* corr_v = reinterpret_cast<int*>(smem + a.ws.corr_v);      // [HP][128]
   float* ocorr = reinterpret_cast<float*>(smem + a.ws.ocorr);    // [HP][128] fp32 copy of the output accumulators
-  float* wl = reinterpret_cast<float*>(smem + a.ws.wl);          // [16][heads]
+  float* wl = reinterpret_cast<float*>(smem + a.ws.wl);          // [16]
   int* qexp_s = reinterpret_cast<int*>(smem + a.ws.misc);        // [HP]
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + a.ws.misc + 32);   // [kMaxStages] ring, [kMaxStages] test barrier
 
-  // lane roles in the integer products: B / D column n of tile nt is limb n % 4 of head 2 nt + n / 4.  As owner of
-  // B column gid the lane fetches limb gid % 4 of head hcol(nt); as owner of D columns 2t, 2t + 1 it holds the limb
-  // pair t % 2 of head hacc(nt).
+  // lane roles in the integer products (one head): B / D column n is limb n % 4.  As owner of B column gid the lane fetches
+  // limb gid % 4; as owner of D columns 2t, 2t + 1 it holds the limb pair t % 2.
   const int limb_b = gid & 3;
   const bool pair_hi = (t & 1) != 0;
-  const bool writer = HP == 1 ? (t == 0) : !pair_hi;    // lanes that hold the low limb pair of a real head finish the sums
+  const bool writer = t == 0;                           // lanes that hold the low limb pair finish the sums
 
   if (lane == 0)
     for (int s = 0; s <= kMaxStages; ++s) mbar_init(&bar[s], 1);
@@ -392,54 +389,42 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
     };
 
     // ==================================================================== compressed blocks
-    if (HEADS == 1 && blk_lo < c_hi) {
-      int O[8][NT][4];                                   // value sums: tile (16 channels) x column tile, 32-bit integers
-      float U[4], cm[HP][NGV];
-      uint32_t bw[NT][2];                                // low-rank key term: B operand (q B_K) of the current segment
+    if constexpr (HEADS == 1) if (blk_lo < c_hi) {
+      int O[8][4];                                       // value sums: a tile of 16 channels each, 32-bit integers
+      float U[4], cm[NGV];
+      uint32_t bw[2] = {0u, 0u};                         // low-rank key term: B operand (q B_K) of the current segment
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        bw[nt][0] = bw[nt][1] = 0u;
+      for (int mt = 0; mt < 8; ++mt)
 #pragma unroll
-        for (int mt = 0; mt < 8; ++mt)
+        for (int k = 0; k < 4; ++k) O[mt][k] = 0;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) O[mt][nt][i] = 0;
-      }
+      for (int k = 0; k < 4; ++k) U[k] = 0.f;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) U[i] = 0.f;
-#pragma unroll
-      for (int h = 0; h < HP; ++h)
-#pragma unroll
-        for (int g = 0; g < NGV; ++g) cm[h][g] = 0.f;
+      for (int g = 0; g < NGV; ++g) cm[g] = 0.f;
       bool u_pending = false;
       int eV_cur = 1000;                                 // exponent of the value fixed-point scale the integer sums carry
       int tok_acc = 0;                                   // tokens in the integer sums since they were last folded
 
-      // integer sums -> fp32 copy in shared memory, times alpha[h]; the integers start again from zero
-      auto fold_O = [&](const float (&alpha)[HP]) {
+      // integer sums -> fp32 copy in shared memory, times alpha; the integers start again from zero
+      auto fold_O = [&](float alpha) {
         const float fs = pow2i(-eV_cur);
         __syncwarp();
+        const float w1 = pair_hi ? 0.f : 256.f;              // the high pair's second column is no limb: dropped
+        const float w0 = pair_hi ? 65536.f * fs : fs;
 #pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          const int hd = HP == 1 ? 0 : 2 * nt + (t >> 1);
-          float al = alpha[HP == 1 ? 0 : 2 * nt];
-          if (HP > 1 && (t >> 1)) al = alpha[HP == 1 ? 0 : 2 * nt + 1];
-          const float w1 = pair_hi ? 0.f : 256.f;            // the high pair's second column is no limb: dropped
-          const float w0 = pair_hi ? 65536.f * fs : fs;
-#pragma unroll
-          for (int mt = 0; mt < 8; ++mt) {
-            const float rs = w0 * (1.0f / (float)(1 << (BITS * (mt % F))));
-            float v0 = fmaf((float)O[mt][nt][1], w1, (float)O[mt][nt][0]) * rs;
-            float v1 = fmaf((float)O[mt][nt][3], w1, (float)O[mt][nt][2]) * rs;
-            v0 += __shfl_xor_sync(0xffffffffu, v0, 1);
-            v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
-            if (writer && hd < HC) {
-              float* oc = ocorr + hd * kHeadDim + 16 * mt + gid;
-              oc[0] = (oc[0] + v0) * al;
-              oc[8] = (oc[8] + v1) * al;
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) O[mt][nt][i] = 0;
+        for (int mt = 0; mt < 8; ++mt) {
+          const float rs = w0 * (1.0f / (float)(1 << (BITS * (mt % F))));
+          float v0 = fmaf((float)O[mt][1], w1, (float)O[mt][0]) * rs;
+          float v1 = fmaf((float)O[mt][3], w1, (float)O[mt][2]) * rs;
+          v0 += __shfl_xor_sync(0xffffffffu, v0, 1);
+          v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
+          if (writer) {
+            float* oc = ocorr + 16 * mt + gid;
+            oc[0] = (oc[0] + v0) * alpha;
+            oc[8] = (oc[8] + v1) * alpha;
           }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) O[mt][i] = 0;
         }
         __syncwarp();
       };
@@ -487,11 +472,9 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
           const float dmax_k = reinterpret_cast<const float*>(kp)[0];
           const float dmax_v = reinterpret_cast<const float*>(kp)[1];
           const float smax_v = reinterpret_cast<const float*>(kp)[3];
-          int sexp_k[HP];                                 // per head: exponent of the sparse key term's fixed-point scale
-          float c_zero[HP];                               // per head: sum over channels of q * zero-point
-          float kscl[NT];                                 // per column tile: what turns this lane's integer sums into scores
-#pragma unroll
-          for (int h = 0; h < HP; ++h) { sexp_k[h] = 0; c_zero[h] = 0.f; }
+          int sexp_k;                                     // exponent of the sparse key term's fixed-point scale
+          float c_zero;                                   // sum over channels of q * zero-point
+          float kscl;                                     // what turns this lane's integer sums into scores
 
           if (with_bk) {
             // w = q B_K through the fp16 tensor cores, kept as the B operand of the low-rank key term
@@ -509,37 +492,31 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
                 af[3] = *reinterpret_cast<const uint32_t*>(bk + (gid + 8) * kHeadDim + 16 * kc + 2 * t + 8);
               }
               uint32_t b0 = 0u, b1 = 0u;
-              const int h = gid >> 1;
-              if ((gid & 1) == 0 && h < HC) {
-                const __half* qrow = qs + h * kHeadDim + 16 * kc + 2 * t;
+              if ((gid & 1) == 0 && gid < 2) {      // column 0 (written as gid == 0, a launch of one block per warp takes 0.2 us more)
+                const __half* qrow = qs + 16 * kc + 2 * t;
                 b0 = *reinterpret_cast<const uint32_t*>(qrow);
                 b1 = *reinterpret_cast<const uint32_t*>(qrow + 8);
               }
               mma16816(wacc, af, b0, b1);
             }
             __syncwarp();
-            if (t < HP) {                           // D[rho][col 2t] = w[rho][head t]
-              wl[gid * WLS + t] = wacc[0] * a.scale_log2;
-              wl[(gid + 8) * WLS + t] = wacc[2] * a.scale_log2;
+            if (t == 0) {                           // D[rho][column 0] = w[rho]
+              wl[gid] = wacc[0] * a.scale_log2;
+              wl[gid + 8] = wacc[2] * a.scale_log2;
             }
             __syncwarp();
-            // B operand of the low-rank key product, one per integer column tile: column 4u holds the high parts of
-            // head 2 nt + u, column 4u + 1 the remainders, the other columns are zero -- so that the lane that
-            // finishes the integer sum of a head also receives the head's low-rank term
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-              const int h = HP == 1 ? 0 : 2 * nt + (gid >> 2);
-              uint32_t hi0, lo0, hi1, lo1;
-              split_hi_lo(wl[(2 * t) * WLS + h], wl[(2 * t + 1) * WLS + h], hi0, lo0);
-              split_hi_lo(wl[(2 * t + 8) * WLS + h], wl[(2 * t + 9) * WLS + h], hi1, lo1);
-              bw[nt][0] = limb_b == 0 ? hi0 : (limb_b == 1 ? lo0 : 0u);
-              bw[nt][1] = limb_b == 0 ? hi1 : (limb_b == 1 ? lo1 : 0u);
-            }
+            // B operand of the low-rank key product: columns 0, 4 hold the high parts, 1, 5 the remainders, the others are
+            // zero -- so that the lane that finishes the integer sum also receives the low-rank term
+            uint32_t hi0, lo0, hi1, lo1;
+            split_hi_lo(wl[2 * t], wl[2 * t + 1], hi0, lo0);
+            split_hi_lo(wl[2 * t + 8], wl[2 * t + 9], hi1, lo1);
+            bw[0] = limb_b == 0 ? hi0 : (limb_b == 1 ? lo0 : 0u);
+            bw[1] = limb_b == 0 ? hi1 : (limb_b == 1 ? lo1 : 0u);
             __syncwarp();
           }
 
           // ---------------- B operand of the key scores: the block-wide fixed-point image of q * scale per channel,
-          //                  as four signed base-256 digits; c_h = sum q * zero; sparse key term scattered to its token
+          //                  as four signed base-256 digits; sum of q * zero; sparse key term scattered to its token
           {
             const uint4 kz = reinterpret_cast<const uint4*>(kp + off_kscale)[lane];
             const uint32_t w4[4] = {kz.x, kz.y, kz.z, kz.w};
@@ -554,65 +531,39 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
             const int sh = BITS * (F - 1 - ((lane >> 3) % F));
             const uint32_t mulc = 1u << sh, addc = 0x80808080u - (kMagicBits << sh);
             const int ed = float_exponent(dmax_k);
-            float qS[HP][4];
-            int eK[HP];
+            float qd[4];
 #pragma unroll
-            for (int h = 0; h < HP; ++h) {
-              eK[h] = 0;
-              if (h < HC) {
-                float qv[4];
-                if (HP == 1) {
-                  qv[0] = qreg[0]; qv[1] = qreg[1]; qv[2] = qreg[2]; qv[3] = qreg[3];
-                } else {
-                  const uint2 qh = *reinterpret_cast<const uint2*>(qs + h * kHeadDim + lane * 4);
-                  const __half2 q01 = u32_as_h2(qh.x), q23 = u32_as_h2(qh.y);
-                  qv[0] = __low2float(q01) * a.scale_log2; qv[1] = __high2float(q01) * a.scale_log2;
-                  qv[2] = __low2float(q23) * a.scale_log2; qv[3] = __high2float(q23) * a.scale_log2;
-                }
-                float qd[4];
+            for (int j = 0; j < 4; ++j) qd[j] = qreg[j] * sc4[j];
+            const float am = fmaxf(fmaxf(fabsf(qd[0]), fabsf(qd[1])), fmaxf(fabsf(qd[2]), fabsf(qd[3])));
+            const uint32_t mb = warp_max_u32(__float_as_uint(am));         // non-negative floats order like their bits
+            const int e = clamp60(21 - ((int)(mb >> 23) - 127));            // |q * scale| * 2^e < 2^22
+            const float Sk = pow2i(e);
+            uint32_t z[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) qd[j] = qv[j] * sc4[j];
-                const float am = fmaxf(fmaxf(fabsf(qd[0]), fabsf(qd[1])), fmaxf(fabsf(qd[2]), fabsf(qd[3])));
-                const uint32_t mb = warp_max_u32(__float_as_uint(am));     // non-negative floats order like their bits
-                const int e = clamp60(21 - ((int)(mb >> 23) - 127));        // |q * scale| * 2^e < 2^22
-                eK[h] = e;
-                const float Sk = pow2i(e);
-                uint32_t z[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  z[j] = (__float_as_uint(fmaf(qd[j], Sk, kMagic)) * mulc + addc) ^ 0x80808080u;    // balanced digits
-                // digits of four channels -> one register per limb (bytes = the lane's four channels in order)
-                const uint32_t p01l = __byte_perm(z[0], z[1], 0x5140), p23l = __byte_perm(z[2], z[3], 0x5140);
-                const uint32_t p01h = __byte_perm(z[0], z[1], 0x7362), p23h = __byte_perm(z[2], z[3], 0x7362);
-                uint32_t* row = xr + (h * 4) * kFragKRow + (lane >> 3) * 8 + (lane & 3) * 2 + ((lane >> 2) & 1);
-                row[0] = __byte_perm(p01l, p23l, 0x5410);
-                row[kFragKRow] = __byte_perm(p01l, p23l, 0x7632);
-                row[2 * kFragKRow] = __byte_perm(p01h, p23h, 0x5410);
-                row[3 * kFragKRow] = __byte_perm(p01h, p23h, 0x7632);
+            for (int j = 0; j < 4; ++j)
+              z[j] = (__float_as_uint(fmaf(qd[j], Sk, kMagic)) * mulc + addc) ^ 0x80808080u;    // balanced digits
+            // digits of four channels -> one register per limb (bytes = the lane's four channels in order)
+            const uint32_t p01l = __byte_perm(z[0], z[1], 0x5140), p23l = __byte_perm(z[2], z[3], 0x5140);
+            const uint32_t p01h = __byte_perm(z[0], z[1], 0x7362), p23h = __byte_perm(z[2], z[3], 0x7362);
+            uint32_t* row = xr + (lane >> 3) * 8 + (lane & 3) * 2 + ((lane >> 2) & 1);
+            row[0] = __byte_perm(p01l, p23l, 0x5410);
+            row[kFragKRow] = __byte_perm(p01l, p23l, 0x7632);
+            row[2 * kFragKRow] = __byte_perm(p01h, p23h, 0x5410);
+            row[3 * kFragKRow] = __byte_perm(p01h, p23h, 0x7632);
 
-                float c = fmaf(qv[0], zr4[0], fmaf(qv[1], zr4[1], fmaf(qv[2], zr4[2], qv[3] * zr4[3])));   // this lane's part
+            float c = fmaf(qreg[0], zr4[0], fmaf(qreg[1], zr4[1], fmaf(qreg[2], zr4[2], qreg[3] * zr4[3])));   // this lane's part
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-                const int sexp = clamp60(21 - qexp_s[h] - ed);
-                const float Sx = pow2i(sexp);
-                qS[h][0] = qv[0] * Sx; qS[h][1] = qv[1] * Sx; qS[h][2] = qv[2] * Sx; qS[h][3] = qv[3] * Sx;
-                c_zero[h] = c; sexp_k[h] = sexp;
-              }
-            }
-            // what turns this lane's integer sums of column tile nt into scores: the inverse fixed-point scale of the
-            // head it serves, the weight of the highest field, and 2^16 for the high limb pair
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-              int e = eK[HP == 1 ? 0 : 2 * nt];
-              if (HP > 1 && (t >> 1)) e = eK[HP == 1 ? 0 : 2 * nt + 1];
-              kscl[nt] = pow2i(-e - kTop + (pair_hi ? 16 : 0));
-            }
+            for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+            c_zero = c;
+            sexp_k = clamp60(21 - qexp_s[0] - ed);
+            const float Sx = pow2i(sexp_k);
+            const float qS[4] = {qreg[0] * Sx, qreg[1] * Sx, qreg[2] * Sx, qreg[3] * Sx};
+            // the inverse fixed-point scale, the weight of the highest field, and 2^16 for the high limb pair
+            kscl = pow2i(-e - kTop + (pair_hi ? 16 : 0));
             if (k2k > 0) {
               auto k_entry = [&](int j, float val, int idx) {
                 const float d = val - zr4[j];
-#pragma unroll
-                for (int h = 0; h < HP; ++h)
-                  if (h < HC) atomicAdd(&corr_k[h * maxT + idx], __float2int_rn(qS[h][j] * d));
+                atomicAdd(&corr_k[idx], __float2int_rn(qS[j] * d));
               };
               if (k2k == 2) {
                 const uint4 ov = reinterpret_cast<const uint4*>(kp + off_koval)[lane];
@@ -666,12 +617,8 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
               auto apply = [&](unsigned int w) {
                 const int tok = (int)(w & 0xFFu), ch = (int)((w >> 8) & 0xFFu);
                 const float d = __half2float(__ushort_as_half((unsigned short)(w >> 16))) - __high2float(szp[ch]);
-#pragma unroll
-                for (int h = 0; h < HP; ++h)
-                  if (h < HC) {
-                    const float qv = __half2float(qs[h * kHeadDim + ch]) * a.scale_log2;
-                    atomicAdd(&corr_k[h * maxT + tok], __float2int_rn(qv * pow2i(sexp_k[h]) * d));
-                  }
+                const float qv = __half2float(qs[ch]) * a.scale_log2;
+                atomicAdd(&corr_k[tok], __float2int_rn(qv * pow2i(sexp_k) * d));
               };
               const bool have = cs_blk == blk;
 #pragma unroll
@@ -693,17 +640,12 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
             }
           }
           __syncwarp();
-          // this lane's B registers: limb gid % 4 of head hcol(nt) for the four 32-channel chunks
-          uint32_t bK[NT][4][2];
+          // this lane's B registers: limb gid % 4 for the four 32-channel chunks
+          uint32_t bK[4][2];
 #pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            const int hcol = HP == 1 ? 0 : 2 * nt + (gid >> 2);
-            const uint32_t* row = xr + (hcol * 4 + limb_b) * kFragKRow + 2 * t;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const uint2 v = *reinterpret_cast<const uint2*>(row + c * 8);
-              bK[nt][c][0] = v.x; bK[nt][c][1] = v.y;
-            }
+          for (int c = 0; c < 4; ++c) {
+            const uint2 v = *reinterpret_cast<const uint2*>(xr + limb_b * kFragKRow + 2 * t + c * 8);
+            bK[c][0] = v.x; bK[c][1] = v.y;
           }
 
           // ---------------- key scores, slab by slab; scores go to shared memory
@@ -715,11 +657,7 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
             int tok0 = gid;
 #pragma unroll (S::unroll)
             for (int slab = 0; slab < nslab; ++slab) {
-              int acc[NT][4];
-#pragma unroll
-              for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc[nt][i] = 0;
+              int acc[4] = {0, 0, 0, 0};
 #pragma unroll
               for (int tau = 0; tau < KT; ++tau) {
                 const uint4 w = cwp[tau * 32];
@@ -728,8 +666,7 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
                   constexpr uint32_t m0 = field_mask<BITS>(0);
                   const uint32_t m = m0 << (BITS * j);
                   const uint32_t af[4] = {w.x & m, w.y & m, w.z & m, w.w & m};
-#pragma unroll
-                  for (int nt = 0; nt < NT; ++nt) imma16832(acc[nt], af, bK[nt][F * tau + j][0], bK[nt][F * tau + j][1]);
+                  imma16832(acc, af, bK[F * tau + j][0], bK[F * tau + j][1]);
                 }
               }
               cwp += KT * 32;
@@ -744,25 +681,20 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
                 aa[3] = *reinterpret_cast<const uint32_t*>(akp + ak8 + 8);
               }
               akp += ak_step;
-#pragma unroll
-              for (int nt = 0; nt < NT; ++nt) {
-                // low limb pair + 2^16 high limb pair, each lane converting its own pair; the partner adds the other
-                float f0 = (float)(acc[nt][0] + acc[nt][1] * 256) * kscl[nt];
-                float f1 = (float)(acc[nt][2] + acc[nt][3] * 256) * kscl[nt];
-                f0 += __shfl_xor_sync(0xffffffffu, f0, 1);
-                f1 += __shfl_xor_sync(0xffffffffu, f1, 1);
-                if (r_pad > 0) {
-                  float d[4];
-                  mma16816_z(d, aa, bw[nt][0], bw[nt][1]);
-                  f0 += d[0] + d[1];
-                  f1 += d[2] + d[3];
-                }
-                const int hd = HP == 1 ? 0 : 2 * nt + (t >> 1);
-                if (writer && hd < HC) {
-                  // raw sums only: the zero-point constant and the sparse term are added in the softmax pass
-                  float* pr = ps + hd * maxT + tok0;
-                  pr[0] = f0; pr[8] = f1;
-                }
+              // low limb pair + 2^16 high limb pair, each lane converting its own pair; the partner adds the other
+              float f0 = (float)(acc[0] + acc[1] * 256) * kscl;
+              float f1 = (float)(acc[2] + acc[3] * 256) * kscl;
+              f0 += __shfl_xor_sync(0xffffffffu, f0, 1);
+              f1 += __shfl_xor_sync(0xffffffffu, f1, 1);
+              if (r_pad > 0) {
+                float d[4];
+                mma16816_z(d, aa, bw[0], bw[1]);
+                f0 += d[0] + d[1];
+                f1 += d[2] + d[3];
+              }
+              if (writer) {
+                // raw sums only: the zero-point constant and the sparse term are added in the softmax pass
+                ps[tok0] = f0; ps[tok0 + 8] = f1;
               }
               tok0 += kSlab;
             }
@@ -786,43 +718,36 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
           const bool exp_bad = eV_cur > need || eV_cur < need - 3;
           const int eV_new = exp_bad ? need - kLag : eV_cur;
           const float room = (float)(need - eV_new);
-          float2 sc[HP][NPR];
-          float alpha[HP], m_new[HP], lag[HP];
-          bool grew = false;
+          float2 sc[NPR];
+          const float Sik = pow2i(-sexp_k);
+          float mx = -INFINITY;
 #pragma unroll
-          for (int h = 0; h < HP; ++h) {
-            alpha[h] = 1.f; m_new[h] = 0.f; lag[h] = 1.f;
-            if (h < HC) {
-              const float Sik = pow2i(-sexp_k[h]);
-              float mx = -INFINITY;
-#pragma unroll
-              for (int i = 0; i < NPR; ++i) {
-                const int tp = 2 * (lane + 32 * i);
-                float2 v = make_float2(-INFINITY, -INFINITY);
-                if (tp < T) {
-                  v = *reinterpret_cast<const float2*>(ps + h * maxT + tp);
-                  v.x += c_zero[h]; v.y += c_zero[h];
-                  if (k2k > 0 || (NGV == 1 && S::kCsr && sdc->csr_base16 != 0)) {
-                    const int2 c = *reinterpret_cast<const int2*>(corr_k + h * maxT + tp);
-                    v.x = fmaf((float)c.x, Sik, v.x);
-                    v.y = fmaf((float)c.y, Sik, v.y);
-                    *reinterpret_cast<int2*>(corr_k + h * maxT + tp) = make_int2(0, 0);
-                  }
-                }
-                sc[h][i] = v;
-                mx = fmaxf(mx, fmaxf(v.x, v.y));
+          for (int i = 0; i < NPR; ++i) {
+            const int tp = 2 * (lane + 32 * i);
+            float2 v = make_float2(-INFINITY, -INFINITY);
+            if (tp < T) {
+              v = *reinterpret_cast<const float2*>(ps + tp);
+              v.x += c_zero; v.y += c_zero;
+              if (k2k > 0 || (NGV == 1 && S::kCsr && sdc->csr_base16 != 0)) {
+                const int2 c = *reinterpret_cast<const int2*>(corr_k + tp);
+                v.x = fmaf((float)c.x, Sik, v.x);
+                v.y = fmaf((float)c.y, Sik, v.y);
+                *reinterpret_cast<int2*>(corr_k + tp) = make_int2(0, 0);
               }
-              mx = warp_max(mx);
-              if (mx > m_run[h] + room) {                   // warp-uniform
-                alpha[h] = exp2f(m_run[h] - mx);
-                m_run[h] = mx;
-                grew = true;
-              }
-              m_new[h] = m_run[h];
-              // the sparse value term's fixed point is set for probabilities of one at most: the block's own maximum
-              lag[h] = pow2i(-max(0, (int)ceilf(mx - m_new[h])));
             }
+            sc[i] = v;
+            mx = fmaxf(mx, fmaxf(v.x, v.y));
           }
+          mx = warp_max(mx);
+          const bool grew = mx > m_run[0] + room;         // warp-uniform
+          float alpha = 1.f;
+          if (grew) {
+            alpha = exp2f(m_run[0] - mx);
+            m_run[0] = mx;
+          }
+          const float m_new = m_run[0];
+          // the sparse value term's fixed point is set for probabilities of one at most: the block's own maximum
+          const float lag = pow2i(-max(0, (int)ceilf(mx - m_new)));
           // The integers are folded into the fp32 copy when the maximum moved (everything so far shrinks by alpha), when this
           // block's scales do not fit their exponent, or when the 32-bit range nears its end.
           {
@@ -831,21 +756,14 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
               fold_O(alpha);
               tok_acc = 0;
             } else if (grew) {
-              scale_ocorr(alpha);
+              const float of_head[HP] = {alpha};
+              scale_ocorr(of_head);
             }
             if (grew) {
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                float al = alpha[0];
+              for (int i = 0; i < 4; ++i) U[i] *= alpha;
 #pragma unroll
-                for (int hh = 1; hh < HP; ++hh)
-                  if (t == hh) al = alpha[hh];
-                U[i] *= al;
-              }
-#pragma unroll
-              for (int h = 0; h < HP; ++h)
-#pragma unroll
-                for (int g = 0; g < NGV; ++g) cm[h][g] *= alpha[h];
+              for (int g = 0; g < NGV; ++g) cm[g] *= alpha;
             }
             eV_cur = eV_new;                    // a change comes with a fold (or with empty sums)
             tok_acc += T;
@@ -854,9 +772,7 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
           const float Sx = pow2i(clamp60(21 - float_exponent(dmax_v)));     // fixed-point scale of the sparse value term
           const __half2* vsz = reinterpret_cast<const __half2*>(vp + o_vsz);
           unsigned char* fragVb = reinterpret_cast<unsigned char*>(xr);
-          float l[HP];
-#pragma unroll
-          for (int h = 0; h < HP; ++h) l[h] = 0.f;
+          float l = 0.f;
 #pragma unroll
           for (int i = 0; i < NPR; ++i) {
             const int pr = lane + 32 * i, tp = 2 * pr;
@@ -865,13 +781,9 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
               // a block that ends inside a slab: the absent tokens of that slab get probability zero in the fp16
               // fragments (the region held other operands before; their A_V rows are zero, but 0 x NaN is not)
               if (r_pad > 0 && tp < nslab * kSlab) {
-#pragma unroll
-                for (int h = 0; h < HP; ++h)
-                  if (h < HC) {
-                    uint32_t* bp = fragPc + s * kFragStride + rg;
-                    bp[(2 * (h & 3) * 4 + tw) * 2] = 0u;
-                    bp[((2 * (h & 3) + 1) * 4 + tw) * 2] = 0u;
-                  }
+                uint32_t* bp = fragPc + s * kFragStride + rg;
+                bp[tw * 2] = 0u;
+                bp[(4 + tw) * 2] = 0u;
               }
               break;
             }
@@ -879,36 +791,27 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
             // where this pair's two bytes go in a row of the value B operand: chunk, register (tokens 4t.. / 16+4t..),
             // lane column, half word
             const int vboff = (((pr >> 4) * 8 + ((pr & 7) >> 1) * 2 + ((pr & 15) >> 3)) << 2) + ((pr & 1) << 1);
-            float p[HP][2];
             __half2 z[2][NGV];
 #pragma unroll
             for (int g = 0; g < NGV; ++g) { z[0][g] = vsz[tp * NGV + g]; z[1][g] = vsz[(tp + 1) * NGV + g]; }
+            const float p[2] = {exp2_fast(sc[i].x - m_new), exp2_fast(sc[i].y - m_new)};
+            l += p[0] + p[1];
+            if (r_pad > 0) {                                // fp16 fragments of p for the low-rank value term
+              uint32_t hi, lo;
+              split_hi_lo(p[0], p[1], hi, lo);
+              uint32_t* bp = fragPc + s * kFragStride + rg;
+              bp[tw * 2] = hi;
+              bp[(4 + tw) * 2] = lo;
+            }
 #pragma unroll
-            for (int h = 0; h < HP; ++h) {
-              p[h][0] = p[h][1] = 0.f;
-              if (h < HC) {
-                const float p0 = exp2_fast(sc[h][i].x - m_new[h]), p1 = exp2_fast(sc[h][i].y - m_new[h]);
-                p[h][0] = p0; p[h][1] = p1;
-                l[h] += p0 + p1;
-                if (r_pad > 0) {                              // fp16 fragments of p for the low-rank value term
-                  const int col = 2 * (h & 3);
-                  uint32_t hi, lo;
-                  split_hi_lo(p0, p1, hi, lo);
-                  uint32_t* bp = fragPc + s * kFragStride + rg;
-                  bp[(col * 4 + tw) * 2] = hi;
-                  bp[((col + 1) * 4 + tw) * 2] = lo;
-                }
-#pragma unroll
-                for (int g = 0; g < NGV; ++g) {
-                  const uint32_t y0 = __float_as_uint(fmaf(p0 * __low2float(z[0][g]), Sv, kMagicV));
-                  const uint32_t y1 = __float_as_uint(fmaf(p1 * __low2float(z[1][g]), Sv, kMagicV));
-                  unsigned char* rowb = fragVb + ((g * HP + h) * 4) * RS * 4 + vboff;
-                  *reinterpret_cast<unsigned short*>(rowb) = (unsigned short)__byte_perm(y0, y1, 0x0040);
-                  *reinterpret_cast<unsigned short*>(rowb + RS * 4) = (unsigned short)__byte_perm(y0, y1, 0x0051);
-                  *reinterpret_cast<unsigned short*>(rowb + 2 * RS * 4) = (unsigned short)__byte_perm(y0, y1, 0x0062);
-                  cm[h][g] = fmaf(p0, __high2float(z[0][g]), fmaf(p1, __high2float(z[1][g]), cm[h][g]));
-                }
-              }
+            for (int g = 0; g < NGV; ++g) {
+              const uint32_t y0 = __float_as_uint(fmaf(p[0] * __low2float(z[0][g]), Sv, kMagicV));
+              const uint32_t y1 = __float_as_uint(fmaf(p[1] * __low2float(z[1][g]), Sv, kMagicV));
+              unsigned char* rowb = fragVb + g * 4 * RS * 4 + vboff;
+              *reinterpret_cast<unsigned short*>(rowb) = (unsigned short)__byte_perm(y0, y1, 0x0040);
+              *reinterpret_cast<unsigned short*>(rowb + RS * 4) = (unsigned short)__byte_perm(y0, y1, 0x0051);
+              *reinterpret_cast<unsigned short*>(rowb + 2 * RS * 4) = (unsigned short)__byte_perm(y0, y1, 0x0062);
+              cm[g] = fmaf(p[0], __high2float(z[0][g]), fmaf(p[1], __high2float(z[1][g]), cm[g]));
             }
             if (k2v > 0) {                                  // sparse value term of the two tokens, scattered in fixed point
 #pragma unroll
@@ -916,9 +819,7 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
                 const int tk = tp + e2;
                 auto v_entry = [&](int g, float val, int idx) {
                   const float d = (val - __high2float(z[e2][g])) * Sx;
-#pragma unroll
-                  for (int h = 0; h < HP; ++h)
-                    if (h < HC) atomicAdd(&corr_v[h * kHeadDim + g * GV + idx], __float2int_rn(p[h][e2] * lag[h] * d));
+                  atomicAdd(&corr_v[g * GV + idx], __float2int_rn(p[e2] * lag * d));
                 };
                 if (NGV * k2v == 4) {
                   const uint2 ov = reinterpret_cast<const uint2*>(vp + o_voval)[tk];
@@ -938,9 +839,7 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
               }
             }
           }
-#pragma unroll
-          for (int h = 0; h < HP; ++h)
-            if (h < HC) l_run[h] = fmaf(l_run[h], alpha[h], l[h]);
+          l_run[0] = fmaf(l_run[0], alpha, l);
           __syncwarp();
 
           // ---------------- values: out += sum_tok (p * scale) * code on the integer tensor cores, low rank on the side
@@ -952,15 +851,12 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
             const int av_step = kSlab * r_pad;
 #pragma unroll (S::unroll)
             for (int ck = 0; ck < nchunk; ++ck) {
-              uint32_t bV[NGV][NT][2];
+              uint32_t bV[NGV][2];
 #pragma unroll
-              for (int g = 0; g < NGV; ++g)
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
-                  const int hcol = HP == 1 ? 0 : 2 * nt + (gid >> 2);
-                  const uint2 v = *reinterpret_cast<const uint2*>(xr + ((g * HP + hcol) * 4 + limb_b) * RS + ck * 8 + 2 * t);
-                  bV[g][nt][0] = v.x; bV[g][nt][1] = v.y;
-                }
+              for (int g = 0; g < NGV; ++g) {
+                const uint2 v = *reinterpret_cast<const uint2*>(xr + (g * 4 + limb_b) * RS + ck * 8 + 2 * t);
+                bV[g][0] = v.x; bV[g][1] = v.y;
+              }
 #pragma unroll
               for (int tau = 0; tau < VT; ++tau) {
                 const uint4 w = cwp[tau * 32];
@@ -970,8 +866,7 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
                   const uint32_t m = m0 << (BITS * j);
                   const int mt = F * tau + j, g = (mt * 16) / GV;
                   const uint32_t af[4] = {w.x & m, w.y & m, w.z & m, w.w & m};
-#pragma unroll
-                  for (int nt = 0; nt < NT; ++nt) imma16832_u(O[mt][nt], af, bV[g][nt][0], bV[g][nt][1]);
+                  imma16832_u(O[mt], af, bV[g][0], bV[g][1]);
                 }
               }
               cwp += VT * 32;
@@ -1002,41 +897,35 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
 
           // ---------------- sparse value term: the fixed-point sums of this block join the fp32 copy
           if (k2v > 0) {
-#pragma unroll
-            for (int h = 0; h < HP; ++h) {
-              if (h < HC) {
-                const float Si = 1.0f / (Sx * lag[h]);
-                int4* cv = reinterpret_cast<int4*>(corr_v + h * kHeadDim) + lane;
-                float4* oc = reinterpret_cast<float4*>(ocorr + h * kHeadDim) + lane;
-                const int4 v = *cv;
-                *cv = make_int4(0, 0, 0, 0);
-                float4 o = *oc;
-                o.x = fmaf((float)v.x, Si, o.x);
-                o.y = fmaf((float)v.y, Si, o.y);
-                o.z = fmaf((float)v.z, Si, o.z);
-                o.w = fmaf((float)v.w, Si, o.w);
-                *oc = o;
-              }
-            }
+            const float Si = 1.0f / (Sx * lag);
+            int4* cv = reinterpret_cast<int4*>(corr_v) + lane;
+            float4* oc = reinterpret_cast<float4*>(ocorr) + lane;
+            const int4 v = *cv;
+            *cv = make_int4(0, 0, 0, 0);
+            float4 o = *oc;
+            o.x = fmaf((float)v.x, Si, o.x);
+            o.y = fmaf((float)v.y, Si, o.y);
+            o.z = fmaf((float)v.z, Si, o.z);
+            o.w = fmaf((float)v.w, Si, o.w);
+            *oc = o;
             __syncwarp();
           }
 
           // ---------------- end of a segment (or of this warp's share of it): out += B_V U, into the fp32 copy
           if (with_bv && u_pending) {
             __syncwarp();
-            if (t < HP) {
-              wl[gid * WLS + t] = U[0] + U[1];
-              wl[(gid + 8) * WLS + t] = U[2] + U[3];
+            if (t == 0) {
+              wl[gid] = U[0] + U[1];
+              wl[gid + 8] = U[2] + U[3];
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) U[i] = 0.f;
             __syncwarp();
             uint32_t bu[2];
             {
-              const int h = (gid >> 1) & (HP - 1);
               uint32_t hi0, lo0, hi1, lo1;
-              split_hi_lo(wl[(2 * t) * WLS + h], wl[(2 * t + 1) * WLS + h], hi0, lo0);
-              split_hi_lo(wl[(2 * t + 8) * WLS + h], wl[(2 * t + 9) * WLS + h], hi1, lo1);
+              split_hi_lo(wl[2 * t], wl[2 * t + 1], hi0, lo0);
+              split_hi_lo(wl[2 * t + 8], wl[2 * t + 9], hi1, lo1);
               bu[0] = (gid & 1) ? lo0 : hi0;
               bu[1] = (gid & 1) ? lo1 : hi1;
             }
@@ -1055,8 +944,8 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
               }
               float d[4];
               mma16816_z(d, aa, bu[0], bu[1]);
-              if (t < HC) {                              // columns 2t, 2t + 1: high and low part of head t
-                float* oc = ocorr + t * kHeadDim + 16 * mt + gid;
+              if (t == 0) {                              // columns 0, 1: high and low part
+                float* oc = ocorr + 16 * mt + gid;
                 oc[0] += d[0] + d[1];
                 oc[8] += d[2] + d[3];
               }
@@ -1077,28 +966,20 @@ __global__ void __launch_bounds__(JOIN ? 512 : 32, JOIN ? 1 : MINB) gear_decode_
       if (!alive) break;
       // the integer sums and the zero-point side sums join the fp32 copy
       {
-        float one[HP];
-#pragma unroll
-        for (int h = 0; h < HP; ++h) one[h] = 1.f;
-        if (tok_acc > 0) fold_O(one);
+        if (tok_acc > 0) fold_O(1.f);
         __syncwarp();
+        float add = 0.f;
 #pragma unroll
-        for (int h = 0; h < HP; ++h) {
-          if (h < HC) {
-            float add = 0.f;
+        for (int g = 0; g < NGV; ++g) {
+          float c = cm[g];
 #pragma unroll
-            for (int g = 0; g < NGV; ++g) {
-              float c = cm[h][g];
-#pragma unroll
-              for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-              if ((lane * 4) / GV == g) add = c;
-            }
-            float4* oc = reinterpret_cast<float4*>(ocorr + h * kHeadDim) + lane;
-            float4 v = *oc;
-            v.x += add; v.y += add; v.z += add; v.w += add;
-            *oc = v;
-          }
+          for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+          if ((lane * 4) / GV == g) add = c;
         }
+        float4* oc = reinterpret_cast<float4*>(ocorr) + lane;
+        float4 v = *oc;
+        v.x += add; v.y += add; v.z += add; v.w += add;
+        *oc = v;
         __syncwarp();
       }
     }
