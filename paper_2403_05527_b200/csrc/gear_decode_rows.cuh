@@ -9,9 +9,10 @@
 //   D  values          16-channel tiles by warp, all rows; outlier entries by thread; low-rank sums by slab
 // with a CTA barrier after A, B and C (D runs on into A of the next block).  One warp per CTA doing all of it for four rows
 // (the kernel this one replaced) needs 248 registers and 31 KB per warp: seven warps per SM, which issue on 39 % of the
-// cycles; sixteen warps here issue on 50 to 60 %.  Grouped queries over 32k tokens (four rows, 118 MB): 75 -> 63 us.
-// Sixteen rows: two passes of eight rows here (54 us over 8k tokens, 22 MB), four passes of four before (58 us), one pass of
-// sixteen rows with eight warps per CTA 72 us (spills, two CTAs per SM).  Rows cost about 260 instructions per warp and
+// cycles; sixteen warps here issue on 55 %.  Grouped queries over 32k tokens (four rows, 118 MB): 75 -> 63 us.
+// Sixteen rows over 8k tokens (22 MB): four passes of four rows 48 us (58 in the kernel before), two of eight 54, one pass of
+// sixteen rows with eight warps per CTA 72 us (spills, two CTAs per SM); eight rows pay over longer caches (rows_per_pass in
+// gear_api.cu).  Rows cost about 260 instructions per warp and
 // block each, half of them for the outlier entries (a product, a conversion and a shared-memory add per entry and row).
 //
 // Columns of the integer B operands: a pair of 8-column tiles carries four rows, limbs 0 and 1 of row 4 u + t in columns
