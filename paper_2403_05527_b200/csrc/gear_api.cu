@@ -323,7 +323,12 @@ static bool scratch_zeroed(gear_cache* c, cudaStream_t st) {
 // groups of 64 and 128, 2 and 4 bits): below 2 0.48 to 1.04, 6 to 8 0.87 to 1.06, 10 to 12 0.98 to 1.12, above 12 1.03 to 1.15;
 // with the last pass half empty 1.02 at most.  16 rows, 2 bits, groups of 64, 4096 tokens, us for fours and eights: 8 heads 18.9 / 27.1, 16
 // 28.8 / 32.6, 32 51.7 / 50.5, 128 166.6 / 153.7; 12 rows, 32 heads x 16384 124 / 148.
+// Two rows go one at a time through the kernel of one row where the ranges are long: the fours' kernel does most of its work for
+// rows that are absent then (us for four and one at a time, blocks per SM: 2 bits, groups of 64 110 85.8 / 61.7, 55 47.9 / 36.8,
+// 28 29.4 / 27.0 and 33.2 / 28.4, 14 21.0 / 23.3; groups of 128 55 62.2 / 56.2; 4 bits 110 85.5 / 73.7, 28 32.8 / 35.7; groups
+// of 32 110 117.1 / 94.3, but of 16, with eight value scales a token, 126 / 157).
 static int rows_per_pass(const gear_cache* c, int G, long long nb) {
+  if (G == 2 && c->cc.ngv <= 4 && c->cc.BH * nb >= 40LL * c->sm_count) return 1;
   if (G <= 4) return G == 1 ? 1 : 4;
   if (decode_passes(G, 4) % 2) return 4;
   return c->cc.BH * nb * decode_passes(G, 8) >= 10LL * c->sm_count * kRowsCtasPerSm ? 8 : 4;
@@ -333,7 +338,7 @@ static int rows_per_pass(const gear_cache* c, int G, long long nb) {
 // the first and the last of which may be shared with its neighbours), and the bytes of all slots.
 static int partial_slots(const gear_cache* c, int G, int hp) {
   const size_t units = (size_t)c->cc.BH * decode_passes(G, hp);
-  const size_t ctas = (size_t)c->sm_count * (G == 1 ? 32 : kRowsCtasPerSm);
+  const size_t ctas = (size_t)c->sm_count * (hp == 1 ? 32 : kRowsCtasPerSm);
   return (int)(ctas / units + 3);
 }
 static size_t partial_bytes_for(const gear_cache* c, int G, int hp) {
@@ -419,7 +424,8 @@ extern "C" gear_status gear_create(gear_cache** out, const gear_config* cfg) {
   c->units_alloc = 0; c->partial_bytes = 0;
   for (int nq = 1; nq <= c->max_queries; ++nq) {
     const int G = c->G * nq;
-    for (int hp = G == 1 ? 1 : 4; hp <= (G > 4 ? 8 : G == 1 ? 1 : 4); hp += 4) {
+    for (int hp : {1, 4, 8}) {
+      if (hp == 1 ? G > 2 : hp == 4 ? G == 1 : G <= 4) continue;          // what rows_per_pass may return
       const size_t n = partial_bytes_for(c, G, hp);
       if (n > c->partial_bytes) c->partial_bytes = n;
       const int un = (int)(BH * decode_passes(G, hp));
@@ -589,13 +595,13 @@ static gear_status plan_decode(gear_cache* c, int Gq, int hp) {
   // long streams run with twelve resident warps.  Short streams (few blocks per warp) keep sixteen: there the
   // fixed cost per warp and the granularity of the split weigh more.
   int warps_cap = 0;
-  if (Gq == 1) {
-    const long long blocks = (long long)c->cc.BH * (c->n_blocks_c + (c->buf_len + 15) / 16);
+  if (hp == 1) {
+    const long long blocks = (long long)c->cc.BH * Gq * (c->n_blocks_c + (c->buf_len + 15) / 16);
     if (blocks >= 24LL * 16 * c->sm_count) warps_cap = 12;
   }
   // everything else the plan depends on is fixed by the segments: a push that does not flush keeps it (asking the driver
   // for the occupancy again costs a microsecond and a half per decoding step)
-  const long long key = ((long long)c->segs.size() * 4096 + Gq) * 2 + (warps_cap || hp == 8 ? 1 : 0);
+  const long long key = (((long long)c->segs.size() * 8192 + Gq) * 2 + (warps_cap ? 1 : 0)) * 16 + hp;
   if (c->plan_key == key) return GEAR_OK;
   int max_k = 0, max_v = 0, max_bfac = 0, max_T = 16;
   for (const SegDesc& s : c->segs) {
@@ -604,12 +610,12 @@ static gear_status plan_decode(gear_cache* c, int Gq, int hp) {
     if (s.bfac_bytes > max_bfac) max_bfac = s.bfac_bytes;
     if ((s.T + 31) / 32 * 32 > max_T) max_T = (s.T + 31) / 32 * 32;
   }
-  if (Gq == 1 ? !decode_plan(c->cc.bits, Gq, c->cc.ngv, max_k, max_v, max_bfac, max_T, kDecodeSmemBudget, warps_cap, &c->plan)
+  if (hp == 1 ? !decode_plan(c->cc.bits, hp, c->cc.ngv, max_k, max_v, max_bfac, max_T, kDecodeSmemBudget, warps_cap, &c->plan)
               : !rows_plan(hp, c->cc.ngv, max_k, max_v, max_bfac, max_T, &c->plan))
     return GEAR_ERR_SHAPE;
-  int occ = Gq == 1 ? decode_occupancy(c->cc.bits, Gq, c->cc.ngv, c->plan.wide, (size_t)c->plan.ws.total)
+  int occ = hp == 1 ? decode_occupancy(c->cc.bits, hp, c->cc.ngv, c->plan.wide, (size_t)c->plan.ws.total)
                     : rows_occupancy(c->plan, c->cc.bits, c->cc.ngv);
-  if (Gq > 1 && occ > kRowsCtasPerSm) occ = kRowsCtasPerSm;      // what the partial slots are for
+  if (hp > 1 && occ > kRowsCtasPerSm) occ = kRowsCtasPerSm;      // what the partial slots are for
   if (occ < 1) return GEAR_ERR_CUDA;
   c->plan_occ = occ;
   c->plan_key = key;
@@ -622,9 +628,9 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
   if (((uintptr_t)q | (uintptr_t)out) & 15) return GEAR_ERR_ALIGN;
   if (c->n_compressed == 0 && c->buf_len == 0) return GEAR_ERR_STATE;
   note_stream(c, (cudaStream_t)stream);
-  const int buf_block = Gq == 1 ? 16 : kRowsBufBlock;
+  const int hp = rows_per_pass(c, Gq, c->n_blocks_c), passes = decode_passes(Gq, hp);
+  const int buf_block = hp == 1 ? 16 : kRowsBufBlock;
   const long long nblocks = c->n_blocks_c + (c->buf_len + buf_block - 1) / buf_block;
-  const int hp = rows_per_pass(c, Gq, nblocks), passes = decode_passes(Gq, hp);
   gear_status s = plan_decode(c, Gq, hp);
   if (s != GEAR_OK) return s;
   DecodeArgs a = c->plan;
@@ -706,7 +712,7 @@ static gear_status decode_rows(gear_cache* c, const void* q, float* out, int Gq,
       grid = start;                                                     // = units * pb + ua
     }
   }
-  if ((Gq == 1 ? launch_decode(a, (int)grid, (cudaStream_t)stream) : launch_rows(a, (int)grid, (cudaStream_t)stream)) != cudaSuccess) {
+  if ((hp == 1 ? launch_decode(a, (int)grid, (cudaStream_t)stream) : launch_rows(a, (int)grid, (cudaStream_t)stream)) != cudaSuccess) {
     cudaGetLastError();
     return GEAR_ERR_CUDA;
   }

@@ -1256,7 +1256,7 @@ static bool with_decode_kernel(int bits, int heads, int ngv, int wide, bool join
 cudaError_t launch_decode(const DecodeArgs& a, int grid, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   const size_t smem = (size_t)a.ws.total;
-  const bool ok = with_decode_kernel(a.cc.bits, a.group_heads, a.cc.ngv, a.wide, a.unit_ctas > 0, [&](auto kern) {
+  const bool ok = with_decode_kernel(a.cc.bits, a.hpa, a.cc.ngv, a.wide, a.unit_ctas > 0, [&](auto kern) {
     // Programmatic dependent launch: the CTAs of this launch may become resident while the kernel before it on the
     // stream drains (the kernel below announces that at once, and waits for its predecessor before its first read of
     // global memory), so that back-to-back decode calls do not pay the launch ramp one after the other.

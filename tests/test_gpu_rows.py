@@ -168,3 +168,46 @@ def test_rows_in_eights_against_rows_in_fours(hkv, bits, group, s, rank, n, rows
         assert G.gear_last_device_status(cache) == 0
     finally:
         G.gear_free(cache)
+
+
+@pytest.mark.parametrize("hkv,group_heads,bits,group,s,rank,n", [
+    (32, 1, 2, 64, 2.0, 4, 12032),       # 188 blocks per unit, two passes of one row
+    (32, 2, 4, 64, 1.0, 8, 12032),       # two query heads per kv head instead of two positions
+    (30, 2, 2, 128, 2.0, 4, 26624),
+    (48, 1, 4, 0, 2.0, 4, 8192),         # per-vector lists
+    (24, 2, 4, 16, 6.0, 2, 4096),        # groups of 16 keep their kernel
+    (64, 1, 2, 32, 0.0, 0, 3072),
+])
+def test_two_rows_over_long_caches(hkv, group_heads, bits, group, s, rank, n):
+    """Two rows per kv head take the kernel of one row twice once the cache is long.  Each has to be what it is alone (a second
+    cache with one query head per kv head), before and after the line."""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").half()   # noqa: E731
+    rows = 2 // group_heads
+    nb = 64 if group != 0 else 20
+    cfg = lambda heads, most: G.make_config(1, hkv * heads, hkv, bits, group, s, nb, min(rank, nb), n + nb,   # noqa: E731
+                                            rank_max=rank, seed=1, max_queries=most)
+    k, v, q, tail = draw(1, hkv, n, 128), draw(1, hkv, n, 128), draw(1, hkv, 2, 128), draw(7, 2, 1, hkv, 128)
+    both, single = G.gear_create(cfg(group_heads, rows)), G.gear_create(cfg(1, 1))
+    try:
+        first = n // 8 // 128 * 128
+        for lo, hi in ((0, first), (first, n)):
+            part = k[:, :, lo:hi].contiguous(), v[:, :, lo:hi].contiguous()
+            for cache in (both, single):
+                G.gear_compress(cache, None, *part, hi - lo, rank)
+                for t in tail if hi == n else ():
+                    G.gear_append_buffer(cache, t[0], t[1])
+            got = torch.full(q.shape, float("nan"), device="cuda")
+            for _ in range(2):
+                G.gear_decode_attn_multi(both, q, got, rows)
+            want = torch.empty((1, hkv, 128), device="cuda")
+            for r in range(2):
+                G.gear_decode_attn(single, q[:, :, r].contiguous(), want)
+                err = (got[:, :, r] - want).abs().amax(-1) / want.abs().amax(-1)
+                assert err.max().item() <= 8e-5          # twice what a kernel's own arithmetic may be off
+        assert G.gear_last_device_status(both) == 0
+    finally:
+        G.gear_free(both)
+        G.gear_free(single)
