@@ -55,3 +55,42 @@ def test_steps_queued_beyond_the_ring_match_the_device_calls(where, B, Hq, H, nb
         G.gear_free(cache)
     G.gear_free(ref)
     G.gear_release_workspace()
+
+
+def test_steps_captured_into_a_graph_match_the_eager_calls():
+    """Pushes and attentions of two caches captured token after token: what may be read ahead of the kernel in front is decided
+    inside the capture, and the replay gives the bits of the same calls made one by one, flushes among them."""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+
+    B, Hq, H, nb, steps = 2, 8, 4, 16, 20
+    k, v, q = (t.cuda() for t in _rows(torch, steps, B, H, Hq))
+    eager, graphed = ([_cache(torch, G, B, Hq, H, nb) for _ in range(2)] for _ in range(2))
+    want, got = (torch.full((steps, 2, B, Hq, 128), float("nan"), device="cuda") for _ in range(2))
+
+    def run(caches, out):
+        for i in range(steps):
+            for j, c in enumerate(caches):
+                G.gear_append_buffer(c, k[i], v[i])
+                G.gear_decode_attn(c, q[i], out[i, j])
+            for j, c in enumerate(caches):               # each behind a call on the other cache
+                G.gear_decode_attn(c, q[i], out[i, j])
+
+    run(eager, want)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run(graphed, got)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(got, want)
+    # and the caches go on outside the graph
+    a, b = torch.empty((B, Hq, 128), device="cuda"), torch.empty((B, Hq, 128), device="cuda")
+    for c, out in ((eager[0], a), (graphed[0], b)):
+        G.gear_append_buffer(c, k[0], v[0])
+        G.gear_decode_attn(c, q[0], out)
+    torch.cuda.synchronize()
+    assert torch.equal(a, b) and all(G.gear_last_device_status(c) == 0 for c in eager + graphed)
+    del graph
+    for c in eager + graphed:
+        G.gear_free(c)
