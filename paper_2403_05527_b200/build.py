@@ -16,7 +16,7 @@ LIB = os.path.join(HERE, "libgear_b200.so")
 STAMP = os.path.join(HERE, "libgear_b200.stamp")
 SOURCES = ["gear_api.cu", "gear_compress.cu", "gear_decode.cu", "gear_decode_rows.cu",
            "gear_decode_rows_b2.cu", "gear_decode_rows_b4.cu", "gear_export.cu", "gear_fp16_attn.cu",
-           "gear_gram.cu", "gear_kcvt.cu"]
+           "gear_gram.cu", "gear_kcvt.cu", "gear_pass_codes.cu", "gear_quant_gram.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
               "-Xcompiler", "-fPIC", "--threads", "0"]
 

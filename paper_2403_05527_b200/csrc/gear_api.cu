@@ -496,13 +496,12 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
     // Bounded transient workspace, (batch, head) pairs processed in ranges.  Flushes of buffers too long for one launch take it
     // from the pool like prompts: held by every cache it was 235 MB for 256 pairs of 256 tokens at rank 4, 7.5 GB for 32 layers.
     // (Kept small by ranges instead, 88 MB, such a flush took 350 us and not 235, of 64 pairs 365 and not 110.)
-    const int csr_k = per_vector ? sd.csr_k : -1;
     const size_t budget = (size_t)3 << 30;
-    auto bytes_of = [&](int nbh) { return compress_workspace_bytes(nbh, n, rank, c->sm_count, csr_k); };
+    auto bytes_of = [&](int nbh) { return compress_workspace_bytes(nbh, sd, c->cc, c->sm_count); };
     int ranges = 1, chunk = c->cc.BH;
     while (chunk > 1 && bytes_of(chunk) > budget) chunk = (c->cc.BH + ++ranges - 1) / ranges;      // equal ranges
     unsigned char* ws = nullptr;
-    const size_t ws_bytes = compress_workspace_bytes(chunk, n, rank, c->sm_count, csr_k);
+    const size_t ws_bytes = bytes_of(chunk);
     cudaMemPool_t pool = workspace_pool(c->device);
     if (pool == nullptr || cudaMallocFromPoolAsync((void**)&ws, ws_bytes, pool, st) != cudaSuccess) {
       cudaGetLastError();

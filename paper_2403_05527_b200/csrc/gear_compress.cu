@@ -9,6 +9,7 @@
 #include <string.h>
 
 #include "gear_internal.cuh"
+#include "gear_pass.cuh"
 #include "gear_pi.cuh"
 #include "gear_quant.cuh"
 
@@ -309,21 +310,6 @@ struct BlockFeed {
   }
 };
 
-// Entry of the first set bit of L mask bits: bit t of the low / high half of word w stands for entry 2 (16 w + t) / that + 1 of
-// a group whose pairs are rotated by `turn` (a multiple of four).  An entry of the group also if no bit is set (all NaN).
-template <int L>
-__device__ __forceinline__ int first_set(const unsigned int (&m)[4], int turn) {
-  auto first = [&](unsigned int sel) {
-    const unsigned int lo = __byte_perm(m[0], m[L == 32 ? 0 : 1], sel);            // 32 entries: their 16 bits twice
-    if (L <= 64) return __ffs((int)__funnelshift_l(lo, lo, turn)) - 1;
-    const unsigned int hi = __byte_perm(m[2], m[3], sel);
-    const unsigned int l = __funnelshift_l(hi, lo, turn), h = __funnelshift_l(lo, hi, turn);
-    return l ? __ffs((int)l) - 1 : h ? 32 + __ffs((int)h) - 1 : -1;
-  };
-  const int even = first(0x5410), odd = first(0x7632);
-  return min(L - 1, min(even < 0 ? L : 2 * even, odd < 0 ? L : 2 * odd + 1));
-}
-
 template <int BITS, int SIDE, int L, int K>
 __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_kernel(CompressArgs p, int nbh) {
   constexpr int F = 8 / BITS, side = SIDE, kGroups = kHeadDim / L, kPieces = L / 8;
@@ -373,43 +359,9 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
         xp[4 * q + 3] = *reinterpret_cast<const __half2*>(&v.w);
       }
     }
-    // Filter_s (Eq. 4), one entry per side: the largest and the smallest entry leave the group, the second largest and
-    // second smallest instances bound what is kept (no outliers: the largest and the smallest).  Comparisons of fp16 values
-    // are exact in fp16, so the search runs on the packed pairs: even and odd entries keep their own two largest / smallest
-    // and are merged at the end.
     float mx, mn;
-    int imax = 0, imin = 1;
-    {
-      const __half2 ninf = __float2half2_rn(-INFINITY), pinf = __float2half2_rn(INFINITY);
-      __half2 M1 = ninf, M2 = ninf, m1 = pinf, m2 = pinf;
-#pragma unroll
-      for (int q = 0; q < L / 2; ++q) {
-        if (K == 1) {
-          M2 = __hmax2(M2, __hmin2(xp[q], M1));
-          m2 = __hmin2(m2, __hmax2(xp[q], m1));
-        }
-        M1 = __hmax2(M1, xp[q]);
-        m1 = __hmin2(m1, xp[q]);
-      }
-      const float2 fM1 = __half22float2(M1), fM2 = __half22float2(M2), fm1 = __half22float2(m1), fm2 = __half22float2(m2);
-      const float max1 = fmaxf(fM1.x, fM1.y), min1 = fminf(fm1.x, fm1.y);
-      mx = K == 0 ? max1 : fmaxf(fminf(fM1.x, fM1.y), fmaxf(fM2.x, fM2.y));
-      mn = K == 0 ? min1 : fminf(fmaxf(fm1.x, fm1.y), fminf(fm2.x, fm2.y));
-      // first index of the maximum and of the minimum (ties go to the lower index): one mask bit per entry
-      if (K == 1) {
-        const __half2 vM = __float2half2_rn(max1), vm = __float2half2_rn(min1);
-        unsigned int a[4] = {0u, 0u, 0u, 0u}, b[4] = {0u, 0u, 0u, 0u};   // bit t of a half of word w: pair 16 w + t
-#pragma unroll
-        for (int q = 0; q < L / 2; ++q) {
-          const unsigned int bit = 0x00010001u << (q & 15);
-          a[q >> 4] |= __heq2_mask(xp[q], vM) & bit;
-          b[q >> 4] |= __heq2_mask(xp[q], vm) & bit;
-        }
-        imax = first_set<L>(a, 4 * rot);
-        imin = first_set<L>(b, 4 * rot);
-        if (imin == imax) imin = 1;           // all entries equal: the bottom entry is the next index
-      }
-    }
+    int imax, imin;
+    filter_one<L, K>(xp, 4 * rot, mn, mx, imax, imin);
     // Eq. 2 on the kept entries: binary32, one rounding per operation
     const float levels = (float)((1 << BITS) - 1);
     const float range = __fsub_rn(mx, mn);
@@ -834,20 +786,10 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
 // R_h [n_c, 128] in the workspace.  Factor buffers are [128][16] fp32, zero
 // beyond the rank.
 // ---------------------------------------------------------------------------
-// ---- helpers of the tensor-core pass
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-constexpr int kChunkRows = 512;
-constexpr int kPassWarps = 4;
 constexpr int kPassPitch = kHeadDim * 4 + 16;    // bytes per residual row in shared memory (the lanes' 128-bit reads of two rows hit different banks)
 constexpr int kPassStage = 16 * kPassPitch;      // the 16 rows a warp takes at a time
 constexpr int kPassStages = 2;
 constexpr int kPassSmem = kPassWarps * kPassStages * kPassStage;
-constexpr int kRtaParts = 4;
 
 // The last loop's pass over the residual: the rows A0 = R b, stored, and this chunk's part of A0^T A0.  The loops before it
 // run on R^T R alone (gear_gram.cu), which also gives R^T A0 = (R^T R) b, so this is the only product of the residual
@@ -865,11 +807,8 @@ constexpr int kRtaParts = 4;
 // remainder each) per tile.
 template <int NT>
 __global__ void __launch_bounds__(kPassWarps * 32, 3) pi_pass_kernel(PiArgs p) {
-  constexpr int RP = 4 * NT;                       // rank columns: each gives a (head, remainder) column pair of n
-  constexpr bool kGram = NT <= 2;                  // A0^T A0 here (in registers), else by pi_gram2_kernel
-  __shared__ __align__(16) __half bsplit[2 * RP][kHeadDim];   // [2 rho + (0: head, 1: remainder)][channel]
-  __shared__ float colmax[kPassWarps][RP];
-  __shared__ float gred[kGram ? kPassWarps : 1][RP][RP];
+  constexpr int RP = 4 * NT;
+  __shared__ typename PassFactor<NT>::Shared sh;
   __shared__ uint64_t full[kPassWarps][kPassStages];
   extern __shared__ __align__(128) unsigned char ring_all[];
   const int tile = blockIdx.y, chunk = blockIdx.x;
@@ -898,56 +837,19 @@ __global__ void __launch_bounds__(kPassWarps * 32, 3) pi_pass_kernel(PiArgs p) {
 #pragma unroll
   for (int s = 0; s < kPassStages; ++s) request(row0 + (s * kPassWarps + warp) * 16, s);
 
-  // ---- the scaled, split factor columns
   const int er = pow2_exponent(__uint_as_float(p.Rmax[tile]));
   const float sr = exp2_int(-er);
-  int eb[RP];
-  {
-    const int j = threadIdx.x;                     // one channel per thread (kPassWarps * 32 == kHeadDim)
-    float bj[RP];
-#pragma unroll
-    for (int r = 0; r < RP; ++r) {
-      bj[r] = p.Bcur[((size_t)tile * kHeadDim + j) * kMaxRank + r];
-      const float m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fabsf(bj[r]))));
-      if (lane == 0) colmax[warp][r] = m;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < RP; ++r) {
-      float m = 0.f;
-#pragma unroll
-      for (int w = 0; w < kPassWarps; ++w) m = fmaxf(m, colmax[w][r]);
-      eb[r] = pow2_exponent(m);
-      const float v = bj[r] * exp2_int(-eb[r]);
-      const __half h = __float2half_rn(v);
-      bsplit[2 * r][j] = h;
-      bsplit[2 * r + 1][j] = __float2half_rn(v - __half2float(h));
-    }
-    __syncthreads();
-  }
+  PassFactor<NT> factor;
+  factor.load(p, tile, er, sh);
   // B fragments of a = R b: column n = gid of tile nt is (rho = 4 nt + gid / 2, head | remainder), k as described above
   uint32_t bf[8][NT][2];
 #pragma unroll
   for (int c = 0; c < 8; ++c)
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
-      const uint2 v = *reinterpret_cast<const uint2*>(&bsplit[8 * nt + gid][16 * c + 4 * t]);
+      const uint2 v = *reinterpret_cast<const uint2*>(&sh.bsplit[8 * nt + gid][16 * c + 4 * t]);
       bf[c][nt][0] = v.x; bf[c][nt][1] = v.y;
     }
-  float inv_a[NT];                                 // back to a for column rho = 4 nt + t
-#pragma unroll
-  for (int nt = 0; nt < NT; ++nt) {
-    int ebt = eb[4 * nt];
-#pragma unroll
-    for (int q = 1; q < 4; ++q) ebt = t == q ? eb[4 * nt + q] : ebt;
-    inv_a[nt] = exp2_int(er + ebt);
-  }
-  float gram[kGram ? NT : 1][kGram ? RP : 1];      // gram[nt][v]: row rho = 4 nt + t of A0^T A0, column v
-#pragma unroll
-  for (int nt = 0; nt < (kGram ? NT : 1); ++nt)
-#pragma unroll
-    for (int v = 0; v < (kGram ? RP : 1); ++v) gram[nt][v] = 0.f;
-
   int stage = 0;
   uint32_t parity = 0;
   for (int rb = row0 + warp * 16; rb < row1; rb += kPassWarps * 16) {
@@ -977,53 +879,17 @@ __global__ void __launch_bounds__(kPassWarps * 32, 3) pi_pass_kernel(PiArgs p) {
       split_pair(b.z * sr, b.w * sr, fh[3], fl[3]);
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
-        mma16816(d[nt], fh, bf[c][nt][0], bf[c][nt][1]);
-        mma16816(d[nt], fl, bf[c][nt][0], bf[c][nt][1]);
+        mma16816_f16(d[nt], fh, bf[c][nt][0], bf[c][nt][1]);
+        mma16816_f16(d[nt], fl, bf[c][nt][0], bf[c][nt][1]);
       }
     }
     const int used = stage;
     if (++stage == kPassStages) { stage = 0; parity ^= 1; }
-    float mine[2][NT];                             // a[row gid | gid + 8][rho 4 nt + t]; rows past the chunk are zero
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      mine[0][nt] = (d[nt][0] + d[nt][1]) * inv_a[nt];
-      mine[1][nt] = (d[nt][2] + d[nt][3]) * inv_a[nt];
-      if (va) A0[(size_t)ra * RP + 4 * nt + t] = mine[0][nt];
-      if (vc) A0[(size_t)rc * RP + 4 * nt + t] = mine[1][nt];
-    }
+    factor.store(d, A0, ra, rc, va, vc);           // rows past the chunk are zero
     request(rb + kPassStages * kPassWarps * 16, used);             // behind stores that need every load from the stage
-    if (kGram) {
-#pragma unroll
-      for (int half = 0; half < 2; ++half)
-#pragma unroll
-        for (int nv = 0; nv < NT; ++nv)
-#pragma unroll
-          for (int tv = 0; tv < 4; ++tv) {
-            const float other = __shfl_sync(0xffffffffu, mine[half][nv], (lane & ~3) | tv);   // a[row][4 nv + tv]
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-              gram[kGram ? nt : 0][kGram ? 4 * nv + tv : 0] = fmaf(mine[half][nt], other, gram[kGram ? nt : 0][kGram ? 4 * nv + tv : 0]);
-          }
-    }
+    factor.add_gram();
   }
-  if (kGram) {                                     // rows of the warp (over gid), then the warps, in a fixed order
-#pragma unroll
-    for (int nt = 0; nt < (kGram ? NT : 1); ++nt)
-#pragma unroll
-      for (int v = 0; v < (kGram ? RP : 1); ++v) {
-        float g = gram[nt][v];
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
-        if (gid == 0) gred[kGram ? warp : 0][4 * nt + t][v] = g;
-      }
-    __syncthreads();
-    for (int i = threadIdx.x; i < RP * RP; i += blockDim.x) {
-      const int u = i / RP, v = i % RP;
-      float g = 0.f;
-      for (int w = 0; w < kPassWarps; ++w) g += gred[kGram ? w : 0][u][v];
-      p.Gp[((size_t)tile * p.nchunk + chunk) * 256 + u * kMaxRank + v] = g;
-    }
-  }
+  factor.leave_gram(p, tile, chunk, sh);
 }
 
 // R^T A0 from the residual itself, for tiles whose factor columns differ so much in norm that (R^T R) b would lose digits
@@ -1065,6 +931,7 @@ template <int RP>
 __global__ void __launch_bounds__(256) pi_store_a_kernel(PiArgs p) {
   __shared__ __align__(16) float Wm[RP][RP];
   const int tile = blockIdx.y;
+  after_previous();
   for (int i = threadIdx.x; i < RP * RP; i += blockDim.x) Wm[i / RP][i % RP] = p.W[(size_t)tile * 256 + (i / RP) * kMaxRank + i % RP];
   __syncthreads();
   const int row = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1118,6 +985,7 @@ template <int RP>
 __global__ void __launch_bounds__(kHeadDim) pi_finish_kernel(PiArgs p) {
   __shared__ float Gm[RP][RP + 1], Wm[RP][RP + 1];
   const int tile = blockIdx.x, j = threadIdx.x, lane = j & 31, warp = j >> 5, r = p.rank;
+  after_previous();
   for (int e = j; e < r * r; e += kHeadDim) {
     const float* src = p.Gp + (size_t)tile * p.nchunk * 256 + (e / r) * kMaxRank + e % r;
     float s = 0.f;
@@ -1169,9 +1037,10 @@ __global__ void __launch_bounds__(256) pi_gram2_kernel(PiArgs p) {
   __shared__ float red[8][256];
   const int tile = blockIdx.y, chunk = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = p.rank, u0 = (lane >> 2) * 2, v0 = (lane & 3) * 4;
-  const int row0 = chunk * kChunkRows, row1 = min(p.n_c, row0 + kChunkRows);
+  const int row0 = chunk * p.chunk_rows, row1 = min(p.n_c, row0 + p.chunk_rows);
   const float4* A0 = reinterpret_cast<const float4*>(p.A0 + (size_t)tile * p.n_c * kMaxRank);
   float g[2][4] = {};
+  after_previous();
   for (int base = row0 + warp * 32; base < row1; base += 8 * 32) {
     const int row = base + lane;
 #pragma unroll
@@ -1648,13 +1517,19 @@ static cudaError_t launch_pass(const PiArgs& p, cudaStream_t st) {
 static int a0_columns(int rank) { return rank <= 4 ? 4 : (rank <= 8 ? 8 : kMaxRank); }   // of the A0 rows in the workspace
 
 // bytes of the power iteration's part of the workspace (a multiple of 256)
-static size_t pi_workspace_bytes(int nbh, int n_c, int rank, int sms) {
+static size_t pi_workspace_bytes(int nbh, const SegDesc& sd, const CacheConst& cc, int sms) {
+  const int rank = sd.rank, n_c = sd.n_c;
   if (rank == 0) return 256;
   const size_t ntiles = (size_t)nbh * 2;
-  const size_t nchunk = (n_c + kChunkRows - 1) / kChunkRows;
+  const size_t chunk_rows = pass_chunk_rows(nbh, sd, cc, sms), nchunk = (n_c + chunk_rows - 1) / chunk_rows;
   size_t b = 0;
-  b += ntiles * n_c * kHeadDim * 4;               // R
-  b += pi_gram_workspace_bytes((int)ntiles, n_c, sms);   // Gpart
+  if (qg_fits(sd, cc)) {
+    b += ntiles * kHeadDim * kHeadDim * 4;        // G
+    b += qg_partials(nbh, sd, sms) * (kHeadDim * kHeadDim + 1) * 4;    // Gpart, Gexp
+  } else {
+    b += ntiles * n_c * kHeadDim * 4;             // R
+    b += pi_gram_workspace_bytes((int)ntiles, n_c, sms);   // G, Gpart
+  }
   b += ntiles * kHeadDim * kMaxRank * 4;          // Bcur
   b += ntiles * kHeadDim * kMaxRank * 4;          // Bg
   b += ntiles * kRtaParts * kHeadDim * kMaxRank * 4;   // Bp
@@ -1665,26 +1540,33 @@ static size_t pi_workspace_bytes(int nbh, int n_c, int rank, int sms) {
   return (b + 1024 + 255) / 256 * 256;
 }
 
-// csr_k < 0: a segment with per-block key groups; otherwise one with per-vector keys and csr_k outliers per channel
-size_t compress_workspace_bytes(int nbh, int n_c, int rank, int sms, int csr_k) {
-  return pi_workspace_bytes(nbh, n_c, rank, sms) + (csr_k >= 0 ? kcvt_workspace_bytes(nbh, n_c, csr_k) : 0);
+size_t compress_workspace_bytes(int nbh, const SegDesc& sd, const CacheConst& cc, int sms) {
+  return pi_workspace_bytes(nbh, sd, cc, sms) + (sd.csr_base16 != 0 ? kcvt_workspace_bytes(nbh, sd.n_c, sd.csr_k) : 0);
 }
 
 cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned char* ws, cudaStream_t st) {
   const SegDesc& sd = job.seg;
   const size_t ntiles = (size_t)nbh * 2;
-  const int nchunk = (sd.n_c + kChunkRows - 1) / kChunkRows;
+  const int chunk_rows = pass_chunk_rows(nbh, sd, job.cc, job.sms), nchunk = (sd.n_c + chunk_rows - 1) / chunk_rows;
   float* wsf = reinterpret_cast<float*>(ws);
   PiArgs pa;
   pa.seg = sd; pa.arena = job.arena; pa.bh0 = bh0; pa.ntiles = (int)ntiles; pa.n_c = sd.n_c; pa.rank = sd.rank;
-  pa.nchunk = nchunk;
+  pa.nchunk = nchunk; pa.chunk_rows = chunk_rows;
   pa.status = job.status; pa.a0_pitch = a0_columns(sd.rank);
-  pa.R = nullptr; pa.Rmax = nullptr; pa.Gpart = nullptr; pa.G = nullptr; pa.Bcur = nullptr; pa.Bp = nullptr; pa.Bg = nullptr; pa.ill = nullptr; pa.A0 = nullptr; pa.Gp = nullptr; pa.W = nullptr;
+  pa.K = job.K + (size_t)bh0 * sd.n_c * kHeadDim; pa.V = job.V + (size_t)bh0 * sd.n_c * kHeadDim; pa.cc = job.cc;
+  pa.R = nullptr; pa.Rmax = nullptr; pa.Gpart = nullptr; pa.Gexp = nullptr; pa.G = nullptr; pa.Bcur = nullptr; pa.Bp = nullptr; pa.Bg = nullptr; pa.ill = nullptr; pa.A0 = nullptr; pa.Gp = nullptr; pa.W = nullptr;
   pa.dbgA = job.dbgA; pa.dbgB = job.dbgB;
+  const bool from_codes = qg_fits(sd, job.cc);         // the residual is not kept
   if (sd.rank > 0) {
-    pa.R = wsf;       wsf += ntiles * sd.n_c * kHeadDim;
-    pa.G = wsf;       pa.Gpart = wsf + ntiles * kHeadDim * kHeadDim;
-    wsf += pi_gram_workspace_bytes((int)ntiles, sd.n_c, job.sms) / 4;
+    if (from_codes) {
+      const size_t parts = qg_partials(nbh, sd, job.sms);
+      pa.G = wsf;     wsf += ntiles * kHeadDim * kHeadDim;
+      pa.Gpart = wsf; wsf += parts * kHeadDim * kHeadDim;
+    } else {
+      pa.R = wsf;     wsf += ntiles * sd.n_c * kHeadDim;
+      pa.G = wsf;     pa.Gpart = wsf + ntiles * kHeadDim * kHeadDim;
+      wsf += pi_gram_workspace_bytes((int)ntiles, sd.n_c, job.sms) / 4;
+    }
     pa.Bcur = wsf;    wsf += ntiles * kHeadDim * kMaxRank;
     pa.Bg = wsf;      wsf += ntiles * kHeadDim * kMaxRank;
     pa.Bp = wsf;      wsf += ntiles * kRtaParts * kHeadDim * kMaxRank;
@@ -1693,41 +1575,50 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
     pa.W = wsf;       wsf += ntiles * 256;
     pa.Rmax = reinterpret_cast<unsigned int*>(wsf);
     pa.ill = reinterpret_cast<int*>(wsf) + ntiles;
+    pa.Gexp = pa.ill + ntiles;
     if (cudaMemsetAsync(pa.Rmax, 0, ntiles * 4, st) != cudaSuccess) return cudaGetLastError();
   }
   CompressArgs ca;
   ca.seg = sd; ca.cc = job.cc; ca.arena = job.arena; ca.bh0 = bh0;
-  ca.K = job.K + (size_t)bh0 * sd.n_c * kHeadDim;
-  ca.V = job.V + (size_t)bh0 * sd.n_c * kHeadDim;
-  ca.R = pa.R; ca.Rmax = pa.Rmax; ca.status = job.status;
+  ca.K = pa.K; ca.V = pa.V;
+  ca.R = pa.R; ca.Rmax = pa.Rmax; ca.status = job.status; ca.Gpart = pa.Gpart; ca.Gexp = pa.Gexp;
   const int kneed = sd.k_k > job.cc.k_v ? sd.k_k : job.cc.k_v;
   const bool per_vector = sd.csr_base16 != 0;          // keys: one group per channel over the whole segment
   ca.side0 = per_vector ? 1 : 0;
-  int n_quant = 0;
-  cudaError_t e = job.cc.bits == 2 ? launch_quant<2>(ca, nbh, kneed, job.sms, st, &n_quant) : launch_quant<4>(ca, nbh, kneed, job.sms, st, &n_quant);
-  if (e != cudaSuccess) return e;
-  count_launches(n_quant);
-  if (per_vector) {
-    KcvtArgs ka;
-    ka.seg = sd; ka.arena = job.arena; ka.K = ca.K; ka.R = pa.R; ka.Rmax = pa.Rmax; ka.bh0 = bh0;
-    e = launch_kcvt_keys(ka, nbh, job.cc.bits, ws + pi_workspace_bytes(nbh, sd.n_c, sd.rank, job.sms), st);
+  cudaError_t e = cudaSuccess;
+  if (from_codes) {
+    e = launch_quant_gram(ca, pa, nbh, job.sms, st);                 // R^T R too
+    if (e == cudaSuccess) e = launch_pi_iterate(pa, job.B0, job.seed, job.segment_index, job.iters, st);
+    if (e == cudaSuccess) e = launch_pass_codes(pa, st);             // A0 = R B; for ranks up to 8 also A0^T A0
     if (e != cudaSuccess) return e;
+  } else {
+    int n_quant = 0;
+    e = job.cc.bits == 2 ? launch_quant<2>(ca, nbh, kneed, job.sms, st, &n_quant) : launch_quant<4>(ca, nbh, kneed, job.sms, st, &n_quant);
+    if (e != cudaSuccess) return e;
+    count_launches(n_quant);
+    if (per_vector) {
+      KcvtArgs ka;
+      ka.seg = sd; ka.arena = job.arena; ka.K = ca.K; ka.R = pa.R; ka.Rmax = pa.Rmax; ka.bh0 = bh0;
+      e = launch_kcvt_keys(ka, nbh, job.cc.bits, ws + pi_workspace_bytes(nbh, sd, job.cc, job.sms), st);
+      if (e != cudaSuccess) return e;
+    }
+    if (sd.rank == 0) return cudaSuccess;
+    e = launch_pi_gram(pa, job.B0, job.seed, job.segment_index, job.iters, job.sms, st);   // the loops, B <- Q(B), its scaling
+    if (e != cudaSuccess) return e;
+    e = launch_pass(pa, st);                                          // A0 = R B; for ranks up to 8 also A0^T A0
+    if (e != cudaSuccess) return e;
+    pi_rta_kernel<<<dim3(kRtaParts, (int)ntiles), kHeadDim, 0, st>>>(pa);                // R^T A0 of ill-conditioned tiles
+    count_launches(2);
   }
-  if (sd.rank == 0) return cudaSuccess;
-  e = launch_pi_gram(pa, job.B0, job.seed, job.segment_index, job.iters, job.sms, st);   // the loops, B <- Q(B), its scaling
+  if (sd.rank > 8) e = launch_dependent(pi_gram2_kernel, dim3(nchunk, (int)ntiles), 256, 0, st, pa);
   if (e != cudaSuccess) return e;
-  e = launch_pass(pa, st);                                          // A0 = R B; for ranks up to 8 also A0^T A0
+  auto finish = sd.rank <= 4 ? pi_finish_kernel<4> : sd.rank <= 8 ? pi_finish_kernel<8> : pi_finish_kernel<16>;
+  e = launch_dependent(finish, dim3((int)ntiles), kHeadDim, 0, st, pa);                  // W, B
   if (e != cudaSuccess) return e;
-  pi_rta_kernel<<<dim3(kRtaParts, (int)ntiles), kHeadDim, 0, st>>>(pa);                  // R^T A0 of ill-conditioned tiles
-  if (sd.rank > 8) pi_gram2_kernel<<<dim3(nchunk, (int)ntiles), 256, 0, st>>>(pa);
-  if (sd.rank <= 4) pi_finish_kernel<4><<<(int)ntiles, kHeadDim, 0, st>>>(pa);           // W, B
-  else if (sd.rank <= 8) pi_finish_kernel<8><<<(int)ntiles, kHeadDim, 0, st>>>(pa);
-  else pi_finish_kernel<16><<<(int)ntiles, kHeadDim, 0, st>>>(pa);
-  const dim3 sgrid((sd.n_c + 255) / 256, (int)ntiles);                                   // A = A0 W
-  if (sd.rank <= 4) pi_store_a_kernel<4><<<sgrid, 256, 0, st>>>(pa);
-  else if (sd.rank <= 8) pi_store_a_kernel<8><<<sgrid, 256, 0, st>>>(pa);
-  else pi_store_a_kernel<16><<<sgrid, 256, 0, st>>>(pa);
-  count_launches(sd.rank > 8 ? 5 : 4);
+  auto store = sd.rank <= 4 ? pi_store_a_kernel<4> : sd.rank <= 8 ? pi_store_a_kernel<8> : pi_store_a_kernel<16>;
+  e = launch_dependent(store, dim3((sd.n_c + 255) / 256, (int)ntiles), 256, 0, st, pa);  // A = A0 W
+  if (e != cudaSuccess) return e;
+  count_launches(sd.rank > 8 ? 3 : 2);
   return cudaGetLastError();
 }
 

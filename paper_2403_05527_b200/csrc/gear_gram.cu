@@ -7,31 +7,9 @@
 
 #include "gear_internal.cuh"
 #include "gear_pi.cuh"
+#include "gear_umma.cuh"
 
 namespace gear {
-
-// ------------------------------------------------------------------ tcgen05 helpers
-namespace {
-__device__ __forceinline__ void umma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-               ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t* b) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(b)) : "memory");
-}
-__device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t addr) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,"
-      "%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]),
-        "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]),
-        "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(addr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-}  // namespace
 
 // ------------------------------------------------------------------ G = R^T R
 // Work: the 32-row blocks of all tiles, one after the other, cut into equal contiguous ranges, one per CTA (two CTAs per
@@ -266,6 +244,7 @@ __global__ void __launch_bounds__(256, 2) pi_iterate_kernel(PiArgs p, const floa
 #pragma unroll
     for (int k = 0; k < 64; ++k) g[k] = __ldcg(src + (size_t)k * kHeadDim);
   };
+  after_previous();
   load_g();
   if (half == 0) {
     const size_t gtile = (size_t)p.bh0 * 2 + tile;
@@ -422,10 +401,15 @@ cudaError_t launch_pi_gram(const PiArgs& p, const float* B0, unsigned long long 
   if (e != cudaSuccess) return e;
   pi_gram_kernel<<<sp.ctas, kGramWarps * 32 + 32, kGramSmem, st>>>(p, sms);
   pi_gram_sum_kernel<<<dim3(kHeadDim / kSumRows, p.ntiles), kHeadDim, 0, st>>>(p, sp.ctas, sms);
-  if (p.rank <= 4) pi_iterate_kernel<4><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters);
-  else if (p.rank <= 8) pi_iterate_kernel<8><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters);
-  else pi_iterate_kernel<16><<<p.ntiles, 256, 0, st>>>(p, B0, seed, segment, iters);
-  count_launches(3);
+  count_launches(2);
+  return launch_pi_iterate(p, B0, seed, segment, iters, st);
+}
+
+cudaError_t launch_pi_iterate(const PiArgs& p, const float* B0, unsigned long long seed, int segment, int iters, cudaStream_t st) {
+  auto iterate = p.rank <= 4 ? pi_iterate_kernel<4> : p.rank <= 8 ? pi_iterate_kernel<8> : pi_iterate_kernel<16>;
+  const cudaError_t e = launch_dependent(iterate, dim3(p.ntiles), 256, 0, st, p, B0, seed, segment, iters);
+  if (e != cudaSuccess) return e;
+  count_launches(1);
   return cudaGetLastError();
 }
 

@@ -12,6 +12,27 @@ namespace gear {
 // process-wide count of kernels this library launched (read through gear_kernel_launches)
 void count_launches(int n);
 
+// A launch that may start while the kernel in front of it on the stream drains (programmatic dependent launch); that kernel's results
+// are there behind after_previous().
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+#ifdef __CUDACC__
+// Waits for the kernel in front, and only then lets the next one start: whoever starts early knows that everything two launches back
+// is complete.
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 struct CompressArgs {
   SegDesc seg;
   CacheConst cc;
@@ -23,6 +44,8 @@ struct CompressArgs {
   int bh0;              // first (batch, head) of the range, for addressing the records
   int side0;            // first side the launch covers (blockIdx.z + side0: 0 keys, 1 values)
   int* status;          // the cache's status word
+  float* Gpart;         // quant_gram_kernel: see PiArgs
+  int* Gexp;
 };
 
 // Key side of a segment with per-vector grouping (gear_kcvt.cu)
@@ -46,7 +69,12 @@ struct PiArgs {
   unsigned char* arena;
   float* R;             // [ntiles][n_c][128]
   unsigned int* Rmax;   // [ntiles] bit pattern of the tile's largest |R|
-  float* Gpart;         // partials of R^T R, [CTA + tile][2][128][128] (gear_gram.cu)
+  const __half* K;      // [nbh][n_c][128]: the range's rows, and the constants of its codes (residual not kept)
+  const __half* V;
+  CacheConst cc;
+  float* Gpart;         // partials of R^T R: [CTA + tile][2][128][128] (gear_gram.cu), or, where the residual is not kept,
+                        // [side][CTA + (batch, head)][128][128] (gear_quant_gram.cu)
+  int* Gexp;            // and the power of two that each of these was scaled by
   float* G;             // [ntiles][128][128]: R^T R (of R scaled by the tile's power of two)
   int* status;          // the cache's status word
   float* Bcur;          // [ntiles][128][16]
@@ -59,6 +87,7 @@ struct PiArgs {
   float* dbgA;          // fp32 copies for export, whole segment: [BH][2][n_c][rank] / [BH][2][128][rank]
   float* dbgB;
   int bh0, ntiles, n_c, rank, nchunk;
+  int chunk_rows;       // rows per CTA of the pass, and per partial of A0^T A0
   int a0_pitch;         // 4, 8 or 16 columns, zero past the rank
 };
 
@@ -78,11 +107,21 @@ struct CompressJob {
   int* status;
 };
 
-size_t compress_workspace_bytes(int nbh, int n_c, int rank, int sms, int csr_k = -1);
+size_t compress_workspace_bytes(int nbh, const SegDesc& sd, const CacheConst& cc, int sms);
 // R^T R of every tile, then everything of Algorithm 2 that runs on it: leaves the last loop's factor in p.Bcur
 size_t pi_gram_workspace_bytes(int ntiles, int n_c, int sms);
 cudaError_t launch_pi_gram(const PiArgs& p, const float* B0, unsigned long long seed, int segment, int iters, int sms,
                            cudaStream_t st);
+// Filter, Quant, packing and R^T R of segments whose residual is not kept (gear_quant_gram.cu), A0 = R b of them (gear_pass_codes.cu)
+constexpr int kRtaParts = 4;      // CTAs per tile that sum R^T A0 where it is asked for
+struct QgSplit { long long blocks; int ctas; };
+QgSplit qg_split(int nbh, const SegDesc& sd, int sms);
+int pass_chunk_rows(int nbh, const SegDesc& sd, const CacheConst& cc, int sms);
+bool qg_fits(const SegDesc& sd, const CacheConst& cc);
+size_t qg_partials(int nbh, const SegDesc& sd, int sms);
+cudaError_t launch_quant_gram(const CompressArgs& a, const PiArgs& p, int nbh, int sms, cudaStream_t st);
+cudaError_t launch_pass_codes(const PiArgs& p, cudaStream_t st);
+cudaError_t launch_pi_iterate(const PiArgs& p, const float* B0, unsigned long long seed, int segment, int iters, cudaStream_t st);
 // whole-tile path for short segments (one launch): usable when compress_tile_fits()
 bool compress_tile_fits(int T, int n_c, int rank);
 cudaError_t compress_tile(const CompressJob& job, int BH, cudaStream_t st);

@@ -1,0 +1,59 @@
+"""Prompts whose residual is not kept: R^T R summed while the blocks are quantized, A0 = R b from the codes.  Residuals that grow past
+the range that the sums were scaled for, blocks without a residual, ranges that end inside tiles, chunks that end early."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _compress(p, k16, v16, rank, seed):
+    import torch
+    from paper_2403_05527_b200 import binding as G
+    B, H, n = k16.shape[:3]
+    b0 = np.random.default_rng(seed).standard_normal((B, H, 2, 128, rank)).astype(np.float32)
+    p.oracle.compress(k16, v16, rank, b0)
+    G.gear_compress(p.cache, None, torch.from_numpy(k16).cuda(), torch.from_numpy(v16).cuda(), n, rank, torch.from_numpy(b0).cuda())
+    torch.cuda.synchronize()
+    assert G.gear_last_device_status(p.cache) == 0
+    p.check_segment(0)
+
+
+@pytest.mark.parametrize("bits,s_pct,B,H,n,rank", [
+    (2, 2.0, 1, 1, 192, 4),         # the shortest; one range per side
+    (4, 2.0, 1, 3, 704, 8),         # eleven blocks a tile: ranges end inside tiles, the second chunk of rows is short
+    (2, 0.0, 2, 2, 576, 16),        # no outliers, sixteen columns
+    (4, 0.0, 1, 2, 1024, 1),
+    (4, 3.0, 1, 40, 320, 2),
+])
+def test_group_shapes(bits, s_pct, B, H, n, rank):
+    from paper_2403_05527_b200 import synth
+    from tests.gear_harness import Pair
+    p = Pair(31, B, H, H, bits, 64, s_pct, 64, min(rank, 4), n + 128, r_max=rank)
+    try:
+        k16, v16 = synth.make_kv(31, B, H, n, 128)
+        _compress(p, k16, v16, rank, n)
+        # on the factors as stored: fp16 storage moves the attention over short prompts by up to 2e-3, the kernels' arithmetic by less than 1e-4
+        p.oracle = p.with_stored_factors()
+        p.check_attention(tol=1e-4)
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("first", [2.0 ** -10, 0.0])
+@pytest.mark.parametrize("bits", [2, 4])
+def test_residuals_that_grow(bits, first):
+    """The first 64 tokens, then the next ones, are smaller than the rest by factors that fp16 does not span (with `first` zero: without
+    any residual), so that the scale of the sums moves inside a range; 1088 tokens, i.e. 17 blocks in four or five ranges."""
+    from tests.gear_harness import Pair
+    p = Pair(32, 1, 2, 2, bits, 64, 2.0, 64, 4, 2048, r_max=4)
+    try:
+        gen = np.random.default_rng(bits)
+        x = gen.standard_normal((2, 1, 2, 1088, 128)) * np.exp(gen.standard_normal((2, 1, 2, 1, 128)))
+        for start in range(0, 1088, 256):                   # whatever range a block belongs to: small ones ahead of large ones
+            x[..., start:start + 64, :] *= first
+            x[..., start + 64:start + 128, :] *= 2.0 ** -6
+            x[..., start + 128:start + 256, :] *= 2.0 ** 7
+        k16, v16 = np.clip(x, -6e4, 6e4).astype(np.float16) + np.float16(0)      # no negative zeros: either may be the zero point
+        _compress(p, k16, v16, 4, 7)
+    finally:
+        p.close()
