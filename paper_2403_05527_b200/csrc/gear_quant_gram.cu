@@ -6,6 +6,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "gear_internal.cuh"
 #include "gear_pi.cuh"
 #include "gear_quant.cuh"
@@ -14,9 +16,9 @@
 
 namespace gear {
 
-constexpr int kQgThreads = 128;                    // a thread per quantization group of a block
-constexpr int kQgRows = 64;                        // tokens whose operands are in shared memory at a time
-constexpr int kQgOperand = kQgRows * kHeadDim * 2; // fp16 heads, or remainders, of those
+constexpr int kQgPart = 64;                        // entries of a thread: a group of 64, or half a group of 128
+__host__ __device__ constexpr int qg_threads(int len) { return 2 * len; }                     // 128 channels times `len` tokens a block
+__host__ __device__ constexpr int qg_operand(int len) { return len * kHeadDim * 2; }          // fp16 heads, or remainders, of a block
 constexpr int kQgCodeKey = kHeadDim + 4;           // bytes per row of packed key codes
 // Tokens per CTA at least, a partial sum being 64 KB; where there are fewer blocks than SMs a block each.
 constexpr int kQgMinRows = 128;
@@ -24,12 +26,12 @@ constexpr int kQgMinRows = 128;
 // fp16 ends at 2^16.
 constexpr int kQgStart = 4, kQgGrow = 14;
 
-__host__ __device__ constexpr int qg_ctas_per_sm(int len) { return len == 64 ? 4 : 3; }
+__host__ __device__ constexpr int qg_ctas_per_sm(int len) { return len == 64 ? 4 : 2; }
 __host__ __device__ constexpr int qg_code_bytes(int bits, int side, int len) {
   return side == 0 ? len * bits / 8 * kQgCodeKey : kHeadDim * bits / 8 * (len + 4);
 }
 __host__ __device__ constexpr int qg_smem(int bits, int side, int len) {
-  return 1024 + 2 * kQgOperand + len * kHeadDim * 2 + qg_code_bytes(bits, side, len);
+  return 1024 + 2 * qg_operand(len) + len * kHeadDim * 2 + qg_code_bytes(bits, side, len);
 }
 
 QgSplit qg_split(int nbh, const SegDesc& sd, int sms) {
@@ -41,13 +43,59 @@ QgSplit qg_split(int nbh, const SegDesc& sd, int sms) {
 }
 bool qg_fits(const SegDesc& sd, const CacheConst& cc) {
   if (sd.rank == 0 || sd.csr_base16 != 0 || sd.T != cc.g_v) return false;
-  return sd.T == 64 && sd.k_k == cc.k_v && sd.k_k <= 1;
+  return sd.k_k == cc.k_v && (sd.T == 64 ? sd.k_k <= 1 : sd.T == 128 && sd.k_k <= 2);
 }
 size_t qg_partials(int nbh, const SegDesc& sd, int sms) { return 2 * (size_t)(qg_split(nbh, sd, sms).ctas + nbh); }
 
-// Bound: instruction issue, with the 2 bytes per entry of X behind it.  A thread owns a group (keys: a channel's L
-// tokens, values: L channels of a token), which it keeps in registers as packed pairs; see quant_fast_kernel for the filter
-// and the order of the arithmetic.  The residual of an entry, scaled by a power of two, leaves as an fp16 head and an
+// Largest and smallest instances of a thread's entries and of its partner's (K = 0: one of each, 1: two, 2: three), as pairs (i-th largest,
+// minus the i-th smallest), so that one comparison serves both sides.  An entry that is NaN makes
+// the first of them NaN.
+template <int K> struct Ends { __half2 v[K + 1]; };
+// the first K + 1 of the union: the k-th largest is the maximum over i + j = k of min(a_i, b_j), a_0 = b_0 = infinity
+template <int K>
+__device__ __forceinline__ Ends<K> merge_ends(const Ends<K>& a, const Ends<K>& b) {
+  Ends<K> r;
+  r.v[0] = __hmax2_nan(a.v[0], b.v[0]);
+  if constexpr (K > 0) r.v[1] = __hmax2_nan(__hmin2_nan(a.v[0], b.v[0]), __hmax2_nan(a.v[1], b.v[1]));
+  if constexpr (K > 1)
+    r.v[2] = __hmax2_nan(__hmax2_nan(__hmin2_nan(a.v[0], b.v[1]), __hmin2_nan(a.v[1], b.v[0])), __hmax2_nan(a.v[2], b.v[2]));
+  return r;
+}
+// of 64 entries in packed pairs.  Sorting networks of four pairs, merged one after the other per half of the pairs (largest and smallest
+// apart), the halves at the end: 7 instructions per pair for K = 2, where a chain that keeps three of each takes 10.
+template <int K>
+__device__ __forceinline__ Ends<K> ends_of(const __half2 (&xp)[kQgPart / 2]) {
+  Ends<K> top, bot;                                // bot: negated
+#pragma unroll
+  for (int q = 0; q < kQgPart / 2; q += 4) {
+    __half2 a = xp[q], b = xp[q + 1], c = xp[q + 2], d = xp[q + 3];
+    auto order = [](__half2& hi, __half2& lo) { const __half2 h = __hmax2_nan(hi, lo); lo = __hmin2_nan(hi, lo); hi = h; };
+    order(a, b); order(c, d); order(a, c); order(b, d);
+    if (K > 0) order(b, c);
+    Ends<K> t, u;
+    t.v[0] = a; u.v[0] = __hneg2(d);
+    if constexpr (K > 0) { t.v[1] = b; u.v[1] = __hneg2(c); }
+    if constexpr (K > 1) { t.v[2] = c; u.v[2] = __hneg2(b); }
+    top = q == 0 ? t : merge_ends(top, t);
+    bot = q == 0 ? u : merge_ends(bot, u);
+  }
+  Ends<K> even, odd;
+#pragma unroll
+  for (int i = 0; i <= K; ++i) { even.v[i] = __lows2half2(top.v[i], bot.v[i]); odd.v[i] = __highs2half2(top.v[i], bot.v[i]); }
+  return merge_ends(even, odd);
+}
+// first set entry of 64 mask bits (even entries, odd entries), removed from them; 64 if none
+__device__ __forceinline__ int take_entry(unsigned int& even, unsigned int& odd) {
+  const int fe = even ? 2 * (__ffs((int)even) - 1) : 64, fo = odd ? 2 * (__ffs((int)odd) - 1) + 1 : 64;
+  if (fe < fo) { even &= even - 1; return fe; }
+  if (fo < 64) odd &= odd - 1;
+  return fo;
+}
+
+// Bound: instruction issue, with the 2 bytes per entry of X behind it.  A thread owns 64 entries of a group (keys: tokens of a
+// channel, values: channels of a token), which it keeps in registers as packed pairs; groups of 128 belong to two threads, which
+// exchange what the filter has to know of the other half.  See quant_fast_kernel for the order of the arithmetic.  The residual of
+// an entry, scaled by a power of two, leaves as an fp16 head and an
 // fp16 remainder (22 bits) for the products h^T h and h^T 2l: with l h the transpose of h l, the mean of the accumulator
 // and its transpose is h h + h l + l h, in 128 columns of tensor memory instead of 256, so that four CTAs fit on an SM.
 // Keys are stored [channel][token] (K-major), as the thread of a channel has them, values [token][channel] (MN-major);
@@ -58,27 +106,30 @@ size_t qg_partials(int nbh, const SegDesc& sd, int sms) { return 2 * (size_t)(qg
 // times its field's weight; what the filtered entries left there is taken out again afterwards (modulo 256).
 // 2 bits, 8 x 32 heads x 4096: keys 157, values 155 us (quant_fast_kernel 154 and 168, and 182 for R^T R from the fp32
 // residual); 22 to 24 instructions per entry, 60 % of the issue slots, tensor cores 22 %.  The whole call 851 -> 575 us; 4 bits, 16 x
-// 40 heads x 8192 4162 -> 2888 us, one head of 192 to 2048 tokens 70 -> 45 to 68 us (half of that from launches that overlap).
+// 40 heads x 8192 4162 -> 2854 us, one head of 192 to 2048 tokens 70 -> 45 to 68 us (half of that from launches that overlap).
+// Groups of 128 with two outliers per side, 2 bits, 2 x 8 heads x 16384: keys 64, values 58 us (one thread per group 74 and 82: three
+// CTAs of four warps, and more code than the instruction cache holds); the call for two such layers 603 -> 455 us.
 template <int BITS, int SIDE, int L, int K>
-__global__ void __launch_bounds__(kQgThreads, qg_ctas_per_sm(L))
+__global__ void __launch_bounds__(qg_threads(L), qg_ctas_per_sm(L))
 quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap value_rows) {
-  constexpr int F = 8 / BITS, ROWS = L / F, kSegRows = 64 / F;      // rows of packed codes of a group / of 64 of its entries
-  constexpr int kGroups = kHeadDim / L;
+  constexpr int F = 8 / BITS, kPartRows = kQgPart / F;              // rows of packed codes of a thread's entries
+  constexpr int kThreads = qg_threads(L), kOperand = qg_operand(L);
   constexpr int kCodePitch = SIDE == 0 ? kQgCodeKey : L + 4;
-  constexpr int kSubs = L / kQgRows;
+  constexpr bool kShared = L > kQgPart;            // two threads per group
   extern __shared__ unsigned char smem_raw[];
   __shared__ uint64_t full, mma_done;
   __shared__ uint32_t tmem_slot;
   __shared__ unsigned int dmax_bits[2], smax_bits[2], rmax_bits[2];    // of even and odd blocks
+  __shared__ __half2 ends_s[kShared ? K + 1 : 1][kShared ? kThreads : 1];
   unsigned char* op_hi = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
-  unsigned char* op_lo = op_hi + kQgOperand;
-  unsigned char* tile = op_lo + kQgOperand;        // keys: [token][channel]; values: boxes, [64-channel half][token]
+  unsigned char* op_lo = op_hi + kOperand;
+  unsigned char* tile = op_lo + kOperand;          // keys: [token][channel]; values: boxes, [64-channel half][token]
   unsigned char* codes = tile + L * kHeadDim * 2;
   const SegDesc& sd = p.seg;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // values: a warp's lanes are consecutive tokens of the same channels
-  const int tok = SIDE == 0 ? 0 : tid % L, grp = SIDE == 0 ? 0 : tid / L;
-  const int gi = SIDE == 0 ? tid : tok * kGroups + grp;             // the group's number in the record
+  // keys: channel and which 64 tokens; values: token and which 64 channels.  A warp's lanes are neighbours.
+  const int line = SIDE == 0 ? tid % kHeadDim : tid % L, part = SIDE == 0 ? tid / kHeadDim : tid / L;
+  const int gi = SIDE == 1 && !kShared ? 2 * line + part : line;    // the group's number in the record
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) { dmax_bits[i] = 0u; smax_bits[i] = 0u; rmax_bits[i] = 0u; }
     bar_init(&full);
@@ -105,28 +156,24 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
       bulk_copy(tile, p.K + (size_t)(f0 + it) * L * kHeadDim, L * kHeadDim * 2, &full);
     } else {
 #pragma unroll
-      for (int b = 0; b < 2 * kSubs; ++b)
-        load_box(tile + b * kBoxBytes, &value_rows, b / kSubs * kBoxChannels, (int)(f0 + it) * L + b % kSubs * kBoxRows, &full);
+      for (int b = 0; b < 2 * (L / kBoxRows); ++b)
+        load_box(tile + b * kBoxBytes, &value_rows, b / (L / kBoxRows) * kBoxChannels, (int)(f0 + it) * L + b % (L / kBoxRows) * kBoxRows, &full);
     }
   };
   if (tid == 0 && count > 0) request(0);
 
-  // entry e of the group in the tile
-  auto entry = [&](int e) -> __half {
-    if (SIDE == 0) return reinterpret_cast<const __half*>(tile)[e * kHeadDim + tid];
-    const int ch = grp * L + e;
-    return *reinterpret_cast<const __half*>(tile + (ch / kBoxChannels) * (L * 128) + box_at(tok, ch % kBoxChannels));
+  // entry e of part q of the thread's line
+  auto entry_of = [&](int q, int e) -> __half {
+    if (SIDE == 0) return reinterpret_cast<const __half*>(tile)[(q * kQgPart + e) * kHeadDim + line];
+    return *reinterpret_cast<const __half*>(tile + q * (L * 128) + box_at(line, e));
   };
-  // where entries e .. e + 7 go as operands (e a multiple of eight, of the present 64 tokens)
-  auto op_at = [&](int e) {
-    const int c = e / 8 % 8;
-    if (SIDE == 0) return tid * 128 + ((c ^ (tid & 7)) << 4);
-    return (grp + e / 64) * (kQgOperand / 2) + ((tok & 63) >> 3) * 1024 + (tok & 7) * 128 + ((c ^ (tok & 7)) << 4);
-  };
+  // where the thread's entries e .. e + 7 go as operands (e a multiple of eight)
+  unsigned char* const op_line = op_hi + (SIDE == 0 ? part * (kHeadDim * 128) + line * 128 : part * (L * 128) + line * 128);
+  auto op_at = [&](int e) { return ((e / 8) ^ (line & 7)) << 4; };
   // row of the packed codes and field of entry e
-  auto code_row = [&](int e) { return SIDE == 0 ? e / 64 * kSegRows + e % kSegRows : e / (16 * F) * 16 + e % 16; };
-  auto code_field = [&](int e) { return SIDE == 0 ? e % 64 / kSegRows : e % (16 * F) / 16; };
-  unsigned char* mine = codes + (SIDE == 0 ? tid : grp * ROWS * kCodePitch + tok);
+  auto code_row = [&](int e) { return SIDE == 0 ? e % kPartRows : e / (16 * F) * 16 + e % 16; };
+  auto code_field = [&](int e) { return SIDE == 0 ? e / kPartRows : e % (16 * F) / 16; };
+  unsigned char* mine = codes + part * kPartRows * kCodePitch + line;
 
   int exp_cur = 0;
   bool exp_set = false;
@@ -137,16 +184,16 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
     ok = ok && bar_wait(&full, parity);
     parity ^= 1u;
     unsigned char* rec = p.arena + sd.seg_base + (size_t)(p.bh0 + bhl) * sd.bh_stride + sd.bfac_bytes + (size_t)blk * sd.rec_bytes;
-    __half2 xp[L / 2];                             // entries 2q, 2q + 1
+    __half2 xp[kQgPart / 2];                       // entries 2q, 2q + 1
     if (SIDE == 0) {
-      const __half* col = reinterpret_cast<const __half*>(tile) + tid;
+      const __half* col = reinterpret_cast<const __half*>(tile) + part * kQgPart * kHeadDim + line;
 #pragma unroll
-      for (int q = 0; q < L / 2; ++q) xp[q] = __halves2half2(col[(2 * q) * kHeadDim], col[(2 * q + 1) * kHeadDim]);
+      for (int q = 0; q < kQgPart / 2; ++q) xp[q] = __halves2half2(col[(2 * q) * kHeadDim], col[(2 * q + 1) * kHeadDim]);
     } else {
-      const unsigned char* row = tile + grp * (L * 128) + tok * 128;
+      const unsigned char* row = tile + part * (L * 128) + line * 128;
 #pragma unroll
-      for (int q = 0; q < L / 8; ++q) {
-        const uint4 v = *reinterpret_cast<const uint4*>(row + q / 8 * (L * 128) + ((q % 8 ^ (tok & 7)) << 4));
+      for (int q = 0; q < kQgPart / 8; ++q) {
+        const uint4 v = *reinterpret_cast<const uint4*>(row + ((q ^ (line & 7)) << 4));
         xp[4 * q] = *reinterpret_cast<const __half2*>(&v.x);
         xp[4 * q + 1] = *reinterpret_cast<const __half2*>(&v.y);
         xp[4 * q + 2] = *reinterpret_cast<const __half2*>(&v.z);
@@ -154,13 +201,108 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
       }
     }
     float mn, mx;
-    int oi[2 * K + 1];                             // the filtered entries, ascending
-    __half ov[2 * K + 1];
-    {
+    int oi[2 * K + 1];                             // the thread's filtered entries, ascending; kQgPart and more: none
+    oi[2 * K] = kQgPart;
+    int before = 0;                                // filtered entries of the group in the part ahead
+    if constexpr (!kShared) {
+      static_assert(K <= 1, "");
       int imax, imin;
       filter_one<L, K, true>(xp, 0, mn, mx, imax, imin);
       if (K == 1) { oi[0] = min(imax, imin); oi[2 * K - 1] = max(imax, imin); }
+    } else {
+      Ends<K> ends = ends_of<K>(xp), other;
+#pragma unroll
+      for (int i = 0; i <= K; ++i) ends_s[i][tid] = ends.v[i];
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i <= K; ++i) other.v[i] = ends_s[i][tid ^ (kThreads / 2)];
+      ends = merge_ends(ends, other);
+      float top[K + 1], bot[K + 1];
+#pragma unroll
+      for (int i = 0; i <= K; ++i) { top[i] = __low2float(ends.v[i]); bot[i] = -__high2float(ends.v[i]); }
+      mx = top[K]; mn = bot[K];
+      if constexpr (K > 0) {
+        if (bot[K - 1] < top[K - 1]) {
+          // The K entries above or at the K-th largest instance, of equal ones the first; the smallest likewise
+          const __half2 vT = __float2half2_rn(top[K - 1]), vB = __float2half2_rn(bot[K - 1]);
+          unsigned int t[2] = {0u, 0u}, b[2] = {0u, 0u};            // bit i of a half of word w: pair 16 w + i
+#pragma unroll
+          for (int q = 0; q < kQgPart / 2; ++q) {
+            const unsigned int bit = 0x00010001u << (q & 15);
+            t[q >> 4] |= __hge2_mask(xp[q], vT) & bit;
+            b[q >> 4] |= __hle2_mask(xp[q], vB) & bit;
+          }
+          unsigned int even = 0u, odd = 0u;
+          auto collect = [&](const unsigned int (&m)[2], const float (&end)[K + 1], auto of_other) {
+            unsigned int me = __byte_perm(m[0], m[1], 0x5410), mo = __byte_perm(m[0], m[1], 0x7632);
+            if (end[K] == end[K - 1]) {              // more than K entries reach the bound: one group in fifty of ordinary data
+              int take = K, ahead = 0;
+#pragma unroll
+              for (int i = 0; i < K; ++i) take -= end[i] != end[K - 1];
+#pragma unroll
+              for (int i = 0; i <= K; ++i) ahead += of_other(i) == end[K - 1];
+              if (part > 0) take -= min(take, ahead);
+              unsigned int ke = 0u, ko = 0u;
+#pragma unroll 1
+              while (me | mo) {
+                const int e = take_entry(me, mo);
+                if (__half2float(entry_of(part, e)) == end[K - 1] && --take < 0) continue;
+                if (e & 1) ko |= 1u << (e >> 1); else ke |= 1u << (e >> 1);
+              }
+              me = ke; mo = ko;
+            }
+            even |= me; odd |= mo;
+          };
+          collect(t, top, [&](int i) { return __low2float(other.v[i]); });
+          collect(b, bot, [&](int i) { return -__high2float(other.v[i]); });
+#pragma unroll
+          for (int a = 0; a < 2 * K; ++a) oi[a] = take_entry(even, odd);
+          int own = 0;
+#pragma unroll
+          for (int a = 0; a < 2 * K; ++a) own += oi[a] < kQgPart;
+          before = part == 0 ? 0 : 2 * K - own;
+        } else {
+          // The sides share entries (or NaN): one after the other, ties to the lower index, the largest K, then the smallest K of what
+          // is left, then the bounds of the rest
+          int pick[2 * K];
+          mn = INFINITY; mx = -INFINITY;
+#pragma unroll 1
+          for (int n = 0; n <= 2 * K; ++n) {
+            int best = -1;
+            float v = 0.f;
+#pragma unroll 1
+            for (int e = 0; e < L; ++e) {
+              bool gone = false;
+#pragma unroll
+              for (int a = 0; a < 2 * K; ++a) gone = gone || (a < n && pick[a] == e);
+              if (gone) continue;
+              const float x = __half2float(entry_of(e / kQgPart, e % kQgPart));
+              if (n == 2 * K) { mn = fminf(mn, x); mx = fmaxf(mx, x); }
+              else if (best < 0 || (n < K ? x > v : x < v)) { best = e; v = x; }
+            }
+#pragma unroll
+            for (int a = 0; a < 2 * K; ++a) pick[a] = a == n ? best : pick[a];
+          }
+#pragma unroll
+          for (int a = 0; a < 2 * K; ++a)
+#pragma unroll
+            for (int b = a + 1; b < 2 * K; ++b) { const int lo = min(pick[a], pick[b]), hi = max(pick[a], pick[b]); pick[a] = lo; pick[b] = hi; }
+          int n = 0;
+#pragma unroll
+          for (int a = 0; a < 2 * K; ++a) oi[a] = kQgPart;
+#pragma unroll
+          for (int a = 0; a < 2 * K; ++a) {
+            if (pick[a] / kQgPart < part) ++before;
+            if (pick[a] / kQgPart == part) {
+#pragma unroll
+              for (int b = 0; b < 2 * K; ++b) oi[b] = b == n ? pick[a] % kQgPart : oi[b];
+              ++n;
+            }
+          }
+        }
+      }
     }
+    auto filtered = [&](int a) { return !kShared || oi[a] < kQgPart; };
     // Eq. 2 on the kept entries: binary32, one rounding per operation
     const float levels = (float)((1 << BITS) - 1);
     const float range = __fsub_rn(mx, mn);
@@ -169,22 +311,28 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
     const float d = __half2float(d16);
     const float inv = d != 0.f ? __fdiv_rn(1.0f, d) : 0.f;
     float dm = 0.f;
+    __half ov[2 * K + 1];
     // Stored ahead of the barrier: the next block's copy is requested behind it and does not wait for loads that are still on
     // their way, so everything loaded from the block has to be used before it.
-    if (K > 0) {
+    if constexpr (K > 0) {
 #pragma unroll
-      for (int a = 0; a < 2 * K; ++a) ov[a] = entry(oi[a]);
+      for (int a = 0; a < 2 * K; ++a) ov[a] = entry_of(part, kShared ? min(oi[a], kQgPart - 1) : oi[a]);
+      __half* dv = reinterpret_cast<__half*>(rec + (SIDE == 0 ? sd.off_koval : sd.off_voval)) + gi * 2 * K + before;
+      unsigned char* di = rec + (SIDE == 0 ? sd.off_koidx : sd.off_voidx) + gi * 2 * K + before;
 #pragma unroll
-      for (int a = 0; a < 2 * K; ++a) dm = fmaxf(dm, fabsf(__half2float(ov[a]) - mn));
-      __half2* dv = reinterpret_cast<__half2*>(rec + (SIDE == 0 ? sd.off_koval : sd.off_voval)) + gi * K;
-      uchar2* di = reinterpret_cast<uchar2*>(rec + (SIDE == 0 ? sd.off_koidx : sd.off_voidx)) + gi * K;
+      for (int a = 0; a < 2 * K; ++a)
+        if (filtered(a)) dm = fmaxf(dm, fabsf(__half2float(ov[a]) - mn));
+      if constexpr (!kShared) {
+        *reinterpret_cast<__half2*>(dv) = __halves2half2(ov[0], ov[1]);
+        *reinterpret_cast<uchar2*>(di) = make_uchar2((unsigned char)oi[0], (unsigned char)oi[1]);
+      } else {
 #pragma unroll
-      for (int a = 0; a < K; ++a) {
-        dv[a] = __halves2half2(ov[2 * a], ov[2 * a + 1]);
-        di[a] = make_uchar2((unsigned char)oi[2 * a], (unsigned char)oi[2 * a + 1]);
+        for (int a = 0; a < 2 * K; ++a)
+          if (filtered(a)) { dv[a] = ov[a]; di[a] = (unsigned char)(part * kQgPart + oi[a]); }
       }
     }
-    reinterpret_cast<__half2*>(rec + (SIDE == 0 ? sd.off_kscale : sd.off_vscale))[gi] = __halves2half2(d16, __float2half_rn(mn));
+    if (!kShared || part == 0)
+      reinterpret_cast<__half2*>(rec + (SIDE == 0 ? sd.off_kscale : sd.off_vscale))[gi] = __halves2half2(d16, __float2half_rn(mn));
     {
       // A bound on the group's residuals: half a step for a kept entry, the whole range if the step rounded to zero, plus the
       // rounding of the dequantised value.  Non-negative floats order like their bit patterns.
@@ -205,6 +353,9 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
     const float rmax = __uint_as_float(rmax_bits[it & 1]);
     const int er = max(-150, min(130, pow2_exponent(rmax)));
     if (mma_pending) ok = ok && bar_wait(&mma_done, mma_parity);    // the operands may be written, the sums are current
+    // accumulator row 32 (warp % 4) + lane, and the columns from c0 on that the warp takes
+    const uint32_t sums = tmem + ((uint32_t)(warp % 4 * 32) << 16);
+    const int c0 = warp / 4 * (kHeadDim / (kThreads / 128)), c1 = c0 + kHeadDim / (kThreads / 128);
     if (rmax > 0.f) {
       if (!exp_set) {
         exp_cur = er - kQgStart;
@@ -214,14 +365,13 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
         if (!fresh) {
           tmem_fence_after();
           const float f = exp2_int(2 * (exp_cur - e_new));
-          const uint32_t at = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
-          for (int c = 0; c < kHeadDim; c += 32) {
+          for (int c = c0; c < c1; c += 32) {
             uint32_t v[32];
-            tmem_ld32(v, at + c);
+            tmem_ld32(v, sums + c);
 #pragma unroll
             for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * f);
-            tmem_st32(at + c, v);
+            tmem_st32(sums + c, v);
           }
           tmem_fence_before();
         }
@@ -231,93 +381,83 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
     // Codes and residuals are computed for every entry as if it were kept.
     const PairQuantSplit quantize(mn, inv, d, levels, exp2_int(-exp_cur));
 #pragma unroll
-    for (int sub = 0; sub < kSubs; ++sub) {
-      if (SIDE == 0 || kSubs == 1 || tid / kQgRows == sub) {
+    for (int r8 = 0; r8 < kPartRows / 8; ++r8) {
+      unsigned int acc[8];
 #pragma unroll
-        for (int r8 = 0; r8 < (SIDE == 0 ? kSegRows : ROWS) / 8; ++r8) {
-          unsigned int acc[8];
+      for (int f = 0; f < F; ++f) {
+        const int e = SIDE == 0 ? f * kPartRows + r8 * 8 : r8 / 2 * 16 * F + f * 16 + r8 % 2 * 8;
+        uint32_t h[4], l[4];
 #pragma unroll
-          for (int f = 0; f < F; ++f) {
-            const int e = SIDE == 0 ? sub * 64 + f * kSegRows + r8 * 8 : r8 / 2 * 16 * F + f * 16 + r8 % 2 * 8;
-            uint32_t h[4], l[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              unsigned int c0, c1;
-              quantize(xp[e / 2 + k], c0, c1, h[k], l[k]);
-              acc[2 * k] = f == 0 ? c0 : c0 * (1u << (BITS * f)) + acc[2 * k];
-              acc[2 * k + 1] = f == 0 ? c1 : c1 * (1u << (BITS * f)) + acc[2 * k + 1];
-            }
-            *reinterpret_cast<uint4*>(op_hi + op_at(e)) = make_uint4(h[0], h[1], h[2], h[3]);
-            *reinterpret_cast<uint4*>(op_lo + op_at(e)) = make_uint4(l[0], l[1], l[2], l[3]);
-          }
-          const int row = (SIDE == 0 ? sub * kSegRows : 0) + r8 * 8;
-#pragma unroll
-          for (int i = 0; i < 8; ++i) mine[(row + i) * kCodePitch] = (unsigned char)acc[i];
+        for (int k = 0; k < 4; ++k) {
+          unsigned int k0, k1;
+          quantize(xp[e / 2 + k], k0, k1, h[k], l[k]);
+          acc[2 * k] = f == 0 ? k0 : k0 * (1u << (BITS * f)) + acc[2 * k];
+          acc[2 * k + 1] = f == 0 ? k1 : k1 * (1u << (BITS * f)) + acc[2 * k + 1];
         }
-        // the filtered entries: no residual, code zero
-#pragma unroll
-        for (int a = 0; a < K; ++a) {
-          unsigned int c[2];
-          uint32_t h, l;
-          quantize(__halves2half2(ov[2 * a], ov[2 * a + 1]), c[0], c[1], h, l);
-#pragma unroll
-          for (int b = 0; b < 2; ++b) {
-            const int e = oi[2 * a + b];
-            if (SIDE == 0 && kSubs > 1 && e / kQgRows != sub) continue;
-            const int at = op_at(e) + (e & 7) * 2;
-            *reinterpret_cast<unsigned short*>(op_hi + at) = 0;
-            *reinterpret_cast<unsigned short*>(op_lo + at) = 0;
-            unsigned char* byte = mine + code_row(e) * kCodePitch;
-            *byte = (unsigned char)(*byte - (c[b] << (BITS * code_field(e))));
-          }
-        }
+        *reinterpret_cast<uint4*>(op_line + op_at(e)) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4*>(op_line + kOperand + op_at(e)) = make_uint4(l[0], l[1], l[2], l[3]);
       }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      tmem_fence_before();
-      __syncthreads();
-      if (tid == 0) {
-        tmem_fence_after();
-        // 128B swizzle, 8-row groups 1 KB apart (stride); values MN-major, their 64-channel halves 8 KB apart (leading); fp32
-        // accumulator, fp16 operands, M = N = 128
-        constexpr uint64_t kDesc = (SIDE == 0 ? 1ull << 16 : (uint64_t)(kQgOperand / 2 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
-                                   (1ull << 46) | (2ull << 61);
-        constexpr uint32_t kIdesc = (1u << 4) | (SIDE == 0 ? 0u : (1u << 15) | (1u << 16)) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-        constexpr uint32_t kStep = (SIDE == 0 ? 32 : 2048) >> 4;                  // 16 tokens further
-        const uint64_t dh = kDesc | (smem_addr(op_hi) >> 4), dl = kDesc | (smem_addr(op_lo) >> 4);
 #pragma unroll
-        for (int k = 0; k < kQgRows / 16; ++k) {
-          umma_f16(tmem, dh + k * kStep, dh + k * kStep, kIdesc, fresh && sub == 0 && k == 0 ? 0u : 1u);
-          umma_f16(tmem, dh + k * kStep, dl + k * kStep, kIdesc, 1u);
-        }
-        umma_commit(&mma_done);
-      }
-      if (mma_pending) mma_parity ^= 1u;
-      mma_pending = true;
-      if (sub + 1 < kSubs) ok = ok && bar_wait(&mma_done, mma_parity);
+      for (int i = 0; i < 8; ++i) mine[(r8 * 8 + i) * kCodePitch] = (unsigned char)acc[i];
     }
-    fresh = false;
+    // the filtered entries: no residual, code zero
+#pragma unroll
+    for (int a = 0; a < K; ++a) {
+      unsigned int c[2];
+      uint32_t h, l;
+      quantize(__halves2half2(ov[2 * a], ov[2 * a + 1]), c[0], c[1], h, l);
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        if (!filtered(2 * a + b)) continue;
+        const int e = oi[2 * a + b], at = op_at(e) + (e & 7) * 2;
+        *reinterpret_cast<unsigned short*>(op_line + at) = 0;
+        *reinterpret_cast<unsigned short*>(op_line + kOperand + at) = 0;
+        unsigned char* byte = mine + code_row(e) * kCodePitch;
+        *byte = (unsigned char)(*byte - (c[b] << (BITS * code_field(e))));
+      }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    tmem_fence_before();
+    __syncthreads();
     if (tid == 0) {
+      tmem_fence_after();
+      // 128B swizzle, 8-row groups 1 KB apart (stride).  Keys K-major, 64 tokens a row; values MN-major, their 64-channel halves
+      // L rows apart (leading).  fp32 accumulator, fp16 operands, M = N = 128.
+      constexpr uint64_t kDesc = (SIDE == 0 ? 1ull << 16 : (uint64_t)(L * 128 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+                                 (1ull << 46) | (2ull << 61);
+      constexpr uint32_t kIdesc = (1u << 4) | (SIDE == 0 ? 0u : (1u << 15) | (1u << 16)) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+      const uint64_t dh = kDesc | (smem_addr(op_hi) >> 4), dl = kDesc | (smem_addr(op_lo) >> 4);
+#pragma unroll
+      for (int k = 0; k < L / 16; ++k) {           // 16 tokens further
+        const uint32_t at = (SIDE == 0 ? k / 4 * (kHeadDim * 128) + k % 4 * 32 : k * 2048) >> 4;
+        umma_f16(tmem, dh + at, dh + at, kIdesc, fresh && k == 0 ? 0u : 1u);
+        umma_f16(tmem, dh + at, dl + at, kIdesc, 1u);
+      }
+      umma_commit(&mma_done);
       const int s = it & 1;
       reinterpret_cast<float*>(rec)[SIDE] = __uint_as_float(dmax_bits[s]);
       reinterpret_cast<float*>(rec)[2 + SIDE] = __uint_as_float(smax_bits[s]);
       atomicMax(p.Rmax + bhl * 2 + SIDE, rmax_bits[s]);
       dmax_bits[s] = 0u; smax_bits[s] = 0u; rmax_bits[s] = 0u;      // used again two blocks on, behind the next block's first barrier
     }
+    if (mma_pending) mma_parity ^= 1u;
+    mma_pending = true;
+    fresh = false;
     // the codes in fragment order (code_coord_k / code_coord_v)
     unsigned int* dst = reinterpret_cast<unsigned int*>(rec + (SIDE == 0 ? sd.off_kcodes : sd.off_vcodes));
     if (SIDE == 0) {
       // word (w, lane, tau) of a slab: four neighbouring channels of a token in each of its fields; a row of packed bytes holds the
       // channels' codes of F tokens, 64 / F apart
-      constexpr int kWords = kSlab * kHeadDim * BITS / 32, kSegSlabs = kSegRows / kSlab;      // words per slab
+      constexpr int kWords = kSlab * kHeadDim * BITS / 32, kPartSlabs = kPartRows / kSlab;    // words per slab
 #pragma unroll
-      for (int li = tid; li < ROWS / kSlab * kWords; li += kQgThreads) {
+      for (int li = tid; li < L / F / kSlab * kWords; li += kThreads) {
         const int slab = li / kWords, wl = li % kWords;            // slab of rows
         const int w = wl & 3, ln = (wl >> 2) & 31, tau = wl >> 7;
         const int row = slab * kSlab + (ln >> 2) + 8 * (w & 1), ch = 32 * F * tau + 16 * (w >> 1) + 4 * (ln & 3);
         unsigned int v[F];
 #pragma unroll
         for (int j = 0; j < F; ++j) v[j] = *reinterpret_cast<const unsigned int*>(codes + row * kCodePitch + ch + 32 * j);
-        unsigned int* out = dst + (slab / kSegSlabs * (64 / kSlab) + slab % kSegSlabs) * kWords + wl;
+        unsigned int* out = dst + (slab / kPartSlabs * (kQgPart / kSlab) + slab % kPartSlabs) * kWords + wl;
 #pragma unroll
         for (int f = 0; f < F; ++f) {
           unsigned int word = 0;
@@ -326,14 +466,14 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
             const unsigned int m = field_of_bytes<BITS>() << (BITS * j);
             word |= (j >= f ? v[j] << (BITS * (j - f)) : v[j] >> (BITS * (f - j))) & m;
           }
-          out[f * kSegSlabs * kWords] = word;
+          out[f * kPartSlabs * kWords] = word;
         }
       }
     } else {
       // a row of packed bytes is the byte rows of one channel of a tuple: four tokens are a word
       constexpr int kWords = 32 * kHeadDim * BITS / 32;               // words per 32-token chunk
 #pragma unroll
-      for (int li = tid; li < L / 32 * kWords; li += kQgThreads) {
+      for (int li = tid; li < L / 32 * kWords; li += kThreads) {
         const int chunk = li / kWords, wl = li % kWords;
         const int w = wl & 3, ln = (wl >> 2) & 31, tau = wl >> 7;
         dst[li] = *reinterpret_cast<const unsigned int*>(codes + (tau * 16 + (ln >> 2) + 8 * (w & 1)) * kCodePitch + chunk * 32 +
@@ -345,14 +485,13 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
       tmem_fence_after();
       __syncwarp();
       const size_t at = (size_t)blockIdx.x + bhl + (SIDE == 0 ? 0 : gridDim.x + nbh);
-      float* part = p.Gpart + at * (kHeadDim * kHeadDim) + tid;
-      const uint32_t from = tmem + ((uint32_t)(warp * 32) << 16);
+      float* part_sum = p.Gpart + at * (kHeadDim * kHeadDim) + warp % 4 * 32 + lane;
 #pragma unroll 1
-      for (int c = 0; c < kHeadDim; c += 32) {     // accumulator row i is thread i's: row c of the partial gets its column c
+      for (int c = c0; c < c1; c += 32) {          // row c of the partial gets the accumulator's column c
         uint32_t v[32];
-        tmem_ld32(v, from + c);
+        tmem_ld32(v, sums + c);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) part[(size_t)(c + i) * kHeadDim] = __uint_as_float(v[i]);
+        for (int i = 0; i < 32; ++i) part_sum[(size_t)(c + i) * kHeadDim] = __uint_as_float(v[i]);
       }
       tmem_fence_before();
       if (tid == 0) p.Gexp[at] = exp_cur;
@@ -421,7 +560,7 @@ template <int BITS, int SIDE, int L, int K>
 static cudaError_t launch_side(const CompressArgs& a, int nbh, int ctas, const CUtensorMap& value_rows, cudaStream_t st) {
   const int smem = qg_smem(BITS, SIDE, L);
   const cudaError_t e = cudaFuncSetAttribute(quant_gram_kernel<BITS, SIDE, L, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  return e == cudaSuccess ? launch_dependent(quant_gram_kernel<BITS, SIDE, L, K>, dim3(ctas), kQgThreads, smem, st, a, nbh, value_rows) : e;
+  return e == cudaSuccess ? launch_dependent(quant_gram_kernel<BITS, SIDE, L, K>, dim3(ctas), qg_threads(L), smem, st, a, nbh, value_rows) : e;
 }
 template <int BITS, int L, int K>
 static cudaError_t launch_sides(const CompressArgs& a, int nbh, int ctas, const CUtensorMap& value_rows, cudaStream_t st) {
@@ -433,8 +572,13 @@ cudaError_t launch_quant_gram(const CompressArgs& a, const PiArgs& p, int nbh, i
   CUtensorMap rows;
   cudaError_t e = make_row_map(&rows, a.V, (long long)nbh * a.seg.n_c);
   if (e != cudaSuccess) return e;
-  if (a.cc.bits == 2) e = k == 0 ? launch_sides<2, 64, 0>(a, nbh, ctas, rows, st) : launch_sides<2, 64, 1>(a, nbh, ctas, rows, st);
-  else e = k == 0 ? launch_sides<4, 64, 0>(a, nbh, ctas, rows, st) : launch_sides<4, 64, 1>(a, nbh, ctas, rows, st);
+  auto run = [&](auto bits) {
+    constexpr int B = decltype(bits)::value;
+    if (a.seg.T == 64) return k == 0 ? launch_sides<B, 64, 0>(a, nbh, ctas, rows, st) : launch_sides<B, 64, 1>(a, nbh, ctas, rows, st);
+    return k == 0 ? launch_sides<B, 128, 0>(a, nbh, ctas, rows, st) : k == 1 ? launch_sides<B, 128, 1>(a, nbh, ctas, rows, st)
+                                                                              : launch_sides<B, 128, 2>(a, nbh, ctas, rows, st);
+  };
+  e = a.cc.bits == 2 ? run(std::integral_constant<int, 2>()) : run(std::integral_constant<int, 4>());
   if (e != cudaSuccess) return e;
   e = ctas < 8 * nbh ? launch_dependent(quant_gram_sum_kernel<1>, dim3(kQgPairs, p.ntiles), 256, 0, st, p, ctas)
                      : launch_dependent(quant_gram_sum_kernel<4>, dim3(kQgPairs, p.ntiles), 1024, 0, st, p, ctas);

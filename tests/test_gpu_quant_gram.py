@@ -18,23 +18,50 @@ def _compress(p, k16, v16, rank, seed):
     p.check_segment(0)
 
 
-@pytest.mark.parametrize("bits,s_pct,B,H,n,rank", [
-    (2, 2.0, 1, 1, 192, 4),         # the shortest; one range per side
-    (4, 2.0, 1, 3, 704, 8),         # eleven blocks a tile: ranges end inside tiles, the second chunk of rows is short
-    (2, 0.0, 2, 2, 576, 16),        # no outliers, sixteen columns
-    (4, 0.0, 1, 2, 1024, 1),
-    (4, 3.0, 1, 40, 320, 2),
+@pytest.mark.parametrize("bits,group,s_pct,B,H,n,rank", [
+    (2, 64, 2.0, 1, 1, 192, 4),     # the shortest; one range per side
+    (4, 64, 2.0, 1, 3, 704, 8),     # eleven blocks a tile: ranges end inside tiles, the second chunk of rows is short
+    (2, 64, 0.0, 2, 2, 576, 16),    # no outliers, sixteen columns
+    (4, 64, 0.0, 1, 2, 1024, 1),
+    (4, 64, 3.0, 1, 40, 320, 2),
+    (2, 128, 2.0, 1, 1, 256, 4),    # two outliers per side: two blocks
+    (4, 128, 2.0, 1, 5, 1152, 8),   # nine blocks a tile
+    (2, 128, 1.0, 1, 2, 640, 2),    # one outlier
+    (4, 128, 1.0, 1, 30, 384, 16),
+    (2, 128, 0.0, 1, 3, 384, 5),
 ])
-def test_group_shapes(bits, s_pct, B, H, n, rank):
+def test_group_shapes(bits, group, s_pct, B, H, n, rank):
     from paper_2403_05527_b200 import synth
     from tests.gear_harness import Pair
-    p = Pair(31, B, H, H, bits, 64, s_pct, 64, min(rank, 4), n + 128, r_max=rank)
+    p = Pair(31, B, H, H, bits, group, s_pct, 64, min(rank, 4), n + 128, r_max=rank)
     try:
         k16, v16 = synth.make_kv(31, B, H, n, 128)
         _compress(p, k16, v16, rank, n)
         # on the factors as stored: fp16 storage moves the attention over short prompts by up to 2e-3, the kernels' arithmetic by less than 1e-4
         p.oracle = p.with_stored_factors()
         p.check_attention(tol=1e-4)
+    finally:
+        p.close()
+
+
+@pytest.mark.parametrize("bits,group,s_pct", [(2, 64, 2.0), (4, 128, 2.0), (2, 128, 1.0), (4, 64, 0.0)])
+def test_flat_groups_among_others(bits, group, s_pct):
+    """Groups whose entries are all equal, equal but for one, two or three, or equal on two levels: the sides of the filter share
+    candidates there, and what they clear has to stay out of the sums."""
+    from tests.gear_harness import Pair
+    p = Pair(33, 1, 1, 1, bits, group, s_pct, 64, 2, 1024, r_max=2)
+    try:
+        gen = np.random.default_rng(group + bits)
+        x = gen.standard_normal((2, 1, 1, 512, 128)).astype(np.float16)
+        x[:, 0, 0, :group] = 1.25                           # whole blocks of keys, whole groups of values
+        x[:, 0, 0, group:2 * group] = 0.5
+        for at in range(group, 2 * group, 9):               # one to three other entries in a key's and a value's group
+            for e in range(1 + at % 3):
+                x[:, 0, 0, group + (at * 5 + 11 * e) % group, (at * 7) % 128] = gen.standard_normal()
+                x[:, 0, 0, at, (at * 3 + 17 * e) % 128] = gen.standard_normal()
+        x[:, 0, 0, 2 * group:2 * group + 64, ::2] = -3.0    # two levels
+        x[:, 0, 0, 2 * group:2 * group + 64, 1::2] = 3.0
+        _compress(p, x[0], x[1], 2, 3)
     finally:
         p.close()
 
