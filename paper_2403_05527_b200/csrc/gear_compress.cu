@@ -200,6 +200,7 @@ __global__ void __launch_bounds__(128) quant_pack_kernel(CompressArgs p) {
   auto x_of = [&](int idx) { return __half2float(__ushort_as_half(xs[idx])); };
   __shared__ unsigned int dmax_bits, smax_bits;
   if (tid == 0) { dmax_bits = 0u; smax_bits = 0u; }
+  after_previous();
 
   const __half* X = (side == 0 ? p.K : p.V) + ((size_t)bhl * sd.n_c + (size_t)blk * T) * kHeadDim;
   for (int i = tid; i < T * 16; i += 128) {
@@ -323,6 +324,8 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
   const int T = SIDE == 1 && L == kHeadDim ? sd.T : L;              // tokens of a block; values: 128 / L groups each
   const bool active = L < kHeadDim || SIDE == 0 || tid < T;         // a thread per group
   BlockFeed feed{tile, &full, side == 0 ? p.K : p.V, sd.n_c, sd.nblk, T, sd.nblk * nbh, 0u};
+  if (SIDE == 0) after_previous();                 // the values' CTAs run beside the keys' and wait at their end (see quant_gram_kernel)
+  else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;
     bar_init(&full);
@@ -496,6 +499,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
       }
     }
   }
+  if (SIDE == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -554,6 +558,8 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
   const int T = sd.T;                               // keys: 128; values: tokens (= groups) of the block
   const int tid = threadIdx.x;
   BlockFeed feed{tile, &full, SIDE == 0 ? p.K : p.V, sd.n_c, sd.nblk, T, sd.nblk * nbh, 0u};
+  if (SIDE == 0) after_previous();                 // the values' CTAs run beside the keys' and wait at their end (see quant_gram_kernel)
+  else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;
     bar_init(&full);
@@ -779,6 +785,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
       }
     }
   }
+  if (SIDE == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -817,6 +824,7 @@ __global__ void __launch_bounds__(kPassWarps * 32, 3) pi_pass_kernel(PiArgs p) {
   const int row1 = min(p.n_c, row0 + kChunkRows);
   const float* R = p.R + (size_t)tile * p.n_c * kHeadDim;
   float* A0 = p.A0 + (size_t)tile * p.n_c * RP;
+  after_previous();
 
   // ---- the warp's ring: rows [rb, rb + 16) of its it-th group go to stage it % kPassStages
   unsigned char* ring = ring_all + warp * kPassStages * kPassStage;
@@ -899,6 +907,7 @@ __global__ void __launch_bounds__(kHeadDim) pi_rta_kernel(PiArgs p) {
   constexpr int kRows = 32;
   __shared__ float a[kRows * kMaxRank];
   const int tile = blockIdx.y, part = blockIdx.x, j = threadIdx.x;
+  after_previous();
   if (!p.ill[tile]) return;
   const int RP = p.a0_pitch;
   const int row0 = (int)((long long)part * p.n_c / kRtaParts), row1 = (int)((long long)(part + 1) * p.n_c / kRtaParts);
@@ -1187,6 +1196,7 @@ __global__ void __launch_bounds__(128) compress_tile_kernel(TileArgs p) {
   const __half* Xt = (side == 0 ? p.K : p.V) + (size_t)bh * n_c * kHeadDim;
   unsigned char* seg_bh = p.arena + sd.seg_base + (size_t)bh * sd.bh_stride;
   auto x_of = [&](int idx) { return __half2float(__ushort_as_half(xs[idx])); };
+  after_previous();
 
   // ---- Filter, Quant, pack, residual: block by block (one key group per channel spans one block)
   for (int blk = 0; blk < sd.nblk; ++blk) {
@@ -1397,7 +1407,7 @@ cudaError_t compress_tile(const CompressJob& job, int BH, cudaStream_t st) {
   {                                                                                                                  \
     e = cudaFuncSetAttribute(compress_tile_kernel<B, KM, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
     if (e != cudaSuccess) return e;                                                                                  \
-    compress_tile_kernel<B, KM, R><<<grid, 128, smem, st>>>(a);                                                      \
+    e = launch_dependent(compress_tile_kernel<B, KM, R>, grid, 128, smem, st, a);                                    \
   }
 #define GEAR_TILE_R(B, KM) \
   { if (rp == 4) GEAR_TILE(B, KM, 4) else if (rp == 8) GEAR_TILE(B, KM, 8) else GEAR_TILE(B, KM, 16) }
@@ -1415,6 +1425,7 @@ cudaError_t compress_tile(const CompressJob& job, int BH, cudaStream_t st) {
 // Segment with rank 0: nothing to fit, but the A sections of the records do not exist either.
 // Segment descriptor table entry, written by the device so that no host copy is needed.
 __global__ void write_desc_kernel(SegDesc* table, int* blk2seg, int index, SegDesc d) {
+  after_previous();
   if (threadIdx.x == 0) table[index] = d;
   for (int b = threadIdx.x; b < d.nblk; b += blockDim.x) blk2seg[d.blk_start + b] = index;
 }
@@ -1454,7 +1465,7 @@ __global__ void __launch_bounds__(256) push_kernel(PushArgs p) {
 // Filter / Quant / pack / residual of a long segment: per side, the register-resident kernel that fits the group
 // shape, else the general one.  side0 = 1: the value side only.  Returns the number of launches through *launches.
 template <int BITS>
-static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, int sms, cudaStream_t st, int* launches) {
+static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, int sms, bool overlap, cudaStream_t st, int* launches) {
   const int T = a.seg.T;
   const size_t smem = round_up(T * kXPitch * 2, 16) + (size_t)T * kRPitch * 4;
   const dim3 grid(a.seg.nblk, nbh, 1);
@@ -1471,7 +1482,7 @@ static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, int sm
     auto launch = [&](auto kern) {
       const int tile = T * kHeadDim * 2;
       if (len == kHeadDim) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadDim * kHeadDim * 2);
-      if (e == cudaSuccess) kern<<<ctas, 128, tile, st>>>(a, nbh);
+      if (e == cudaSuccess) e = launch_after(overlap, kern, dim3(ctas), 128, tile, st, a, nbh);
     };
 #define GEAR_LAUNCH_FAST(LEN, K) \
   if (side == 0) launch(quant_fast_kernel<BITS, 0, LEN, K>); else launch(quant_fast_kernel<BITS, 1, LEN, K>);
@@ -1491,7 +1502,7 @@ static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, int sm
     e = cudaFuncSetAttribute(quant_pack_kernel<BITS, KM>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                              (int)smem);                                                                   \
     if (e != cudaSuccess) return e;                                                                         \
-    quant_pack_kernel<BITS, KM><<<grid, 128, smem, st>>>(a);                                                \
+    e = launch_after(overlap, quant_pack_kernel<BITS, KM>, grid, 128, smem, st, a);                                              \
   }
       if (kmax_needed <= 1) GEAR_LAUNCH_Q(1)
       else if (kmax_needed <= 2) GEAR_LAUNCH_Q(2)
@@ -1505,11 +1516,10 @@ static cudaError_t launch_quant(CompressArgs a, int nbh, int kmax_needed, int sm
   return cudaGetLastError();
 }
 
-static cudaError_t launch_pass(const PiArgs& p, cudaStream_t st) {
+static cudaError_t launch_pass(const PiArgs& p, bool overlap, cudaStream_t st) {
   auto launch = [&](auto kern) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassSmem);
-    if (e == cudaSuccess) kern<<<dim3(p.nchunk, p.ntiles), kPassWarps * 32, kPassSmem, st>>>(p);
-    return e;
+    return e == cudaSuccess ? launch_after(overlap, kern, dim3(p.nchunk, p.ntiles), kPassWarps * 32, kPassSmem, st, p) : e;
   };
   return p.rank <= 4 ? launch(pi_pass_kernel<1>) : p.rank <= 8 ? launch(pi_pass_kernel<2>) : launch(pi_pass_kernel<4>);
 }
@@ -1592,22 +1602,28 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
     if (e == cudaSuccess) e = launch_pass_codes(pa, st);             // A0 = R B; for ranks up to 8 also A0^T A0
     if (e != cudaSuccess) return e;
   } else {
+    // Launches that overlap pay where they are short (256 tokens x 32 heads, us without and with: groups of 16 68.4 / 58.5, of 32 63.9 / 53.2,
+    // per-vector keys 93.0 / 86.6; one head of 4096 75.5 / 68.6, 70.8 / 66.8, 124 / 114) and without a low-rank part (128 heads x 4096 120 /
+    // 110); long chains over a kept residual run 1 to 7 % longer with them (4096 tokens x 32 heads 214.7 / 226.3, 167.7 / 174.0, 265 / 275).
+    const bool overlap = sd.rank == 0 || (long long)nbh * sd.n_c <= 16384;
     int n_quant = 0;
-    e = job.cc.bits == 2 ? launch_quant<2>(ca, nbh, kneed, job.sms, st, &n_quant) : launch_quant<4>(ca, nbh, kneed, job.sms, st, &n_quant);
+    e = job.cc.bits == 2 ? launch_quant<2>(ca, nbh, kneed, job.sms, overlap, st, &n_quant)
+                           : launch_quant<4>(ca, nbh, kneed, job.sms, overlap, st, &n_quant);
     if (e != cudaSuccess) return e;
     count_launches(n_quant);
     if (per_vector) {
       KcvtArgs ka;
       ka.seg = sd; ka.arena = job.arena; ka.K = ca.K; ka.R = pa.R; ka.Rmax = pa.Rmax; ka.bh0 = bh0;
-      e = launch_kcvt_keys(ka, nbh, job.cc.bits, ws + pi_workspace_bytes(nbh, sd, job.cc, job.sms), st);
+      e = launch_kcvt_keys(ka, nbh, job.cc.bits, ws + pi_workspace_bytes(nbh, sd, job.cc, job.sms), overlap, st);
       if (e != cudaSuccess) return e;
     }
     if (sd.rank == 0) return cudaSuccess;
-    e = launch_pi_gram(pa, job.B0, job.seed, job.segment_index, job.iters, job.sms, st);   // the loops, B <- Q(B), its scaling
+    e = launch_pi_gram(pa, job.B0, job.seed, job.segment_index, job.iters, job.sms, overlap, st);   // the loops, B <- Q(B), its scaling
     if (e != cudaSuccess) return e;
-    e = launch_pass(pa, st);                                          // A0 = R B; for ranks up to 8 also A0^T A0
+    e = launch_pass(pa, overlap, st);                                          // A0 = R B; for ranks up to 8 also A0^T A0
     if (e != cudaSuccess) return e;
-    pi_rta_kernel<<<dim3(kRtaParts, (int)ntiles), kHeadDim, 0, st>>>(pa);                // R^T A0 of ill-conditioned tiles
+    e = launch_after(overlap, pi_rta_kernel, dim3(kRtaParts, (int)ntiles), kHeadDim, 0, st, pa);   // R^T A0 of ill-conditioned tiles
+    if (e != cudaSuccess) return e;
     count_launches(2);
   }
   if (sd.rank > 8) e = launch_dependent(pi_gram2_kernel, dim3(nchunk, (int)ntiles), 256, 0, st, pa);
@@ -1623,9 +1639,9 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
 }
 
 cudaError_t launch_write_desc(SegDesc* table, int* blk2seg, int index, const SegDesc& d, cudaStream_t st) {
-  write_desc_kernel<<<1, 256, 0, st>>>(table, blk2seg, index, d);
-  count_launches(1);
-  return cudaGetLastError();
+  const cudaError_t e = launch_dependent(write_desc_kernel, dim3(1), 256, 0, st, table, blk2seg, index, d);
+  if (e == cudaSuccess) count_launches(1);
+  return e;
 }
 
 cudaError_t launch_push(const PushArgs& a, cudaStream_t st) {

@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(kGramWarps * 32 + 32, 2) pi_gram_kernel(PiArgs
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_addr(&tmem_slot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  after_previous();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -179,6 +180,7 @@ __global__ void __launch_bounds__(kHeadDim) pi_gram_sum_kernel(PiArgs p, int gra
   const long long NW = gram_ctas, b0 = (long long)tile * sp.nb, b1 = b0 + sp.nb;
   const int w0 = (int)(((b0 + 1) * NW + sp.blocks - 1) / sp.blocks - 1), w1 = (int)((b1 * NW + sp.blocks - 1) / sp.blocks - 1);
   float g[kSumRows];
+  after_previous();
 #pragma unroll
   for (int k = 0; k < kSumRows; ++k) g[k] = 0.f;
   const float* src = p.Gpart + (size_t)(w0 + tile) * kGramPartial;
@@ -395,12 +397,12 @@ __global__ void __launch_bounds__(256, 2) pi_iterate_kernel(PiArgs p, const floa
 }
 
 cudaError_t launch_pi_gram(const PiArgs& p, const float* B0, unsigned long long seed, int segment, int iters, int sms,
-                           cudaStream_t st) {
+                           bool overlap, cudaStream_t st) {
   const GramSplit sp = gram_split(p.ntiles, p.n_c, sms);
   cudaError_t e = cudaFuncSetAttribute(pi_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGramSmem);
+  if (e == cudaSuccess) e = launch_after(overlap, pi_gram_kernel, dim3(sp.ctas), kGramWarps * 32 + 32, kGramSmem, st, p, sms);
+  if (e == cudaSuccess) e = launch_after(overlap, pi_gram_sum_kernel, dim3(kHeadDim / kSumRows, p.ntiles), kHeadDim, 0, st, p, sp.ctas, sms);
   if (e != cudaSuccess) return e;
-  pi_gram_kernel<<<sp.ctas, kGramWarps * 32 + 32, kGramSmem, st>>>(p, sms);
-  pi_gram_sum_kernel<<<dim3(kHeadDim / kSumRows, p.ntiles), kHeadDim, 0, st>>>(p, sp.ctas, sms);
   count_launches(2);
   return launch_pi_iterate(p, B0, seed, segment, iters, st);
 }

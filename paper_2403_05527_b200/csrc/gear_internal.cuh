@@ -15,14 +15,18 @@ void count_launches(int n);
 // A launch that may start while the kernel in front of it on the stream drains (programmatic dependent launch); that kernel's results
 // are there behind after_previous().
 template <class... P, class... A>
-inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+inline cudaError_t launch_after(bool overlap, void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[0].val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
   cfg.attrs = attr; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+  return launch_after(true, kern, grid, block, smem, st, args...);
 }
 #ifdef __CUDACC__
 // Waits for the kernel in front, and only then lets the next one start: whoever starts early knows that everything two launches back
@@ -62,7 +66,7 @@ struct KcvtArgs {
 };
 bool kcvt_fits(int n_c);
 size_t kcvt_workspace_bytes(int nbh, int n_c, int csr_k);
-cudaError_t launch_kcvt_keys(KcvtArgs a, int nbh, int bits, unsigned char* ws, cudaStream_t st);
+cudaError_t launch_kcvt_keys(KcvtArgs a, int nbh, int bits, unsigned char* ws, bool overlap, cudaStream_t st);
 
 struct PiArgs {
   SegDesc seg;
@@ -111,7 +115,7 @@ size_t compress_workspace_bytes(int nbh, const SegDesc& sd, const CacheConst& cc
 // R^T R of every tile, then everything of Algorithm 2 that runs on it: leaves the last loop's factor in p.Bcur
 size_t pi_gram_workspace_bytes(int ntiles, int n_c, int sms);
 cudaError_t launch_pi_gram(const PiArgs& p, const float* B0, unsigned long long seed, int segment, int iters, int sms,
-                           cudaStream_t st);
+                           bool overlap, cudaStream_t st);
 // Filter, Quant, packing and R^T R of segments whose residual is not kept (gear_quant_gram.cu), A0 = R b of them (gear_pass_codes.cu)
 constexpr int kRtaParts = 4;      // CTAs per tile that sum R^T A0 where it is asked for
 struct QgSplit { long long blocks; int ctas; };

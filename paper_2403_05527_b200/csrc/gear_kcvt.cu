@@ -242,6 +242,7 @@ __global__ void __launch_bounds__(kSelChannels * 32, 2) kcvt_select_kernel(KcvtA
   unsigned int* hist = hist_all + warp * 512;
 
   const __half* X = p.K + (size_t)bhl * n_c * kHeadDim;
+  after_previous();
 #pragma unroll 4
   for (int t2 = tid; t2 < n_c / 2; t2 += kSelChannels * 32) {  // 16 bytes (this CTA's 8 channels) of two token rows
     const uint4 a = *reinterpret_cast<const uint4*>(X + (size_t)(2 * t2) * kHeadDim + cg * kSelChannels);
@@ -382,6 +383,7 @@ __global__ void __launch_bounds__(256) kcvt_list_kernel(KcvtArgs p) {
   for (int i = tid; i < nblk * kHeadDim; i += blockDim.x) cnt[i] = 0u;
   for (int i = tid; i < nblk; i += blockDim.x) dmax[i] = 0u;
   if (tid == 0) smax_bits = 0u;
+  after_previous();
   __syncthreads();
   const unsigned int* olist = p.olist + (size_t)bhl * kHeadDim * k2;
   const __half2* sz = p.sz + (size_t)bhl * kHeadDim;
@@ -453,6 +455,7 @@ __global__ void __launch_bounds__(128) kcvt_pack_kernel(KcvtArgs p) {
   __shared__ __align__(16) unsigned char codes[kBlockTok * kPitch];
   const SegDesc& sd = p.seg;
   const int blk = blockIdx.x, bhl = blockIdx.y, tid = threadIdx.x;
+  after_previous();
   const unsigned char* C8 = p.codes8 + ((size_t)bhl * sd.n_c + (size_t)blk * kBlockTok) * kHeadDim;
   for (int i = tid; i < kBlockTok * 8; i += 128) {          // 16-byte pieces
     const int tok = i >> 3, q = i & 7;
@@ -493,7 +496,7 @@ size_t kcvt_workspace_bytes(int nbh, int n_c, int csr_k) {
 }
 
 // Key side of a per-vector segment for the (batch, head) range of `a`; three launches.
-cudaError_t launch_kcvt_keys(KcvtArgs a, int nbh, int bits, unsigned char* ws, cudaStream_t st) {
+cudaError_t launch_kcvt_keys(KcvtArgs a, int nbh, int bits, unsigned char* ws, bool overlap, cudaStream_t st) {
   const SegDesc& sd = a.seg;
   a.codes8 = ws;
   a.olist = reinterpret_cast<unsigned int*>(ws + (size_t)nbh * sd.n_c * kHeadDim);
@@ -503,19 +506,18 @@ cudaError_t launch_kcvt_keys(KcvtArgs a, int nbh, int bits, unsigned char* ws, c
   if (bits == 2) {
     e = cudaFuncSetAttribute(kcvt_select_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_sel);
     if (e != cudaSuccess) return e;
-    kcvt_select_kernel<2><<<dim3(kHeadDim / kSelChannels, nbh), kSelChannels * 32, sm_sel, st>>>(a);
+    e = launch_after(overlap, kcvt_select_kernel<2>, dim3(kHeadDim / kSelChannels, nbh), kSelChannels * 32, sm_sel, st, a);
   } else {
     e = cudaFuncSetAttribute(kcvt_select_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_sel);
     if (e != cudaSuccess) return e;
-    kcvt_select_kernel<4><<<dim3(kHeadDim / kSelChannels, nbh), kSelChannels * 32, sm_sel, st>>>(a);
+    e = launch_after(overlap, kcvt_select_kernel<4>, dim3(kHeadDim / kSelChannels, nbh), kSelChannels * 32, sm_sel, st, a);
   }
-  e = cudaFuncSetAttribute(kcvt_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_list);
   if (e != cudaSuccess) return e;
-  kcvt_list_kernel<<<nbh, 256, sm_list, st>>>(a);
-  if (bits == 2) kcvt_pack_kernel<2><<<dim3(sd.nblk, nbh), 128, 0, st>>>(a);
-  else kcvt_pack_kernel<4><<<dim3(sd.nblk, nbh), 128, 0, st>>>(a);
-  count_launches(3);
-  return cudaGetLastError();
+  e = cudaFuncSetAttribute(kcvt_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_list);
+  if (e == cudaSuccess) e = launch_after(overlap, kcvt_list_kernel, dim3(nbh), 256, sm_list, st, a);
+  if (e == cudaSuccess) e = launch_after(overlap, bits == 2 ? kcvt_pack_kernel<2> : kcvt_pack_kernel<4>, dim3(sd.nblk, nbh), 128, 0, st, a);
+  if (e == cudaSuccess) count_launches(3);
+  return e;
 }
 
 }  // namespace gear
