@@ -324,7 +324,9 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
   const int T = SIDE == 1 && L == kHeadDim ? sd.T : L;              // tokens of a block; values: 128 / L groups each
   const bool active = L < kHeadDim || SIDE == 0 || tid < T;         // a thread per group
   BlockFeed feed{tile, &full, side == 0 ? p.K : p.V, sd.n_c, sd.nblk, T, sd.nblk * nbh, 0u};
-  if (SIDE == 0) after_previous();                 // the values' CTAs run beside the keys' and wait at their end (see quant_gram_kernel)
+  // The values' CTAs run beside the keys' and wait at their end (see quant_gram_kernel); without keys in front of them (per-vector
+  // key groups) the kernel in front may be the one that writes V.
+  if (SIDE == 0 || p.side0 == 1) after_previous();
   else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;
@@ -558,7 +560,9 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
   const int T = sd.T;                               // keys: 128; values: tokens (= groups) of the block
   const int tid = threadIdx.x;
   BlockFeed feed{tile, &full, SIDE == 0 ? p.K : p.V, sd.n_c, sd.nblk, T, sd.nblk * nbh, 0u};
-  if (SIDE == 0) after_previous();                 // the values' CTAs run beside the keys' and wait at their end (see quant_gram_kernel)
+  // The values' CTAs run beside the keys' and wait at their end (see quant_gram_kernel); without keys in front of them (per-vector
+  // key groups) the kernel in front may be the one that writes V.
+  if (SIDE == 0 || p.side0 == 1) after_previous();
   else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;

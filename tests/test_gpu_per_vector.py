@@ -162,3 +162,35 @@ def test_selection_of_the_outliers(pair_factory, n, s):
     G.gear_compress(p.cache, None, torch.from_numpy(k16).to(p.dev), torch.from_numpy(v16).to(p.dev), n, 0, None)
     torch.cuda.synchronize()
     p.check_segment(0)
+
+
+# Lets the kernel behind it start at once, and writes what that kernel reads some thirty microseconds later.
+_LATE_COPY = r"""
+extern "C" __global__ void late_copy(const uint4* src, uint4* dst, int n) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int i = 0; i < 60; ++i) __nanosleep(500);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
+"""
+
+
+@pytest.mark.parametrize("group,s,rank", [(0, 0.0, 0), (0, 1.0, 0), (0, 2.0, 0), (0, 2.0, 4), (64, 2.0, 0), (128, 2.0, 0)])
+def test_keys_and_values_that_the_kernel_in_front_writes(pair_factory, group, s, rank):
+    """The producer of a segment's rows may let its dependents start before it has written them: every kernel of the call has to
+    wait for it, also the values' where no keys' kernel is in front of it.  The second segment: a new cache clears scratch first."""
+    import torch
+    from paper_2403_05527_b200 import binding as G, synth
+    p = pair_factory(6, 1, 2, 2, 4, group, s, 64, 0, 1024, r_max=4)
+    p.compress(256, 0)
+    k16, v16 = synth.make_kv(6, 1, 2, 256, 128, extra=1)
+    b0 = synth.make_b0(6, 1, 2, 128, rank, extra=1)
+    p.oracle.compress(k16, v16, rank, b0)
+    made = torch.from_numpy(np.stack([k16, v16])).to(p.dev)
+    rows = torch.zeros_like(made)
+    b0d = torch.from_numpy(np.ascontiguousarray(b0)).to(p.dev) if rank else None
+    late_copy = torch.cuda._compile_kernel(_LATE_COPY, "late_copy")
+    torch.cuda.synchronize()
+    late_copy(grid=(8, 1, 1), block=(256, 1, 1), args=[made, rows, made.numel() // 8])
+    G.gear_compress(p.cache, None, rows[0], rows[1], 256, rank, b0d)
+    torch.cuda.synchronize()
+    p.check_segment(1)
