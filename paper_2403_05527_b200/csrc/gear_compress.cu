@@ -444,10 +444,8 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
         }
       }
     }
-    // A bound on the group's residuals instead of their maximum (it only picks the power of two the power iteration
-    // scales by): half a step for a kept entry, the whole range if the step rounded to zero, plus the rounding of the
-    // dequantised value
-    float rmax = active ? (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx)) : 0.f;
+    // a bound on the group's residuals instead of their maximum (it only picks the power of two the power iteration scales by)
+    float rmax = active ? residual_bound(mn, mx, range, d, levels) : 0.f;
     {
       float dm = K == 1 && active ? fmaxf(fabsf(__half2float(vmax) - mn), fabsf(__half2float(vmin) - mn)) : 0.f;
       float sm = active ? d : 0.f;
@@ -728,7 +726,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
           if (R != nullptr) R[SIDE == 0 ? oi[a] * kHeadDim + tid : first + oi[a]] = 0.f;
           dm = fmaxf(dm, fabsf(__half2float(__ushort_as_half(ov[a])) - mn));
         }
-        rmax = (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
+        rmax = residual_bound(mn, mx, range, d, levels);
       } else {
         rmax = 0.f;
         GroupResult g = process_group<BITS, 2>(

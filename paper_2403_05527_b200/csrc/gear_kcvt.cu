@@ -330,9 +330,8 @@ __global__ void __launch_bounds__(kSelChannels * 32, 2) kcvt_select_kernel(KcvtA
   if (lane == 0) {
     quant[warp] = make_float4(mn, inv, d, 0.f);
     p.sz[(size_t)bhl * kHeadDim + ch] = __halves2half2(d16, __float2half_rn(mn));
-    if (p.Rmax != nullptr) {        // a bound on the residuals of the channel (see quant_fast_kernel)
-      const float rb = (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
-      atomicMax(p.Rmax + bhl * 2, __float_as_uint(rb));
+    if (p.Rmax != nullptr) {        // a bound on the residuals of the channel
+      atomicMax(p.Rmax + bhl * 2, __float_as_uint(residual_bound(mn, mx, range, d, levels)));
     }
   }
   // ---- codes and residuals: a thread takes four tokens of all eight channels, so that it has whole 32-byte sectors to store

@@ -51,6 +51,13 @@ struct PairQuant {
   }
 };
 
+// Bound on the residuals of a group's kept entries; it picks the powers of two that residuals are scaled by.  Half a step, or, where the
+// step is subnormal in fp16 and its rounding leaves the top entries beyond the last code (up to fourteen times that; a step of
+// zero: the whole range), what they lie beyond it; and the rounding of the dequantised value.
+__device__ __forceinline__ float residual_bound(float mn, float mx, float range, float d, float levels) {
+  return fmaxf(0.50390625f * d, fmaf(-levels, d, range)) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
+}
+
 // Entry of the first set bit of L mask bits: bit t of the low / high half of word w stands for entry 2 (16 w + t) / that + 1 of
 // a group whose pairs are rotated by `turn` (a multiple of four).  An entry of the group also if no bit is set (all NaN).
 template <int L>

@@ -334,9 +334,8 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
     if (!kShared || part == 0)
       reinterpret_cast<__half2*>(rec + (SIDE == 0 ? sd.off_kscale : sd.off_vscale))[gi] = __halves2half2(d16, __float2half_rn(mn));
     {
-      // A bound on the group's residuals: half a step for a kept entry, the whole range if the step rounded to zero, plus the
-      // rounding of the dequantised value.  Non-negative floats order like their bit patterns.
-      const float rm = (d != 0.f ? 0.50390625f * d : range) + 2.4e-7f * (fabsf(mn) + fabsf(mx));
+      // Non-negative floats order like their bit patterns.
+      const float rm = residual_bound(mn, mx, range, d, levels);
       const unsigned int wr = __reduce_max_sync(0xffffffffu, __float_as_uint(rm)), ws = __reduce_max_sync(0xffffffffu, __float_as_uint(d)),
                          wd = __reduce_max_sync(0xffffffffu, __float_as_uint(dm));
       if (lane == 0) {

@@ -84,3 +84,48 @@ def test_residuals_that_grow(bits, first):
         _compress(p, k16, v16, 4, 7)
     finally:
         p.close()
+
+
+def _heads_for_ranges(group, blocks_per_tile):
+    """Heads with which a CTA sums two blocks or more of each side, whole pairs of blocks: below one block per SM each has a CTA of
+    its own; from there on two blocks of 64 tokens, one of 128, until four (two) CTAs per SM are used up."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return (sms if group == 64 else 4 * sms) // blocks_per_tile + 1
+
+
+@pytest.mark.parametrize("group,s_pct,blocks", [(64, 2.0, 34), (64, 0.0, 34), (128, 2.0, 16), (128, 0.0, 16)])
+def test_steps_that_are_subnormal_behind_blocks_of_equal_entries(group, s_pct, blocks):
+    """A range of 16 to 22 units of 2^-24 has a step of one unit at 4 bits, so that the top entries lie up to seven steps beyond the
+    last code; the blocks in front of such blocks have no residual, so that the sums are scaled for the rounding of their zero
+    point alone, 2^-35.  fp16 does not span the two."""
+    import torch
+    from paper_2403_05527_b200 import binding as G
+    from tests.gear_harness import Pair, rel_max
+    H, n = _heads_for_ranges(group, blocks), group * blocks
+    p = Pair(34, 1, H, H, 4, group, s_pct, 64, 0, n + 128, r_max=4)
+    try:
+        gen = np.random.default_rng(group)
+        top = gen.integers(16, 23, (2, 1, H, blocks // 2, 1, 1))
+        x = gen.integers(0, top + 1, (2, 1, H, blocks // 2, group, 128))
+        x[0][..., :3, :], x[0][..., 3:6, :] = 0, top[0]                 # three of either end in every group: two leave it at most
+        values = x[1].reshape(1, H, blocks // 2, group, 128 // group, group)
+        values[..., :3], values[..., 3:6] = 0, top[1][..., None]
+        flat = np.zeros_like(x)
+        units = 1500 + np.stack([flat, x], 4).reshape(2, 1, H, n, 128)  # all of them below 2^-13: spaced 2^-24
+        k16, v16 = (units * 2.0 ** -24).astype(np.float16)
+        b0 = gen.standard_normal((1, H, 2, 128, 4)).astype(np.float32)
+        p.oracle.compress(k16, v16, 4, b0)
+        G.gear_compress(p.cache, None, torch.from_numpy(k16).cuda(), torch.from_numpy(v16).cuda(), n, 4, torch.from_numpy(b0).cuda())
+        torch.cuda.synchronize()
+        assert G.gear_last_device_status(p.cache) == 0
+        p.check_segment(0, tol=1.0)     # codes, scales, outliers; the factors as stored are themselves of a few units of fp16
+        for side in "KV":
+            a, b = (G.gear_export(p.cache, 0, f"{side}_{w}_FP32", 1, H)[0].astype(np.float64) for w in "AB")
+            for h in range(H):
+                t = p.oracle.segments[0][side][0][h]
+                assert rel_max(a[h] @ b[h].T, t["A"] @ t["B"].T) <= 1e-3
+        p.oracle = p.with_stored_factors()
+        p.check_attention(tol=1e-4)
+    finally:
+        p.close()
