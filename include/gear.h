@@ -302,7 +302,8 @@ gear_status gear_fp16_attn_status(void* scratch, int32_t* code);
 gear_status gear_fp16_attn_static_status(int32_t* code);
 /* Test only: while `on`, every decode call on the cache first waits, with a limit of a few dozen polls, on a
  * barrier that nothing completes, so that the give-up path runs: the kernel drains its copies, records
- * GEAR_ERR_TIMEOUT and returns.  Nothing faults, traps or hangs. */
+ * GEAR_ERR_TIMEOUT and returns.  So do, behind their last blocks, the kernels that quantize a prompt whose
+ * residual is not kept.  Nothing faults, traps or hangs. */
 gear_status gear_test_dead_wait(gear_cache* cache, int32_t on);
 
 const char* gear_strerror(gear_status s);

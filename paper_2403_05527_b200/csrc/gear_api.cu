@@ -196,7 +196,7 @@ struct gear_cache {
   // cached launch plan of the decode kernel (depends on the segments' shapes)
   long long plan_key; int plan_occ;
   DecodeArgs plan;
-  int test_dead_wait;            // gear_test_dead_wait: the next decode calls wait on a barrier nothing completes
+  int test_dead_wait;            // gear_test_dead_wait: the next decode and compress calls wait on a barrier nothing completes
   int max_queries, units_alloc;  // query rows per head the scratch was sized for; units of that size
   CallOrder::Write seg_write, buf_write;   // the last calls that wrote the segments (records, descriptors) and the buffer rows
 };
@@ -479,7 +479,7 @@ static gear_status compress_segment(gear_cache* c, const void* K, const void* V,
   job.K = (const __half*)K; job.V = (const __half*)V; job.B0 = B0;
   job.dbgA = dbgA; job.dbgB = dbgB;
   job.seed = c->cfg.seed; job.segment_index = (int)c->segs.size(); job.iters = c->cfg.power_iters;
-  job.sms = c->sm_count; job.status = c->status;
+  job.sms = c->sm_count; job.status = c->status; job.test_dead_wait = c->test_dead_wait;
 
   const CallOrder::Key key = order_key(st);
   const uint64_t begun = g_order.begin();

@@ -393,6 +393,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
     }
     if (__syncthreads_or(!ok)) {              // every thread has read the block
       if (tid == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
+      bar_wait(&full, feed.parity ^ 1u);       // the copy lands before its memory goes (bounded)
       break;
     }
     if (tid == 0 && item + (int)gridDim.x < feed.total) feed.request(item + gridDim.x);
@@ -673,6 +674,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
     }
     if (__syncthreads_or(!ok)) {                    // every thread has read the block
       if (tid == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
+      bar_wait(&full, feed.parity ^ 1u);       // the copy lands before its memory goes (bounded)
       break;
     }
     if (tid == 0 && item + (int)gridDim.x < feed.total) feed.request(item + gridDim.x);
@@ -1594,6 +1596,7 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
   ca.seg = sd; ca.cc = job.cc; ca.arena = job.arena; ca.bh0 = bh0;
   ca.K = pa.K; ca.V = pa.V;
   ca.R = pa.R; ca.Rmax = pa.Rmax; ca.status = job.status; ca.Gpart = pa.Gpart; ca.Gexp = pa.Gexp;
+  ca.test_dead_wait = job.test_dead_wait;
   const int kneed = sd.k_k > job.cc.k_v ? sd.k_k : job.cc.k_v;
   const bool per_vector = sd.csr_base16 != 0;          // keys: one group per channel over the whole segment
   ca.side0 = per_vector ? 1 : 0;

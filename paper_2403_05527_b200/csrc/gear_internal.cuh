@@ -50,6 +50,7 @@ struct CompressArgs {
   int* status;          // the cache's status word
   float* Gpart;         // quant_gram_kernel: see PiArgs
   int* Gexp;
+  int test_dead_wait;   // test only: quant_gram_kernel waits behind a CTA's last block for a copy that nothing requests, with a short limit
 };
 
 // Key side of a segment with per-vector grouping (gear_kcvt.cu)
@@ -109,6 +110,7 @@ struct CompressJob {
   int iters;
   int sms;
   int* status;
+  int test_dead_wait;   // see CompressArgs
 };
 
 size_t compress_workspace_bytes(int nbh, const SegDesc& sd, const CacheConst& cc, int sms);

@@ -153,9 +153,9 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 4 ? 3 : 4) pi_codes_pas
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    if (__syncthreads_or(!ok)) {                   // gave up: report, let the other stage's copies land (bounded)
+    if (__syncthreads_or(!ok)) {                   // gave up: report, let the copies of both stages land (bounded)
       if (tid == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
-      if (item + 1 < items) bar_wait(&full[(item + 1) % kCpStages], (uint32_t)((item + 1) / kCpStages) & 1u);
+      for (int i = item; i < items && i < item + kCpStages; ++i) bar_wait(&full[i % kCpStages], (uint32_t)(i / kCpStages) & 1u);
       break;
     }
     float d[NT][4];

@@ -16,10 +16,10 @@ __device__ __forceinline__ void bar_arrive(uint64_t* b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(b)) : "memory");
 }
 // bounded: false when the phase did not complete within the limit
-__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity) {
+__device__ __forceinline__ bool bar_wait(uint64_t* b, uint32_t parity, int limit = kDecodeSpinLimit) {
   uint32_t ok = 0;
 #pragma unroll 1
-  for (int i = 0; i < kDecodeSpinLimit && !ok; ++i)
+  for (int i = 0; i < limit && !ok; ++i)
     asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\nselp.u32 %0, 1, 0, p;\n}"
                  : "=r"(ok) : "r"(smem_addr(b)), "r"(parity), "r"(kWaitHintNs) : "memory");
   return ok != 0;

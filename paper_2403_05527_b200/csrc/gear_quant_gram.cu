@@ -345,7 +345,7 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
       }
     }
     if (__syncthreads_or(!ok)) {                   // every thread has read the block
-      if (tid == 0) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
+      bar_wait(&full, parity ^ 1u);                // gave up, reported below: the copy lands before its memory goes (bounded)
       break;
     }
     if (tid == 0 && it + 1 < count) request(it + 1);
@@ -481,6 +481,7 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
     }
     if (it + 1 == count || blk + 1 == sd.nblk) {   // the tile's last block in this range: leave the partial
       ok = ok && bar_wait(&mma_done, mma_parity);
+      if (p.test_dead_wait && it + 1 == count) ok = bar_wait(&full, parity, 64) && ok;
       tmem_fence_after();
       __syncwarp();
       const size_t at = (size_t)blockIdx.x + bhl + (SIDE == 0 ? 0 : gridDim.x + nbh);
@@ -498,7 +499,8 @@ quant_gram_kernel(CompressArgs p, int nbh, const __grid_constant__ CUtensorMap v
     }
     if (++blk == sd.nblk) { blk = 0; ++bhl; }
   }
-  if (mma_pending) bar_wait(&mma_done, mma_parity);                 // also when a wait gave up: the products end before their operands' memory does
+  if (mma_pending) ok = bar_wait(&mma_done, mma_parity) && ok;      // also when a wait gave up: the products end before their operands' memory does
+  if (!ok) atomicExch(p.status, -7 /* GEAR_ERR_TIMEOUT */);
   tmem_fence_before();
   __syncthreads();
   if (warp == 0) tmem_free<kHeadDim>(tmem);

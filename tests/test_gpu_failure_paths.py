@@ -40,6 +40,26 @@ def test_a_wait_that_runs_out_sets_the_status_word_and_the_cache_recovers():
             p.close()
 
 
+@pytest.mark.parametrize("group,n", [(64, 192), (128, 1024)])
+def test_a_wait_of_a_prompt_that_runs_out_sets_the_status_word(group, n):
+    """The last wait of a kernel: nothing after it looks at the block any more."""
+    import torch
+    from tests.gear_harness import Pair
+    from paper_2403_05527_b200 import binding as G
+    p = Pair(13, 1, 2, 2, 2, group, 2.0, 64, 4, 4096)
+    try:
+        G.gear_test_dead_wait(p.cache, True)
+        p.compress(n, 4)                                        # returns by itself: every wait is bounded
+        assert G.gear_last_device_status(p.cache) == G.GEAR_ERR_TIMEOUT
+        assert G.gear_last_device_status(p.cache) == 0
+        G.gear_test_dead_wait(p.cache, False)
+        p.compress(n, 4, extra=1)
+        assert G.gear_last_device_status(p.cache) == 0
+        p.check_segment(1)
+    finally:
+        p.close()
+
+
 def test_status_word_of_the_fp16_entry_points_is_readable():
     import torch
     from paper_2403_05527_b200 import binding as G, synth
