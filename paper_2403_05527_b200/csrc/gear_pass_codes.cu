@@ -174,12 +174,10 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 4 ? 3 : 4) pi_codes_pas
       const unsigned char* xa = st + (warp * kSlab + gid) * 128 + 8 * (t & 1);     // piece 2 c + t / 2 of row gid, box c / 4
       const int swz = ((t >> 1) ^ gid) << 4;
       const uint4* cw = reinterpret_cast<const uint4*>(st + cs.codes) + warp * (256 * BITS / 16) + lane;
+      uint4 w = make_uint4(0u, 0u, 0u, 0u);        // the codes of 2 F steps
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
-        constexpr int KT = 4 / F;
-        uint4 w4[KT];
-        if (c % (2 * F) == 0) w4[c / (2 * F)] = cw[c / (2 * F) * 32];
-        const uint4 w = w4[c / (2 * F)];
+        if (c % (2 * F) == 0) w = cw[c / (2 * F) * 32];
         const unsigned int wa = (((c & 1) ? w.z : w.x) >> (BITS * (c / 2 % F))) & mask, wc = (((c & 1) ? w.w : w.y) >> (BITS * (c / 2 % F))) & mask;
         const unsigned char* xc = xa + c / 4 * kBoxBytes + (swz ^ (c % 4 << 5));
         const uint2 va = *reinterpret_cast<const uint2*>(xc), vc = *reinterpret_cast<const uint2*>(xc + 8 * 128);
@@ -211,12 +209,11 @@ __global__ void __launch_bounds__(kPassWarps * 32, NT == 4 ? 3 : 4) pi_codes_pas
       const int xrow = 4 * (kp >> 1) + (kp & 1) + 2 * ((mi & 1) ^ (kp >> 2));      // piece 2 c + mi / 2 of this row, box c / 4
       const uint32_t xaddr = smem_addr(st) + (warp * kSlab + xrow) * 128, swz = ((mi >> 1) ^ (xrow & 7)) << 4;
       const unsigned char* cw = st + cs.codes + (warp >> 1) * (512 * BITS) + lane * 16 + 8 * (warp & 1);
+      uint2 w = make_uint2(0u, 0u);                // the codes of F steps
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
-        constexpr int VT = 8 / F;
-        uint2 w2[VT];
-        if (c % F == 0) w2[c / F] = *reinterpret_cast<const uint2*>(cw + c / F * 512);
-        const unsigned int w0 = (w2[c / F].x >> (BITS * (c % F))) & mask, w1 = (w2[c / F].y >> (BITS * (c % F))) & mask;
+        if (c % F == 0) w = *reinterpret_cast<const uint2*>(cw + c / F * 512);
+        const unsigned int w0 = (w.x >> (BITS * (c % F))) & mask, w1 = (w.y >> (BITS * (c % F))) & mask;
         const int g = c * 16 / (kHeadDim / NGV);
         uint32_t x[4], fh[4], fl[4];
         asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
