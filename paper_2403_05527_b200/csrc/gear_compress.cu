@@ -325,8 +325,9 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
   const bool active = L < kHeadDim || SIDE == 0 || tid < T;         // a thread per group
   BlockFeed feed{tile, &full, side == 0 ? p.K : p.V, sd.n_c, sd.nblk, T, sd.nblk * nbh, 0u};
   // The values' CTAs run beside the keys' and wait at their end (see quant_gram_kernel); without keys in front of them (per-vector
-  // key groups) the kernel in front may be the one that writes V.
-  if (SIDE == 0 || p.side0 == 1) after_previous();
+  // key groups) the kernel in front may be the one that writes V, and the keys' kernel starts at their end (launch_kcvt_keys).
+  if (SIDE == 0) after_previous();
+  else if (p.side0 == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
   else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;
@@ -500,7 +501,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
       }
     }
   }
-  if (SIDE == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (SIDE == 1) after_previous();
 }
 
 // ---------------------------------------------------------------------------
@@ -560,8 +561,9 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
   const int tid = threadIdx.x;
   BlockFeed feed{tile, &full, SIDE == 0 ? p.K : p.V, sd.n_c, sd.nblk, T, sd.nblk * nbh, 0u};
   // The values' CTAs run beside the keys' and wait at their end (see quant_gram_kernel); without keys in front of them (per-vector
-  // key groups) the kernel in front may be the one that writes V.
-  if (SIDE == 0 || p.side0 == 1) after_previous();
+  // key groups) the kernel in front may be the one that writes V, and the keys' kernel starts at their end (launch_kcvt_keys).
+  if (SIDE == 0) after_previous();
+  else if (p.side0 == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
   else asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     dmax_bits = 0u; smax_bits = 0u; rmax_bits = 0u;
@@ -789,7 +791,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, kFast2Len)) quant_
       }
     }
   }
-  if (SIDE == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (SIDE == 1) after_previous();
 }
 
 // ---------------------------------------------------------------------------
@@ -1607,9 +1609,13 @@ cudaError_t compress_range(const CompressJob& job, int bh0, int nbh, unsigned ch
     if (e == cudaSuccess) e = launch_pass_codes(pa, st);             // A0 = R B; for ranks up to 8 also A0^T A0
     if (e != cudaSuccess) return e;
   } else {
-    // Launches that overlap pay where they are short (256 tokens x 32 heads, us without and with: groups of 16 68.4 / 58.5, of 32 63.9 / 53.2,
-    // per-vector keys 93.0 / 86.6; one head of 4096 75.5 / 68.6, 70.8 / 66.8, 124 / 114) and without a low-rank part (128 heads x 4096 120 /
-    // 110); long chains over a kept residual run 1 to 7 % longer with them (4096 tokens x 32 heads 214.7 / 226.3, 167.7 / 174.0, 265 / 275).
+    // Launches that overlap pay where they are short (256 tokens x 32 heads, us without and with: groups of 16 66.3 / 59.2, of 32 61.9 / 53.8,
+    // per-vector keys 91.1 / 86.0; one head of 4096 77.6 / 68.9, 72.5 / 67.4, 125.8 / 112.4) and without a low-rank part (128 heads x 4096
+    // 120 / 110).  Over a kept residual the two cross between 12288 rows (384 tokens x 32 heads 76.7 / 68.5, 70.5 / 61.4, 101.8 / 97.1) and
+    // 32768 (1024 x 32 100.9 / 103.7, 86.8 / 86.6; four heads of 8192 121.8 / 131.7, 107.6 / 116.8), at 16384 by shape and group
+    // (512 x 32 78.1 / 81.7, 69.9 / 64.8, 102.3 / 101.6; 1024 x 16 77.5 / 77.7, 69.9 / 63.6, 96.6 / 91.7; 4096 x 4 82.2 / 84.9, 73.9 /
+    // 75.8, 125.0 / 124.5), and long chains run 4 to 9 % longer (4096 x 32 215 / 227, 167 / 175): all of it the early start of the kernel
+    // that sums the partials of R^T R.  What follows that kernel overlaps always.
     const bool overlap = sd.rank == 0 || (long long)nbh * sd.n_c <= 16384;
     int n_quant = 0;
     e = job.cc.bits == 2 ? launch_quant<2>(ca, nbh, kneed, job.sms, overlap, st, &n_quant)

@@ -494,7 +494,10 @@ size_t kcvt_workspace_bytes(int nbh, int n_c, int csr_k) {
   return (size_t)nbh * n_c * kHeadDim + (size_t)nbh * kHeadDim * csr_k * 4 + (size_t)nbh * kHeadDim * 4 + 256;
 }
 
-// Key side of a per-vector segment for the (batch, head) range of `a`; three launches.
+// Key side of a per-vector segment for the (batch, head) range of `a`; three launches.  Where they overlap, the select kernel may start
+// when the values' CTAs end: those that came beside running ones shared SMs two by two while others fell idle (us, from the start / from
+// the end, 4 bits without a low-rank part: three heads of 3072 tokens 62.4 / 47.2, four of 2560 56.7 / 45.2, eight of 4096 66.8 / 58.4;
+// rank 4: three heads of 3072 128.2 / 107.4; nine heads of 4096 67.4 / 69.5; at 1024 tokens and less, or one head, as before).
 cudaError_t launch_kcvt_keys(KcvtArgs a, int nbh, int bits, unsigned char* ws, bool overlap, cudaStream_t st) {
   const SegDesc& sd = a.seg;
   a.codes8 = ws;

@@ -27,6 +27,20 @@ def test_factors_match_the_oracle(B, H, n, bits, group, rank, iters):
         p.close()
 
 
+@pytest.mark.parametrize("group,n", [(32, 2048), (32, 2080), (0, 2048), (0, 2112)])
+def test_rows_on_both_sides_of_the_line_between_launches_that_overlap(group, n):
+    """A kept residual: up to 16384 rows every launch of the chain may start early, above that the last ones."""
+    from tests.gear_harness import Pair
+    p = Pair(17, 1, 8, 8, 4, group, 2.0, 64, 4, n + 128)
+    try:
+        p.compress(n, 4)
+        p.check_segment(0)
+        p.oracle = p.with_stored_factors()
+        p.check_attention(tol=1e-4)
+    finally:
+        p.close()
+
+
 def test_residuals_of_zeros_and_of_rank_one():
     """Entries on the quantization grid leave no residual (factors zero); a column off the grid leaves a residual of rank
     one, of which a rank-4 fit must reproduce exactly that and invent nothing."""
