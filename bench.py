@@ -406,7 +406,7 @@ def compress_roofline(w, res, peak):
     in_bytes = 2 * B * H * w.n * 128 * 2
     pre_ms = statistics.median(res["compress_ms"])
     pre_alg = in_bytes + res["prefill_out_bytes"]
-    out = {"prefill": {"bound": "hbm", "kernel": "Filter/Quant kernel of the group shape (quant_fast*_kernel, quant_pack_kernel, kcvt_*) + pi_pass_kernel (dominant)", "ms": pre_ms,
+    out = {"prefill": {"bound": "hbm", "kernel": ("quant_gram_kernel + pi_codes_pass_kernel" if w.group else "kcvt_select_kernel, quant_fast2_kernel, pi_gram_kernel, pi_pass_kernel") + " (dominant)", "ms": pre_ms,
                        "input_gbs": in_bytes / (pre_ms * 1e-3) / 1e9, "algorithmic_bytes": pre_alg,
                        "achieved": pre_alg / (pre_ms * 1e-3) / 1e9, "peak": peak, "unit": "GB/s",
                        "frac": pre_alg / (pre_ms * 1e-3) / 1e9 / peak}}

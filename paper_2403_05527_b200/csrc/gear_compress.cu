@@ -288,7 +288,9 @@ __global__ void __launch_bounds__(128) quant_pack_kernel(CompressArgs p) {
 // scalar arithmetic and a residual staged through shared memory (2 bits, 8 x 32 heads x 4096): keys 181 -> 153 us, values
 // 261 -> 168 us; 4 bits, 16 x 40 heads x 8192: 469 -> 415 and 652 -> 434 us.  Against quant_pack_kernel (8 x 32 heads x 4096,
 // keys / values): groups of 32 283 / 298 -> 165 / 175 us, of 64 without outliers 266 / 299 -> 150 / 159, of 128 with one
-// outlier 581 / 604 -> 172 / 169, without 441 / 480 -> 146 / 162, values of per-vector keys 517 -> 209.
+// outlier 581 / 604 -> 172 / 169, without 441 / 480 -> 146 / 162, values of per-vector keys 517 -> 209.  All with the residual
+// stored; key blocks of 64 and 128 tokens with value groups as long come here without a low-rank part only (quant_gram_kernel
+// takes the others), where it is not.
 // ---------------------------------------------------------------------------
 constexpr int kCodePitchK = kHeadDim + 4;   // bytes per token row of the key codes  [token][channel]
 // CTAs per SM.  L = 64 (128 registers): five or six are slower, keys 153 -> 166 -> 196 us, values 168 -> 169 -> 171 (8 x 32 heads
@@ -511,7 +513,7 @@ __global__ void __launch_bounds__(128, fast_ctas_per_sm(SIDE, L)) quant_fast_ker
 // below / equal to the second smallest) are found as bit masks, which give the two filtered entries per side in
 // (value, index) order.  A group in which the two sides would share an entry (nearly constant groups) takes the
 // general routine instead.  Same binary32 sequence per entry as everywhere else.  Bound and layout as above (2 bits, 4 x 8
-// heads x 32768: keys 279 -> 204 us, values 290 -> 184 us).
+// heads x 32768 with the residual stored: keys 279 -> 204 us, values 290 -> 184 us; today that is the values of per-vector keys alone).
 // ---------------------------------------------------------------------------
 constexpr int kFast2Len = 128;
 constexpr int kCodePitch2 = kFast2Len + 4;
